@@ -86,13 +86,20 @@ extern "C" {
                                  n >= 14 and reps >= 2 write layers 1..min(4, reps - 1)
                                  from contracted tables of those matrices (a write-only pass per state)
                                  instead of running their tile passes.  Same results up to FP32 rounding;
-                                 the last layer always runs as tile passes. */
+                                 the last layer always runs as tile passes.
+                                 At 0, evaluations of a diagonal H (gvqe_energy, gvqe_energy_grad, parameter
+                                 shift, staged batches) whose CNOTs cross the middle of the register at most
+                                 six times in all (linear, full, reverse linear, pairwise: once per layer;
+                                 circular, SCA: twice) are taken from the circuits of its two halves, with no
+                                 2^n state at all (FP32 from 14 qubits, FP64 from 10 to 28); any other value
+                                 keeps them on stored states.  Same results up to rounding in either precision. */
 #define GVQE_OPT_MPS_TENSOR 6 /* closed-form layers at bond dimension 16 (four closed-form layers): 0 = auto
                                  (the writer's product per 2^13-amplitude chunk, 128 x 16 x 64, and the
                                  gradient pass's two lambda contractions, 64 x 128 x 16 and 128 x 64 x 16, on
                                  the tensor cores as tcgen05 TF32 MMAs with every operand split into two TF32
-                                 parts, FP32 accumulators), -1 = both on the FP32 pipe.  Same results up to
-                                 FP32 rounding. */
+                                 parts, FP32 accumulators), -1 = both on the FP32 pipe, which also keeps
+                                 FP32 evaluations off the two-half form, whose contraction runs on the tensor
+                                 cores.  Same results up to FP32 rounding. */
 
 /* gate sets of a rotation layer (Eq. 8).
  * RY:    RY on every qubit; P = n (reps+1), theta[r*n + q]; real amplitudes.
@@ -225,8 +232,9 @@ int gvqe_batch_run(gvqe_batch b, const double *const *params, const uint8_t *con
  *     states, partial sums and diagonal tables sit job after job, and each
  *     group runs its plan's passes as launches of the regular pass kernels over
  *     all its jobs (as gvqe_energy_grad runs a batch of vectors), on its own
- *     branch of the graph; the branches run side by side.  Results equal those
- *     of single gvqe_energy_grad calls bit for bit, and every instance with RY
+ *     branch of the graph; the branches run side by side (the instances evaluated
+ *     from their halves share their launches instead, see GVQE_OPT_MPS_LAYERS).
+ *     Results equal those of single gvqe_energy_grad calls bit for bit, and every instance with RY
  *     layers and a diagonal H takes part, whatever its n.
  *     GVQE_BATCH_PERSISTENT: one persistent launch whose CTAs claim items
  *     (one 2^tile-bits tile of one pass) in ticket order and wait, with a

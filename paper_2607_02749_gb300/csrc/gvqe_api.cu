@@ -1312,6 +1312,81 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
   return GVQE_OK;
 }
 
+// ------------------------------------------------- two-half evaluation --
+// A diagonal H and RY layers whose crossing CNOTs leave at most 64 terms: the state is
+// never stored (gvqe_cut.cuh).  GVQE_OPT_MPS_LAYERS other than 0 and GVQE_OPT_MPS_TENSOR = -1
+// name the other evaluations.  FP64 runs on the FP64 pipe: 2 D multiply-adds per amplitude
+// and contraction against about 2 per gate and sweep of the tile passes.
+gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec) {
+  if (a->gates != 1 || a->mps != 0 || (!prec && a->mps_tc != 0)) return nullptr;
+  gvqe_cut_plan &c = a->cut[prec];
+  if (!c.known) {
+    c.ok = cut_build(a->n, a->reps, a->ent, prec, &c.d) && (!prec || c.d.D <= a->n * a->reps);
+    c.known = true;
+  }
+  return c.ok ? &c : nullptr;
+}
+
+int gvqe::cut_upload(gvqe_cut_plan *c) {
+  if (c->dev.ptr) return GVQE_OK;
+  PendingBuf guard(c->dev);
+  GV_TRY(c->dev.reserve(sizeof(CutDesc)));
+  GV_CUDA(cudaMemcpy(c->dev.ptr, &c->d, sizeof(CutDesc), cudaMemcpyHostToDevice));
+  guard.done = true;
+  return GVQE_OK;
+}
+
+int gvqe::ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool grad, cudaStream_t s) {
+  GV_TRY(ensure_tables(h, prec, s));
+  if (prec || !grad || h->T32t.ptr) return GVQE_OK;
+  PendingBuf guard(h->T32t);
+  GV_TRY(h->T32t.reserve(((size_t)1 << h->n) * 4));
+  GV_CUDA(launch_transpose_table({(const float *)h->T32.ptr, (float *)h->T32t.ptr, d.half[0].m, d.half[1].m}, s));
+  GV_CUDA(cudaStreamSynchronize(s));
+  guard.done = true;
+  return GVQE_OK;
+}
+
+static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, const void *cs, const uint8_t *mask,
+                   int batch, double *E, double *grad, int prec, cudaStream_t s) {
+  GV_TRY(cut_upload(c));
+  const int P = a->n * (a->reps + 1);
+  CutArgs A;
+  memset(&A, 0, sizeof(A));
+  A.job0.lay = cut_layout(c->d, prec, grad != nullptr);
+  const size_t per_job = (size_t)A.job0.lay.total;
+  size_t freeb = 0, total = 0;
+  GV_CUDA(cudaMemGetInfo(&freeb, &total));
+  size_t have = freeb + a->ws.bytes;
+  const long long left = budget_left();
+  if (left >= 0) have = std::min(have, (size_t)left + a->ws.bytes);
+  if (per_job > have)
+    return fail(GVQE_ENOMEM, "one evaluation needs %.3f GiB of workspace, %.3f GiB available", per_job / 1073741824.0,
+                have / 1073741824.0);
+  // as many vectors per launch as 4 GiB hold: far more than fill the GPU
+  const size_t cap = std::max(per_job, std::min(have, (size_t)4 << 30));
+  const int J = (int)std::min<size_t>((size_t)batch, cap / per_job);
+  GV_TRY(a->ws.reserve(per_job * (size_t)J));
+  A.job0.desc = (const CutDesc *)c->dev.ptr;
+  A.job0.table = prec ? h->T64.ptr : h->T32.ptr;
+  A.job0.table_t = prec ? nullptr : h->T32t.ptr;
+  A.job0.ws = (char *)a->ws.ptr;
+  A.ws_stride = (long long)per_job;
+  A.cs_stride = (long long)P * (prec ? 16 : 8);
+  A.P = P;
+  for (int j0 = 0; j0 < batch; j0 += J) {
+    A.njobs = std::min(J, batch - j0);
+    A.job0.cs = (const char *)cs + (long long)j0 * A.cs_stride;
+    A.job0.mask = mask ? mask + (size_t)j0 * P : nullptr;
+    A.job0.E = E + j0;
+    A.job0.grad = grad ? grad + (size_t)j0 * P : nullptr;
+    int nl = 0;
+    GV_CUDA(launch_cut(prec, A, CutGrid{c->d.half[0].m, c->d.D, 0, 0, nullptr, nullptr}, grad != nullptr, s, &nl));
+    count_launches(nl);
+  }
+  return GVQE_OK;
+}
+
 static bool is_ham(const void *p) { return p && ((const gvqe_hamiltonian_s *)p)->magic == MAGIC_HAM; }
 static bool is_ansatz(const void *p) { return p && ((const gvqe_ansatz_s *)p)->magic == MAGIC_ANSATZ; }
 
@@ -1327,6 +1402,14 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
                       double *E, double *grad, int prec, cudaStream_t s) {
   const bool cplx = a->gates == 2;
   const bool diag = cplx ? h->cgm.empty() : h->gm.empty();
+  if (gvqe_cut_plan *c = diag ? get_cut(a, prec) : nullptr) {
+    GV_TRY(ensure_cut_tables(h, prec, c->d, grad != nullptr, s));
+    const long long count = (long long)batch * a->n * (a->reps + 1);
+    GV_TRY(a->aux.reserve((size_t)count * (prec ? 16 : 8)));
+    GV_CUDA(launch_trig(prec, params, count, a->aux.ptr, s));
+    count_launches(1);
+    return run_cut(a, h, c, a->aux.ptr, mask, batch, E, grad, prec, s);
+  }
   GV_TRY(ensure_tables(h, prec, s, cplx));
   Plan *pl = get_plan(a, prec, grad != nullptr, diag);
   const int P = pl->P;
@@ -1847,6 +1930,12 @@ int gvqe_ansatz_describe(gvqe_ansatz a, int flags, char *buf, int buflen) {
     return fail(GVQE_EINVAL, "tile bits %d too large", eff_tile_bits(a, prec));
   const Plan *pl = get_plan(a, prec, true, true);
   std::string s = describe_plan(*pl);
+  if (const gvqe_cut_plan *c = get_cut(a, prec)) {
+    char line[160];
+    snprintf(line, sizeof(line), "diagonal H: evaluated from the halves [0,%d) and [%d,%d), %d terms%s\n", c->d.half[1].q0,
+             c->d.half[1].q0, a->n, c->d.D, prec ? "" : " (tensor cores, TF32 split)");
+    s += line;
+  }
   if (!a->tune_report.empty()) s += a->tune_report;
   if (buf && buflen > 0) {
     const size_t m = std::min<size_t>((size_t)buflen - 1, s.size());
@@ -1865,6 +1954,7 @@ int gvqe_destroy(void *handle) {
     gvqe_hamiltonian_s *h = (gvqe_hamiltonian_s *)handle;
     h->T64.release();
     h->T32.release();
+    h->T32t.release();
     h->G.release();
     h->magic = 0;
     delete h;
@@ -1879,6 +1969,7 @@ int gvqe_destroy(void *handle) {
     a->ro.release();
     a->tune.release();
     for (auto &kv : a->plans) kv.second.d_dir.release();
+    for (auto &c : a->cut) c.dev.release();
     a->magic = 0;
     delete a;
     return GVQE_OK;

@@ -45,13 +45,6 @@ struct BatchStep {
   int n, reps;       // PREP: register size and repetitions
 };
 
-struct BatchIO {
-  const double *params;  // P doubles
-  const uint8_t *mask;   // P bytes or NULL (all active)
-  double *grad;          // P doubles or NULL
-  double *energy;        // one double
-};
-
 struct BatchArgs {
   const BatchStep *steps;
   const unsigned *seg_start;  // first ticket of each step in schedule order
@@ -85,7 +78,7 @@ __device__ void batch_prep(const BatchStep &st, const BatchIO &io) {
     v.y = (T)s;
     cs[p] = v;
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && A.minlayer) {
     int m = st.reps + 1;  // nothing active: no backward pass needed
     if (io.mask == nullptr) {
       m = 0;
@@ -656,6 +649,9 @@ int batch_loop(gvqe_batch_s *b, const double *const *params, const uint8_t *cons
 // graph: a PREP launch (one CTA per job: its cos/sin table and lowest active
 // layer), the plan's passes, and a REDUCE launch (one CTA per job: its energy
 // and gradient into the caller's buffers).  The branches run side by side.
+// Instances with a two-half evaluation (gvqe_cut.cuh) take one branch per number of
+// terms and CTA size instead, whatever their circuits: a PREP launch and the kernels of
+// that evaluation, each over all of the branch's instances, largest first.
 int build_grouped(gvqe_batch_s *b, int want_grad) {
   BatchSchedule &sc = b->sched[want_grad];
   const int prec = b->prec;
@@ -665,8 +661,22 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
   auto A_of = [&](int k) { return b->a[b->pidx[k]]; };
   auto H_of = [&](int k) { return b->h[b->pidx[k]]; };
   std::map<std::vector<int>, std::vector<int>> by_plan;  // plan key -> slots
-  for (int k = 0; k < ni; ++k)
-    by_plan[{A_of(k)->n, A_of(k)->reps, A_of(k)->ent, eff_split(A_of(k), prec)}].push_back(k);
+  struct CutGroup {
+    std::vector<int> slots;
+    CutGrid grid{};
+    std::vector<CutJob> jobs;
+    std::vector<int4> half, con;
+    std::vector<CutDesc> desc;
+    size_t o_jobs, o_half, o_con, o_desc;
+  };
+  std::map<std::pair<int, int>, CutGroup> cuts;  // (terms, threads of a half circuit's CTA)
+  for (int k = 0; k < ni; ++k) {
+    if (const gvqe_cut_plan *c = get_cut(A_of(k), prec)) {
+      cuts[{cut_k(c->d.D), cut_threads(c->d.half[0].m)}].slots.push_back(k);
+    } else {
+      by_plan[{A_of(k)->n, A_of(k)->reps, A_of(k)->ent, eff_split(A_of(k), prec)}].push_back(k);
+    }
+  }
   struct Group {
     std::vector<int> slots;
     Plan plan;
@@ -704,6 +714,47 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     off = up256(off + sizeof(RedEntry) * std::max<size_t>(1, g.plan.dir.size()));
     groups.push_back(std::move(g));
   }
+  // an instance's cos/sin table, then its workspace; FP32 gradients: the transposed
+  // diagonal tables, one per Hamiltonian (one allocation and one launch for all of them)
+  std::vector<size_t> cut_cs(ni, 0);
+  std::map<gvqe_hamiltonian, size_t> cut_tt;
+  std::vector<TransposeJob> tjobs;
+  for (auto &kv : cuts) {
+    CutGroup &g = kv.second;
+    std::stable_sort(g.slots.begin(), g.slots.end(), [&](int x, int y) { return A_of(x)->n > A_of(y)->n; });
+    for (int k : g.slots) {
+      const CutDesc &d = get_cut(A_of(k), prec)->d;
+      const int j = (int)g.jobs.size();
+      CutJob job{};
+      job.lay = cut_layout(d, prec, want_grad != 0);
+      cut_cs[k] = off;
+      off = up256(off + (size_t)d.n * (d.reps + 1) * 2 * es);
+      off = up256(off + (size_t)job.lay.total);
+      if (!prec && want_grad && cut_tt.find(H_of(k)) == cut_tt.end()) {
+        cut_tt[H_of(k)] = off;
+        off = up256(off + ((size_t)1 << d.n) * 4);
+      }
+      g.desc.push_back(d);
+      g.grid.m0 = std::max(g.grid.m0, d.half[0].m);
+      g.grid.D = std::max(g.grid.D, d.D);
+      for (int h = 0; h < 2; ++h) {
+        for (int a = 0; a < d.D; ++a) g.half.push_back(make_int4(j, h, a, 0));
+        if (h == 0 || want_grad)
+          for (int i = 0; i < job.lay.rb[h] * job.lay.ns[h]; ++i) g.con.push_back(make_int4(j, h, i, 0));
+      }
+      g.jobs.push_back(job);
+    }
+    g.o_jobs = off;
+    off = up256(off + sizeof(CutJob) * g.jobs.size());
+    g.o_half = off;
+    off = up256(off + sizeof(int4) * g.half.size());
+    g.o_con = off;
+    off = up256(off + sizeof(int4) * g.con.size());
+    g.o_desc = off;
+    off = up256(off + sizeof(CutDesc) * g.desc.size());
+  }
+  const size_t o_tj = off;
+  off = up256(off + sizeof(TransposeJob) * std::max<size_t>(1, cut_tt.size()));
   // larger groups first: their longer chains of passes start early
   std::stable_sort(groups.begin(), groups.end(), [](const Group &x, const Group &y) {
     return x.slots.size() * (size_t)x.plan.state_elems * x.plan.steps.size() >
@@ -747,12 +798,63 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     if (!g.plan.dir.empty())
       GB_CUDA(cudaMemcpy(base + g.o_dir, g.plan.dir.data(), sizeof(RedEntry) * g.plan.dir.size(), cudaMemcpyHostToDevice));
   }
+  std::map<gvqe_hamiltonian, const void *> done_tt;
+  for (auto &kv : cuts) {
+    CutGroup &g = kv.second;
+    for (size_t j = 0; j < g.slots.size(); ++j) {
+      const int k = g.slots[j];
+      const CutDesc &d = g.desc[j];
+      const size_t cs_bytes = (size_t)d.n * (d.reps + 1) * 2 * es;
+      CutJob &job = g.jobs[j];
+      job.desc = (const CutDesc *)(base + g.o_desc) + j;
+      job.cs = base + cut_cs[k];
+      job.table = prec ? H_of(k)->T64.ptr : H_of(k)->T32.ptr;
+      const auto tt = cut_tt.find(H_of(k));
+      if (tt != cut_tt.end()) {
+        job.table_t = base + tt->second;
+        tjobs.push_back({(const float *)job.table, (float *)(base + tt->second), d.half[0].m, d.half[1].m});
+        cut_tt.erase(tt);
+        done_tt[H_of(k)] = job.table_t;
+      } else if (!prec && want_grad) {
+        job.table_t = done_tt[H_of(k)];
+      }
+      job.ws = base + up256(cut_cs[k] + cs_bytes);
+      job.io = (const BatchIO *)(base + o_io) + k;
+      BatchStep &pr = steps[2 * (size_t)k];
+      pr = BatchStep{};
+      pr.kind = S_PREP;
+      pr.inst = k;
+      pr.dep = -1;
+      pr.n = d.n;
+      pr.reps = d.reps;
+      pr.A.P = d.n * (d.reps + 1);
+      pr.A.cs = job.cs;
+    }
+    GB_CUDA(cudaMemcpy(base + g.o_jobs, g.jobs.data(), sizeof(CutJob) * g.jobs.size(), cudaMemcpyHostToDevice));
+    GB_CUDA(cudaMemcpy(base + g.o_half, g.half.data(), sizeof(int4) * g.half.size(), cudaMemcpyHostToDevice));
+    GB_CUDA(cudaMemcpy(base + g.o_con, g.con.data(), sizeof(int4) * g.con.size(), cudaMemcpyHostToDevice));
+    GB_CUDA(cudaMemcpy(base + g.o_desc, g.desc.data(), sizeof(CutDesc) * g.desc.size(), cudaMemcpyHostToDevice));
+    g.grid.half_blocks = (int)g.half.size();
+    g.grid.con_blocks = (int)g.con.size();
+    g.grid.half_items = (const int4 *)(base + g.o_half);
+    g.grid.con_items = (const int4 *)(base + g.o_con);
+  }
+  if (!tjobs.empty()) {
+    GB_CUDA(cudaMemcpy(base + o_tj, tjobs.data(), sizeof(TransposeJob) * tjobs.size(), cudaMemcpyHostToDevice));
+    int nmax = 0;
+    for (const TransposeJob &t : tjobs) nmax = std::max(nmax, t.m0 + t.m1);
+    GB_CUDA(launch_transpose_tables((const TransposeJob *)(base + o_tj), (int)tjobs.size(), nmax, nullptr));
+    GB_CUDA(cudaStreamSynchronize(nullptr));
+  }
   // PREP and REDUCE ids in group order (a launch covers one group's contiguous range)
   std::vector<int> ids;
   for (const Group &g : groups)
     for (int k : g.slots) ids.push_back(2 * k);
   for (const Group &g : groups)
     for (int k : g.slots) ids.push_back(2 * k + 1);
+  const size_t cut_ids = ids.size();
+  for (const auto &kv : cuts)
+    for (int k : kv.second.slots) ids.push_back(2 * k);
   GB_CUDA(cudaMemcpy(base + o_steps, steps.data(), sizeof(BatchStep) * steps.size(), cudaMemcpyHostToDevice));
   GB_CUDA(cudaMemcpy(base + o_ids, ids.data(), sizeof(int) * ids.size(), cudaMemcpyHostToDevice));
   GB_CUDA(cudaMemset(base + o_ctr, 0, sizeof(unsigned) * 2));
@@ -764,7 +866,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
   B.err = (int *)(base + o_ctr + sizeof(unsigned));
   B.io = (const BatchIO *)(base + o_io);
   sc.smem = 0;
-  sc.groups = (int)groups.size();
+  sc.groups = (int)(groups.size() + cuts.size());
   const int *d_ids = (const int *)(base + o_ids);
 
   cudaStream_t cap;
@@ -831,7 +933,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
         A.minlayer = (const int *)(base + g.o_ml);
         le = launch_pass(prec, A, J, 0, gs);
       }
-      if (le == cudaSuccess) le = launch_stage_tb(prec, 12, B, d_ids + ni + first, 1, (unsigned)J, 0, gs);
+      if (le == cudaSuccess) le = launch_stage_tb(prec, 12, B, d_ids + cut_ids / 2 + first, 1, (unsigned)J, 0, gs);
       cudaEvent_t join = nullptr;
       if (le == cudaSuccess) le = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
       if (le == cudaSuccess) {
@@ -840,6 +942,39 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
       }
       if (le == cudaSuccess) le = cudaStreamWaitEvent(cap, join, 0);
       first += (size_t)J;
+    }
+    if (le == cudaSuccess && !cuts.empty()) {
+      cudaEvent_t cfork = nullptr;
+      le = cudaEventCreateWithFlags(&cfork, cudaEventDisableTiming);
+      if (le == cudaSuccess) {
+        evs.push_back(cfork);
+        le = cudaEventRecord(cfork, cap);
+      }
+      size_t at = cut_ids;
+      for (auto &kv : cuts) {
+        if (le != cudaSuccess) break;
+        const CutGroup &g = kv.second;
+        const unsigned J = (unsigned)g.slots.size();
+        cudaStream_t gs = nullptr;
+        le = cudaStreamCreateWithFlags(&gs, cudaStreamNonBlocking);
+        if (le != cudaSuccess) break;
+        streams.push_back(gs);
+        le = cudaStreamWaitEvent(gs, cfork, 0);
+        if (le == cudaSuccess) le = launch_stage_tb(prec, 12, B, d_ids + at, 1, J, 0, gs);
+        at += J;
+        CutArgs A{};
+        A.jobs = (const CutJob *)(base + g.o_jobs);
+        A.njobs = (int)J;
+        int nl = 0;
+        if (le == cudaSuccess) le = launch_cut(prec, A, g.grid, want_grad != 0, gs, &nl);
+        cudaEvent_t join = nullptr;
+        if (le == cudaSuccess) le = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+        if (le == cudaSuccess) {
+          evs.push_back(join);
+          le = cudaEventRecord(join, gs);
+        }
+        if (le == cudaSuccess) le = cudaStreamWaitEvent(cap, join, 0);
+      }
     }
     e = cudaStreamEndCapture(cap, &sc.graph);
     if (e == cudaSuccess) e = le;

@@ -1,0 +1,404 @@
+// gvqe_cut_tc.cu -- the FP32 contraction of the two half tables on the tensor cores.
+//
+// An item is 128 rows of one half (i) against a run of the other half's columns (j), in
+// tiles of 64 columns.  Per tile, with K terms (16, 32 or 64):
+//   S(i, j) = sum_a A(i, a) B(j, a)            128 x K by K x 64
+//   lambda = E(i, j) S                         on the FP32 pipe, S read from tensor memory
+//   G(i, a) += sum_j lambda(i, j) B(j, a)      128 x 64 by 64 x K
+// as tcgen05.mma kind::tf32 with FP32 accumulators.  Every operand is split into two
+// TF32 parts (x_hi rounded to nearest, x_lo = x - x_hi exactly, its last bits cut by the
+// tensor core: about 2^-22 of x), and each product is x_lo y_hi + x_hi y_lo + x_hi y_hi,
+// the small parts first so that they meet a small accumulator.  The accumulators round
+// toward zero, so G is taken out after every tile (8 full-size steps) and summed on the
+// FP32 pipe.
+//
+// Both A operands (the rows, and lambda) sit in tensor memory: lambda never touches shared
+// memory, its high part overwrites S in place, and the MMAs read only B from shared
+// memory (64 bytes per clock of its 128).  B comes in ready-made operand images
+// (k_cut_fwd) by one bulk copy per tile.  Warps 0-3 and 4-7 take alternate tiles, a row
+// per thread; warp 8 copies, warp 9 issues the MMAs.  E is read straight into registers
+// one tile ahead, lanes along i (for the second contraction from its transposed copy).
+//
+// What bounds it: at K = 64 the MMAs (768 multiply-adds per amplitude over the two
+// contractions); at K = 16 the FP32 pipe's nine instructions per amplitude.
+#include "gvqe_cut.cuh"
+
+namespace gvqe {
+namespace {
+
+constexpr int NT = 320;
+constexpr int COLS = 64;
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// K-major operand in shared memory, no swizzle: core matrices of 8 rows x 16 bytes, 128
+// bytes apart along K, sbo bytes apart along the rows
+__device__ __forceinline__ uint64_t op_desc(uint32_t addr, uint32_t sbo) {
+  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) |
+         (1ull << 46);
+}
+// FP32 accumulator, TF32 operands, K-major, M = 128
+__host__ __device__ constexpr uint32_t idesc(int N) {
+  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24);
+}
+__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint64_t b, uint32_t id, bool acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+      "r"(a), "l"(b), "r"(id), "r"(acc ? 1 : 0)
+      : "memory");
+}
+__device__ __forceinline__ void commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void ld16(uint32_t ta, float *v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(ta)
+      : "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+__device__ __forceinline__ void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void st16(uint32_t ta, const float *v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+          ta),
+      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+      "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+      : "memory");
+}
+__device__ __forceinline__ void st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// A wait that gives up: after its limit, or once another wait of this CTA has given up
+// (every MMA and copy completes, so neither is expected).
+__device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, volatile int *bad) {
+  uint32_t done = 0;
+  for (int it = 0; it < (1 << 22) && !done; ++it) {
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (!done && *bad) return false;
+  }
+  if (!done) *bad = 1;
+  return done != 0;
+}
+
+__device__ __forceinline__ void two_sum(float &hi, float &lo, float x) {
+  const float s = hi + x, b = s - hi;
+  lo += (hi - (s - b)) + (x - b);
+  hi = s;
+}
+
+template <int K>
+struct Cfg {
+  static constexpr int BUFS = K <= 32 ? 3 : 2;  // S / lambda buffers
+  static constexpr int STAGES = K <= 32 ? 4 : 3;
+  // tensor-memory columns
+  static constexpr int A_HI = 0, A_LO = K, S0 = 2 * K, G0 = S0 + 128 * BUFS;
+  static_assert(G0 + 2 * K <= 512, "tensor memory");
+  static constexpr int PARTS = 64 * K;  // floats of one operand image part
+};
+
+template <int K, bool GRAD>
+__global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
+  using C = Cfg<K>;
+  constexpr int STAGE_F = (GRAD ? 4 : 2) * C::PARTS;
+  extern __shared__ __align__(128) float dyn[];
+  __shared__ __align__(8) unsigned long long bars[2 * C::STAGES + 2 * C::BUFS + 2];
+  __shared__ uint32_t tslot;
+  __shared__ int bad_s;
+  __shared__ double es[2][8];
+  volatile int *bad = &bad_s;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  int job, h, idx;
+  if (A.items) {
+    const int4 it = A.items[blockIdx.x];
+    job = it.x;
+    h = it.y;
+    idx = it.z;
+  } else {  // the vectors of one item next to each other: they read the same part of E
+    job = blockIdx.x % A.njobs;
+    idx = blockIdx.x / A.njobs;
+    h = idx >= A.blk0;
+    if (h) idx -= A.blk0;
+  }
+  const CutJob J = cut_job(A, job);
+  const int mr = J.desc->half[h].m, mc = J.desc->half[1 - h].m, D = J.desc->D;
+  const int ns = J.lay.ns[h], split = idx % ns, row0 = (idx / ns) * 128;
+  const int nt = (1 << (mc - 6)) / ns, t0 = split * nt;
+  const float *ap = reinterpret_cast<const float *>(J.ws + J.lay.pack[h]);
+  const float *bp = reinterpret_cast<const float *>(J.ws + J.lay.pack[1 - h]);
+  const float *E = reinterpret_cast<const float *>(h ? J.table_t : J.table);
+  const uint32_t bar0 = smem_addr(bars);
+  auto full = [&](int s) { return bar0 + 8 * s; };
+  auto empty = [&](int s) { return bar0 + 8 * (C::STAGES + s); };
+  auto sbar = [&](int b) { return bar0 + 8 * (2 * C::STAGES + b); };
+  auto lbar = [&](int b) { return bar0 + 8 * (2 * C::STAGES + C::BUFS + b); };
+  auto gbar = [&](int b) { return bar0 + 8 * (2 * C::STAGES + 2 * C::BUFS + b); };
+  if (w == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(&tslot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 256) {
+    bad_s = 0;
+    for (int s = 0; s < C::STAGES; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full(s)));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(empty(s)));
+    }
+    for (int b = 0; b < C::BUFS; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sbar(b)));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(lbar(b)));
+    }
+    for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(gbar(b)));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = tslot;
+  const int r = 32 * (w & 3) + lane;                       // this thread's row (warps 0-7)
+  const uint32_t tw = tmem + ((uint32_t)(32 * (w & 3)) << 16);  // ... and lane quarter
+  if (w < 4) {
+    // the rows' operand: hi and lo parts into tensor memory
+    const float *src = ap + (size_t)((row0 + r) >> 6) * (256 * K) + ((r & 63) >> 3) * (K * 8) + (r & 7) * 4;
+#pragma unroll
+    for (int c = 0; c < 2 * K; c += 16) {
+      const float *p = src + (c < K ? 0 : C::PARTS) + ((c % K) >> 2) * 32;
+      float v[16];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4 x = *reinterpret_cast<const float4 *>(p + 32 * k);
+        v[4 * k] = x.x;
+        v[4 * k + 1] = x.y;
+        v[4 * k + 2] = x.z;
+        v[4 * k + 3] = x.w;
+      }
+      st16(tw + C::A_HI + c, v);
+    }
+    st_wait();
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+
+  float acc[K];
+  if (w < 8) {
+    // ------------------------------------------------------------ rows --
+    const int g = w >> 2;
+    const float *Ei = E + row0 + r;
+    float e_hi = 0.f, e_lo = 0.f, z_hi = 0.f, z_lo = 0.f;
+    float tv[COLS];
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k] = 0.f;
+    auto load = [&](int t) {
+      const float *p = Ei + ((long long)(t0 + t) << (6 + mr));
+#pragma unroll
+      for (int j = 0; j < COLS; ++j) tv[j] = __ldg(p + ((long long)j << mr));
+    };
+    if (g < nt) load(g);
+    bool ok = true;
+    for (int t = g; t < nt; t += 2) {
+      const int b = t % C::BUFS;
+      ok = wait_bounded(sbar(b), (t / C::BUFS) & 1, bad);
+      if (!ok) break;
+      fence_after();
+      const uint32_t ts = tw + C::S0 + 128 * b;
+      float es_ = 0.f, zs_ = 0.f;
+#pragma unroll
+      for (int c = 0; c < COLS; c += 16) {
+        float v[16], l[16];
+        ld16(ts + c, v);
+        ld_wait();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float lam = v[j] * tv[c + j];
+          es_ = fmaf(lam, v[j], es_);
+          zs_ = fmaf(v[j], v[j], zs_);
+          if constexpr (GRAD) {
+            float hi;
+            asm("cvt.rna.tf32.f32 %0, %1;" : "=f"(hi) : "f"(lam));
+            v[j] = hi;
+            l[j] = lam - hi;
+          }
+        }
+        if constexpr (GRAD) {
+          st16(ts + c, v);
+          st16(ts + 64 + c, l);
+        }
+      }
+      if constexpr (GRAD) st_wait();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) arrive(lbar(b));
+      if (t + 2 < nt) load(t + 2);
+      two_sum(e_hi, e_lo, es_);
+      two_sum(z_hi, z_lo, zs_);
+      if constexpr (GRAD) {
+        ok = wait_bounded(gbar(g), (t >> 1) & 1, bad);
+        if (!ok) break;
+        fence_after();
+#pragma unroll
+        for (int c = 0; c < K; c += 16) {
+          float v[16];
+          ld16(tw + C::G0 + K * g + c, v);
+          ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) acc[c + j] += v[j];
+        }
+        fence_before();
+      }
+    }
+    if (h == 0) {
+      double e = (double)e_hi + e_lo, z = (double)z_hi + z_lo;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        e += __shfl_xor_sync(0xffffffffu, e, o);
+        z += __shfl_xor_sync(0xffffffffu, z, o);
+      }
+      if (lane == 0) {
+        es[0][w] = e;
+        es[1][w] = z;
+      }
+    }
+  } else if (w == 8) {
+    // ---------------------------------------------------------- copies --
+    if (lane == 0) {
+      const float *src = bp + (size_t)t0 * (256 * K);
+      for (int t = 0; t < nt; ++t) {
+        const int s = t % C::STAGES;
+        if (t >= C::STAGES && !wait_bounded(empty(s), (t / C::STAGES - 1) & 1, bad)) break;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(STAGE_F * 4)
+                     : "memory");
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                smem_addr(dyn + s * STAGE_F)),
+            "l"(src + (size_t)t * (256 * K)), "r"(STAGE_F * 4), "r"(full(s))
+            : "memory");
+      }
+      // the last commits have arrived before the CTA leaves
+      for (int t = nt > C::STAGES ? nt - C::STAGES : 0; t < nt; ++t)
+        wait_bounded(empty(t % C::STAGES), (t / C::STAGES) & 1, bad);
+    }
+  } else {
+    // ------------------------------------------------------------ MMAs --
+    if (lane == 0) {
+      bool ok = true;
+      for (int t = 0; t <= nt && ok; ++t) {
+        if (t < nt) {  // S of tile t
+          const int s = t % C::STAGES, b = t % C::BUFS;
+          ok = wait_bounded(full(s), (t / C::STAGES) & 1, bad);
+          // the buffer's previous tile: its lambda has been contracted (or, energies only, read)
+          const int u = t - C::BUFS;
+          if (ok && u >= 0)
+            ok = GRAD ? wait_bounded(gbar(u & 1), (u >> 1) & 1, bad)
+                      : wait_bounded(lbar(b), (u / C::BUFS) & 1, bad);
+          if (!ok) break;
+          fence_after();
+          const uint32_t bs = smem_addr(dyn + s * STAGE_F), d = tmem + C::S0 + 128 * b;
+          const uint64_t bh = op_desc(bs, K * 32), bl = op_desc(bs + C::PARTS * 4, K * 32);
+#pragma unroll
+          for (int k = 0; k < K / 8; ++k) mma(d, tmem + C::A_LO + 8 * k, bh + 16 * k, idesc(COLS), k > 0);
+#pragma unroll
+          for (int k = 0; k < K / 8; ++k) mma(d, tmem + C::A_HI + 8 * k, bl + 16 * k, idesc(COLS), true);
+#pragma unroll
+          for (int k = 0; k < K / 8; ++k) mma(d, tmem + C::A_HI + 8 * k, bh + 16 * k, idesc(COLS), true);
+          commit(sbar(b));
+          if (!GRAD) commit(empty(s));
+        }
+        if (GRAD && t > 0) {  // G of tile t - 1
+          const int u = t - 1, s = u % C::STAGES, b = u % C::BUFS;
+          ok = wait_bounded(lbar(b), (u / C::BUFS) & 1, bad);
+          if (!ok) break;
+          fence_after();
+          const uint32_t bs = smem_addr(dyn + s * STAGE_F) + 2 * C::PARTS * 4;
+          const uint32_t lh = tmem + C::S0 + 128 * b, ll = lh + 64, d = tmem + C::G0 + K * (u & 1);
+          const uint64_t bh = op_desc(bs, 2048), bl = op_desc(bs + C::PARTS * 4, 2048);
+#pragma unroll
+          for (int k = 0; k < COLS / 8; ++k) mma(d, ll + 8 * k, bh + 16 * k, idesc(K), k > 0);
+#pragma unroll
+          for (int k = 0; k < COLS / 8; ++k) mma(d, lh + 8 * k, bl + 16 * k, idesc(K), true);
+#pragma unroll
+          for (int k = 0; k < COLS / 8; ++k) mma(d, lh + 8 * k, bh + 16 * k, idesc(K), true);
+          commit(gbar(u & 1));
+          commit(empty(s));
+        }
+      }
+    }
+  }
+  __syncwarp();
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const bool good = bad_s == 0;
+  // every stage copied has been read: full and empty of the last STAGES tiles are complete
+  // unless a wait gave up, and then the copies in flight are waited for before leaving
+  if (!good && tid == 256) {
+    int dummy = 0;
+    for (int s = 0; s < C::STAGES; ++s)
+      for (int p = 0; p < 2; ++p) wait_bounded(full(s), p, &dummy);
+  }
+  if constexpr (GRAD) {
+    // rows' sums of the two warp groups, through shared memory (all copies are consumed)
+    if (good) {
+      float *x = dyn;
+      if (w >= 4 && w < 8) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) x[k * 128 + r] = acc[k];
+      }
+      __syncthreads();
+      if (w < 4) {
+        float *gout = reinterpret_cast<float *>(J.ws + J.lay.g[h]) + ((size_t)split * D << mr) + row0 + r;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+          if (k < D) gout[(size_t)k << mr] = acc[k] + x[k * 128 + r];
+      }
+    } else if (w < 4) {
+      float *gout = reinterpret_cast<float *>(J.ws + J.lay.g[h]) + ((size_t)split * D << mr) + row0 + r;
+      for (int k = 0; k < D; ++k) gout[(size_t)k << mr] = __int_as_float(0x7fc00000);
+    }
+  }
+  if (h == 0 && tid == 0) {
+    double e = 0.0, z = 0.0;
+    for (int k = 0; k < 8; ++k) {
+      e += es[0][k];
+      z += es[1][k];
+    }
+    double *ep = reinterpret_cast<double *>(J.ws + J.lay.ep) + 2 * idx;
+    ep[0] = good ? e : __longlong_as_double(0x7ff8000000000000ll);
+    ep[1] = good ? z : 1.0;
+  }
+  __syncthreads();
+  if (w == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
+
+template <int K, bool GRAD>
+cudaError_t launch_k(const CutArgs &A, cudaStream_t s) {
+  const size_t smem = (size_t)Cfg<K>::STAGES * (GRAD ? 4 : 2) * Cfg<K>::PARTS * 4;
+  const size_t need = GRAD && smem < (size_t)K * 512 ? (size_t)K * 512 : smem;
+  auto k = k_cut_contract_tc<K, GRAD>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+  if (e != cudaSuccess) return e;
+  k<<<A.nblk, NT, need, s>>>(A);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_cut_tc(const CutArgs &A, int K, bool grad, cudaStream_t s) {
+  if (K == 16) return grad ? launch_k<16, true>(A, s) : launch_k<16, false>(A, s);
+  if (K == 32) return grad ? launch_k<32, true>(A, s) : launch_k<32, false>(A, s);
+  return grad ? launch_k<64, true>(A, s) : launch_k<64, false>(A, s);
+}
+
+}  // namespace gvqe

@@ -5,6 +5,7 @@
 #include <string>
 #include <vector>
 
+#include "gvqe_cut.cuh"
 #include "gvqe_engine.cuh"
 
 #define GVQE_VERSION_MAJOR 0
@@ -124,12 +125,20 @@ struct gvqe_hamiltonian_s {
   void *d_ctr[2] = {nullptr, nullptr}, *d_cti[2] = {nullptr, nullptr};  // FP32, FP64
   double abs_sum = 0.0;
   gvqe::DevBuf T64, T32, G;
+  gvqe::DevBuf T32t;  // T32 with the halves of its index exchanged (two-half evaluation, gvqe_cut.cuh)
   gvqe::DevBuf TC[2];  // complex path: each table entry twice (re/im), FP32 and FP64
   uint32_t *d_gm = nullptr;
   int *d_gs = nullptr;
   uint32_t *d_tz = nullptr;
   double *d_tc64 = nullptr;
   float *d_tc32 = nullptr;
+};
+
+// The two-half evaluation of a circuit (gvqe_cut.cuh) in one precision.
+struct gvqe_cut_plan {
+  bool known = false, ok = false;
+  gvqe::CutDesc d;
+  gvqe::DevBuf dev;  // d on the device
 };
 
 struct gvqe_ansatz_s {
@@ -147,6 +156,7 @@ struct gvqe_ansatz_s {
   int mps = 0;                   // GVQE_OPT_MPS_LAYERS (0 auto, -1 none, 1..4 at most that many)
   int mps_tc = 0;                // GVQE_OPT_MPS_TENSOR (0 auto = tensor cores, -1 = FP32 pipe)
   std::map<int, gvqe::Plan> plans;
+  gvqe_cut_plan cut[2];          // per precision
   gvqe::DevBuf ws, aux, shift, ro, tune;
   std::string tune_report;  // the last gvqe_autotune sweep and its choice (empty: not tuned)
 };
@@ -164,6 +174,12 @@ inline int eff_xy_tb(const gvqe_ansatz_s *a, int prec) { return a->tuned_xy_tb[p
 // ansatz is destroyed or one of its options changes.
 // allow_mps = false: no closed-form layers (callers without a table region).
 Plan *get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state_only = false, bool allow_mps = true);
+// The ansatz's two-half plan for this precision when its options and circuit let it take
+// the place of the tile passes for a diagonal H, else NULL.  cut_upload: its descriptor
+// on the device.  ensure_cut_tables: what its contraction reads of the Hamiltonian.
+gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec);
+int cut_upload(gvqe_cut_plan *c);
+int ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool grad, cudaStream_t s);
 // Energies (and adjoint gradients when grad != NULL) of a batch: the body of
 // gvqe_energy / gvqe_energy_grad after their argument checks.
 int energy_impl(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const double *params, const uint8_t *mask, int batch,

@@ -1,0 +1,97 @@
+"""The two-half evaluation (gvqe_cut.cuh) against the oracle and the tile passes.
+
+A diagonal H with RY layers whose entanglers cross the middle of the register at
+most six times in all is evaluated from two half-register tables instead of a
+2^n state.  Sizes: the smallest registers of each precision, odd ones (uneven
+halves), every number of terms (2 to 64), every entangler, several row blocks and
+column splits, many vectors per launch, masks.  Tolerances as in
+test_gpu_parity.py, and against the tile passes of the same precision the FP32
+level of both (a few units of 2^-22 per product, averaged over the sums: 5e-6
+relative L2 leaves a factor of ten) and 1e-12 in FP64.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2607_02749_gb300 import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - CPU containers
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2607_02749_gb300 as gv  # noqa: E402
+
+ALL = [gv.GVQE_ENT_LINEAR, gv.GVQE_ENT_CIRCULAR, gv.GVQE_ENT_FULL, gv.GVQE_ENT_REVERSE_LINEAR, gv.GVQE_ENT_PAIRWISE,
+       gv.GVQE_ENT_SCA]
+TWO = (gv.GVQE_ENT_CIRCULAR, gv.GVQE_ENT_SCA)  # two crossings per layer
+
+
+def _run(n, reps, ent, ham, th, fp64, mps=0, mask=None):
+    a = gv.Ansatz(n, reps, entangler=ent)
+    a.set_mps_layers(mps)
+    h = gv.Hamiltonian.from_workload(ham)
+    t = torch.as_tensor(th, device="cuda")
+    m = None if mask is None else torch.as_tensor(mask, dtype=torch.uint8, device="cuda")
+    e0 = gv.energy(a, h, t, fp64=fp64).cpu().numpy()
+    e, g = gv.energy_grad(a, h, t, mask=m, fp64=fp64)
+    d = a.describe(fp64=fp64)
+    a.close()
+    h.close()
+    return e0, e.cpu().numpy(), g.cpu().numpy(), d
+
+
+CASES = [(n, r, e, fp64) for e in ALL
+         for n, r, fp64 in [(14, 1, False), (15, 3, False), (17, 2, False), (16, 6, False), (18, 5, False),
+                            (10, 2, True), (11, 1, True), (12, 3, True), (13, 2, True), (15, 6, True)]
+         if not (e in TWO and r > 3)]
+
+
+@pytest.mark.parametrize("n,reps,ent,fp64", CASES)
+def test_against_oracle_and_tile_passes(n, reps, ent, fp64):
+    ham = wl.z_hamiltonian(n, 5 * n + 3, seed=n + reps)
+    th = wl.thetas(n, reps, 2, seed=10 * n + ent)
+    e0, e, g, d = _run(n, reps, ent, ham, th, fp64)
+    kappa = (2 if ent in TWO else 1) * reps
+    if not fp64:
+        assert f"{2 ** kappa} terms" in d, d
+    scale = ham.abs_sum()
+    te, tg = (1e-10, 1e-9) if fp64 else (2e-5, 1e-4)
+    b = 1
+    with oracle.entangler(ent):
+        er, gr = oracle.energy_grad(n, reps, th[b], ham.strings, ham.coeffs)
+    assert abs(e[b] - er) <= te * scale and abs(e0[b] - er) <= te * scale
+    if fp64:
+        assert np.max(np.abs(g[b] - gr)) <= tg * scale
+    else:
+        assert np.linalg.norm(g[b] - gr) <= tg * np.linalg.norm(gr)
+    _, et, gt, dt = _run(n, reps, ent, ham, th, fp64, mps=-1)
+    assert "terms" not in dt
+    rel = np.linalg.norm(g - gt) / np.linalg.norm(gt)
+    print(f"n={n} reps={reps} ent={ent} fp64={fp64}: oracle grad {np.linalg.norm(g[b] - gr) / np.linalg.norm(gr):.2e} "
+          f"(tile passes {np.linalg.norm(gt[b] - gr) / np.linalg.norm(gr):.2e}), E {abs(e[b] - er) / scale:.1e} "
+          f"({abs(et[b] - er) / scale:.1e})")
+    assert rel <= (1e-12 if fp64 else 5e-6), rel
+
+
+@pytest.mark.parametrize("n,reps,ent,batch,fp64", [(22, 4, gv.GVQE_ENT_LINEAR, 3, False), (25, 6, gv.GVQE_ENT_FULL, 2, False),
+                                                   (24, 2, gv.GVQE_ENT_CIRCULAR, 5, False), (20, 3, gv.GVQE_ENT_PAIRWISE, 2, True)])
+def test_many_items_and_vectors(n, reps, ent, batch, fp64):
+    """Several row blocks and column splits, E and its transposed copy at unequal
+    halves, more items than multiprocessors, masks; single vectors give the same bits."""
+    ham = wl.z_hamiltonian(n, 200, seed=n)
+    th = wl.thetas(n, reps, batch, seed=n + 1)
+    mask = wl.active_mask(n * (reps + 1), batch, seed=n + 2)
+    e0, e, g, d = _run(n, reps, ent, ham, th, fp64, mask=mask)
+    assert "terms" in d
+    _, et, gt, _ = _run(n, reps, ent, ham, th, fp64, mps=-1, mask=mask)
+    assert np.all(g[mask == 0] == 0.0)
+    scale = ham.abs_sum()
+    assert np.max(np.abs(e - et)) <= (1e-12 if fp64 else 1e-7) * scale
+    assert np.max(np.abs(e0 - et)) <= (1e-12 if fp64 else 1e-7) * scale
+    rel = np.linalg.norm(g - gt) / np.linalg.norm(gt)
+    print(f"n={n} reps={reps} ent={ent}: vs tile passes grad {rel:.2e}, E {np.max(np.abs(e - et)) / scale:.1e}")
+    assert rel <= (1e-12 if fp64 else 5e-6)
+    _, e1, g1, _ = _run(n, reps, ent, ham, th[1:2], fp64, mask=mask[1:2])
+    assert e1[0] == e[1] and np.array_equal(g1[0], g[1])
