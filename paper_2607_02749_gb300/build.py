@@ -23,7 +23,7 @@ LIB = os.path.join(HERE, "libgvqe.so")
 LIB_DEBUG = os.path.join(HERE, "libgvqe_debug.so")
 SOURCES = ["gvqe_api.cu", "gvqe_kernels.cu", "gvqe_static.cu", "gvqe_batch.cu", "gvqe_grad_l0.cu", "gvqe_readout.cu",
            "gvqe_graph.cu", "gvqe_tune.cu", "gvqe_mps.cu", "gvqe_cut.cu", "gvqe_cut_tc.cu"]
-# gvqe_inst.cu is compiled once per (amplitude type, tile bits) pair
+# gvqe_inst.cu is compiled once per (amplitude type, tile bits) pair, gvqe_cut_half.cu once per type
 INSTANCES = [("float", tb) for tb in (10, 11, 12, 13)] + [("double", tb) for tb in (10, 11, 12)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
@@ -68,9 +68,10 @@ def build(force: bool = False, verbose: bool = False, extra: Optional[List[str]]
     os.makedirs(out_dir, exist_ok=True)
     extra = list(extra or []) + (["-DGVQE_DEBUG"] if debug else [])
     jobs = [(s, [], "") for s in SOURCES]
+    jobs += [("gvqe_cut_half.cu", [f"-DGVQE_INST_T={t}"], f"_{t}") for t in ("float", "double")]
     jobs += [("gvqe_inst.cu", [f"-DGVQE_INST_T={t}", f"-DGVQE_INST_TB={tb}"], f"_{t}_{tb}") for t, tb in INSTANCES]
     # the heaviest units first
-    jobs.sort(key=lambda j: (j[0] != "gvqe_inst.cu", -int(j[1][1].split("=")[1]) if j[1] else 0))
+    jobs.sort(key=lambda j: (not j[1], -int(j[1][1].split("=")[1]) if len(j[1]) > 1 else -99))
     workers = max(1, min(len(jobs), os.cpu_count() or 4))
     with cf.ThreadPoolExecutor(max_workers=workers) as ex:
         objs = list(ex.map(lambda j: _compile(j, extra, out_dir), jobs))

@@ -1337,13 +1337,16 @@ int gvqe::cut_upload(gvqe_cut_plan *c) {
 }
 
 int gvqe::ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool grad, cudaStream_t s) {
-  GV_TRY(ensure_tables(h, prec, s));
-  if (prec || !grad || h->T32t.ptr) return GVQE_OK;
-  PendingBuf guard(h->T32t);
-  GV_TRY(h->T32t.reserve(((size_t)1 << h->n) * 4));
-  GV_CUDA(launch_transpose_table({(const float *)h->T32.ptr, (float *)h->T32t.ptr, d.half[0].m, d.half[1].m}, s));
+  GV_TRY(build_table64(h, s));
+  if (prec || (h->TT[0].ptr && (!grad || h->TT[1].ptr))) return GVQE_OK;
+  // energies alone read the first order only; a later gradient rebuilds both
+  PendingBuf g0(h->TT[0]), g1(h->TT[1]);
+  GV_TRY(h->TT[0].reserve(((size_t)1 << h->n) * 4));
+  if (grad) GV_TRY(h->TT[1].reserve(((size_t)1 << h->n) * 4));
+  GV_CUDA(launch_tile_table({(const double *)h->T64.ptr, (float *)h->TT[0].ptr, (float *)h->TT[1].ptr, d.half[0].m,
+                             d.half[1].m}, s));
   GV_CUDA(cudaStreamSynchronize(s));
-  guard.done = true;
+  g0.done = g1.done = true;
   return GVQE_OK;
 }
 
@@ -1355,21 +1358,24 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
   memset(&A, 0, sizeof(A));
   A.job0.lay = cut_layout(c->d, prec, grad != nullptr);
   const size_t per_job = (size_t)A.job0.lay.total;
-  size_t freeb = 0, total = 0;
-  GV_CUDA(cudaMemGetInfo(&freeb, &total));
-  size_t have = freeb + a->ws.bytes;
-  const long long left = budget_left();
-  if (left >= 0) have = std::min(have, (size_t)left + a->ws.bytes);
-  if (per_job > have)
-    return fail(GVQE_ENOMEM, "one evaluation needs %.3f GiB of workspace, %.3f GiB available", per_job / 1073741824.0,
-                have / 1073741824.0);
-  // as many vectors per launch as 4 GiB hold: far more than fill the GPU
-  const size_t cap = std::max(per_job, std::min(have, (size_t)4 << 30));
-  const int J = (int)std::min<size_t>((size_t)batch, cap / per_job);
+  int J = batch;
+  if (per_job * (size_t)batch > a->ws.bytes) {  // else the workspace of an earlier call serves
+    size_t freeb = 0, total = 0;
+    GV_CUDA(cudaMemGetInfo(&freeb, &total));
+    size_t have = freeb + a->ws.bytes;
+    const long long left = budget_left();
+    if (left >= 0) have = std::min(have, (size_t)left + a->ws.bytes);
+    if (per_job > have)
+      return fail(GVQE_ENOMEM, "one evaluation needs %.3f GiB of workspace, %.3f GiB available",
+                  per_job / 1073741824.0, have / 1073741824.0);
+    // as many vectors per launch as 4 GiB hold: far more than fill the GPU
+    const size_t cap = std::max(per_job, std::min(have, (size_t)4 << 30));
+    J = (int)std::min<size_t>((size_t)batch, cap / per_job);
+  }
   GV_TRY(a->ws.reserve(per_job * (size_t)J));
   A.job0.desc = (const CutDesc *)c->dev.ptr;
-  A.job0.table = prec ? h->T64.ptr : h->T32.ptr;
-  A.job0.table_t = prec ? nullptr : h->T32t.ptr;
+  A.job0.table = prec ? h->T64.ptr : h->TT[0].ptr;
+  A.job0.table_t = prec ? nullptr : h->TT[1].ptr;
   A.job0.ws = (char *)a->ws.ptr;
   A.ws_stride = (long long)per_job;
   A.cs_stride = (long long)P * (prec ? 16 : 8);
@@ -1381,7 +1387,7 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
     A.job0.E = E + j0;
     A.job0.grad = grad ? grad + (size_t)j0 * P : nullptr;
     int nl = 0;
-    GV_CUDA(launch_cut(prec, A, CutGrid{c->d.half[0].m, c->d.D, 0, 0, nullptr, nullptr}, grad != nullptr, s, &nl));
+    GV_CUDA(launch_cut(prec, A, CutGrid{c->d.half[0].m, c->d.half[1].m, c->d.D, 0, 0, 0, nullptr, nullptr, nullptr}, grad != nullptr, s, &nl));
     count_launches(nl);
   }
   return GVQE_OK;
@@ -1954,7 +1960,8 @@ int gvqe_destroy(void *handle) {
     gvqe_hamiltonian_s *h = (gvqe_hamiltonian_s *)handle;
     h->T64.release();
     h->T32.release();
-    h->T32t.release();
+    h->TT[0].release();
+    h->TT[1].release();
     h->G.release();
     h->magic = 0;
     delete h;

@@ -20,6 +20,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <set>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -650,7 +651,7 @@ int batch_loop(gvqe_batch_s *b, const double *const *params, const uint8_t *cons
 // layer), the plan's passes, and a REDUCE launch (one CTA per job: its energy
 // and gradient into the caller's buffers).  The branches run side by side.
 // Instances with a two-half evaluation (gvqe_cut.cuh) take one branch per number of
-// terms and CTA size instead, whatever their circuits: a PREP launch and the kernels of
+// terms and class of half circuit instead, whatever their circuits: a PREP launch and the kernels of
 // that evaluation, each over all of the branch's instances, largest first.
 int build_grouped(gvqe_batch_s *b, int want_grad) {
   BatchSchedule &sc = b->sched[want_grad];
@@ -665,14 +666,14 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     std::vector<int> slots;
     CutGrid grid{};
     std::vector<CutJob> jobs;
-    std::vector<int4> half, con;
+    std::vector<int4> half, con, pack;
     std::vector<CutDesc> desc;
-    size_t o_jobs, o_half, o_con, o_desc;
+    size_t o_jobs, o_half, o_con, o_pack, o_desc;
   };
-  std::map<std::pair<int, int>, CutGroup> cuts;  // (terms, threads of a half circuit's CTA)
+  std::map<std::pair<int, int>, CutGroup> cuts;  // (terms, class of the larger half)
   for (int k = 0; k < ni; ++k) {
     if (const gvqe_cut_plan *c = get_cut(A_of(k), prec)) {
-      cuts[{cut_k(c->d.D), cut_threads(c->d.half[0].m)}].slots.push_back(k);
+      cuts[{cut_k(c->d.D), cut_class(prec, c->d.half[0].m)}].slots.push_back(k);
     } else {
       by_plan[{A_of(k)->n, A_of(k)->reps, A_of(k)->ent, eff_split(A_of(k), prec)}].push_back(k);
     }
@@ -714,11 +715,11 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     off = up256(off + sizeof(RedEntry) * std::max<size_t>(1, g.plan.dir.size()));
     groups.push_back(std::move(g));
   }
-  // an instance's cos/sin table, then its workspace; FP32 gradients: the transposed
-  // diagonal tables, one per Hamiltonian (one allocation and one launch for all of them)
+  // an instance's cos/sin table, then its workspace; FP32: the diagonal tables in tile
+  // order, one pair per Hamiltonian (one allocation and one launch for all of them)
   std::vector<size_t> cut_cs(ni, 0);
   std::map<gvqe_hamiltonian, size_t> cut_tt;
-  std::vector<TransposeJob> tjobs;
+  std::vector<TableJob> tjobs;
   for (auto &kv : cuts) {
     CutGroup &g = kv.second;
     std::stable_sort(g.slots.begin(), g.slots.end(), [&](int x, int y) { return A_of(x)->n > A_of(y)->n; });
@@ -730,15 +731,18 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
       cut_cs[k] = off;
       off = up256(off + (size_t)d.n * (d.reps + 1) * 2 * es);
       off = up256(off + (size_t)job.lay.total);
-      if (!prec && want_grad && cut_tt.find(H_of(k)) == cut_tt.end()) {
+      if (!prec && cut_tt.find(H_of(k)) == cut_tt.end()) {
         cut_tt[H_of(k)] = off;
-        off = up256(off + ((size_t)1 << d.n) * 4);
+        off = up256(off + (((size_t)1 << d.n) * 4 << (want_grad ? 1 : 0)));
       }
       g.desc.push_back(d);
       g.grid.m0 = std::max(g.grid.m0, d.half[0].m);
+      g.grid.m1 = g.jobs.empty() ? d.half[1].m : std::min(g.grid.m1, d.half[1].m);
       g.grid.D = std::max(g.grid.D, d.D);
       for (int h = 0; h < 2; ++h) {
         for (int a = 0; a < d.D; ++a) g.half.push_back(make_int4(j, h, a, 0));
+        if (!prec)
+          for (int t = 0; t < 1 << (d.half[h].m - 6); ++t) g.pack.push_back(make_int4(j, h, t, 0));
         if (h == 0 || want_grad)
           for (int i = 0; i < job.lay.rb[h] * job.lay.ns[h]; ++i) g.con.push_back(make_int4(j, h, i, 0));
       }
@@ -750,11 +754,13 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     off = up256(off + sizeof(int4) * g.half.size());
     g.o_con = off;
     off = up256(off + sizeof(int4) * g.con.size());
+    g.o_pack = off;
+    off = up256(off + sizeof(int4) * g.pack.size());
     g.o_desc = off;
     off = up256(off + sizeof(CutDesc) * g.desc.size());
   }
   const size_t o_tj = off;
-  off = up256(off + sizeof(TransposeJob) * std::max<size_t>(1, cut_tt.size()));
+  off = up256(off + sizeof(TableJob) * std::max<size_t>(1, cut_tt.size()));
   // larger groups first: their longer chains of passes start early
   std::stable_sort(groups.begin(), groups.end(), [](const Group &x, const Group &y) {
     return x.slots.size() * (size_t)x.plan.state_elems * x.plan.steps.size() >
@@ -798,7 +804,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     if (!g.plan.dir.empty())
       GB_CUDA(cudaMemcpy(base + g.o_dir, g.plan.dir.data(), sizeof(RedEntry) * g.plan.dir.size(), cudaMemcpyHostToDevice));
   }
-  std::map<gvqe_hamiltonian, const void *> done_tt;
+  std::set<gvqe_hamiltonian> done_tt;
   for (auto &kv : cuts) {
     CutGroup &g = kv.second;
     for (size_t j = 0; j < g.slots.size(); ++j) {
@@ -808,15 +814,14 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
       CutJob &job = g.jobs[j];
       job.desc = (const CutDesc *)(base + g.o_desc) + j;
       job.cs = base + cut_cs[k];
-      job.table = prec ? H_of(k)->T64.ptr : H_of(k)->T32.ptr;
-      const auto tt = cut_tt.find(H_of(k));
-      if (tt != cut_tt.end()) {
-        job.table_t = base + tt->second;
-        tjobs.push_back({(const float *)job.table, (float *)(base + tt->second), d.half[0].m, d.half[1].m});
-        cut_tt.erase(tt);
-        done_tt[H_of(k)] = job.table_t;
-      } else if (!prec && want_grad) {
-        job.table_t = done_tt[H_of(k)];
+      job.table = H_of(k)->T64.ptr;
+      if (!prec) {
+        const size_t bytes = ((size_t)1 << d.n) * 4;
+        float *t0 = (float *)(base + cut_tt[H_of(k)]), *t1 = want_grad ? (float *)((char *)t0 + bytes) : nullptr;
+        job.table = t0;
+        job.table_t = t1;
+        if (done_tt.insert(H_of(k)).second)
+          tjobs.push_back({(const double *)H_of(k)->T64.ptr, t0, t1, d.half[0].m, d.half[1].m});
       }
       job.ws = base + up256(cut_cs[k] + cs_bytes);
       job.io = (const BatchIO *)(base + o_io) + k;
@@ -834,16 +839,20 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     GB_CUDA(cudaMemcpy(base + g.o_half, g.half.data(), sizeof(int4) * g.half.size(), cudaMemcpyHostToDevice));
     GB_CUDA(cudaMemcpy(base + g.o_con, g.con.data(), sizeof(int4) * g.con.size(), cudaMemcpyHostToDevice));
     GB_CUDA(cudaMemcpy(base + g.o_desc, g.desc.data(), sizeof(CutDesc) * g.desc.size(), cudaMemcpyHostToDevice));
+    if (!prec)
+      GB_CUDA(cudaMemcpy(base + g.o_pack, g.pack.data(), sizeof(int4) * g.pack.size(), cudaMemcpyHostToDevice));
+    g.grid.pack_blocks = (int)g.pack.size();
+    g.grid.pack_items = (const int4 *)(base + g.o_pack);
     g.grid.half_blocks = (int)g.half.size();
     g.grid.con_blocks = (int)g.con.size();
     g.grid.half_items = (const int4 *)(base + g.o_half);
     g.grid.con_items = (const int4 *)(base + g.o_con);
   }
   if (!tjobs.empty()) {
-    GB_CUDA(cudaMemcpy(base + o_tj, tjobs.data(), sizeof(TransposeJob) * tjobs.size(), cudaMemcpyHostToDevice));
+    GB_CUDA(cudaMemcpy(base + o_tj, tjobs.data(), sizeof(TableJob) * tjobs.size(), cudaMemcpyHostToDevice));
     int nmax = 0;
-    for (const TransposeJob &t : tjobs) nmax = std::max(nmax, t.m0 + t.m1);
-    GB_CUDA(launch_transpose_tables((const TransposeJob *)(base + o_tj), (int)tjobs.size(), nmax, nullptr));
+    for (const TableJob &t : tjobs) nmax = std::max(nmax, t.m0 + t.m1);
+    GB_CUDA(launch_tile_tables((const TableJob *)(base + o_tj), (int)tjobs.size(), nmax, nullptr));
     GB_CUDA(cudaStreamSynchronize(nullptr));
   }
   // PREP and REDUCE ids in group order (a launch covers one group's contiguous range)

@@ -13,6 +13,7 @@
 // sweep of that half's own circuit started from G_a.  No 2^n state is stored, read or
 // written: one pass over E(x) per contraction replaces the tile passes of every layer.
 #pragma once
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -23,15 +24,13 @@ constexpr int CUT_MAX_PATH = 6;    // crossing CNOTs in all: at most 64 terms
 constexpr int CUT_MAX_M = 15;      // qubits of a half
 
 // One entangler layer as seen by one half: the GF(2)-affine map of its basis indices
-// for each value b of the layer's path bits, and its projections.
+// for each value b of the layer's path bits.  Bits 16 and 17 carry the layer's projections
+// through the map: an amplitude is kept where both come out 0.
 struct CutLayer {
-  uint16_t fc[CUT_MAX_M];  // y = XOR of fc[q] over the set bits q of x, ^ fo[b]
-  uint16_t ic[CUT_MAX_M];  // x = XOR of ic[q] over the set bits q of y, ^ io[b]
-  uint16_t fo[4], io[4];
-  uint16_t pm[2];          // projection k keeps x with parity(x & pm[k]) == bit b of pt[k]
-  uint8_t pt[2];
-  uint8_t np;              // projections of this layer in this half
-  uint8_t shift, nb;       // the layer's path bits: (a >> shift) & (2^nb - 1)
+  uint32_t fc[CUT_MAX_M];  // y = XOR of fc[q] over the set bits q of x, ^ fo[b]
+  uint32_t ic[CUT_MAX_M];  // x = XOR of ic[q] over the set bits q of y, ^ io[b]
+  uint32_t fo[4], io[4];
+  int shift, nb;           // the layer's path bits: (a >> shift) & (2^nb - 1)
 };
 
 struct CutHalf {
@@ -46,9 +45,10 @@ struct CutDesc {
 
 // Workspace of one evaluation (byte offsets) and how its contractions are split.
 struct CutLayout {
-  long long tab[2];   // L and R: [a][x], amplitude type
+  long long tab[2];   // L and R: [a][x], amplitude type; with gradients a second time in runs
   long long pack[2];  // FP32: their tensor-core operand images
-  long long phi[2];   // the half states after layers 0 .. reps - 1, one per value of the path bits so far
+  long long phi[2];   // the half states after layers 0 .. reps - 1, one per value of the path bits so
+                      // far: [x], then the same in runs
   long long g[2];     // partial contractions: [split][a][x]
   long long gp;       // gradient partials (doubles): [half][a][(reps + 1) * 16]
   long long ep;       // per item of contraction 0: energy and norm (doubles)
@@ -69,8 +69,8 @@ struct BatchIO {
 struct CutJob {
   const CutDesc *desc;
   const void *cs;       // (cos, sin) of theta/2 per parameter
-  const void *table;    // E(x), amplitude type
-  const void *table_t;  // FP32: E with the halves of its index exchanged
+  const void *table;    // E(x): FP64 in index order, FP32 in contraction 0's tile order
+  const void *table_t;  // FP32: in contraction 1's tile order
   char *ws;
   const uint8_t *mask;  // or NULL
   double *E, *grad;
@@ -93,48 +93,77 @@ struct CutArgs {
 bool cut_build(int n, int reps, int ent, int prec, CutDesc *d);
 CutLayout cut_layout(const CutDesc &d, int prec, bool grad);
 
-// What the launches of one evaluation cover: the largest low half and number of terms,
-// and, for different problems in one launch, the blocks of the half circuits and of the
-// contraction.  The threads of a half circuit's CTA fix the order of its sums, so only
-// problems with equal cut_threads share a launch.
+// What the launches of one evaluation cover: the largest half and number of terms, and,
+// for different problems in one launch, the blocks of the half circuits, of the operand
+// images and of the contraction.  Problems share launches when their larger halves have
+// the same cut_class.
 struct CutGrid {
-  int m0, D;
-  int half_blocks, con_blocks;
-  const int4 *half_items, *con_items;
+  int m0, m1, D;  // m1: the smallest half
+  int half_blocks, con_blocks, pack_blocks;
+  const int4 *half_items, *con_items, *pack_items;  // (job, half, path value | index | 64-row tile, 0)
 };
-int cut_threads(int m0);
+int cut_class(int prec, int m);
 int cut_k(int D);  // terms of the tensor-core operands
 // The kernels of one evaluation, in order.  `grad`: also the gradients.
 cudaError_t launch_cut(int prec, const CutArgs &A, const CutGrid &g, bool grad, cudaStream_t s, int *launches);
-// dst[x_lo][x_hi] = src[x_hi][x_lo], x_lo of m0 and x_hi of m1 bits (both at least 5):
-// one table, or several at once (nmax: the largest m0 + m1).
-struct TransposeJob {
-  const float *src;
-  float *dst;
+// The diagonal table in the order the FP32 contractions read it, rounded from FP64:
+// d0 for contraction 0 (rows x_lo), d1 for contraction 1 (rows x_hi; may be NULL).  Tiles
+// of 128 rows x 64 columns, a row block's tiles after one another, each [j / 4][row][j % 4].
+struct TableJob {
+  const double *src;
+  float *d0, *d1;
   int m0, m1;
 };
-cudaError_t launch_transpose_table(const TransposeJob &t, cudaStream_t s);
-cudaError_t launch_transpose_tables(const TransposeJob *jobs, int njobs, int nmax, cudaStream_t s);
+// one table, or several at once (nmax: the largest m0 + m1)
+cudaError_t launch_tile_table(const TableJob &t, cudaStream_t s);
+cudaError_t launch_tile_tables(const TableJob *jobs, int njobs, int nmax, cudaStream_t s);
+// The half circuits (gvqe_cut_half.cu): mode 0 forward, 1 forward keeping the states the
+// backward reads, 2 backward; m: the class of the larger half.
+constexpr int HALF_WARP_M(int prec) { return prec ? 7 : 10; }  // largest half in one warp
+template <typename T>
+cudaError_t launch_half(const CutArgs &A, int m, int mode, int blocks, cudaStream_t s);
+// A kernel's dynamic shared-memory limit, raised once per device.
+struct SmemLimit {
+  std::atomic<uint64_t> done{0};
+  template <typename K>
+  cudaError_t set(K k, size_t bytes) {
+    int dev = 0;
+    if (const cudaError_t e = cudaGetDevice(&dev)) return e;
+    const uint64_t bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
 // FP32 contraction on the tensor cores (gvqe_cut_tc.cu).
 cudaError_t launch_cut_tc(const CutArgs &A, int K, bool grad, cudaStream_t s);
 
-__device__ __forceinline__ CutJob cut_job(const CutArgs &A, int k) {
-  if (A.jobs) {
-    CutJob j = A.jobs[k];
-    if (j.io) {
-      j.mask = j.io->mask;
-      j.E = j.io->energy;
-      j.grad = j.io->grad;
-    }
-    return j;
+// What a kernel uses of job k (the layout is indexed in place, not copied).
+struct CutView {
+  const CutDesc *desc;
+  const CutLayout *lay;
+  const void *cs, *table, *table_t;
+  char *ws;
+};
+__device__ __forceinline__ CutView cut_view(const CutArgs &A, int k) {
+  const CutJob &j = A.jobs ? A.jobs[k] : A.job0;
+  CutView v{j.desc, &j.lay, j.cs, j.table, j.table_t, j.ws};
+  if (!A.jobs) {
+    v.ws += (long long)k * A.ws_stride;
+    v.cs = (const char *)v.cs + (long long)k * A.cs_stride;
   }
-  CutJob j = A.job0;
-  j.ws += (long long)k * A.ws_stride;
-  j.cs = (const char *)j.cs + (long long)k * A.cs_stride;
-  if (j.mask) j.mask += (long long)k * A.P;
-  j.E += k;
-  if (j.grad) j.grad += (long long)k * A.P;
-  return j;
+  return v;
+}
+struct CutOut {
+  const uint8_t *mask;
+  double *E, *grad;
+};
+__device__ __forceinline__ CutOut cut_out(const CutArgs &A, int k) {
+  const CutJob &j = A.jobs ? A.jobs[k] : A.job0;
+  if (j.io) return {j.io->mask, j.io->energy, j.io->grad};
+  const long long o = A.jobs ? 0 : k;
+  return {j.mask ? j.mask + o * A.P : nullptr, j.E + o, j.grad ? j.grad + o * A.P : nullptr};
 }
 
 }  // namespace gvqe

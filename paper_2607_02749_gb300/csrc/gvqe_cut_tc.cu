@@ -6,46 +6,52 @@
 //   lambda = E(i, j) S                         on the FP32 pipe, S read from tensor memory
 //   G(i, a) += sum_j lambda(i, j) B(j, a)      128 x 64 by 64 x K
 // as tcgen05.mma kind::tf32 with FP32 accumulators.  Every operand is split into two
-// TF32 parts (x_hi rounded to nearest, x_lo = x - x_hi exactly, its last bits cut by the
-// tensor core: about 2^-22 of x), and each product is x_lo y_hi + x_hi y_lo + x_hi y_hi,
-// the small parts first so that they meet a small accumulator.  The accumulators round
-// toward zero, so G is taken out after every tile (8 full-size steps) and summed on the
-// FP32 pipe.
+// TF32 parts (x_hi and x_lo = x - x_hi exactly, its last bits cut by the tensor core:
+// about 2^-22 of x), and each product is x_lo y_hi + x_hi y_lo + x_hi y_hi, the small parts
+// first so that they meet a small accumulator.  The tables' x_hi is rounded to nearest, so
+// that x_lo has no sign of its own and the dropped x_lo y_lo averages out; lambda's x_hi is
+// cut (one instruction).  The accumulators round toward zero, so G is taken out after every
+// tile (8 full-size steps) and summed on the FP32 pipe.
 //
 // Both A operands (the rows, and lambda) sit in tensor memory: lambda never touches shared
 // memory, its high part overwrites S in place, and the MMAs read only B from shared
 // memory (64 bytes per clock of its 128).  B comes in ready-made operand images
-// (k_cut_fwd) by one bulk copy per tile.  Warps 0-3 and 4-7 take alternate tiles, a row
-// per thread; warp 8 copies, warp 9 issues the MMAs.  E is read straight into registers
-// one tile ahead, lanes along i (for the second contraction from its transposed copy).
-//
-// What bounds it: at K = 64 the MMAs (768 multiply-adds per amplitude over the two
-// contractions); at K = 16 the FP32 pipe's nine instructions per amplitude.
+// (k_cut_fwd) by one bulk copy per tile, E from tables in tile order (k_tile_table), 16
+// coalesced 16-byte loads per thread straight into registers two tiles ahead.  Warps 0-3
+// and 4-7 take alternate tiles, a row per thread; warp 8 copies, warps 9 and 10 issue the MMAs.
+// Warps 8-11 hand their registers to the others.
 #include "gvqe_cut.cuh"
 
 namespace gvqe {
 namespace {
 
-constexpr int NT = 320;
+constexpr int NT = 384;
 constexpr int COLS = 64;
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // K-major operand in shared memory, no swizzle: core matrices of 8 rows x 16 bytes, 128
-// bytes apart along K, sbo bytes apart along the rows
-__device__ __forceinline__ uint64_t op_desc(uint32_t addr, uint32_t sbo) {
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) |
-         (1ull << 46);
-}
+// bytes apart along K, sbo bytes apart along the rows.  The descriptor's low word is the
+// address and the K step, the high word the row step and the version.
+__device__ __forceinline__ uint32_t op_lo(uint32_t addr) { return (addr >> 4) | ((128u >> 4) << 16); }
+__host__ __device__ constexpr uint32_t op_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
 // FP32 accumulator, TF32 operands, K-major, M = 128
 __host__ __device__ constexpr uint32_t idesc(int N) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24);
 }
-__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint64_t b, uint32_t id, bool acc) {
+template <uint32_t HI, uint32_t ID, bool ACC>
+__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint32_t blo) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
-      "r"(a), "l"(b), "r"(id), "r"(acc ? 1 : 0)
+      "{\n .reg .pred p;\n .reg .b64 b;\n mov.b64 b, {%2, %3};\n setp.ne.b32 p, %5, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], b, %4, p;\n}\n" ::"r"(d),
+      "r"(a), "r"(blo), "n"(HI), "n"(ID), "n"(ACC ? 1 : 0)
       : "memory");
+}
+// one product over N8 steps of 8 along K
+template <uint32_t HI, uint32_t ID, bool FIRST, int N8>
+__device__ __forceinline__ void mmas(uint32_t d, uint32_t a, uint32_t blo) {
+  mma<HI, ID, !FIRST>(d, a, blo);
+#pragma unroll
+  for (int k = 1; k < N8; ++k) mma<HI, ID, true>(d, a + 8 * k, blo + 16 * k);
 }
 __device__ __forceinline__ void commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -93,28 +99,69 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, vola
   return done != 0;
 }
 
+// The same for a whole warp: one lane polls (32 would keep the barrier unit busy and every
+// other wait of the CTA, above all the MMA warp's, behind them).
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int *bad) {
+  int ok = 1;
+  if ((threadIdx.x & 31) == 0) ok = wait_bounded(bar, parity, bad);
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
 __device__ __forceinline__ void two_sum(float &hi, float &lo, float x) {
   const float s = hi + x, b = s - hi;
   lo += (hi - (s - b)) + (x - b);
   hi = s;
 }
 
+struct Yes {
+  static constexpr bool value = true;
+};
+struct No {
+  static constexpr bool value = false;
+};
+
+using f2 = unsigned long long;  // two packed floats
+__device__ __forceinline__ f2 pk2(float x, float y) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void unpk2(f2 v, float &x, float &y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 template <int K>
 struct Cfg {
-  static constexpr int BUFS = K <= 32 ? 3 : 2;  // S / lambda buffers
+  static constexpr int BUFS = K <= 16 ? 3 : 2;   // S / lambda buffers
+  static constexpr int GBUFS = K <= 32 ? 4 : 2;  // G buffers: two per warp group where they fit
   static constexpr int STAGES = K <= 32 ? 4 : 3;
   // tensor-memory columns
   static constexpr int A_HI = 0, A_LO = K, S0 = 2 * K, G0 = S0 + 128 * BUFS;
-  static_assert(G0 + 2 * K <= 512, "tensor memory");
+  static_assert(G0 + GBUFS * K <= 512, "tensor memory");
   static constexpr int PARTS = 64 * K;  // floats of one operand image part
 };
 
 template <int K, bool GRAD>
-__global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
+__global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant__ CutArgs A) {
   using C = Cfg<K>;
   constexpr int STAGE_F = (GRAD ? 4 : 2) * C::PARTS;
   extern __shared__ __align__(128) float dyn[];
-  __shared__ __align__(8) unsigned long long bars[2 * C::STAGES + 2 * C::BUFS + 2];
+  __shared__ __align__(8) unsigned long long bars[2 * C::STAGES + 2 * C::BUFS + C::GBUFS];
   __shared__ uint32_t tslot;
   __shared__ int bad_s;
   __shared__ double es[2][8];
@@ -132,13 +179,13 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
     h = idx >= A.blk0;
     if (h) idx -= A.blk0;
   }
-  const CutJob J = cut_job(A, job);
+  const CutView J = cut_view(A, job);
   const int mr = J.desc->half[h].m, mc = J.desc->half[1 - h].m, D = J.desc->D;
-  const int ns = J.lay.ns[h], split = idx % ns, row0 = (idx / ns) * 128;
+  const int ns = J.lay->ns[h], split = idx % ns, row0 = (idx / ns) * 128;
   const int nt = (1 << (mc - 6)) / ns, t0 = split * nt;
-  const float *ap = reinterpret_cast<const float *>(J.ws + J.lay.pack[h]);
-  const float *bp = reinterpret_cast<const float *>(J.ws + J.lay.pack[1 - h]);
-  const float *E = reinterpret_cast<const float *>(h ? J.table_t : J.table);
+  const float *ap = reinterpret_cast<const float *>(J.ws + J.lay->pack[h]);
+  const float *bp = reinterpret_cast<const float *>(J.ws + J.lay->pack[1 - h]);
+  const float *E = reinterpret_cast<const float *>(h ? J.table_t : J.table);  // in tile order
   const uint32_t bar0 = smem_addr(bars);
   auto full = [&](int s) { return bar0 + 8 * s; };
   auto empty = [&](int s) { return bar0 + 8 * (C::STAGES + s); };
@@ -159,7 +206,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sbar(b)));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(lbar(b)));
     }
-    for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(gbar(b)));
+    for (int b = 0; b < C::GBUFS; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(gbar(b)));
     asm volatile("fence.mbarrier_init.release.cluster;");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -192,73 +239,97 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
   __syncthreads();
   fence_after();
 
-  float acc[K];
   if (w < 8) {
     // ------------------------------------------------------------ rows --
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
+    float acc[K];
     const int g = w >> 2;
-    const float *Ei = E + row0 + r;
+    // tile (row block, t): [j / 4][row][j % 4]
+    const float *Ei = E + ((size_t)(row0 >> 7) << (mc + 7)) + (size_t)t0 * (128 * COLS) + r * 4;
     float e_hi = 0.f, e_lo = 0.f, z_hi = 0.f, z_lo = 0.f;
-    float tv[COLS];
+    f2 tv[COLS / 2];
 #pragma unroll
     for (int k = 0; k < K; ++k) acc[k] = 0.f;
     auto load = [&](int t) {
-      const float *p = Ei + ((long long)(t0 + t) << (6 + mr));
+      const float *p = Ei + (size_t)t * (128 * COLS);
 #pragma unroll
-      for (int j = 0; j < COLS; ++j) tv[j] = __ldg(p + ((long long)j << mr));
+      for (int j = 0; j < COLS / 4; ++j)  // volatile: issued here, not where the values are used
+        asm volatile("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(tv[2 * j]), "=l"(tv[2 * j + 1]) : "l"(p + 512 * j));
     };
-    if (g < nt) load(g);
-    bool ok = true;
-    for (int t = g; t < nt; t += 2) {
-      const int b = t % C::BUFS;
-      ok = wait_bounded(sbar(b), (t / C::BUFS) & 1, bad);
-      if (!ok) break;
+    auto drain = [&](int t) {  // G of tile t
+      if (!wait_warp(gbar(t % C::GBUFS), (t / C::GBUFS) & 1, bad)) return false;
       fence_after();
-      const uint32_t ts = tw + C::S0 + 128 * b;
-      float es_ = 0.f, zs_ = 0.f;
 #pragma unroll
-      for (int c = 0; c < COLS; c += 16) {
-        float v[16], l[16];
-        ld16(ts + c, v);
+      for (int c = 0; c < K; c += 16) {
+        float v[16];
+        ld16(tw + C::G0 + K * (t % C::GBUFS) + c, v);
         ld_wait();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float lam = v[j] * tv[c + j];
-          es_ = fmaf(lam, v[j], es_);
-          zs_ = fmaf(v[j], v[j], zs_);
+        for (int j = 0; j < 16; ++j) acc[c + j] += v[j];
+      }
+      fence_before();
+      return true;
+    };
+    constexpr int AHEAD = C::GBUFS == 4 ? 2 : 0;  // tiles between a tile's lambda and its G
+    const f2 neg1 = pk2(-1.f, -1.f);
+    if (g < nt) load(g);
+    int t = g;
+    for (; t < nt; t += 2) {
+      const int b = t % C::BUFS;
+      if (!wait_warp(sbar(b), (t / C::BUFS) & 1, bad)) break;
+      fence_after();
+      const uint32_t ts = tw + C::S0 + 128 * b;
+      f2 e0 = 0, e1 = 0, z0 = 0, z1 = 0;
+      auto tile = [&](auto energy) {
+#pragma unroll
+        for (int c = 0; c < COLS; c += 16) {
+          float v[16];
+          [[maybe_unused]] float l[16];
+          ld16(ts + c, v);
+          ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {
+            const f2 s = pk2(v[j], v[j + 1]);
+            const f2 lam = mul2(s, tv[(c + j) / 2]);
+            if constexpr (decltype(energy)::value) {
+              f2 &e = (j & 2) ? e1 : e0, &z = (j & 2) ? z1 : z0;
+              e = fma2(lam, s, e);
+              z = fma2(s, s, z);
+            }
+            if constexpr (GRAD) {
+              const f2 hi = lam & 0xFFFFE000FFFFE000ull;
+              const f2 lo = fma2(hi, neg1, lam);  // exact
+              unpk2(hi, v[j], v[j + 1]);
+              unpk2(lo, l[j], l[j + 1]);
+            }
+          }
           if constexpr (GRAD) {
-            float hi;
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=f"(hi) : "f"(lam));
-            v[j] = hi;
-            l[j] = lam - hi;
+            st16(ts + c, v);
+            st16(ts + 64 + c, l);
           }
         }
-        if constexpr (GRAD) {
-          st16(ts + c, v);
-          st16(ts + 64 + c, l);
-        }
-      }
+      };
+      if (h == 0)
+        tile(Yes{});
+      else
+        tile(No{});
       if constexpr (GRAD) st_wait();
       fence_before();
       __syncwarp();
       if (lane == 0) arrive(lbar(b));
       if (t + 2 < nt) load(t + 2);
-      two_sum(e_hi, e_lo, es_);
-      two_sum(z_hi, z_lo, zs_);
-      if constexpr (GRAD) {
-        ok = wait_bounded(gbar(g), (t >> 1) & 1, bad);
-        if (!ok) break;
-        fence_after();
-#pragma unroll
-        for (int c = 0; c < K; c += 16) {
-          float v[16];
-          ld16(tw + C::G0 + K * g + c, v);
-          ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) acc[c + j] += v[j];
-        }
-        fence_before();
+      if (h == 0) {
+        float x, y;
+        unpk2(add2(e0, e1), x, y);
+        two_sum(e_hi, e_lo, x + y);
+        unpk2(add2(z0, z1), x, y);
+        two_sum(z_hi, z_lo, x + y);
       }
+      if constexpr (GRAD)
+        if (t >= AHEAD && !drain(t - AHEAD)) break;
     }
+    if constexpr (GRAD && AHEAD > 0)
+      if (t >= 2 && !*bad) drain(t - 2);
     if (h == 0) {
       double e = (double)e_hi + e_lo, z = (double)z_hi + z_lo;
 #pragma unroll
@@ -271,7 +342,35 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
         es[1][w] = z;
       }
     }
-  } else if (w == 8) {
+    // the two warp groups' sums of each row, through shared memory: every G is out, so every
+    // MMA and every copy it waited for is complete
+    float *x = dyn;
+    if (GRAD && w >= 4) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) x[k * 128 + r] = acc[k];
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    const bool good = *bad == 0;  // else a wait gave up: NaN out
+    if (GRAD && w < 4) {
+      float *gout = reinterpret_cast<float *>(J.ws + J.lay->g[h]) + ((size_t)split * D << mr) + row0 + r;
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (k < D) gout[(size_t)k << mr] = good ? acc[k] + x[k * 128 + r] : __int_as_float(0x7fc00000);
+    }
+    if (h == 0 && tid == 0) {
+      double e = 0.0, z = 0.0;
+      for (int k = 0; k < 8; ++k) {
+        e += es[0][k];
+        z += es[1][k];
+      }
+      double *ep = reinterpret_cast<double *>(J.ws + J.lay->ep) + 2 * idx;
+      ep[0] = good ? e : __longlong_as_double(0x7ff8000000000000ll);
+      ep[1] = good ? z : 1.0;
+    }
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+  }
+  if (w == 8) {
     // ---------------------------------------------------------- copies --
     if (lane == 0) {
       const float *src = bp + (size_t)t0 * (256 * K);
@@ -290,49 +389,48 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
       for (int t = nt > C::STAGES ? nt - C::STAGES : 0; t < nt; ++t)
         wait_bounded(empty(t % C::STAGES), (t / C::STAGES) & 1, bad);
     }
-  } else {
+  } else if (w == 9 || w == 10) {
     // ------------------------------------------------------------ MMAs --
-    if (lane == 0) {
-      bool ok = true;
-      for (int t = 0; t <= nt && ok; ++t) {
-        if (t < nt) {  // S of tile t
-          const int s = t % C::STAGES, b = t % C::BUFS;
-          ok = wait_bounded(full(s), (t / C::STAGES) & 1, bad);
-          // the buffer's previous tile: its lambda has been contracted (or, energies only, read)
-          const int u = t - C::BUFS;
-          if (ok && u >= 0)
-            ok = GRAD ? wait_bounded(gbar(u & 1), (u >> 1) & 1, bad)
-                      : wait_bounded(lbar(b), (u / C::BUFS) & 1, bad);
-          if (!ok) break;
-          fence_after();
-          const uint32_t bs = smem_addr(dyn + s * STAGE_F), d = tmem + C::S0 + 128 * b;
-          const uint64_t bh = op_desc(bs, K * 32), bl = op_desc(bs + C::PARTS * 4, K * 32);
-#pragma unroll
-          for (int k = 0; k < K / 8; ++k) mma(d, tmem + C::A_LO + 8 * k, bh + 16 * k, idesc(COLS), k > 0);
-#pragma unroll
-          for (int k = 0; k < K / 8; ++k) mma(d, tmem + C::A_HI + 8 * k, bl + 16 * k, idesc(COLS), true);
-#pragma unroll
-          for (int k = 0; k < K / 8; ++k) mma(d, tmem + C::A_HI + 8 * k, bh + 16 * k, idesc(COLS), true);
-          commit(sbar(b));
-          if (!GRAD) commit(empty(s));
-        }
-        if (GRAD && t > 0) {  // G of tile t - 1
-          const int u = t - 1, s = u % C::STAGES, b = u % C::BUFS;
-          ok = wait_bounded(lbar(b), (u / C::BUFS) & 1, bad);
-          if (!ok) break;
-          fence_after();
-          const uint32_t bs = smem_addr(dyn + s * STAGE_F) + 2 * C::PARTS * 4;
-          const uint32_t lh = tmem + C::S0 + 128 * b, ll = lh + 64, d = tmem + C::G0 + K * (u & 1);
-          const uint64_t bh = op_desc(bs, 2048), bl = op_desc(bs + C::PARTS * 4, 2048);
-#pragma unroll
-          for (int k = 0; k < COLS / 8; ++k) mma(d, ll + 8 * k, bh + 16 * k, idesc(K), k > 0);
-#pragma unroll
-          for (int k = 0; k < COLS / 8; ++k) mma(d, lh + 8 * k, bl + 16 * k, idesc(K), true);
-#pragma unroll
-          for (int k = 0; k < COLS / 8; ++k) mma(d, lh + 8 * k, bh + 16 * k, idesc(K), true);
-          commit(gbar(u & 1));
-          commit(empty(s));
-        }
+    // Warp 9 issues S, warp 10 G: a warp's barrier polls queue behind its own MMAs (about
+    // 250 clocks), so with one warp the pipe ran dry at every change.  One elected lane runs
+    // each loop: from a branch on elect.sync an MMA takes 11 clocks to issue, from one on
+    // the lane number 45, more than a 128 x 64 x 8 MMA runs.
+    uint32_t el;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(el));
+    const uint32_t tu = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t dyn0 = smem_addr(dyn);
+    if (el && w == 9) {
+      for (int t = 0; t < nt; ++t) {
+        const int s = t % C::STAGES, b = t % C::BUFS, u = t - C::BUFS;
+        if (!wait_bounded(full(s), (t / C::STAGES) & 1, bad)) break;
+        // the buffer's previous tile: its lambda has been contracted (or, energies only, read)
+        if (u >= 0 && !(GRAD ? wait_bounded(gbar(u % C::GBUFS), (u / C::GBUFS) & 1, bad)
+                             : wait_bounded(lbar(b), (u / C::BUFS) & 1, bad)))
+          break;
+        fence_after();
+        const uint32_t bs = dyn0 + s * (STAGE_F * 4), d = tu + C::S0 + 128 * b;
+        const uint32_t bh = op_lo(bs), bl = op_lo(bs + C::PARTS * 4);
+        constexpr uint32_t HI = op_hi(K * 32), ID = idesc(COLS);
+        mmas<HI, ID, true, K / 8>(d, tu + C::A_LO, bh);
+        mmas<HI, ID, false, K / 8>(d, tu + C::A_HI, bl);
+        mmas<HI, ID, false, K / 8>(d, tu + C::A_HI, bh);
+        commit(sbar(b));
+        if (!GRAD) commit(empty(s));
+      }
+    } else if (GRAD && el && w == 10) {
+      for (int t = 0; t < nt; ++t) {
+        const int s = t % C::STAGES, b = t % C::BUFS;
+        if (!wait_bounded(lbar(b), (t / C::BUFS) & 1, bad)) break;
+        fence_after();
+        const uint32_t bs = dyn0 + s * (STAGE_F * 4) + 2 * C::PARTS * 4;
+        const uint32_t lh = tu + C::S0 + 128 * b, ll = lh + 64, d = tu + C::G0 + K * (t % C::GBUFS);
+        const uint32_t bh = op_lo(bs), bl = op_lo(bs + C::PARTS * 4);
+        constexpr uint32_t HI = op_hi(2048), ID = idesc(K);
+        mmas<HI, ID, true, COLS / 8>(d, ll, bh);
+        mmas<HI, ID, false, COLS / 8>(d, lh, bl);
+        mmas<HI, ID, false, COLS / 8>(d, lh, bh);
+        commit(gbar(t % C::GBUFS));
+        commit(empty(s));
       }
     }
   }
@@ -340,43 +438,12 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const CutArgs A) {
   fence_before();
   __syncthreads();
   fence_after();
-  const bool good = bad_s == 0;
-  // every stage copied has been read: full and empty of the last STAGES tiles are complete
-  // unless a wait gave up, and then the copies in flight are waited for before leaving
-  if (!good && tid == 256) {
-    int dummy = 0;
+  // unless a wait gave up, every stage copied has been read; if one did, the copies in
+  // flight are waited for before leaving
+  if (bad_s && tid == 256) {
+    int none = 0;
     for (int s = 0; s < C::STAGES; ++s)
-      for (int p = 0; p < 2; ++p) wait_bounded(full(s), p, &dummy);
-  }
-  if constexpr (GRAD) {
-    // rows' sums of the two warp groups, through shared memory (all copies are consumed)
-    if (good) {
-      float *x = dyn;
-      if (w >= 4 && w < 8) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) x[k * 128 + r] = acc[k];
-      }
-      __syncthreads();
-      if (w < 4) {
-        float *gout = reinterpret_cast<float *>(J.ws + J.lay.g[h]) + ((size_t)split * D << mr) + row0 + r;
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-          if (k < D) gout[(size_t)k << mr] = acc[k] + x[k * 128 + r];
-      }
-    } else if (w < 4) {
-      float *gout = reinterpret_cast<float *>(J.ws + J.lay.g[h]) + ((size_t)split * D << mr) + row0 + r;
-      for (int k = 0; k < D; ++k) gout[(size_t)k << mr] = __int_as_float(0x7fc00000);
-    }
-  }
-  if (h == 0 && tid == 0) {
-    double e = 0.0, z = 0.0;
-    for (int k = 0; k < 8; ++k) {
-      e += es[0][k];
-      z += es[1][k];
-    }
-    double *ep = reinterpret_cast<double *>(J.ws + J.lay.ep) + 2 * idx;
-    ep[0] = good ? e : __longlong_as_double(0x7ff8000000000000ll);
-    ep[1] = good ? z : 1.0;
+      for (int p = 0; p < 2; ++p) wait_bounded(full(s), p, &none);
   }
   __syncthreads();
   if (w == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
@@ -387,8 +454,8 @@ cudaError_t launch_k(const CutArgs &A, cudaStream_t s) {
   const size_t smem = (size_t)Cfg<K>::STAGES * (GRAD ? 4 : 2) * Cfg<K>::PARTS * 4;
   const size_t need = GRAD && smem < (size_t)K * 512 ? (size_t)K * 512 : smem;
   auto k = k_cut_contract_tc<K, GRAD>;
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-  if (e != cudaSuccess) return e;
+  static SmemLimit limit;
+  if (const cudaError_t e = limit.set(k, need)) return e;
   k<<<A.nblk, NT, need, s>>>(A);
   return cudaGetLastError();
 }

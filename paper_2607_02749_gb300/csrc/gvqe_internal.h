@@ -125,7 +125,7 @@ struct gvqe_hamiltonian_s {
   void *d_ctr[2] = {nullptr, nullptr}, *d_cti[2] = {nullptr, nullptr};  // FP32, FP64
   double abs_sum = 0.0;
   gvqe::DevBuf T64, T32, G;
-  gvqe::DevBuf T32t;  // T32 with the halves of its index exchanged (two-half evaluation, gvqe_cut.cuh)
+  gvqe::DevBuf TT[2];  // FP32 tables in the tile order of the two-half contractions (gvqe_cut.cuh)
   gvqe::DevBuf TC[2];  // complex path: each table entry twice (re/im), FP32 and FP64
   uint32_t *d_gm = nullptr;
   int *d_gs = nullptr;
