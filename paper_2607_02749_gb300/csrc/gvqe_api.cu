@@ -1315,16 +1315,29 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
 // ------------------------------------------------- two-half evaluation --
 // A diagonal H and RY layers whose crossing CNOTs leave at most 64 terms: the state is
 // never stored (gvqe_cut.cuh).  GVQE_OPT_MPS_LAYERS other than 0 and GVQE_OPT_MPS_TENSOR = -1
-// name the other evaluations.  FP64 runs on the FP64 pipe: 2 D multiply-adds per amplitude
-// and contraction against about 2 per gate and sweep of the tile passes.
-gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec) {
-  if (a->gates != 1 || a->mps != 0 || (!prec && a->mps_tc != 0)) return nullptr;
-  gvqe_cut_plan &c = a->cut[prec];
+// name the other evaluations.  FP64 is a matter of FP64 operations: D (energies) or 4 D
+// multiply-adds per amplitude and the half circuits, spread over all SMs, against about 2
+// or 6 per gate and amplitude of the tile passes, on as many SMs as the call has tiles.
+// Up to n reps terms the halves win at any number of vectors; above, only where a call leaves
+// most SMs without a tile (10 qubits, 4 circular repetitions, one vector: 256 terms, 3.5 M
+// operations on 152 SMs against 0.25 M on one).
+gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad) {
+  if (a->mps != 0 || (!prec && a->mps_tc != 0) || (a->gates == 2 && prec)) return nullptr;
+  gvqe_cut_plan &c = a->cut[a->gates == 2 ? 2 : prec];
   if (!c.known) {
-    c.ok = cut_build(a->n, a->reps, a->ent, prec, &c.d) && (!prec || c.d.D <= a->n * a->reps);
+    c.ok = cut_build(a->n, a->reps, a->ent, prec, a->gates, &c.d);
     c.known = true;
   }
-  return c.ok ? &c : nullptr;
+  if (!c.ok) return nullptr;
+  if (prec && c.d.D > a->n * a->reps) {
+    const double S = std::ldexp(1.0, a->n), m = c.d.half[0].m;
+    const double half = 2.0 * c.d.D * std::ldexp(m, c.d.half[0].m) * (a->reps + 1) * (grad ? 6 : 2);
+    const double cut = ((grad ? 4 : 1) * c.d.D * S + half) / 152.0;
+    const double sms = std::min(152.0, vectors * std::max(1.0, S / 4096.0));
+    const double tile = (grad ? 6 : 2) * a->n * a->reps * S / sms;
+    if (cut * 1.5 > tile) return nullptr;
+  }
+  return &c;
 }
 
 int gvqe::cut_upload(gvqe_cut_plan *c) {
@@ -1338,25 +1351,132 @@ int gvqe::cut_upload(gvqe_cut_plan *c) {
 
 int gvqe::ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool grad, cudaStream_t s) {
   GV_TRY(build_table64(h, s));
-  if (prec || (h->TT[0].ptr && (!grad || h->TT[1].ptr))) return GVQE_OK;
+  DevBuf *tt = h->TT[d.cx];
+  if (prec || (tt[0].ptr && (!grad || tt[1].ptr))) return GVQE_OK;
   // energies alone read the first order only; a later gradient rebuilds both
-  PendingBuf g0(h->TT[0]), g1(h->TT[1]);
-  GV_TRY(h->TT[0].reserve(((size_t)1 << h->n) * 4));
-  if (grad) GV_TRY(h->TT[1].reserve(((size_t)1 << h->n) * 4));
-  GV_CUDA(launch_tile_table({(const double *)h->T64.ptr, (float *)h->TT[0].ptr, (float *)h->TT[1].ptr, d.half[0].m,
-                             d.half[1].m}, s));
+  PendingBuf g0(tt[0]), g1(tt[1]);
+  GV_TRY(tt[0].reserve(((size_t)1 << h->n) * 4));
+  if (grad) GV_TRY(tt[1].reserve(((size_t)1 << h->n) * 4));
+  GV_CUDA(launch_tile_table({(const double *)h->T64.ptr, (float *)tt[0].ptr, (float *)tt[1].ptr, d.half[0].m,
+                             d.half[1].m, d.cx}, s));
   GV_CUDA(cudaStreamSynchronize(s));
   g0.done = g1.done = true;
   return GVQE_OK;
 }
 
+void gvqe::split_xy(const gvqe_hamiltonian_s *h, int m0, CutXyDims *dims, std::vector<uint32_t> *xm,
+                    std::vector<uint32_t> *zm, std::vector<int> *start, std::vector<int> *other,
+                    std::vector<double> *coef, std::vector<int> *gstart) {
+  const uint32_t lom = (1u << m0) - 1;
+  std::map<std::pair<uint32_t, uint32_t>, int> id[2];  // (x, z) of a part -> index, in order of x
+  for (int s = 0; s < 2; ++s) {
+    auto part = [&](uint32_t v) { return s ? v >> m0 : v & lom; };
+    for (size_t g = 0; g < h->gm.size(); ++g)
+      for (int t = h->gs[g]; t < h->gs[g + 1]; ++t) id[s][{part(h->gm[g]), part(h->tz[t])}] = 0;
+    int k = 0;
+    for (auto &kv : id[s]) {
+      if (xm[s].empty() || xm[s].back() != kv.first.first) gstart[s].push_back(k);
+      xm[s].push_back(kv.first.first);
+      zm[s].push_back(kv.first.second);
+      kv.second = k++;
+    }
+    gstart[s].push_back(k);
+    dims->U[s] = k;
+    dims->ng[s] = (int)gstart[s].size() - 1;
+  }
+  std::vector<std::vector<std::pair<int, double>>> by[2];
+  for (int s = 0; s < 2; ++s) by[s].resize(dims->U[s]);
+  for (size_t g = 0; g < h->gm.size(); ++g)
+    for (int t = h->gs[g]; t < h->gs[g + 1]; ++t) {
+      const int l = id[0][{h->gm[g] & lom, h->tz[t] & lom}], r = id[1][{h->gm[g] >> m0, h->tz[t] >> m0}];
+      by[0][l].push_back({r, h->tc[t]});
+      by[1][r].push_back({l, h->tc[t]});
+    }
+  for (int s = 0; s < 2; ++s)
+    for (int u = 0; u <= dims->U[s]; ++u) {
+      start[s].push_back((int)other[s].size());
+      if (u == dims->U[s]) break;
+      for (const auto &p : by[s][u]) {
+        other[s].push_back(p.first);
+        coef[s].push_back(p.second);
+      }
+    }
+}
+
+// The device arrays of split_xy in one buffer, the descriptor at its start.
+static int ensure_cut_xy(gvqe_hamiltonian_s *h, int m0) {
+  if (h->XY.ptr) return GVQE_OK;
+  CutXy x{};
+  std::vector<uint32_t> xm[2], zm[2];
+  std::vector<int> start[2], other[2], gstart[2];
+  std::vector<double> coef[2];
+  split_xy(h, m0, &x, xm, zm, start, other, coef, gstart);
+  std::vector<char> img(256);
+  auto put = [&](const void *p, size_t bytes) {
+    const size_t o = img.size();
+    img.resize(o + (bytes + 15) / 16 * 16);
+    memcpy(img.data() + o, p, bytes);
+    return o;
+  };
+  static_assert(sizeof(CutXy) <= 256, "descriptor");
+  size_t o[2][6];
+  for (int s = 0; s < 2; ++s) {
+    o[s][0] = put(xm[s].data(), xm[s].size() * 4);
+    o[s][1] = put(zm[s].data(), zm[s].size() * 4);
+    o[s][2] = put(start[s].data(), start[s].size() * 4);
+    o[s][3] = put(other[s].data(), other[s].size() * 4);
+    o[s][4] = put(gstart[s].data(), gstart[s].size() * 4);
+    o[s][5] = put(coef[s].data(), coef[s].size() * 8);
+  }
+  PendingBuf guard(h->XY);
+  GV_TRY(h->XY.reserve(img.size()));
+  const char *b = (const char *)h->XY.ptr;
+  for (int s = 0; s < 2; ++s) {
+    x.xm[s] = (const uint32_t *)(b + o[s][0]);
+    x.zm[s] = (const uint32_t *)(b + o[s][1]);
+    x.start[s] = (const int *)(b + o[s][2]);
+    x.other[s] = (const int *)(b + o[s][3]);
+    x.gstart[s] = (const int *)(b + o[s][4]);
+    x.coef[s] = (const double *)(b + o[s][5]);
+  }
+  memcpy(img.data(), &x, sizeof(x));
+  GV_CUDA(cudaMemcpy(h->XY.ptr, img.data(), img.size(), cudaMemcpyHostToDevice));
+  h->xy = x;
+  guard.done = true;
+  return GVQE_OK;
+}
+
+// X/Y strings, FP32: the two-half evaluation costs 2 D^2 2^m multiply-adds per part and half
+// (one of the two without gradients), the passes over stored states one signed addition per
+// string and amplitude on top of the tile passes.
+static bool cut_xy_pays(gvqe_hamiltonian_s *h, const CutDesc &d, bool grad) {
+  if (h->xy.U[0] == 0) {  // the sizes alone, once
+    CutXyDims dims{};
+    std::vector<uint32_t> xm[2], zm[2];
+    std::vector<int> start[2], other[2], gstart[2];
+    std::vector<double> coef[2];
+    split_xy(h, d.half[0].m, &dims, xm, zm, start, other, coef, gstart);
+    h->xy.U[0] = dims.U[0];
+    h->xy.U[1] = dims.U[1];
+    h->xy.ng[0] = dims.ng[0];
+    h->xy.ng[1] = dims.ng[1];
+  }
+  const double dp = cut_xy_dp(d.D);
+  const double mac = (std::ldexp((double)h->xy.U[0], d.half[0].m) + std::ldexp((double)h->xy.U[1], d.half[1].m)) * dp *
+                     dp * (grad ? 2 : 1);
+  const double half = mac / 1.5e13, tile = std::ldexp((double)h->tz.size(), d.n) * 2e-13;
+  return half < tile + 50e-6;
+}
+
 static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, const void *cs, const uint8_t *mask,
                    int batch, double *E, double *grad, int prec, cudaStream_t s) {
   GV_TRY(cut_upload(c));
-  const int P = a->n * (a->reps + 1);
+  const int P = a->gates * a->n * (a->reps + 1);
   CutArgs A;
   memset(&A, 0, sizeof(A));
-  A.job0.lay = cut_layout(c->d, prec, grad != nullptr);
+  const bool xy = !h->gm.empty();
+  A.job0.lay = cut_layout(c->d, prec, grad != nullptr, xy ? &h->xy : nullptr);
+  A.xy = xy ? (const CutXy *)h->XY.ptr : nullptr;
   const size_t per_job = (size_t)A.job0.lay.total;
   int J = batch;
   if (per_job * (size_t)batch > a->ws.bytes) {  // else the workspace of an earlier call serves
@@ -1374,8 +1494,8 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
   }
   GV_TRY(a->ws.reserve(per_job * (size_t)J));
   A.job0.desc = (const CutDesc *)c->dev.ptr;
-  A.job0.table = prec ? h->T64.ptr : h->TT[0].ptr;
-  A.job0.table_t = prec ? nullptr : h->TT[1].ptr;
+  A.job0.table = prec ? h->T64.ptr : h->TT[c->d.cx][0].ptr;
+  A.job0.table_t = prec ? nullptr : h->TT[c->d.cx][1].ptr;
   A.job0.ws = (char *)a->ws.ptr;
   A.ws_stride = (long long)per_job;
   A.cs_stride = (long long)P * (prec ? 16 : 8);
@@ -1387,7 +1507,7 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
     A.job0.E = E + j0;
     A.job0.grad = grad ? grad + (size_t)j0 * P : nullptr;
     int nl = 0;
-    GV_CUDA(launch_cut(prec, A, CutGrid{c->d.half[0].m, c->d.half[1].m, c->d.D, 0, 0, 0, nullptr, nullptr, nullptr}, grad != nullptr, s, &nl));
+    GV_CUDA(launch_cut(prec, A, CutGrid{c->d.cx, c->d.half[0].m, c->d.half[1].m, c->d.D, 0, 0, 0, nullptr, nullptr, nullptr}, grad != nullptr, s, &nl, xy ? &h->xy : nullptr));
     count_launches(nl);
   }
   return GVQE_OK;
@@ -1408,9 +1528,11 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
                       double *E, double *grad, int prec, cudaStream_t s) {
   const bool cplx = a->gates == 2;
   const bool diag = cplx ? h->cgm.empty() : h->gm.empty();
-  if (gvqe_cut_plan *c = diag ? get_cut(a, prec) : nullptr) {
+  gvqe_cut_plan *c = diag || (!cplx && !prec) ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
+  if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr))) {
     GV_TRY(ensure_cut_tables(h, prec, c->d, grad != nullptr, s));
-    const long long count = (long long)batch * a->n * (a->reps + 1);
+    if (!diag) GV_TRY(ensure_cut_xy(h, c->d.half[0].m));
+    const long long count = (long long)batch * a->gates * a->n * (a->reps + 1);
     GV_TRY(a->aux.reserve((size_t)count * (prec ? 16 : 8)));
     GV_CUDA(launch_trig(prec, params, count, a->aux.ptr, s));
     count_launches(1);
@@ -1936,7 +2058,7 @@ int gvqe_ansatz_describe(gvqe_ansatz a, int flags, char *buf, int buflen) {
     return fail(GVQE_EINVAL, "tile bits %d too large", eff_tile_bits(a, prec));
   const Plan *pl = get_plan(a, prec, true, true);
   std::string s = describe_plan(*pl);
-  if (const gvqe_cut_plan *c = get_cut(a, prec)) {
+  if (const gvqe_cut_plan *c = get_cut(a, prec, 1, true)) {
     char line[160];
     snprintf(line, sizeof(line), "diagonal H: evaluated from the halves [0,%d) and [%d,%d), %d terms%s\n", c->d.half[1].q0,
              c->d.half[1].q0, a->n, c->d.D, prec ? "" : " (tensor cores, TF32 split)");
@@ -1960,8 +2082,8 @@ int gvqe_destroy(void *handle) {
     gvqe_hamiltonian_s *h = (gvqe_hamiltonian_s *)handle;
     h->T64.release();
     h->T32.release();
-    h->TT[0].release();
-    h->TT[1].release();
+    h->XY.release();
+    for (int k = 0; k < 4; ++k) h->TT[k >> 1][k & 1].release();
     h->G.release();
     h->magic = 0;
     delete h;

@@ -672,7 +672,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
   };
   std::map<std::pair<int, int>, CutGroup> cuts;  // (terms, class of the larger half)
   for (int k = 0; k < ni; ++k) {
-    if (const gvqe_cut_plan *c = get_cut(A_of(k), prec)) {
+    if (const gvqe_cut_plan *c = get_cut(A_of(k), prec, ni, want_grad != 0)) {
       cuts[{cut_k(c->d.D), cut_class(prec, c->d.half[0].m)}].slots.push_back(k);
     } else {
       by_plan[{A_of(k)->n, A_of(k)->reps, A_of(k)->ent, eff_split(A_of(k), prec)}].push_back(k);
@@ -724,7 +724,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     CutGroup &g = kv.second;
     std::stable_sort(g.slots.begin(), g.slots.end(), [&](int x, int y) { return A_of(x)->n > A_of(y)->n; });
     for (int k : g.slots) {
-      const CutDesc &d = get_cut(A_of(k), prec)->d;
+      const CutDesc &d = get_cut(A_of(k), prec, ni, want_grad != 0)->d;
       const int j = (int)g.jobs.size();
       CutJob job{};
       job.lay = cut_layout(d, prec, want_grad != 0);
@@ -821,7 +821,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
         job.table = t0;
         job.table_t = t1;
         if (done_tt.insert(H_of(k)).second)
-          tjobs.push_back({(const double *)H_of(k)->T64.ptr, t0, t1, d.half[0].m, d.half[1].m});
+          tjobs.push_back({(const double *)H_of(k)->T64.ptr, t0, t1, d.half[0].m, d.half[1].m, 0});
       }
       job.ws = base + up256(cut_cs[k] + cs_bytes);
       job.io = (const BatchIO *)(base + o_io) + k;

@@ -50,12 +50,15 @@ static std::vector<std::pair<int, int>> cnot_list(int ent, int n, int r) {
 
 static int parity32(uint32_t x) { return __builtin_parity(x); }
 
-bool cut_build(int n, int reps, int ent, int prec, CutDesc *d) {
+bool cut_build(int n, int reps, int ent, int prec, int gates, CutDesc *d) {
   memset(d, 0, sizeof(*d));
   const int h = (n + 1) / 2;
   // FP32: 128-row and 64-column tiles in the contraction; FP64: 32 x 32 tiles, and a half's
   // state (with its padding) in one CTA's shared memory
-  if (reps < 1 || reps > CUT_MAX_LAYERS || n - h < (prec ? 5 : 7) || h > (prec ? CUT_MAX_M - 1 : CUT_MAX_M)) return false;
+  if (reps < 1 || reps > CUT_MAX_LAYERS || n - h < (prec ? 5 : 7) || h > (prec || gates == 2 ? CUT_MAX_M - 1 : CUT_MAX_M))
+    return false;
+  if (gates == 2 && prec) return false;
+  d->cx = gates == 2;
   d->n = n;
   d->reps = reps;
   const int lo[3] = {0, h, n};
@@ -136,7 +139,7 @@ bool cut_build(int n, int reps, int ent, int prec, CutDesc *d) {
       }
     }
     kappa += nb;
-    if (kappa > CUT_MAX_PATH) return false;
+    if (kappa > (prec ? CUT_MAX_PATH64 : CUT_MAX_PATH) - d->cx) return false;  // complex: two real terms per term
   }
   d->kappa = kappa;
   d->D = 1 << kappa;
@@ -149,7 +152,11 @@ int cut_k(int D) { return D < 16 ? 16 : D; }
 constexpr int CUT_ROWS32 = 128, CUT_COLS32 = 64;  // FP32 contraction tile
 constexpr int CUT_TILE64 = 32;                    // FP64 contraction tile (square)
 
-CutLayout cut_layout(const CutDesc &d, int prec, bool grad) {
+// FP64 contraction with a CTA per row (k_cut_rows64)
+static bool cut_by_rows(int m0, int D) { return m0 <= 8 && D >= 64; }
+static bool cut_by_rows(const CutDesc &d) { return cut_by_rows(d.half[0].m, d.D); }
+
+CutLayout cut_layout(const CutDesc &d, int prec, bool grad, const CutXyDims *xy) {
   CutLayout l;
   memset(&l, 0, sizeof(l));
   const long long es = prec ? 8 : 4;
@@ -160,24 +167,46 @@ CutLayout cut_layout(const CutDesc &d, int prec, bool grad) {
     return o;
   };
   for (int s = 0; s < 2; ++s) {
-    const long long S = 1LL << d.half[s].m;
+    const long long S = 1LL << (d.half[s].m + d.cx), T = (long long)d.D << d.cx;  // rows (with the channel), real terms
     const int mo = d.half[1 - s].m;
-    l.rb[s] = (int)(S / (prec ? CUT_TILE64 : CUT_ROWS32));
+    l.rb[s] = (int)(S / (prec ? (cut_by_rows(d) ? 1 : CUT_TILE64) : CUT_ROWS32));
     const long long tiles = (1LL << mo) / (prec ? CUT_TILE64 : CUT_COLS32);
     // enough items for 152 SMs on a single vector, but runs long enough that an item's
     // set-up (its rows into tensor memory, the first tiles) stays small
     const long long per = prec ? 8 : 32;
-    l.ns[s] = (int)(tiles / per < 1 ? 1 : tiles / per > 4 ? 4 : tiles / per);
-    l.tab[s] = take(d.D * S * es * (grad ? 2 : 1));
-    if (!prec) l.pack[s] = take(S * cut_k(d.D) * 16);
+    l.ns[s] = prec && cut_by_rows(d) ? 1 : (int)(tiles / per < 1 ? 1 : tiles / per > 4 ? 4 : tiles / per);
+    l.tab[s] = take(d.D * S * es * (grad && !d.cx ? 2 : 1));
+    if (!prec) l.pack[s] = take((S >> d.cx) * cut_k(T) * 16);
+    if (d.cx) l.packr[s] = take(S * cut_k(T) * 8);
     if (grad) {
       long long states = 0;
       for (int r = 0; r < d.reps; ++r) states += 1LL << d.half[s].L[r].shift;
+      if (d.cx) states += d.D;  // the last layer's too, before its RZ
       l.phi[s] = take(2 * states * S * es);
-      l.g[s] = take((long long)l.ns[s] * d.D * S * es);
+      l.g[s] = take((l.ns[s] + (xy ? 1 : 0)) * T * S * es);
     }
   }
-  if (grad) l.gp = take(2LL * d.D * (d.reps + 1) * 16 * 8);
+  for (int s = 0; s < 2; ++s) l.gs[s] = l.ns[s] + (xy ? 1 : 0);
+  if (xy) {
+    const long long dp = cut_xy_dp(d.D);
+    for (int s = 0; s < 2; ++s) {
+      const long long S = 1LL << d.half[s].m;
+      // runs of one length for both halves: long enough to pay for their sums, 16 at most
+      l.xrun[s] = (int)(S / 16 < 128 ? 128 : S / 16 > 1024 ? 1024 : S / 16);
+      if (s == 1 && l.xrun[1] > l.xrun[0]) l.xrun[1] = l.xrun[0];
+    }
+    l.xrun[0] = l.xrun[1] = l.xrun[0] < l.xrun[1] ? l.xrun[0] : l.xrun[1];
+    for (int s = 0; s < 2; ++s) {
+      const long long S = 1LL << d.half[s].m;
+      l.rows[s] = take(S * dp * 4);
+      l.mpart[s] = take(S / l.xrun[s] * xy->U[s] * dp * dp * 4);
+      l.mm[s] = take((long long)xy->U[s] * dp * dp * 8);
+      l.nn[s] = grad ? take((long long)xy->U[s] * dp * dp * 4) : -1;
+    }
+    l.nexy = xy->U[0];
+    l.exy = take((long long)xy->U[0] * 8);
+  }
+  if (grad) l.gp = take(2LL * d.D * (d.reps + 1) * (16 << d.cx) * 8);
   l.ep = take((long long)l.rb[0] * l.ns[0] * 16);
   l.total = off;
   return l;
@@ -185,11 +214,29 @@ CutLayout cut_layout(const CutDesc &d, int prec, bool grad) {
 
 // The tensor-core operand images of both tables of a job: per 64 rows x the blocks
 // [hi | lo] of the row form (K-major over a) and [hi | lo] of the column form (rows a,
-// K-major over x), core matrices of 8 rows x 16 bytes; terms from D to K are zero.  One CTA
-// per 64 rows, through shared memory; 16-byte stores.
+// K-major over x), core matrices of 8 rows x 16 bytes; terms beyond the table's are zero.
+// One CTA per 64 rows, through shared memory; 16-byte stores.  A complex table T gives the
+// columns (Re T_a, Im T_a) of real terms 2a, 2a + 1 over x, and in row form alone the rows
+// (x, 0): (Re T_a, -Im T_a) and (x, 1): (Im T_a, Re T_a).
+__device__ __forceinline__ void pack_form(const float *s, float4 *out, int K, bool row) {
+  for (int i = threadIdx.x; i < K * 16; i += 256) {
+    const int r = row ? (i & 7) + 8 * (i / (2 * K)) : 4 * ((i >> 3) & 15);  // [r / 8][a / 4][r % 8]
+    const int a = row ? 4 * ((i >> 3) % (K / 4)) : (i & 7) + 8 * (i >> 7);  // [a / 8][r / 4][a % 8]
+    float hi[4], lo[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float x = row ? s[(a + k) * 65 + r] : s[a * 65 + r + k];
+      asm("cvt.rna.tf32.f32 %0, %1;" : "=f"(hi[k]) : "f"(x));
+      lo[k] = x - hi[k];
+    }
+    out[i] = make_float4(hi[0], hi[1], hi[2], hi[3]);
+    out[16 * K + i] = make_float4(lo[0], lo[1], lo[2], lo[3]);
+  }
+}
+template <bool CX>
 __global__ void __launch_bounds__(256) k_cut_pack(const __grid_constant__ CutArgs A, int K) {
   extern __shared__ __align__(16) unsigned char cut_smem[];
-  float *s = reinterpret_cast<float *>(cut_smem);  // [a][65]
+  float *s = reinterpret_cast<float *>(cut_smem);  // [term][65]
   int job, h, tile;
   if (A.items) {
     const int4 it = A.items[blockIdx.x];
@@ -205,32 +252,33 @@ __global__ void __launch_bounds__(256) k_cut_pack(const __grid_constant__ CutArg
   }
   const CutView J = cut_view(A, job);
   const int D = J.desc->D, m = J.desc->half[h].m;
-  const float *tab = reinterpret_cast<const float *>(J.ws + J.lay->tab[h]) + tile * 64;
+  const float *tab = reinterpret_cast<const float *>(J.ws + J.lay->tab[h]);
+  float4 *out = reinterpret_cast<float4 *>(J.ws + J.lay->pack[h]) + (size_t)tile * (64 * K);
   for (int i = threadIdx.x; i < K * 64; i += 256) {
-    const int a = i >> 6;
-    s[a * 65 + (i & 63)] = a < D ? tab[((size_t)a << m) + (i & 63)] : 0.f;
+    const int a = i >> 6, x = tile * 64 + (i & 63);
+    float v = 0.f;
+    if constexpr (CX) {
+      if (a < 2 * D) v = tab[((size_t)(a >> 1) << (m + 1)) + 2 * x + (a & 1)];
+    } else {
+      if (a < D) v = tab[((size_t)a << m) + x];
+    }
+    s[a * 65 + (i & 63)] = v;
   }
   __syncthreads();
-  float4 *out = reinterpret_cast<float4 *>(J.ws + J.lay->pack[h]) + (size_t)tile * (64 * K);
-  for (int i = threadIdx.x; i < K * 16; i += 256) {
-    float x[2][4];
-    const int r = (i & 7) + 8 * (i / (2 * K)), a = 4 * ((i >> 3) % (K / 4));  // row form: [r / 8][a / 4][r % 8]
-    const int r2 = 4 * ((i >> 3) & 15), a2 = (i & 7) + 8 * (i >> 7);          // column form: [a / 8][r / 4][a % 8]
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      x[0][k] = s[(a + k) * 65 + r];
-      x[1][k] = s[a2 * 65 + r2 + k];
-    }
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      float hi[4], lo[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=f"(hi[k]) : "f"(x[f][k]));
-        lo[k] = x[f][k] - hi[k];
+  pack_form(s, out, K, true);
+  pack_form(s, out + 32 * K, K, false);
+  if constexpr (CX) {  // the two 64-row blocks (x, channel) of these 64 x
+    float4 *rows = reinterpret_cast<float4 *>(J.ws + J.lay->packr[h]) + (size_t)tile * (64 * K);
+    for (int b = 0; b < 2; ++b) {
+      __syncthreads();
+      for (int i = threadIdx.x; i < K * 64; i += 256) {
+        const int a = i >> 6, r = i & 63, x = tile * 64 + b * 32 + (r >> 1), ch = r & 1;
+        float v = 0.f;
+        if (a < 2 * D) v = tab[((size_t)(a >> 1) << (m + 1)) + 2 * x + (ch ^ (a & 1))];
+        s[a * 65 + r] = (a & 1) && !ch ? -v : v;
       }
-      out[f * 32 * K + i] = make_float4(hi[0], hi[1], hi[2], hi[3]);
-      out[f * 32 * K + 16 * K + i] = make_float4(lo[0], lo[1], lo[2], lo[3]);
+      __syncthreads();
+      pack_form(s, rows + b * 32 * K, K, true);
     }
   }
 }
@@ -242,7 +290,7 @@ __global__ void __launch_bounds__(256) k_cut_pack(const __grid_constant__ CutArg
 // amplitude and contraction against 6 (reps + 1) n of the gate-by-gate sweeps.
 constexpr int C64 = CUT_TILE64, C64LD = C64 + 1;
 
-template <bool GRAD>
+template <bool GRAD, int NA>  // NA: terms per thread of G, 8 NA in all
 __global__ void __launch_bounds__(256) k_cut_contract64(const __grid_constant__ CutArgs A) {
   extern __shared__ __align__(16) unsigned char cut_smem[];
   int job, h, idx;
@@ -269,9 +317,9 @@ __global__ void __launch_bounds__(256) k_cut_contract64(const __grid_constant__ 
   double *sR = reinterpret_cast<double *>(cut_smem), *sC = sR + D * C64LD, *sL = sC + D * C64LD;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   for (int i = tid; i < D * C64; i += 256) sR[(i >> 5) * C64LD + (i & 31)] = rt[(i >> 5) * Sr + row0 + (i & 31)];
-  double acc[8], e = 0.0;
+  double acc[NA], e = 0.0;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) acc[k] = 0.0;
+  for (int k = 0; k < NA; ++k) acc[k] = 0.0;
   const int gi = tid & 31, ga = tid >> 5;  // G: row gi, terms ga + 8 k
   for (int c0 = col0; c0 < col0 + cols; c0 += C64) {
     __syncthreads();
@@ -305,7 +353,7 @@ __global__ void __launch_bounds__(256) k_cut_contract64(const __grid_constant__ 
     if constexpr (GRAD) {
       __syncthreads();
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
+      for (int k = 0; k < NA; ++k) {
         const int a = ga + 8 * k;
         if (a < D) {
           double g0 = 0.0, g1 = 0.0;
@@ -322,7 +370,7 @@ __global__ void __launch_bounds__(256) k_cut_contract64(const __grid_constant__ 
   if constexpr (GRAD) {
     double *g = reinterpret_cast<double *>(J.ws + J.lay->g[h]) + (size_t)split * D * Sr;
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
+    for (int k = 0; k < NA; ++k)
       if (ga + 8 * k < D) g[(ga + 8 * k) * Sr + row0 + gi] = acc[k];
   }
   if (h == 0) {
@@ -341,44 +389,130 @@ __global__ void __launch_bounds__(256) k_cut_contract64(const __grid_constant__ 
   }
 }
 
+// Small registers with many terms (halves of at most 8 qubits): one CTA per row, so that the
+// FP64 pipes of many SMs share the work (n = 10, 256 terms: 64 CTAs where 32-row items
+// give 2).  psi of the row's columns with the terms split over the threads, then G with a
+// thread per term; the column table comes from L2 and stays in L1.
+template <bool GRAD>
+__global__ void __launch_bounds__(256) k_cut_rows64(const __grid_constant__ CutArgs A) {
+  __shared__ double row[256], lam[256], part[256], es[8];
+  int job, h, idx;
+  if (A.items) {
+    const int4 it = A.items[blockIdx.x];
+    job = it.x;
+    h = it.y;
+    idx = it.z;
+  } else {
+    job = blockIdx.x % A.njobs;
+    idx = blockIdx.x / A.njobs;
+    h = idx >= A.blk0;
+    if (h) idx -= A.blk0;
+  }
+  const CutView J = cut_view(A, job);
+  const int D = J.desc->D, m0 = J.desc->half[0].m, mr = J.desc->half[h].m, mc = J.desc->half[1 - h].m;
+  const int tid = threadIdx.x, cols = 1 << mc, j = tid & (cols - 1), np = 256 >> mc;
+  const double *rt = reinterpret_cast<const double *>(J.ws + J.lay->tab[h]);
+  const double *ct = reinterpret_cast<const double *>(J.ws + J.lay->tab[1 - h]);
+  if (tid < D) row[tid] = rt[((size_t)tid << mr) + idx];
+  __syncthreads();
+  double s0 = 0.0, s1 = 0.0;
+  for (int a = tid >> mc; a < D; a += 2 * np) {
+    s0 = fma(row[a], ct[((size_t)a << mc) + j], s0);
+    if (a + np < D) s1 = fma(row[a + np], ct[((size_t)(a + np) << mc) + j], s1);
+  }
+  part[tid] = s0 + s1;
+  __syncthreads();
+  double e = 0.0;
+  if (tid < cols) {
+    double s = part[tid];
+    for (int k = 1; k < np; ++k) s += part[k * cols + tid];
+    const long long i = idx, x = h ? ((i << m0) | tid) : (((long long)tid << m0) | i);
+    const double l = reinterpret_cast<const double *>(J.table)[x] * s;
+    e = l * s;
+    lam[tid] = l;
+  }
+  __syncthreads();
+  if constexpr (GRAD)
+    if (tid < D) {
+      const double2 *c = reinterpret_cast<const double2 *>(ct + ((size_t)tid << mc));
+      double g0 = 0.0, g1 = 0.0;
+#pragma unroll 8
+      for (int k = 0; k < cols / 2; ++k) {
+        const double2 x = c[k];
+        g0 = fma(lam[2 * k], x.x, g0);
+        g1 = fma(lam[2 * k + 1], x.y, g1);
+      }
+      reinterpret_cast<double *>(J.ws + J.lay->g[h])[((size_t)tid << mr) + idx] = g0 + g1;
+    }
+  if (h == 0) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if ((tid & 31) == 0) es[tid >> 5] = e;
+    __syncthreads();
+    if (tid == 0) {
+      double s = 0.0;
+      for (int w = 0; w < 8; ++w) s += es[w];
+      double *ep = reinterpret_cast<double *>(J.ws + J.lay->ep) + 2 * idx;
+      ep[0] = s;
+      ep[1] = 0.0;
+    }
+  }
+}
+
 // ------------------------------------------------------------ final sums --
-// One CTA per job: E and, per parameter, the sum over the path values in a fixed
-// order.  The FP32 contraction also sums psi^2: E and the gradients are divided by that
+// One CTA per job: E, and per parameter (a warp each) the sum over the path values, in a
+// fixed order.  The FP32 contraction also sums psi^2: E and the gradients are divided by that
 // norm, which takes the rounding of cos, sin and of the tensor cores' accumulation out
 // of the results to first order (it is 1 up to that rounding).
-__global__ void __launch_bounds__(256) k_cut_reduce(const __grid_constant__ CutArgs A, int prec, int grad) {
+constexpr int RED_NT = 512;
+__device__ __forceinline__ double warp_total(double x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+__global__ void __launch_bounds__(RED_NT) k_cut_reduce(const __grid_constant__ CutArgs A, int prec, int grad) {
   const CutView J = cut_view(A, blockIdx.x);
   const CutOut O = cut_out(A, blockIdx.x);
-  const int tid = threadIdx.x;
-  __shared__ double sh[2][256];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  constexpr int NW = RED_NT / 32;
+  __shared__ double sh[3][NW];
   const double *ep = reinterpret_cast<const double *>(J.ws + J.lay->ep);
+  const double *ex = reinterpret_cast<const double *>(J.ws + J.lay->exy);  // the X/Y strings', part by part
   const int ni = J.lay->rb[0] * J.lay->ns[0];
-  double e = 0.0, z = 0.0;
-  for (int i = tid; i < ni; i += 256) {
+  double e = 0.0, z = 0.0, x = 0.0;
+  for (int i = tid; i < ni; i += RED_NT) {
     e += ep[2 * i];
     z += ep[2 * i + 1];
   }
-  sh[0][tid] = e;
-  sh[1][tid] = z;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (tid < o) {
-      sh[0][tid] += sh[0][tid + o];
-      sh[1][tid] += sh[1][tid + o];
-    }
-    __syncthreads();
+  for (int i = tid; i < J.lay->nexy; i += RED_NT) x += ex[i];
+  e = warp_total(e);
+  z = warp_total(z);
+  x = warp_total(x);
+  if (lane == 0) {
+    sh[0][w] = e;
+    sh[1][w] = z;
+    sh[2][w] = x;
   }
-  const double inv = prec ? 1.0 : 1.0 / sh[1][0];
-  if (tid == 0) *O.E = sh[0][0] * inv;
+  __syncthreads();
+  e = z = x = 0.0;
+  for (int k = 0; k < NW; ++k) {
+    e += sh[0][k];
+    z += sh[1][k];
+    x += sh[2][k];
+  }
+  const double inv = prec ? 1.0 : 1.0 / z;
+  if (tid == 0) *O.E = (e + x) * inv;
   if (!grad) return;
-  const int n = J.desc->n, reps = J.desc->reps, D = J.desc->D, m0 = J.desc->half[0].m;
+  const int n = J.desc->n, reps = J.desc->reps, D = J.desc->D, m0 = J.desc->half[0].m, cx = J.desc->cx;
+  const int row = 16 << cx, per = n << cx;  // complex: RY then RZ of a layer
   const double *gp = reinterpret_cast<const double *>(J.ws + J.lay->gp);
-  for (int p = tid; p < n * (reps + 1); p += 256) {
-    const int r = p / n, q = p % n, h = q >= m0;
-    const double *src = gp + (size_t)h * D * (reps + 1) * 16 + r * 16 + (h ? q - m0 : q);
+  for (int p = w; p < per * (reps + 1); p += NW) {
+    const int r = p / per, zr = p % per >= n, q = p % per - zr * n, h = q >= m0;
+    const double *src = gp + (size_t)h * D * (reps + 1) * row + r * row + 16 * zr + (h ? q - m0 : q);
     double s = 0.0;
-    for (int a = 0; a < D; ++a) s += src[(size_t)a * (reps + 1) * 16];
-    O.grad[p] = (O.mask && !O.mask[p]) ? 0.0 : s * inv;
+    for (int a = lane; a < D; a += 32) s += src[(size_t)a * (reps + 1) * row];
+    s = warp_total(s);
+    if (lane == 0) O.grad[p] = (O.mask && !O.mask[p]) ? 0.0 : s * inv;
   }
 }
 
@@ -395,17 +529,21 @@ __global__ void __launch_bounds__(512) k_tile_table(const TableJob t0, const Tab
   for (int i = threadIdx.x; i < 128 * 128; i += 512)
     t[(i >> 7) * TT_LD + (i & 127)] = (float)src[((long long)(i >> 7) << T.m0) + (i & 127)];
   __syncthreads();
-  float4 *d0 = reinterpret_cast<float4 *>(T.d0 + ((long long)bl << (T.m1 + 7)) + bh * 16384);
-  for (int i = threadIdx.x; i < 4096; i += 512) {  // i = ((tile * 16 + j / 4) * 128 + row)
-    const int r = i & 127, j = 4 * (i >> 7);
-    const float *q = t + j * TT_LD + r;
-    d0[i] = make_float4(q[0], q[TT_LD], q[2 * TT_LD], q[3 * TT_LD]);
+  const int rb = 7 - T.cx, rm = (1 << rb) - 1;  // rows of a tile
+  float4 *d0 = reinterpret_cast<float4 *>(T.d0);
+  for (int i = threadIdx.x; i < 4096; i += 512) {  // ((row block * 2 + tile) * 16 + j / 4) * rows + row
+    const int row = i & rm, j = 4 * ((i >> rb) & 15), tile = (i >> (rb + 4)) & 1, blk = i >> (rb + 5);
+    const float *q = t + (64 * tile + j) * TT_LD + (blk << rb) + row;
+    const long long at = ((((long long)(bl << T.cx) + blk) << (T.m1 - 6)) + 2 * bh + tile) * (16 << rb) + (i & ((16 << rb) - 1));
+    d0[at] = make_float4(q[0], q[TT_LD], q[2 * TT_LD], q[3 * TT_LD]);
   }
   if (!T.d1) return;
-  float4 *d1 = reinterpret_cast<float4 *>(T.d1 + ((long long)bh << (T.m0 + 7)) + bl * 16384);
+  float4 *d1 = reinterpret_cast<float4 *>(T.d1);
   for (int i = threadIdx.x; i < 4096; i += 512) {
-    const float *q = t + (i & 127) * TT_LD + 4 * (i >> 7);
-    d1[i] = make_float4(q[0], q[1], q[2], q[3]);
+    const int row = i & rm, j = 4 * ((i >> rb) & 15), tile = (i >> (rb + 4)) & 1, blk = i >> (rb + 5);
+    const float *q = t + ((blk << rb) + row) * TT_LD + 64 * tile + j;
+    const long long at = ((((long long)(bh << T.cx) + blk) << (T.m0 - 6)) + 2 * bl + tile) * (16 << rb) + (i & ((16 << rb) - 1));
+    d1[at] = make_float4(q[0], q[1], q[2], q[3]);
   }
 }
 constexpr int TT_SMEM = 128 * TT_LD * 4;
@@ -430,11 +568,12 @@ cudaError_t launch_tile_tables(const TableJob *jobs, int njobs, int nmax, cudaSt
 // circuits: one class for every size that runs in one warp, one per size above.
 int cut_class(int prec, int m) { return m <= HALF_WARP_M(prec) ? HALF_WARP_M(prec) : m; }
 
-cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad, cudaStream_t s, int *launches) {
+cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
+                       const CutXyDims *xy) {
   CutArgs A = A0;
   const CutLayout &l = A.job0.lay;
   const int half_blocks = g.half_items ? g.half_blocks : A.njobs * 2 * g.D;
-  const int K = cut_k(g.D);
+  const int K = cut_k(g.D << g.cx);
   cudaError_t e;
 #define CUT_CHECK(x) \
   if ((e = (x)) != cudaSuccess) return e
@@ -443,34 +582,49 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
   if (prec) {
     CUT_CHECK(launch_half<double>(A, cut_class(1, g.m0), grad ? 1 : 0, half_blocks, s));
   } else {
-    CUT_CHECK(launch_half<float>(A, cut_class(0, g.m0), grad ? 1 : 0, half_blocks, s));
+    CUT_CHECK(g.cx ? launch_halfc(A, g.m0, grad ? 1 : 0, half_blocks, s)
+                   : launch_half<float>(A, cut_class(0, g.m0), grad ? 1 : 0, half_blocks, s));
     A.items = g.pack_items;
     A.blk0 = 1 << (g.m0 - 6);
     A.nblk = A.blk0 + (1 << (g.m1 - 6));
-    k_cut_pack<<<g.pack_items ? g.pack_blocks : A.njobs * A.nblk, 256, K * 65 * 4, s>>>(A, K);
+    auto k = g.cx ? k_cut_pack<true> : k_cut_pack<false>;
+    k<<<g.pack_items ? g.pack_blocks : A.njobs * A.nblk, 256, K * 65 * 4, s>>>(A, K);
     CUT_CHECK(cudaGetLastError());
     *launches += 1;
   }
   A.blk0 = l.rb[0] * l.ns[0];
   A.nblk = g.con_items ? g.con_blocks : A.njobs * (A.blk0 + (grad ? l.rb[1] * l.ns[1] : 0));
   A.items = g.con_items;
-  if (prec) {
-    auto k = grad ? k_cut_contract64<true> : k_cut_contract64<false>;
+  if (prec && cut_by_rows(g.m0, g.D)) {
+    auto k = grad ? k_cut_rows64<true> : k_cut_rows64<false>;
+    k<<<A.nblk, 256, 0, s>>>(A);
+    CUT_CHECK(cudaGetLastError());
+  } else if (prec) {
     const size_t sm = (size_t)8 * C64LD * (2 * g.D + (grad ? C64 : 0));
-    k<<<A.nblk, 256, sm, s>>>(A);
+    if (g.D <= 64) {
+      auto k = grad ? k_cut_contract64<true, 8> : k_cut_contract64<false, 8>;
+      k<<<A.nblk, 256, sm, s>>>(A);
+    } else {
+      static SmemLimit lim[2];
+      auto k = grad ? k_cut_contract64<true, 32> : k_cut_contract64<false, 32>;
+      CUT_CHECK(lim[grad].set(k, (size_t)8 * C64LD * (2 * 256 + C64)));
+      k<<<A.nblk, 256, sm, s>>>(A);
+    }
     CUT_CHECK(cudaGetLastError());
   } else {
     CUT_CHECK(launch_cut_tc(A, K, grad, s));
   }
   *launches += 3;
+  if (xy) CUT_CHECK(launch_cut_xy(A, g, *xy, grad, s, launches));
   if (grad) {
     A.blk0 = g.D;
     A.items = g.half_items;
     CUT_CHECK(prec ? launch_half<double>(A, cut_class(1, g.m0), 2, half_blocks, s)
+              : g.cx ? launch_halfc(A, g.m0, 2, half_blocks, s)
                    : launch_half<float>(A, cut_class(0, g.m0), 2, half_blocks, s));
     *launches += 1;
   }
-  k_cut_reduce<<<A.njobs, 256, 0, s>>>(A, prec, grad ? 1 : 0);
+  k_cut_reduce<<<A.njobs, RED_NT, 0, s>>>(A, prec, grad ? 1 : 0);
 #undef CUT_CHECK
   return cudaGetLastError();
 }

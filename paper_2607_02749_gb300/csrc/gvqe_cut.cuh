@@ -20,7 +20,8 @@
 namespace gvqe {
 
 constexpr int CUT_MAX_LAYERS = 6;  // entangler layers, each with at least one crossing CNOT
-constexpr int CUT_MAX_PATH = 6;    // crossing CNOTs in all: at most 64 terms
+constexpr int CUT_MAX_PATH = 6;    // FP32: crossing CNOTs in all, at most 64 terms
+constexpr int CUT_MAX_PATH64 = 8;  // FP64: at most 256
 constexpr int CUT_MAX_M = 15;      // qubits of a half
 
 // One entangler layer as seen by one half: the GF(2)-affine map of its basis indices
@@ -40,13 +41,15 @@ struct CutHalf {
 
 struct CutDesc {
   int n, reps, kappa, D;  // D = 2^kappa terms
+  int cx;                 // 1: RY then RZ (complex amplitudes), FP32
   CutHalf half[2];        // 0: qubits [0, h), 1: qubits [h, n)
 };
 
 // Workspace of one evaluation (byte offsets) and how its contractions are split.
 struct CutLayout {
   long long tab[2];   // L and R: [a][x], amplitude type; with gradients a second time in runs
-  long long pack[2];  // FP32: their tensor-core operand images
+  long long pack[2];  // FP32: their tensor-core operand images (as rows and as columns)
+  long long packr[2]; // complex: as rows, (x, channel) by two real terms per term; pack as columns
   long long phi[2];   // the half states after layers 0 .. reps - 1, one per value of the path bits so
                       // far: [x], then the same in runs
   long long g[2];     // partial contractions: [split][a][x]
@@ -54,6 +57,27 @@ struct CutLayout {
   long long ep;       // per item of contraction 0: energy and norm (doubles)
   long long total;
   int rb[2], ns[2];   // row blocks and column splits of each contraction
+  int gs[2];          // slices of g the backward adds up: ns, and one more with X/Y strings
+  // X/Y strings (gvqe_cut_xy.cu)
+  long long rows[2];   // the tables as [x][a]
+  long long mpart[2];  // M of every part: [run][part][a][b]
+  long long mm[2];     // ... summed, FP64
+  long long nn[2];     // N: [part][b][a] (-1 without gradients)
+  long long exy;       // energies per part of half 0 (doubles)
+  int xrun[2];         // rows in one run of M's sum
+  int nexy;            // parts of half 0 (0: no X/Y strings)
+};
+
+// The X/Y strings of a Hamiltonian as parts on the two halves (device arrays): part u of half
+// h flips xm and signs with zm; its strings t in [start[u], start[u + 1]) pair it with part
+// other[t] of the other half and carry coef[t].  Parts in order of xm; gstart: where xm changes.
+struct CutXyDims {
+  int U[2], ng[2];
+};
+struct CutXy : CutXyDims {
+  const uint32_t *xm[2], *zm[2];
+  const int *start[2], *other[2], *gstart[2];
+  const double *coef[2];
 };
 
 // The caller's buffers of one batch instance (read when the kernels run).
@@ -80,6 +104,7 @@ struct CutJob {
 
 struct CutArgs {
   CutJob job0;
+  const CutXy *xy;      // or NULL (diagonal H)
   const CutJob *jobs;   // NULL: job k is job0 stepped k times
   const int4 *items;    // with jobs: (job, half, index, 0) of each block of this launch
   long long ws_stride, cs_stride;  // bytes
@@ -90,14 +115,15 @@ struct CutArgs {
 
 // The cut plan of a circuit; false when it has none (no layer, too many layers or
 // crossing CNOTs, halves out of range).
-bool cut_build(int n, int reps, int ent, int prec, CutDesc *d);
-CutLayout cut_layout(const CutDesc &d, int prec, bool grad);
+bool cut_build(int n, int reps, int ent, int prec, int gates, CutDesc *d);
+CutLayout cut_layout(const CutDesc &d, int prec, bool grad, const CutXyDims *xy = nullptr);
 
 // What the launches of one evaluation cover: the largest half and number of terms, and,
 // for different problems in one launch, the blocks of the half circuits, of the operand
 // images and of the contraction.  Problems share launches when their larger halves have
 // the same cut_class.
 struct CutGrid {
+  int cx;        // complex amplitudes
   int m0, m1, D;  // m1: the smallest half
   int half_blocks, con_blocks, pack_blocks;
   const int4 *half_items, *con_items, *pack_items;  // (job, half, path value | index | 64-row tile, 0)
@@ -105,14 +131,18 @@ struct CutGrid {
 int cut_class(int prec, int m);
 int cut_k(int D);  // terms of the tensor-core operands
 // The kernels of one evaluation, in order.  `grad`: also the gradients.
-cudaError_t launch_cut(int prec, const CutArgs &A, const CutGrid &g, bool grad, cudaStream_t s, int *launches);
+cudaError_t launch_cut(int prec, const CutArgs &A, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
+                       const CutXyDims *xy = nullptr);
+int cut_xy_dp(int D);  // row length of its matrices
+cudaError_t launch_cut_xy(const CutArgs &A, const CutGrid &g, const CutXyDims &x, bool grad, cudaStream_t s, int *launches);
 // The diagonal table in the order the FP32 contractions read it, rounded from FP64:
 // d0 for contraction 0 (rows x_lo), d1 for contraction 1 (rows x_hi; may be NULL).  Tiles
-// of 128 rows x 64 columns, a row block's tiles after one another, each [j / 4][row][j % 4].
+// of 128 rows x 64 columns, a row block's tiles after one another, each [j / 4][row][j % 4]
+// (cx: the rows are (x, channel), and a tile holds one value for both channels, 64 rows).
 struct TableJob {
   const double *src;
   float *d0, *d1;
-  int m0, m1;
+  int m0, m1, cx;
 };
 // one table, or several at once (nmax: the largest m0 + m1)
 cudaError_t launch_tile_table(const TableJob &t, cudaStream_t s);
@@ -122,6 +152,7 @@ cudaError_t launch_tile_tables(const TableJob *jobs, int njobs, int nmax, cudaSt
 constexpr int HALF_WARP_M(int prec) { return prec ? 7 : 10; }  // largest half in one warp
 template <typename T>
 cudaError_t launch_half(const CutArgs &A, int m, int mode, int blocks, cudaStream_t s);
+cudaError_t launch_halfc(const CutArgs &A, int m, int mode, int blocks, cudaStream_t s);  // complex (gvqe_cut_halfc.cu)
 // A kernel's dynamic shared-memory limit, raised once per device.
 struct SmemLimit {
   std::atomic<uint64_t> done{0};

@@ -180,10 +180,13 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     if (h) idx -= A.blk0;
   }
   const CutView J = cut_view(A, job);
-  const int mr = J.desc->half[h].m, mc = J.desc->half[1 - h].m, D = J.desc->D;
+  // complex: rows (x, channel), two real terms per term, one value of E for both channels
+  const int cx = J.desc->cx;
+  const int mr = J.desc->half[h].m + cx, mc = J.desc->half[1 - h].m, D = J.desc->D << cx;
   const int ns = J.lay->ns[h], split = idx % ns, row0 = (idx / ns) * 128;
   const int nt = (1 << (mc - 6)) / ns, t0 = split * nt;
-  const float *ap = reinterpret_cast<const float *>(J.ws + J.lay->pack[h]);
+  const float *ap = reinterpret_cast<const float *>(J.ws + (cx ? J.lay->packr[h] : J.lay->pack[h]));
+  const int ap_ld = (cx ? 128 : 256) * K;  // floats per 64 rows
   const float *bp = reinterpret_cast<const float *>(J.ws + J.lay->pack[1 - h]);
   const float *E = reinterpret_cast<const float *>(h ? J.table_t : J.table);  // in tile order
   const uint32_t bar0 = smem_addr(bars);
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
   const uint32_t tw = tmem + ((uint32_t)(32 * (w & 3)) << 16);  // ... and lane quarter
   if (w < 4) {
     // the rows' operand: hi and lo parts into tensor memory
-    const float *src = ap + (size_t)((row0 + r) >> 6) * (256 * K) + ((r & 63) >> 3) * (K * 8) + (r & 7) * 4;
+    const float *src = ap + (size_t)((row0 + r) >> 6) * ap_ld + ((r & 63) >> 3) * (K * 8) + (r & 7) * 4;
 #pragma unroll
     for (int c = 0; c < 2 * K; c += 16) {
       const float *p = src + (c < K ? 0 : C::PARTS) + ((c % K) >> 2) * 32;
@@ -245,16 +248,17 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     float acc[K];
     const int g = w >> 2;
     // tile (row block, t): [j / 4][row][j % 4]
-    const float *Ei = E + ((size_t)(row0 >> 7) << (mc + 7)) + (size_t)t0 * (128 * COLS) + r * 4;
+    const int erow = 128 >> cx;
+    const float *Ei = E + ((size_t)(row0 >> 7) << mc) * erow + (size_t)t0 * (erow * COLS) + (r >> cx) * 4;
     float e_hi = 0.f, e_lo = 0.f, z_hi = 0.f, z_lo = 0.f;
     f2 tv[COLS / 2];
 #pragma unroll
     for (int k = 0; k < K; ++k) acc[k] = 0.f;
     auto load = [&](int t) {
-      const float *p = Ei + (size_t)t * (128 * COLS);
+      const float *p = Ei + (size_t)t * (erow * COLS);
 #pragma unroll
       for (int j = 0; j < COLS / 4; ++j)  // volatile: issued here, not where the values are used
-        asm volatile("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(tv[2 * j]), "=l"(tv[2 * j + 1]) : "l"(p + 512 * j));
+        asm volatile("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(tv[2 * j]), "=l"(tv[2 * j + 1]) : "l"(p + 4 * erow * j));
     };
     auto drain = [&](int t) {  // G of tile t
       if (!wait_warp(gbar(t % C::GBUFS), (t / C::GBUFS) & 1, bad)) return false;

@@ -125,7 +125,9 @@ struct gvqe_hamiltonian_s {
   void *d_ctr[2] = {nullptr, nullptr}, *d_cti[2] = {nullptr, nullptr};  // FP32, FP64
   double abs_sum = 0.0;
   gvqe::DevBuf T64, T32, G;
-  gvqe::DevBuf TT[2];  // FP32 tables in the tile order of the two-half contractions (gvqe_cut.cuh)
+  gvqe::CutXy xy{};          // the X/Y strings by halves (host copy of the device descriptor), built on first use
+  gvqe::DevBuf XY;
+  gvqe::DevBuf TT[2][2];  // [complex][contraction]: FP32 tables in the tile order of the two-half contractions
   gvqe::DevBuf TC[2];  // complex path: each table entry twice (re/im), FP32 and FP64
   uint32_t *d_gm = nullptr;
   int *d_gs = nullptr;
@@ -156,7 +158,7 @@ struct gvqe_ansatz_s {
   int mps = 0;                   // GVQE_OPT_MPS_LAYERS (0 auto, -1 none, 1..4 at most that many)
   int mps_tc = 0;                // GVQE_OPT_MPS_TENSOR (0 auto = tensor cores, -1 = FP32 pipe)
   std::map<int, gvqe::Plan> plans;
-  gvqe_cut_plan cut[2];          // per precision
+  gvqe_cut_plan cut[3];          // FP32, FP64, FP32 with RZ layers
   gvqe::DevBuf ws, aux, shift, ro, tune;
   std::string tune_report;  // the last gvqe_autotune sweep and its choice (empty: not tuned)
 };
@@ -177,9 +179,14 @@ Plan *get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state
 // The ansatz's two-half plan for this precision when its options and circuit let it take
 // the place of the tile passes for a diagonal H, else NULL.  cut_upload: its descriptor
 // on the device.  ensure_cut_tables: what its contraction reads of the Hamiltonian.
-gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec);
+// vectors, grad: of the call.
+gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad);
 int cut_upload(gvqe_cut_plan *c);
 int ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool grad, cudaStream_t s);
+// The X/Y strings split into parts on the halves (host only); and whether their two-half
+// evaluation is the cheaper one.
+void split_xy(const gvqe_hamiltonian_s *h, int m0, CutXyDims *dims, std::vector<uint32_t> *xm, std::vector<uint32_t> *zm,
+              std::vector<int> *start, std::vector<int> *other, std::vector<double> *coef, std::vector<int> *gstart);
 // Energies (and adjoint gradients when grad != NULL) of a batch: the body of
 // gvqe_energy / gvqe_energy_grad after their argument checks.
 int energy_impl(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const double *params, const uint8_t *mask, int batch,

@@ -95,3 +95,83 @@ def test_many_items_and_vectors(n, reps, ent, batch, fp64):
     assert rel <= (1e-12 if fp64 else 5e-6)
     _, e1, g1, _ = _run(n, reps, ent, ham, th[1:2], fp64, mask=mask[1:2])
     assert e1[0] == e[1] and np.array_equal(g1[0], g[1])
+
+
+@pytest.mark.parametrize("n,reps,ent,batch", [(14, 1, gv.GVQE_ENT_LINEAR, 2), (15, 3, gv.GVQE_ENT_CIRCULAR, 1),
+                                              (16, 4, gv.GVQE_ENT_PAIRWISE, 3), (17, 5, gv.GVQE_ENT_FULL, 2),
+                                              (19, 2, gv.GVQE_ENT_SCA, 2), (21, 5, gv.GVQE_ENT_LINEAR, 2)])
+def test_xy_strings(n, reps, ent, batch):
+    """X/Y strings as parts on the halves: 8 to 64 terms, even and odd numbers of Y on a
+    half, parts shared by many strings, uneven halves; also no I/Z string at all."""
+    for fraction in (0.6, 1.0):
+        ham = wl.pauli_hamiltonian(n, 40 * n, seed=n, xy_fraction=fraction)
+        th = wl.thetas(n, reps, batch, seed=n + 5)
+        e0, e, g, _ = _run(n, reps, ent, ham, th, False)
+        _, et, gt, _ = _run(n, reps, ent, ham, th, False, mps=-1)
+        scale = ham.abs_sum()
+        assert np.max(np.abs(e - et)) <= 1e-6 * scale and np.max(np.abs(e0 - et)) <= 1e-6 * scale
+        rel = np.linalg.norm(g - gt) / np.linalg.norm(gt)
+        print(f"n={n} reps={reps} ent={ent} xy={fraction}: vs tile passes grad {rel:.2e}, E {np.max(np.abs(e - et)) / scale:.1e}")
+        assert rel <= 5e-6
+        if n <= 16:
+            with oracle.entangler(ent):
+                er, gr = oracle.energy_grad(n, reps, th[0], ham.strings, ham.coeffs)
+            assert abs(e[0] - er) <= 2e-5 * scale
+            assert np.linalg.norm(g[0] - gr) <= 1e-4 * np.linalg.norm(gr)
+
+
+@pytest.mark.parametrize("n,reps,ent", [(14, 1, gv.GVQE_ENT_LINEAR), (15, 3, gv.GVQE_ENT_REVERSE_LINEAR), (16, 2, gv.GVQE_ENT_CIRCULAR),
+                                        (17, 4, gv.GVQE_ENT_PAIRWISE), (18, 2, gv.GVQE_ENT_SCA), (19, 5, gv.GVQE_ENT_FULL),
+                                        (20, 3, gv.GVQE_ENT_LINEAR), (21, 3, gv.GVQE_ENT_LINEAR), (23, 2, gv.GVQE_ENT_LINEAR),
+                                        (26, 3, gv.GVQE_ENT_LINEAR), (27, 2, gv.GVQE_ENT_LINEAR)])
+def test_su2_layers(n, reps, ent):
+    """Full EfficientSU2 layers (complex amplitudes, FP32): every register-round layout of the
+    complex half circuits (8 to 15 index bits), uneven halves, 4 to 64 real terms, masks."""
+    ham = wl.z_hamiltonian(n, 6 * n, seed=n)
+    batch = 2
+    P = 2 * n * (reps + 1)
+    th = np.random.default_rng(n).uniform(-np.pi, np.pi, (batch, P))
+    mask = wl.active_mask(P, batch, seed=n + 1)
+    out = []
+    for mps in (0, -1):
+        a = gv.Ansatz(n, reps, entangler=ent, gates=gv.GVQE_GATES_RY_RZ)
+        a.set_mps_layers(mps)
+        h = gv.Hamiltonian.from_workload(ham)
+        t = torch.as_tensor(th, device="cuda")
+        e0 = gv.energy(a, h, t).cpu().numpy()
+        e, g = gv.energy_grad(a, h, t, mask=torch.as_tensor(mask, device="cuda"))
+        out.append((e0, e.cpu().numpy(), g.cpu().numpy()))
+        assert ("terms" in a.describe()) == (mps == 0)
+        a.close()
+        h.close()
+    (e0, e, g), (_, et, gt) = out
+    scale = ham.abs_sum()
+    assert np.all(g[mask == 0] == 0.0)
+    assert np.max(np.abs(e - et)) <= 1e-6 * scale and np.max(np.abs(e0 - et)) <= 1e-6 * scale
+    rel = np.linalg.norm(g - gt) / np.linalg.norm(gt)
+    print(f"n={n} reps={reps} ent={ent}: vs tile passes grad {rel:.2e}, E {np.max(np.abs(e - et)) / scale:.1e}")
+    assert rel <= 5e-6
+    if n <= 16:
+        with oracle.entangler(ent), oracle.gates(oracle.GATES_RY_RZ):
+            er, gr = oracle.energy_grad(n, reps, th[0], ham.strings, ham.coeffs)
+        gr = np.where(mask[0] == 1, gr, 0.0)
+        assert abs(e[0] - er) <= 2e-5 * scale
+        assert np.linalg.norm(g[0] - gr) <= 1e-4 * np.linalg.norm(gr)
+
+
+@pytest.mark.parametrize("n,reps,ent,batch", [(10, 4, gv.GVQE_ENT_CIRCULAR, 1), (11, 4, gv.GVQE_ENT_SCA, 2), (12, 3, gv.GVQE_ENT_CIRCULAR, 1),
+                                              (13, 4, gv.GVQE_ENT_CIRCULAR, 1), (16, 4, gv.GVQE_ENT_CIRCULAR, 1),
+                                              (15, 3, gv.GVQE_ENT_SCA, 1), (12, 4, gv.GVQE_ENT_CIRCULAR, 64)])
+def test_fp64_many_terms(n, reps, ent, batch):
+    """FP64 with 64 and 256 terms on small registers (a CTA per row of the contraction); with
+    many vectors the tile passes keep the call."""
+    ham = wl.z_hamiltonian(n, 8 * n, seed=n)
+    th = wl.thetas(n, reps, batch, seed=n)
+    e0, e, g, _ = _run(n, reps, ent, ham, th, True)
+    _, et, gt, _ = _run(n, reps, ent, ham, th, True, mps=-1)
+    scale = ham.abs_sum()
+    assert np.max(np.abs(e - et)) <= 1e-12 * scale and np.max(np.abs(e0 - et)) <= 1e-12 * scale
+    assert np.linalg.norm(g - gt) <= 1e-12 * np.linalg.norm(gt)
+    with oracle.entangler(ent):
+        er, gr = oracle.energy_grad(n, reps, th[0], ham.strings, ham.coeffs)
+    assert abs(e[0] - er) <= 1e-10 * scale and np.max(np.abs(g[0] - gr)) <= 1e-9 * scale
