@@ -8,18 +8,23 @@
 // as tcgen05.mma kind::tf32 with FP32 accumulators.  Every operand is split into two
 // TF32 parts (x_hi and x_lo = x - x_hi exactly, its last bits cut by the tensor core:
 // about 2^-22 of x), and each product is x_lo y_hi + x_hi y_lo + x_hi y_hi, the small parts
-// first so that they meet a small accumulator.  The tables' x_hi is rounded to nearest, so
+// first so that they meet a small accumulator.  S takes two accumulators, the second half of
+// the full-size steps in one of its own: they round toward zero at every step, and what that
+// does to E shows where E is near zero.  The tables' x_hi is rounded to nearest, so
 // that x_lo has no sign of its own and the dropped x_lo y_lo averages out; lambda's x_hi is
-// cut (one instruction).  The accumulators round toward zero, so G is taken out after every
-// tile (8 full-size steps) and summed on the FP32 pipe.
+// cut (one instruction).  For the same reason G is taken out after every tile (8 full-size
+// steps) and summed on the FP32 pipe.
 //
 // Both A operands (the rows, and lambda) sit in tensor memory: lambda never touches shared
-// memory, its high part overwrites S in place, and the MMAs read only B from shared
+// memory, its parts overwrite the two of S in place, and the MMAs read only B from shared
 // memory (64 bytes per clock of its 128).  B comes in ready-made operand images
-// (k_cut_fwd) by one bulk copy per tile, E from tables in tile order (k_tile_table), 16
-// coalesced 16-byte loads per thread straight into registers two tiles ahead.  Warps 0-3
-// and 4-7 take alternate tiles, a row per thread; warp 8 copies, warps 9 and 10 issue the MMAs.
-// Warps 8-11 hand their registers to the others.
+// (k_cut_pack) by bulk copies, E in tile order (k_tile_table).  Warps 0-3 and 4-7 take
+// alternate tiles, a row per thread; warps 8 and 11 copy, 9 and 10 issue the MMAs.
+// E is loaded straight into registers two tiles ahead (16 coalesced 16-byte loads a thread; warps
+// 8-11 hand their registers over) up to 32 terms, and copied into shared memory at 64 terms,
+// where the sums of G take the registers: one vector of 30 qubits, 64 terms, 2.20 ms with loads and
+// 2.03 ms with copies; 24 qubits, 16 terms, 0.303 and 0.369 ms (each tile then waits
+// for a second barrier).
 #include "gvqe_cut.cuh"
 
 namespace gvqe {
@@ -87,9 +92,9 @@ __device__ __forceinline__ void st_wait() { asm volatile("tcgen05.wait::st.sync.
 // (every MMA and copy completes, so neither is expected).
 __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, volatile int *bad) {
   uint32_t done = 0;
-  for (int it = 0; it < (1 << 22) && !done; ++it) {
+  for (int it = 0; it < (1 << 16) && !done; ++it) {  // (each sleeps up to 20 us in hardware: about a second)
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, 20000;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
@@ -149,7 +154,8 @@ template <int K>
 struct Cfg {
   static constexpr int BUFS = K <= 16 ? 3 : 2;   // S / lambda buffers
   static constexpr int GBUFS = K <= 32 ? 4 : 2;  // G buffers: two per warp group where they fit
-  static constexpr int STAGES = K <= 32 ? 4 : 3;
+  // stages of the copies: the row-form and column-form halves of B (freed by S and by G), and E
+  static constexpr int RS = K <= 32 ? 4 : 2, CS = K <= 32 ? 4 : 2, ES = K <= 32 ? 0 : 3;
   // tensor-memory columns
   static constexpr int A_HI = 0, A_LO = K, S0 = 2 * K, G0 = S0 + 128 * BUFS;
   static_assert(G0 + GBUFS * K <= 512, "tensor memory");
@@ -159,9 +165,12 @@ struct Cfg {
 template <int K, bool GRAD>
 __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant__ CutArgs A) {
   using C = Cfg<K>;
-  constexpr int STAGE_F = (GRAD ? 4 : 2) * C::PARTS;
+  constexpr int HALF = 2 * C::PARTS;  // floats of one half of B: its hi and lo parts
+  constexpr int ETILE = 128 * COLS;   // floats of a tile of E (complex: half of them used)
+  constexpr int ES = C::ES;
   extern __shared__ __align__(128) float dyn[];
-  __shared__ __align__(8) unsigned long long bars[2 * C::STAGES + 2 * C::BUFS + C::GBUFS];
+  float *sR = dyn, *sE = dyn + C::RS * HALF, *sC = sE + ES * ETILE;
+  __shared__ __align__(8) unsigned long long bars[2 * (C::RS + C::CS + ES) + 2 * C::BUFS + C::GBUFS];
   __shared__ uint32_t tslot;
   __shared__ int bad_s;
   __shared__ double es[2][8];
@@ -190,26 +199,32 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
   const float *bp = reinterpret_cast<const float *>(J.ws + J.lay->pack[1 - h]);
   const float *E = reinterpret_cast<const float *>(h ? J.table_t : J.table);  // in tile order
   const uint32_t bar0 = smem_addr(bars);
-  auto full = [&](int s) { return bar0 + 8 * s; };
-  auto empty = [&](int s) { return bar0 + 8 * (C::STAGES + s); };
-  auto sbar = [&](int b) { return bar0 + 8 * (2 * C::STAGES + b); };
-  auto lbar = [&](int b) { return bar0 + 8 * (2 * C::STAGES + C::BUFS + b); };
-  auto gbar = [&](int b) { return bar0 + 8 * (2 * C::STAGES + 2 * C::BUFS + b); };
+  // per stage a full barrier, then the empty ones
+  auto rfull = [&](int s) { return bar0 + 8 * s; };
+  auto rempty = [&](int s) { return rfull(C::RS + s); };
+  auto cfull = [&](int s) { return rfull(2 * C::RS + s); };
+  auto cempty = [&](int s) { return cfull(C::CS + s); };
+  auto efull = [&](int s) { return cfull(2 * C::CS + s); };
+  auto eempty = [&](int s) { return efull(ES + s); };
+  auto sbar = [&](int b) { return efull(2 * ES + b); };
+  auto lbar = [&](int b) { return sbar(C::BUFS + b); };
+  auto gbar = [&](int b) { return lbar(C::BUFS + b); };
   if (w == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(&tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 256) {
     bad_s = 0;
-    for (int s = 0; s < C::STAGES; ++s) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full(s)));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(empty(s)));
-    }
+    auto init = [](uint32_t bar, int count) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
+    };
+    for (int s = 0; s < 2 * C::RS + 2 * C::CS + ES; ++s) init(bar0 + 8 * s, 1);
+    for (int s = 0; s < ES; ++s) init(eempty(s), 4);
     for (int b = 0; b < C::BUFS; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sbar(b)));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(lbar(b)));
+      init(sbar(b), 1);
+      init(lbar(b), 4);
     }
-    for (int b = 0; b < C::GBUFS; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(gbar(b)));
+    for (int b = 0; b < C::GBUFS; ++b) init(gbar(b), 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -242,24 +257,28 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
   __syncthreads();
   fence_after();
 
+  if constexpr (!ES) {
+    if (w < 8)
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
+    else
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+  }
   if (w < 8) {
     // ------------------------------------------------------------ rows --
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
     float acc[K];
     const int g = w >> 2;
-    // tile (row block, t): [j / 4][row][j % 4]
-    const int erow = 128 >> cx;
-    const float *Ei = E + ((size_t)(row0 >> 7) << mc) * erow + (size_t)t0 * (erow * COLS) + (r >> cx) * 4;
     float e_hi = 0.f, e_lo = 0.f, z_hi = 0.f, z_lo = 0.f;
-    f2 tv[COLS / 2];
-#pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] = 0.f;
+    const int erow = 128 >> cx;  // rows of a tile of E: [j / 4][row][j % 4]
+    const float *Ei = E + ((((size_t)(row0 >> 7) << (mc - 6)) + t0)) * (erow * COLS) + (r >> cx) * 4;
+    f2 ev[ES ? 1 : COLS / 2];
     auto load = [&](int t) {
       const float *p = Ei + (size_t)t * (erow * COLS);
 #pragma unroll
       for (int j = 0; j < COLS / 4; ++j)  // volatile: issued here, not where the values are used
-        asm volatile("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(tv[2 * j]), "=l"(tv[2 * j + 1]) : "l"(p + 4 * erow * j));
+        asm volatile("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(ev[2 * j]), "=l"(ev[2 * j + 1]) : "l"(p + 4 * erow * j));
     };
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k] = 0.f;
     auto drain = [&](int t) {  // G of tile t
       if (!wait_warp(gbar(t % C::GBUFS), (t / C::GBUFS) & 1, bad)) return false;
       fence_after();
@@ -276,25 +295,40 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     };
     constexpr int AHEAD = C::GBUFS == 4 ? 2 : 0;  // tiles between a tile's lambda and its G
     const f2 neg1 = pk2(-1.f, -1.f);
-    if (g < nt) load(g);
     int t = g;
+    if constexpr (!ES) load(t);  // (2 tiles at least)
     for (; t < nt; t += 2) {
-      const int b = t % C::BUFS;
+      const int b = t % C::BUFS, ee = ES ? t % (ES + !ES) : 0;
+      if constexpr (ES > 0)
+        if (!wait_warp(efull(ee), (t / ES) & 1, bad)) break;
       if (!wait_warp(sbar(b), (t / C::BUFS) & 1, bad)) break;
       fence_after();
       const uint32_t ts = tw + C::S0 + 128 * b;
+      const float4 *et = reinterpret_cast<const float4 *>(sE + ee * ETILE) + (r >> cx);
       f2 e0 = 0, e1 = 0, z0 = 0, z1 = 0;
       auto tile = [&](auto energy) {
-#pragma unroll
+#pragma unroll(ES ? 1 : COLS / 16)
         for (int c = 0; c < COLS; c += 16) {
-          float v[16];
-          [[maybe_unused]] float l[16];
+          float v[16], l[16];
+          f2 tv[8];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if constexpr (ES > 0) {
+              const float4 x = et[(c / 4 + k) * erow];
+              tv[2 * k] = pk2(x.x, x.y);
+              tv[2 * k + 1] = pk2(x.z, x.w);
+            } else {
+              tv[2 * k] = ev[c / 2 + 2 * k];
+              tv[2 * k + 1] = ev[c / 2 + 2 * k + 1];
+            }
+          }
           ld16(ts + c, v);
+          ld16(ts + 64 + c, l);
           ld_wait();
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
-            const f2 s = pk2(v[j], v[j + 1]);
-            const f2 lam = mul2(s, tv[(c + j) / 2]);
+            const f2 s = add2(pk2(v[j], v[j + 1]), pk2(l[j], l[j + 1]));
+            const f2 lam = mul2(s, tv[j / 2]);
             if constexpr (decltype(energy)::value) {
               f2 &e = (j & 2) ? e1 : e0, &z = (j & 2) ? z1 : z0;
               e = fma2(lam, s, e);
@@ -320,8 +354,12 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
       if constexpr (GRAD) st_wait();
       fence_before();
       __syncwarp();
-      if (lane == 0) arrive(lbar(b));
-      if (t + 2 < nt) load(t + 2);
+      if (lane == 0) {
+        arrive(lbar(b));
+        if constexpr (ES > 0) arrive(eempty(ee));
+      }
+      if constexpr (!ES)
+        if (t + 2 < nt) load(t + 2);
       if (h == 0) {
         float x, y;
         unpk2(add2(e0, e1), x, y);
@@ -371,27 +409,40 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
       ep[0] = good ? e : __longlong_as_double(0x7ff8000000000000ll);
       ep[1] = good ? z : 1.0;
     }
-  } else {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
-  }
-  if (w == 8) {
+  } else if (w == 8 || w == 11) {
     // ---------------------------------------------------------- copies --
     if (lane == 0) {
-      const float *src = bp + (size_t)t0 * (256 * K);
-      for (int t = 0; t < nt; ++t) {
-        const int s = t % C::STAGES;
-        if (t >= C::STAGES && !wait_bounded(empty(s), (t / C::STAGES - 1) & 1, bad)) break;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full(s)), "r"(STAGE_F * 4)
+      auto copy = [&](float *dst, const float *src, uint32_t bytes, uint32_t bar) {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         smem_addr(dst)),
+                     "l"(src), "r"(bytes), "r"(bar)
                      : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                smem_addr(dyn + s * STAGE_F)),
-            "l"(src + (size_t)t * (256 * K)), "r"(STAGE_F * 4), "r"(full(s))
-            : "memory");
+      };
+      const float *bt = bp + (size_t)t0 * (256 * K);
+      const int et = ETILE >> cx;
+      const float *Ei = E + ((((size_t)(row0 >> 7) << (mc - 6)) + t0)) * et;
+      if (w == 8) {
+        for (int t = 0; t < nt; ++t) {
+          const int s = t % C::RS;
+          if (t >= C::RS && !wait_bounded(rempty(s), (t / C::RS - 1) & 1, bad)) break;
+          copy(sR + s * HALF, bt + (size_t)t * (256 * K), HALF * 4, rfull(s));
+          if constexpr (ES > 0) {
+            const int e = t % ES;
+            if (t >= ES && !wait_bounded(eempty(e), (t / ES - 1) & 1, bad)) break;
+            copy(sE + e * ETILE, Ei + (size_t)t * et, et * 4, efull(e));
+          }
+        }
+        // the last commits have arrived before the CTA leaves
+        for (int t = nt > C::RS ? nt - C::RS : 0; t < nt; ++t) wait_bounded(rempty(t % C::RS), (t / C::RS) & 1, bad);
+      } else if (GRAD) {
+        for (int t = 0; t < nt; ++t) {
+          const int s = t % C::CS;
+          if (t >= C::CS && !wait_bounded(cempty(s), (t / C::CS - 1) & 1, bad)) break;
+          copy(sC + s * HALF, bt + (size_t)t * (256 * K) + HALF, HALF * 4, cfull(s));
+        }
+        for (int t = nt > C::CS ? nt - C::CS : 0; t < nt; ++t) wait_bounded(cempty(t % C::CS), (t / C::CS) & 1, bad);
       }
-      // the last commits have arrived before the CTA leaves
-      for (int t = nt > C::STAGES ? nt - C::STAGES : 0; t < nt; ++t)
-        wait_bounded(empty(t % C::STAGES), (t / C::STAGES) & 1, bad);
     }
   } else if (w == 9 || w == 10) {
     // ------------------------------------------------------------ MMAs --
@@ -402,31 +453,31 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     uint32_t el;
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(el));
     const uint32_t tu = __shfl_sync(0xffffffffu, tmem, 0);
-    const uint32_t dyn0 = smem_addr(dyn);
     if (el && w == 9) {
       for (int t = 0; t < nt; ++t) {
-        const int s = t % C::STAGES, b = t % C::BUFS, u = t - C::BUFS;
-        if (!wait_bounded(full(s), (t / C::STAGES) & 1, bad)) break;
+        const int s = t % C::RS, b = t % C::BUFS, u = t - C::BUFS;
+        if (!wait_bounded(rfull(s), (t / C::RS) & 1, bad)) break;
         // the buffer's previous tile: its lambda has been contracted (or, energies only, read)
         if (u >= 0 && !(GRAD ? wait_bounded(gbar(u % C::GBUFS), (u / C::GBUFS) & 1, bad)
                              : wait_bounded(lbar(b), (u / C::BUFS) & 1, bad)))
           break;
         fence_after();
-        const uint32_t bs = dyn0 + s * (STAGE_F * 4), d = tu + C::S0 + 128 * b;
+        const uint32_t bs = smem_addr(sR) + s * (HALF * 4), d = tu + C::S0 + 128 * b;
         const uint32_t bh = op_lo(bs), bl = op_lo(bs + C::PARTS * 4);
         constexpr uint32_t HI = op_hi(K * 32), ID = idesc(COLS);
         mmas<HI, ID, true, K / 8>(d, tu + C::A_LO, bh);
         mmas<HI, ID, false, K / 8>(d, tu + C::A_HI, bl);
-        mmas<HI, ID, false, K / 8>(d, tu + C::A_HI, bh);
+        mmas<HI, ID, false, K / 16>(d, tu + C::A_HI, bh);
+        mmas<HI, ID, true, K / 16>(d + 64, tu + C::A_HI + K / 2, bh + K);  // (16 per step of 8)
         commit(sbar(b));
-        if (!GRAD) commit(empty(s));
+        commit(rempty(s));
       }
     } else if (GRAD && el && w == 10) {
       for (int t = 0; t < nt; ++t) {
-        const int s = t % C::STAGES, b = t % C::BUFS;
-        if (!wait_bounded(lbar(b), (t / C::BUFS) & 1, bad)) break;
+        const int s = t % C::CS, b = t % C::BUFS;
+        if (!wait_bounded(cfull(s), (t / C::CS) & 1, bad) || !wait_bounded(lbar(b), (t / C::BUFS) & 1, bad)) break;
         fence_after();
-        const uint32_t bs = dyn0 + s * (STAGE_F * 4) + 2 * C::PARTS * 4;
+        const uint32_t bs = smem_addr(sC) + s * (HALF * 4);
         const uint32_t lh = tu + C::S0 + 128 * b, ll = lh + 64, d = tu + C::G0 + K * (t % C::GBUFS);
         const uint32_t bh = op_lo(bs), bl = op_lo(bs + C::PARTS * 4);
         constexpr uint32_t HI = op_hi(2048), ID = idesc(K);
@@ -434,7 +485,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
         mmas<HI, ID, false, COLS / 8>(d, lh, bl);
         mmas<HI, ID, false, COLS / 8>(d, lh, bh);
         commit(gbar(t % C::GBUFS));
-        commit(empty(s));
+        commit(cempty(s));
       }
     }
   }
@@ -446,8 +497,12 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
   // flight are waited for before leaving
   if (bad_s && tid == 256) {
     int none = 0;
-    for (int s = 0; s < C::STAGES; ++s)
-      for (int p = 0; p < 2; ++p) wait_bounded(full(s), p, &none);
+    for (int s = 0; s < C::RS; ++s)
+      for (int p = 0; p < 2; ++p) wait_bounded(rfull(s), p, &none);
+    for (int s = 0; s < ES; ++s)
+      for (int p = 0; p < 2; ++p) wait_bounded(efull(s), p, &none);
+    for (int s = 0; GRAD && s < C::CS; ++s)
+      for (int p = 0; p < 2; ++p) wait_bounded(cfull(s), p, &none);
   }
   __syncthreads();
   if (w == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
@@ -455,8 +510,9 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
 
 template <int K, bool GRAD>
 cudaError_t launch_k(const CutArgs &A, cudaStream_t s) {
-  const size_t smem = (size_t)Cfg<K>::STAGES * (GRAD ? 4 : 2) * Cfg<K>::PARTS * 4;
-  const size_t need = GRAD && smem < (size_t)K * 512 ? (size_t)K * 512 : smem;
+  using C = Cfg<K>;
+  // (the copies' stages, then reused for the rows' sums: K x 128 floats)
+  const size_t need = (size_t)4 * ((C::RS + (GRAD ? C::CS : 0)) * 2 * C::PARTS + C::ES * 128 * COLS);
   auto k = k_cut_contract_tc<K, GRAD>;
   static SmemLimit limit;
   if (const cudaError_t e = limit.set(k, need)) return e;
