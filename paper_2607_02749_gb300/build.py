@@ -23,7 +23,7 @@ LIB = os.path.join(HERE, "libgvqe.so")
 LIB_DEBUG = os.path.join(HERE, "libgvqe_debug.so")
 SOURCES = ["gvqe_api.cu", "gvqe_kernels.cu", "gvqe_static.cu", "gvqe_batch.cu", "gvqe_grad_l0.cu", "gvqe_readout.cu",
            "gvqe_graph.cu", "gvqe_tune.cu", "gvqe_mps.cu", "gvqe_cut.cu", "gvqe_cut_tc.cu", "gvqe_cut_xy.cu",
-           "gvqe_cut_halfc.cu"]
+           "gvqe_cut_halfc.cu", "gvqe_cut_fwd.cu"]
 # gvqe_inst.cu is compiled once per (amplitude type, tile bits) pair, gvqe_cut_half.cu once per type
 INSTANCES = [("float", tb) for tb in (10, 11, 12, 13)] + [("double", tb) for tb in (10, 11, 12)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

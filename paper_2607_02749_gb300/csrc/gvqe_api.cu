@@ -1498,8 +1498,15 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
   A.job0.table_t = prec ? nullptr : h->TT[c->d.cx][1].ptr;
   A.job0.ws = (char *)a->ws.ptr;
   A.ws_stride = (long long)per_job;
-  A.cs_stride = (long long)P * (prec ? 16 : 8);
+  A.cs_stride = (long long)P * 16;
   A.P = P;
+  CutGrid grid{};
+  grid.cx = c->d.cx;
+  grid.m0 = c->d.half[0].m;
+  grid.m1 = c->d.half[1].m;
+  grid.D = c->d.D;
+  grid.reps = c->d.reps;
+  for (int r = 1; r <= c->d.reps; ++r) grid.bits[r] = c->d.half[0].L[r - 1].shift + c->d.half[0].L[r - 1].nb;
   for (int j0 = 0; j0 < batch; j0 += J) {
     A.njobs = std::min(J, batch - j0);
     A.job0.cs = (const char *)cs + (long long)j0 * A.cs_stride;
@@ -1507,7 +1514,7 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
     A.job0.E = E + j0;
     A.job0.grad = grad ? grad + (size_t)j0 * P : nullptr;
     int nl = 0;
-    GV_CUDA(launch_cut(prec, A, CutGrid{c->d.cx, c->d.half[0].m, c->d.half[1].m, c->d.D, 0, 0, 0, nullptr, nullptr, nullptr}, grad != nullptr, s, &nl, xy ? &h->xy : nullptr));
+    GV_CUDA(launch_cut(prec, A, grid, grad != nullptr, s, &nl, xy ? &h->xy : nullptr));
     count_launches(nl);
   }
   return GVQE_OK;
@@ -1533,8 +1540,8 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
     GV_TRY(ensure_cut_tables(h, prec, c->d, grad != nullptr, s));
     if (!diag) GV_TRY(ensure_cut_xy(h, c->d.half[0].m));
     const long long count = (long long)batch * a->gates * a->n * (a->reps + 1);
-    GV_TRY(a->aux.reserve((size_t)count * (prec ? 16 : 8)));
-    GV_CUDA(launch_trig(prec, params, count, a->aux.ptr, s));
+    GV_TRY(a->aux.reserve((size_t)count * 16));
+    GV_CUDA(launch_trig(1, params, count, a->aux.ptr, s));
     count_launches(1);
     return run_cut(a, h, c, a->aux.ptr, mask, batch, E, grad, prec, s);
   }

@@ -729,7 +729,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
       CutJob job{};
       job.lay = cut_layout(d, prec, want_grad != 0);
       cut_cs[k] = off;
-      off = up256(off + (size_t)d.n * (d.reps + 1) * 2 * es);
+      off = up256(off + (size_t)d.n * (d.reps + 1) * 16);
       off = up256(off + (size_t)job.lay.total);
       if (!prec && cut_tt.find(H_of(k)) == cut_tt.end()) {
         cut_tt[H_of(k)] = off;
@@ -739,6 +739,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
       g.grid.m0 = std::max(g.grid.m0, d.half[0].m);
       g.grid.m1 = g.jobs.empty() ? d.half[1].m : std::min(g.grid.m1, d.half[1].m);
       g.grid.D = std::max(g.grid.D, d.D);
+      g.grid.reps = std::max(g.grid.reps, d.reps);
       for (int h = 0; h < 2; ++h) {
         for (int a = 0; a < d.D; ++a) g.half.push_back(make_int4(j, h, a, 0));
         if (!prec)
@@ -810,7 +811,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
     for (size_t j = 0; j < g.slots.size(); ++j) {
       const int k = g.slots[j];
       const CutDesc &d = g.desc[j];
-      const size_t cs_bytes = (size_t)d.n * (d.reps + 1) * 2 * es;
+      const size_t cs_bytes = (size_t)d.n * (d.reps + 1) * 16;
       CutJob &job = g.jobs[j];
       job.desc = (const CutDesc *)(base + g.o_desc) + j;
       job.cs = base + cut_cs[k];
@@ -969,7 +970,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
         if (le != cudaSuccess) break;
         streams.push_back(gs);
         le = cudaStreamWaitEvent(gs, cfork, 0);
-        if (le == cudaSuccess) le = launch_stage_tb(prec, 12, B, d_ids + at, 1, J, 0, gs);
+        if (le == cudaSuccess) le = launch_stage_tb(1, 12, B, d_ids + at, 1, J, 0, gs);  // (FP64 cos and sin)
         at += J;
         CutArgs A{};
         A.jobs = (const CutJob *)(base + g.o_jobs);

@@ -175,14 +175,17 @@ CutLayout cut_layout(const CutDesc &d, int prec, bool grad, const CutXyDims *xy)
     // set-up (its rows into tensor memory, the first tiles) stays small
     const long long per = prec ? 8 : 32;
     l.ns[s] = prec && cut_by_rows(d) ? 1 : (int)(tiles / per < 1 ? 1 : tiles / per > 4 ? 4 : tiles / per);
-    l.tab[s] = take(d.D * S * es * (grad && !d.cx ? 2 : 1));
+    const int sr = prec || d.cx ? 2 : 3;  // numbers kept per amplitude
+    l.tab[s] = take(d.D * S * es * (d.cx ? 1 : sr));
     if (!prec) l.pack[s] = take((S >> d.cx) * cut_k(T) * 16);
     if (d.cx) l.packr[s] = take(S * cut_k(T) * 8);
-    if (grad) {
+    if (grad || (!prec && !d.cx && d.half[0].m > HALF_SMALL_M(0))) {  // FP32 goes layer by layer through them
       long long states = 0;
       for (int r = 0; r < d.reps; ++r) states += 1LL << d.half[s].L[r].shift;
       if (d.cx) states += d.D;  // the last layer's too, before its RZ
-      l.phi[s] = take(2 * states * S * es);
+      l.phi[s] = take(sr * states * S * es);
+    }
+    if (grad) {
       l.g[s] = take((l.ns[s] + (xy ? 1 : 0)) * T * S * es);
     }
   }
@@ -218,6 +221,7 @@ CutLayout cut_layout(const CutDesc &d, int prec, bool grad, const CutXyDims *xy)
 // One CTA per 64 rows, through shared memory; 16-byte stores.  A complex table T gives the
 // columns (Re T_a, Im T_a) of real terms 2a, 2a + 1 over x, and in row form alone the rows
 // (x, 0): (Re T_a, -Im T_a) and (x, 1): (Im T_a, Re T_a).
+template <bool LOW>
 __device__ __forceinline__ void pack_form(const float *s, float4 *out, int K, bool row) {
   for (int i = threadIdx.x; i < K * 16; i += 256) {
     const int r = row ? (i & 7) + 8 * (i / (2 * K)) : 4 * ((i >> 3) & 15);  // [r / 8][a / 4][r % 8]
@@ -225,9 +229,14 @@ __device__ __forceinline__ void pack_form(const float *s, float4 *out, int K, bo
     float hi[4], lo[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float x = row ? s[(a + k) * 65 + r] : s[a * 65 + r + k];
+      const int at = row ? (a + k) * 65 + r : a * 65 + r + k;
+      const float x = s[at];
       asm("cvt.rna.tf32.f32 %0, %1;" : "=f"(hi[k]) : "f"(x));
       lo[k] = x - hi[k];
+      if (LOW) {  // the table's own low part, and the rounding to the tensor cores' 11 bits to nearest
+        const float y = lo[k] + s[K * 65 + at];
+        asm("cvt.rna.tf32.f32 %0, %1;" : "=f"(lo[k]) : "f"(y));
+      }
     }
     out[i] = make_float4(hi[0], hi[1], hi[2], hi[3]);
     out[16 * K + i] = make_float4(lo[0], lo[1], lo[2], lo[3]);
@@ -256,17 +265,20 @@ __global__ void __launch_bounds__(256) k_cut_pack(const __grid_constant__ CutArg
   float4 *out = reinterpret_cast<float4 *>(J.ws + J.lay->pack[h]) + (size_t)tile * (64 * K);
   for (int i = threadIdx.x; i < K * 64; i += 256) {
     const int a = i >> 6, x = tile * 64 + (i & 63);
-    float v = 0.f;
+    float v = 0.f, low = 0.f;
     if constexpr (CX) {
       if (a < 2 * D) v = tab[((size_t)(a >> 1) << (m + 1)) + 2 * x + (a & 1)];
-    } else {
-      if (a < D) v = tab[((size_t)a << m) + x];
+    } else if (a < D) {
+      const float *p = tab + ((size_t)3 * a << m) + x;
+      v = p[0];
+      low = p[(size_t)2 << m];
     }
     s[a * 65 + (i & 63)] = v;
+    if constexpr (!CX) s[(K + a) * 65 + (i & 63)] = low;
   }
   __syncthreads();
-  pack_form(s, out, K, true);
-  pack_form(s, out + 32 * K, K, false);
+  pack_form<!CX>(s, out, K, true);
+  pack_form<!CX>(s, out + 32 * K, K, false);
   if constexpr (CX) {  // the two 64-row blocks (x, channel) of these 64 x
     float4 *rows = reinterpret_cast<float4 *>(J.ws + J.lay->packr[h]) + (size_t)tile * (64 * K);
     for (int b = 0; b < 2; ++b) {
@@ -278,7 +290,7 @@ __global__ void __launch_bounds__(256) k_cut_pack(const __grid_constant__ CutArg
         s[a * 65 + r] = (a & 1) && !ch ? -v : v;
       }
       __syncthreads();
-      pack_form(s, rows + b * 32 * K, K, true);
+      pack_form<false>(s, rows + b * 32 * K, K, true);
     }
   }
 }
@@ -316,14 +328,14 @@ __global__ void __launch_bounds__(256) k_cut_contract64(const __grid_constant__ 
   const double *E = reinterpret_cast<const double *>(J.table);
   double *sR = reinterpret_cast<double *>(cut_smem), *sC = sR + D * C64LD, *sL = sC + D * C64LD;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  for (int i = tid; i < D * C64; i += 256) sR[(i >> 5) * C64LD + (i & 31)] = rt[(i >> 5) * Sr + row0 + (i & 31)];
+  for (int i = tid; i < D * C64; i += 256) sR[(i >> 5) * C64LD + (i & 31)] = rt[(i >> 5) * 2 * Sr + row0 + (i & 31)];
   double acc[NA], e = 0.0;
 #pragma unroll
   for (int k = 0; k < NA; ++k) acc[k] = 0.0;
   const int gi = tid & 31, ga = tid >> 5;  // G: row gi, terms ga + 8 k
   for (int c0 = col0; c0 < col0 + cols; c0 += C64) {
     __syncthreads();
-    for (int i = tid; i < D * C64; i += 256) sC[(i >> 5) * C64LD + (i & 31)] = ct[(i >> 5) * Sc + c0 + (i & 31)];
+    for (int i = tid; i < D * C64; i += 256) sC[(i >> 5) * C64LD + (i & 31)] = ct[(i >> 5) * 2 * Sc + c0 + (i & 31)];
     double t[2][2];
 #pragma unroll
     for (int p = 0; p < 2; ++p)
@@ -413,12 +425,12 @@ __global__ void __launch_bounds__(256) k_cut_rows64(const __grid_constant__ CutA
   const int tid = threadIdx.x, cols = 1 << mc, j = tid & (cols - 1), np = 256 >> mc;
   const double *rt = reinterpret_cast<const double *>(J.ws + J.lay->tab[h]);
   const double *ct = reinterpret_cast<const double *>(J.ws + J.lay->tab[1 - h]);
-  if (tid < D) row[tid] = rt[((size_t)tid << mr) + idx];
+  if (tid < D) row[tid] = rt[((size_t)2 * tid << mr) + idx];
   __syncthreads();
   double s0 = 0.0, s1 = 0.0;
   for (int a = tid >> mc; a < D; a += 2 * np) {
-    s0 = fma(row[a], ct[((size_t)a << mc) + j], s0);
-    if (a + np < D) s1 = fma(row[a + np], ct[((size_t)(a + np) << mc) + j], s1);
+    s0 = fma(row[a], ct[((size_t)2 * a << mc) + j], s0);
+    if (a + np < D) s1 = fma(row[a + np], ct[((size_t)2 * (a + np) << mc) + j], s1);
   }
   part[tid] = s0 + s1;
   __syncthreads();
@@ -434,7 +446,7 @@ __global__ void __launch_bounds__(256) k_cut_rows64(const __grid_constant__ CutA
   __syncthreads();
   if constexpr (GRAD)
     if (tid < D) {
-      const double2 *c = reinterpret_cast<const double2 *>(ct + ((size_t)tid << mc));
+      const double2 *c = reinterpret_cast<const double2 *>(ct + ((size_t)2 * tid << mc));
       double g0 = 0.0, g1 = 0.0;
 #pragma unroll 8
       for (int k = 0; k < cols / 2; ++k) {
@@ -460,59 +472,57 @@ __global__ void __launch_bounds__(256) k_cut_rows64(const __grid_constant__ CutA
 }
 
 // ------------------------------------------------------------ final sums --
-// One CTA per job: E, and per parameter (a warp each) the sum over the path values, in a
-// fixed order.  The FP32 contraction also sums psi^2: E and the gradients are divided by that
-// norm, which takes the rounding of cos, sin and of the tensor cores' accumulation out
+// One warp sums the energy's parts (the FP64 adds of a sum over all warps, by all of them, took
+// longer than the rest), all of them the parameters' path values: a few lanes for a parameter, in
+// an order that depends on the number of terms alone, the parameters next to each other along
+// the lanes as in memory.  8 CTAs for a job where there are few jobs, each a share of the
+// parameters.  The FP32 contraction also sums psi^2: E and the gradients are divided by
+// that norm, which takes the rounding of cos, sin and of the tensor cores' accumulation out
 // of the results to first order (it is 1 up to that rounding).
-constexpr int RED_NT = 512;
-__device__ __forceinline__ double warp_total(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
-}
+constexpr int RED_NT = 256;
 __global__ void __launch_bounds__(RED_NT) k_cut_reduce(const __grid_constant__ CutArgs A, int prec, int grad) {
   const CutView J = cut_view(A, blockIdx.x);
   const CutOut O = cut_out(A, blockIdx.x);
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  constexpr int NW = RED_NT / 32;
-  __shared__ double sh[3][NW];
-  const double *ep = reinterpret_cast<const double *>(J.ws + J.lay->ep);
-  const double *ex = reinterpret_cast<const double *>(J.ws + J.lay->exy);  // the X/Y strings', part by part
-  const int ni = J.lay->rb[0] * J.lay->ns[0];
-  double e = 0.0, z = 0.0, x = 0.0;
-  for (int i = tid; i < ni; i += RED_NT) {
-    e += ep[2 * i];
-    z += ep[2 * i + 1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  __shared__ double inv_s;
+  if (w == 0) {
+    const double *ep = reinterpret_cast<const double *>(J.ws + J.lay->ep);
+    const double *ex = reinterpret_cast<const double *>(J.ws + J.lay->exy);  // the X/Y strings', part by part
+    const int ni = J.lay->rb[0] * J.lay->ns[0];
+    double e = 0.0, z = 0.0;
+#pragma unroll 8
+    for (int i = lane; i < ni; i += 32) {
+      e += ep[2 * i];
+      z += ep[2 * i + 1];
+    }
+    for (int i = lane; i < J.lay->nexy; i += 32) e += ex[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      e += __shfl_xor_sync(0xffffffffu, e, o);
+      z += __shfl_xor_sync(0xffffffffu, z, o);
+    }
+    const double inv = prec ? 1.0 : 1.0 / z;
+    if (lane == 0 && blockIdx.y == 0) *O.E = e * inv;
+    if (lane == 0) inv_s = inv;
   }
-  for (int i = tid; i < J.lay->nexy; i += RED_NT) x += ex[i];
-  e = warp_total(e);
-  z = warp_total(z);
-  x = warp_total(x);
-  if (lane == 0) {
-    sh[0][w] = e;
-    sh[1][w] = z;
-    sh[2][w] = x;
-  }
-  __syncthreads();
-  e = z = x = 0.0;
-  for (int k = 0; k < NW; ++k) {
-    e += sh[0][k];
-    z += sh[1][k];
-    x += sh[2][k];
-  }
-  const double inv = prec ? 1.0 : 1.0 / z;
-  if (tid == 0) *O.E = (e + x) * inv;
   if (!grad) return;
+  __syncthreads();
+  const double inv = inv_s;
   const int n = J.desc->n, reps = J.desc->reps, D = J.desc->D, m0 = J.desc->half[0].m, cx = J.desc->cx;
   const int row = 16 << cx, per = n << cx;  // complex: RY then RZ of a layer
   const double *gp = reinterpret_cast<const double *>(J.ws + J.lay->gp);
-  for (int p = w; p < per * (reps + 1); p += NW) {
+  const int W = D >= 256 ? 32 : D >= 64 ? 8 : D >= 4 ? 4 : D, G = 32 / W;
+  for (int p0 = (w + RED_NT / 32 * blockIdx.y) * G; p0 < per * (reps + 1); p0 += RED_NT / 32 * gridDim.y * G) {
+    const int p = p0 + lane % G;
+    const bool on = p < per * (reps + 1);
     const int r = p / per, zr = p % per >= n, q = p % per - zr * n, h = q >= m0;
     const double *src = gp + (size_t)h * D * (reps + 1) * row + r * row + 16 * zr + (h ? q - m0 : q);
     double s = 0.0;
-    for (int a = lane; a < D; a += 32) s += src[(size_t)a * (reps + 1) * row];
-    s = warp_total(s);
-    if (lane == 0) O.grad[p] = (O.mask && !O.mask[p]) ? 0.0 : s * inv;
+#pragma unroll 8
+    for (int a = lane / G; a < D; a += W)
+      if (on) s += src[(size_t)a * (reps + 1) * row];
+    for (int o = G; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (on && lane < G) O.grad[p] = (O.mask && !O.mask[p]) ? 0.0 : s * inv;
   }
 }
 
@@ -565,8 +575,8 @@ cudaError_t launch_tile_tables(const TableJob *jobs, int njobs, int nmax, cudaSt
 }
 
 // Problems whose larger halves have the same class share the kernels of their half
-// circuits: one class for every size that runs in one warp, one per size above.
-int cut_class(int prec, int m) { return m <= HALF_WARP_M(prec) ? HALF_WARP_M(prec) : m; }
+// circuits: one class for every small size, one per size above.
+int cut_class(int prec, int m) { return m <= HALF_SMALL_M(prec) ? HALF_SMALL_M(prec) : m; }
 
 cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
                        const CutXyDims *xy) {
@@ -582,13 +592,12 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
   if (prec) {
     CUT_CHECK(launch_half<double>(A, cut_class(1, g.m0), grad ? 1 : 0, half_blocks, s));
   } else {
-    CUT_CHECK(g.cx ? launch_halfc(A, g.m0, grad ? 1 : 0, half_blocks, s)
-                   : launch_half<float>(A, cut_class(0, g.m0), grad ? 1 : 0, half_blocks, s));
+    CUT_CHECK(g.cx ? launch_halfc(A, g.m0, grad ? 1 : 0, half_blocks, s) : launch_cut_fwd32(A, g, grad, s, launches));
     A.items = g.pack_items;
     A.blk0 = 1 << (g.m0 - 6);
     A.nblk = A.blk0 + (1 << (g.m1 - 6));
     auto k = g.cx ? k_cut_pack<true> : k_cut_pack<false>;
-    k<<<g.pack_items ? g.pack_blocks : A.njobs * A.nblk, 256, K * 65 * 4, s>>>(A, K);
+    k<<<g.pack_items ? g.pack_blocks : A.njobs * A.nblk, 256, K * 65 * (g.cx ? 4 : 8), s>>>(A, K);
     CUT_CHECK(cudaGetLastError());
     *launches += 1;
   }
@@ -624,7 +633,7 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
                    : launch_half<float>(A, cut_class(0, g.m0), 2, half_blocks, s));
     *launches += 1;
   }
-  k_cut_reduce<<<A.njobs, RED_NT, 0, s>>>(A, prec, grad ? 1 : 0);
+  k_cut_reduce<<<dim3((unsigned)A.njobs, grad && A.njobs <= 19 ? 8 : 1), grad ? RED_NT : 32, 0, s>>>(A, prec, grad ? 1 : 0);
 #undef CUT_CHECK
   return cudaGetLastError();
 }

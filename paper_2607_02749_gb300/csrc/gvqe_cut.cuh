@@ -47,11 +47,13 @@ struct CutDesc {
 
 // Workspace of one evaluation (byte offsets) and how its contractions are split.
 struct CutLayout {
-  long long tab[2];   // L and R: [a][x], amplitude type; with gradients a second time in runs
+  // A state is kept as its amplitudes [x], the same in runs of 16 bytes, and (FP32, RY) its low
+  // parts [x]: SR = 2 or 3 times 2^m numbers.
+  long long tab[2];   // L and R: [a][SR][x]
   long long pack[2];  // FP32: their tensor-core operand images (as rows and as columns)
   long long packr[2]; // complex: as rows, (x, channel) by two real terms per term; pack as columns
-  long long phi[2];   // the half states after layers 0 .. reps - 1, one per value of the path bits so
-                      // far: [x], then the same in runs
+  long long phi[2];   // the half states after layers 0 .. reps - 1 (complex: reps), one per value of
+                      // the path bits so far
   long long g[2];     // partial contractions: [split][a][x]
   long long gp;       // gradient partials (doubles): [half][a][(reps + 1) * 16]
   long long ep;       // per item of contraction 0: energy and norm (doubles)
@@ -92,7 +94,7 @@ struct BatchIO {
 // steps the pointers of job 0; a launch over different problems reads an array.
 struct CutJob {
   const CutDesc *desc;
-  const void *cs;       // (cos, sin) of theta/2 per parameter
+  const void *cs;       // (cos, sin) of theta/2 per parameter, double2
   const void *table;    // E(x): FP64 in index order, FP32 in contraction 0's tile order
   const void *table_t;  // FP32: in contraction 1's tile order
   char *ws;
@@ -125,6 +127,7 @@ CutLayout cut_layout(const CutDesc &d, int prec, bool grad, const CutXyDims *xy 
 struct CutGrid {
   int cx;        // complex amplitudes
   int m0, m1, D;  // m1: the smallest half
+  int reps, bits[CUT_MAX_LAYERS + 1];  // one problem: path bits up to each layer; several: the most layers
   int half_blocks, con_blocks, pack_blocks;
   const int4 *half_items, *con_items, *pack_items;  // (job, half, path value | index | 64-row tile, 0)
 };
@@ -147,9 +150,11 @@ struct TableJob {
 // one table, or several at once (nmax: the largest m0 + m1)
 cudaError_t launch_tile_table(const TableJob &t, cudaStream_t s);
 cudaError_t launch_tile_tables(const TableJob *jobs, int njobs, int nmax, cudaStream_t s);
-// The half circuits (gvqe_cut_half.cu): mode 0 forward, 1 forward keeping the states the
-// backward reads, 2 backward; m: the class of the larger half.
-constexpr int HALF_WARP_M(int prec) { return prec ? 7 : 10; }  // largest half in one warp
+// The half circuits: FP32 forward (gvqe_cut_fwd.cu); the rest (gvqe_cut_half.cu) by mode, 0
+// forward, 1 forward keeping the states the backward reads, 2 backward; m: the class of the
+// larger half.
+constexpr int HALF_SMALL_M(int prec) { return prec ? 7 : 10; }  // halves up to here share one kernel
+cudaError_t launch_cut_fwd32(const CutArgs &A, const CutGrid &g, bool grad, cudaStream_t s, int *launches);  // FP32 forward
 template <typename T>
 cudaError_t launch_half(const CutArgs &A, int m, int mode, int blocks, cudaStream_t s);
 cudaError_t launch_halfc(const CutArgs &A, int m, int mode, int blocks, cudaStream_t s);  // complex (gvqe_cut_halfc.cu)

@@ -55,15 +55,15 @@ __device__ __forceinline__ void half_fwd(const CutView &J, int h, int a, T *st, 
     T *nat, *run;
     bool keep;
     if (r < reps) {
-      phi += 2 * (SZ << l.shift);
+      phi += 2 * (SZ << l.shift);  // (forward: FP64 only)
       const int bits = l.shift + l.nb;
       nat = phi + (size_t)2 * a * SZ;
       run = nat + SZ;
       keep = GRAD && (a >> bits) == 0;
     } else {
       T *tab = reinterpret_cast<T *>(J.ws + J.lay->tab[h]);
-      nat = tab + (size_t)a * SZ;
-      run = tab + (size_t)(J.desc->D + a) * SZ;
+      nat = tab + (size_t)2 * a * SZ;
+      run = nat + SZ;
       keep = true;
     }
     S.low_round([&](int it, T *u) {
@@ -102,10 +102,10 @@ __device__ __forceinline__ void half_bwd(const CutView &J, int h, int a, T *st, 
   }
   S.top_store(v);
   double *gp = reinterpret_cast<double *>(J.ws + J.lay->gp) + ((size_t)h * D + a) * (reps + 1) * 16;
-  const T *tab = reinterpret_cast<const T *>(J.ws + J.lay->tab[h]);
-  const T *nat = tab + (size_t)a * SZ, *run = tab + (size_t)(D + a) * SZ;
+  constexpr int SR = sizeof(T) == 4 ? 3 : 2;  // numbers kept per amplitude
+  const T *nat = reinterpret_cast<const T *>(J.ws + J.lay->tab[h]) + (size_t)SR * a * SZ, *run = nat + SZ;
   const T *phi = reinterpret_cast<const T *>(J.ws + J.lay->phi[h]);
-  for (int r = 0; r < reps; ++r) phi += 2 * (SZ << sh.H.L[r].shift);
+  for (int r = 0; r < reps; ++r) phi += SR * (SZ << sh.H.L[r].shift);
   for (int r = reps;; --r) {
     const typename HF::T2 *cs = sh.cs + r * M;
     T acc[M];
@@ -192,14 +192,14 @@ __device__ __forceinline__ void half_bwd(const CutView &J, int h, int a, T *st, 
     S.gather(v, l.fc, l.fo[(a >> l.shift) & ((1 << l.nb) - 1)]);
     S.sync();
     S.top_store(v);
-    phi -= 2 * (SZ << l.shift);
-    nat = phi + (size_t)2 * (a & ((1 << l.shift) - 1)) * SZ;
+    phi -= SR * (SZ << l.shift);
+    nat = phi + (size_t)SR * (a & ((1 << l.shift) - 1)) * SZ;
     run = nat + SZ;
   }
 }
 
 // MODE 0: forward, 1: forward keeping what the backward reads, 2: backward.  One kernel for
-// all sizes that run in one warp (mixed in a batch), and one per size M above, which also
+// all small sizes (mixed in a batch), and one per size M above, which also
 // takes the other half of an odd register, a qubit smaller, with some threads idle.
 template <typename T, int MODE, int M>
 __device__ __forceinline__ void half_run(const CutView &J, int h, int a, T *st, HalfShared<T> &sh) {
@@ -210,16 +210,16 @@ __device__ __forceinline__ void half_run(const CutView &J, int h, int a, T *st, 
   else
     half_fwd<T, M, MODE == 1>(J, h, a, st, sh);
 }
-constexpr int WARP_M = HALF_WARP_M(sizeof(GVQE_INST_T) == 8);
+constexpr int SMALL_M = HALF_SMALL_M(sizeof(GVQE_INST_T) == 8);
 template <typename T, int MODE, int M>
-__global__ void __launch_bounds__(HalfCfg<T, M>::NT) k_half(const __grid_constant__ CutArgs A) {
+__global__ void __launch_bounds__(half_nt<T, M>()) k_half(const __grid_constant__ CutArgs A) {
   extern __shared__ __align__(16) unsigned char cut_smem[];
   __shared__ HalfShared<T> sh;
   const int3 it = cut_half_item(A);
   const CutView J = cut_view(A, it.x);
   T *st = reinterpret_cast<T *>(cut_smem);
   const int m = J.desc->half[it.y].m;
-  if constexpr (M > WARP_M) {
+  if constexpr (M > SMALL_M) {
     if (m == M)
       half_run<T, MODE, M>(J, it.y, it.z, st, sh);
     else
@@ -243,21 +243,21 @@ static cudaError_t launch_half_m(const CutArgs &A, int blocks, cudaStream_t s) {
   constexpr size_t sm = (size_t)pad<T>(1 << M) * sizeof(T);
   static SmemLimit limit;
   if (const cudaError_t e = limit.set(k_half<T, MODE, M>, sm)) return e;
-  k_half<T, MODE, M><<<blocks, HalfCfg<T, M>::NT, sm, s>>>(A);
+  k_half<T, MODE, M><<<blocks, half_nt<T, M>(), sm, s>>>(A);
   return cudaGetLastError();
 }
 
 template <typename T, int MODE>
 static cudaError_t launch_half_mode(const CutArgs &A, int m, int blocks, cudaStream_t s) {
   switch (m) {
-    case WARP_M: return launch_half_m<T, MODE, WARP_M>(A, blocks, s);
-    case WARP_M + 1: return launch_half_m<T, MODE, WARP_M + 1>(A, blocks, s);
-    case WARP_M + 2: return launch_half_m<T, MODE, WARP_M + 2>(A, blocks, s);
-    case WARP_M + 3: return launch_half_m<T, MODE, WARP_M + 3>(A, blocks, s);
-    case WARP_M + 4: return launch_half_m<T, MODE, WARP_M + 4>(A, blocks, s);
-    case WARP_M + 5: return launch_half_m<T, MODE, WARP_M + 5>(A, blocks, s);
+    case SMALL_M: return launch_half_m<T, MODE, SMALL_M>(A, blocks, s);
+    case SMALL_M + 1: return launch_half_m<T, MODE, SMALL_M + 1>(A, blocks, s);
+    case SMALL_M + 2: return launch_half_m<T, MODE, SMALL_M + 2>(A, blocks, s);
+    case SMALL_M + 3: return launch_half_m<T, MODE, SMALL_M + 3>(A, blocks, s);
+    case SMALL_M + 4: return launch_half_m<T, MODE, SMALL_M + 4>(A, blocks, s);
+    case SMALL_M + 5: return launch_half_m<T, MODE, SMALL_M + 5>(A, blocks, s);
   }
-  if constexpr (WARP_M + 7 == 14) {  // FP64: 14 is the largest half, FP32: 15
+  if constexpr (SMALL_M + 7 == 14) {  // FP64: 14 is the largest half, FP32: 15
     if (m == 13) return launch_half_m<T, MODE, 13>(A, blocks, s);
     if (m == 14) return launch_half_m<T, MODE, 14>(A, blocks, s);
   }
@@ -266,8 +266,10 @@ static cudaError_t launch_half_mode(const CutArgs &A, int m, int blocks, cudaStr
 
 template <>
 cudaError_t launch_half<GVQE_INST_T>(const CutArgs &A, int m, int mode, int blocks, cudaStream_t s) {
-  if (mode == 0) return launch_half_mode<GVQE_INST_T, 0>(A, m, blocks, s);
-  if (mode == 1) return launch_half_mode<GVQE_INST_T, 1>(A, m, blocks, s);
+  if constexpr (sizeof(GVQE_INST_T) == 8) {
+    if (mode == 0) return launch_half_mode<GVQE_INST_T, 0>(A, m, blocks, s);
+    if (mode == 1) return launch_half_mode<GVQE_INST_T, 1>(A, m, blocks, s);
+  }
   return launch_half_mode<GVQE_INST_T, 2>(A, m, blocks, s);
 }
 

@@ -2,32 +2,40 @@
 // two-half evaluation (gvqe_cut_half.cu, gvqe_cut_halfc.cu).
 //
 // One CTA runs one half's circuit for one value a of the path bits, its 2^M amplitudes
-// in shared memory and 2^E per thread in registers (32 from M = 10).  A layer is a gather
+// in shared memory and 2^E per thread in registers (32 from M = 11).  A layer is a gather
 // through the layer's affine map straight into the registers of the top E bits, RY on
 // those, and more register rounds: the bits between (MID) and the lowest (LOW, runs of
 // consecutive amplitudes in 16-byte accesses).  16 bytes of padding per 128 keep runs,
 // rows and columns apart in the banks.  M is a template argument, so that every shared-
 // memory access is a base and an immediate; FP32 rotations run as packed f32x2.
-// One CTA per SM at M = 15 (147 KB, 1024 threads of 64 registers), one warp up to M = 10.
+// One CTA per SM at M = 15 (147 KB, 1024 threads of 64 registers).
 // Bound by shared-memory wavefronts and issue: about 200 and 700 per warp and layer.
 #pragma once
 #include "gvqe_cut.cuh"
 
 namespace gvqe {
 
-// FP64: four warps where the half allows it, one per FP64 pipe of the SM.
+// FP64: four warps where the half allows it, one per FP64 pipe of the SM.  FP32 to 10 qubits: four
+// warps too, a chain of 700 instructions per layer and warp otherwise (64 terms, 19 qubits, one
+// vector, forward and backward: 47 and 25 us with one warp, 19 and 14 with four).  From 11 qubits 32
+// amplitudes a thread save shared-memory rounds (backward, 24 qubits: 37 us, 50 with 16).
 template <typename T>
 __host__ __device__ constexpr int half_e(int M) {
-  return sizeof(T) == 4 ? (M >= 10 ? 5 : M == 9 ? 4 : M >= 7 ? 3 : 2) : (M >= 12 ? 5 : M == 11 ? 4 : M == 10 ? 3 : 2);
+  return sizeof(T) == 4 ? (M >= 11 ? 5 : M >= 7 ? 3 : 2) : (M >= 12 ? 5 : M == 11 ? 4 : M == 10 ? 3 : 2);
 }
-template <typename T, int M>
+template <typename T, int M, int EB = half_e<T>(M)>
 struct HalfCfg {
-  static constexpr int E = half_e<T>(M);      // register bits
+  static constexpr int E = EB;                // register bits
   static constexpr int LT = M - E;            // log2 of the working threads
   static constexpr int G0 = LT < E ? LT : E;  // LOW bits; the other LT - G0 are MID's, at most E at a time
   static constexpr int NT = LT < 5 ? 32 : 1 << LT;
   static_assert(G0 >= 2, "runs of 16 bytes");
 };
+// threads of a kernel that takes halves of M and of M - 1 qubits
+template <typename T, int M>
+constexpr int half_nt() {
+  return HalfCfg<T, M>::NT > HalfCfg<T, M - 1>::NT ? HalfCfg<T, M>::NT : HalfCfg<T, M - 1>::NT;
+}
 
 template <typename T>
 struct CutT;
@@ -168,9 +176,9 @@ struct Int {
 };
 
 // One half circuit of 2^M amplitudes: this thread's share of its state in shared memory.
-template <typename T, int M>
+template <typename T, int M, int EB = half_e<T>(M)>
 struct Half {
-  using C = HalfCfg<T, M>;
+  using C = HalfCfg<T, M, EB>;
   using T2 = typename CutT<T>::T2;
   using V = typename CutT<T>::V;
   static constexpr int N = 1 << C::E, VN = CutT<T>::VN;
@@ -296,7 +304,11 @@ __device__ __forceinline__ void half_setup(HalfShared<T> &sh, const CutView &J, 
     reinterpret_cast<int *>(&sh.H)[i] = reinterpret_cast<const int *>(&J.desc->half[h])[i];
   const int n = J.desc->n, q0 = h ? J.desc->half[0].m : 0, np = (J.desc->reps + 1) * M;
   for (int i = threadIdx.x; i < np; i += blockDim.x)
-    sh.cs[i] = reinterpret_cast<const typename CutT<T>::T2 *>(J.cs)[(i / M) * n + q0 + i % M];
+  {
+    const double2 c = reinterpret_cast<const double2 *>(J.cs)[(i / M) * n + q0 + i % M];
+    sh.cs[i].x = (T)c.x;
+    sh.cs[i].y = (T)c.y;
+  }
   __syncthreads();
 }
 

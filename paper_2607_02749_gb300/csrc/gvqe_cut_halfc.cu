@@ -27,7 +27,8 @@ __device__ __forceinline__ void setup(SharedC &sh, const CutView &J, int h, int 
   const int n = J.desc->n, reps = J.desc->reps, tid = threadIdx.x, NT = blockDim.x;
   for (int i = tid; i < (reps + 1) * 2 * M; i += NT) {
     const int r = i / (2 * M), z = (i / M) & 1, q = i % M;
-    sh.cs[i] = reinterpret_cast<const float2 *>(J.cs)[r * 2 * n + z * n + H.q0 + q];
+    const double2 c = reinterpret_cast<const double2 *>(J.cs)[r * 2 * n + z * n + H.q0 + q];
+    sh.cs[i] = make_float2((float)c.x, (float)c.y);
   }
   for (int i = tid; i < reps * 2 * (M + 1); i += NT) {
     const int r = i / (2 * (M + 1)), d = (i / (M + 1)) & 1, q = i % (M + 1);
@@ -278,7 +279,7 @@ __device__ __forceinline__ void run_c(const CutView &J, int h, int a, float *st,
 
 // MB: index bits of the larger half; the other may have one less
 template <int MODE, int MB>
-__global__ void __launch_bounds__(HalfCfg<float, MB>::NT) k_halfc(const __grid_constant__ CutArgs A) {
+__global__ void __launch_bounds__(half_nt<float, MB>()) k_halfc(const __grid_constant__ CutArgs A) {
   extern __shared__ __align__(16) unsigned char cut_smem[];
   __shared__ SharedC sh;
   const int3 it = cut_half_item(A);
@@ -295,7 +296,7 @@ cudaError_t launch_mb(const CutArgs &A, int blocks, cudaStream_t s) {
   constexpr size_t sm = (size_t)pad<float>(1 << MB) * sizeof(float);
   static SmemLimit limit;
   if (const cudaError_t e = limit.set(k_halfc<MODE, MB>, sm)) return e;
-  k_halfc<MODE, MB><<<blocks, HalfCfg<float, MB>::NT, sm, s>>>(A);
+  k_halfc<MODE, MB><<<blocks, half_nt<float, MB>(), sm, s>>>(A);
   return cudaGetLastError();
 }
 

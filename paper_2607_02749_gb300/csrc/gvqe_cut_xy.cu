@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256) k_xy_rows(const __grid_constant__ CutArgs
   const float *tab = reinterpret_cast<const float *>(J.ws + J.lay->tab[h]);
   for (int i = threadIdx.x; i < DP * 64; i += 256) {
     const int a = i >> 6, x = i & 63;
-    s[a][x] = a < D ? tab[((size_t)a << m) + x0 + x] : 0.f;
+    s[a][x] = a < D ? tab[((size_t)3 * a << m) + x0 + x] : 0.f;
   }
   __syncthreads();
   float *rows = reinterpret_cast<float *>(J.ws + J.lay->rows[h]) + (size_t)x0 * DP;
