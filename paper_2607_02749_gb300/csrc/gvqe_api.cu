@@ -1850,7 +1850,7 @@ int gvqe_readout(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, int fl
   double *part = (double *)(w + o_part);
   unsigned long long *mass = (unsigned long long *)(w + o_mass), *ext = (unsigned long long *)(w + o_ext);
   GV_CUDA(launch_ro_prob(prec, psi, n, csum, cmax, cidx, cdf, stats, (long long *)argmax, s));
-  count_launches(2);
+  count_launches(nch > 1024 ? 3 : 2);
   if (n_shots > 0) {
     GV_CUDA(launch_ro_sample(prec, psi, n, cdf, uniforms, n_shots, (long long *)shots, s));
     count_launches(1);
@@ -1909,18 +1909,18 @@ int gvqe_readout(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, int fl
   // mass below and above it); otherwise the search starts from the full range.
   if (n_shots >= 256 && alpha < 1.0) {
     double *es = (double *)(w + o_es);
-    GV_CUDA(launch_ro_gather(E, (const long long *)shots, n_shots, es, s));
-    count_launches(1);
-    std::vector<double> hes((size_t)n_shots);
-    GV_CUDA(cudaMemcpyAsync(hes.data(), es, 8 * (size_t)n_shots, cudaMemcpyDeviceToHost, s));
-    GV_CUDA(cudaStreamSynchronize(s));
-    std::sort(hes.begin(), hes.end());
     const double K = n_shots, d = 4.0 * std::sqrt(alpha * (1.0 - alpha) / K) + 2.0 / K;
     if (alpha - d > 0.0 && alpha + d < 1.0) {
       const long long ilo = (long long)std::floor((alpha - d) * K);
       const long long ihi = std::min<long long>(n_shots - 1, (long long)std::ceil((alpha + d) * K));
-      lo = hes[(size_t)ilo];
-      hi = std::nextafter(hes[(size_t)ihi], HUGE_VAL);
+      double ends[2];
+      GV_CUDA(launch_ro_gather(E, (const long long *)shots, n_shots, es, s));
+      GV_CUDA(launch_ro_rank(es, n_shots, (int)ilo, (int)ihi, part, s));
+      count_launches(2);
+      GV_CUDA(cudaMemcpyAsync(ends, part, sizeof(ends), cudaMemcpyDeviceToHost, s));
+      GV_CUDA(cudaStreamSynchronize(s));
+      lo = ends[0];
+      hi = std::nextafter(ends[1], HUGE_VAL);
       GV_TRY(hist_pass(true));
       tot = hext[0] + in_range_mass() + hext[3];
       GV_TRY(set_target());

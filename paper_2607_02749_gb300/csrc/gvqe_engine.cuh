@@ -353,6 +353,8 @@ cudaError_t launch_ro_hist(int prec, const void *psi, const double *E, int n, co
                            unsigned long long *gmass, unsigned long long *ext, int below, cudaStream_t s);
 // out[k] = E[shots[k]] for k < nshots.
 cudaError_t launch_ro_gather(const double *E, const long long *shots, int nshots, double *out, cudaStream_t s);
+// out[0], out[1] = the energies of ranks r0 and r1 (from 0, below nshots) among es.
+cudaError_t launch_ro_rank(const double *es, int nshots, int r0, int r1, double *out, cudaStream_t s);
 // part: 3 * readout_tail_parts() doubles; writes stats[1].
 cudaError_t launch_ro_cvar(int prec, const void *psi, const double *E, int n, double alpha, double tau,
                            double *part, double *stats, cudaStream_t s);

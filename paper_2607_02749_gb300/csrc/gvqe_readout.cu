@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(RO_NT) k_ro_chunks(const T *psi, int cb, doubl
   const int len = 1 << cb;
   T s = T(0), m = T(-1);
   long long mi = base;
+#pragma unroll 16
   for (int i = tid; i < len; i += RO_NT) {
     const T v = __ldcg(psi + base + i);
     const T av = v < T(0) ? -v : v;
@@ -110,86 +111,113 @@ __global__ void __launch_bounds__(RO_NT) k_ro_chunks(const T *psi, int cb, doubl
   }
 }
 
-// One CTA: cdf[0] = 0, cdf[c + 1] = sum of chunks 0..c (block scans in a fixed
-// order), the overall maximum (smallest index on ties) and the total.
-__global__ void __launch_bounds__(1024) k_ro_scan(const double *csum, const double *cmax, const long long *cidx,
-                                                  long long nch, double *cdf, double *stats, long long *argmax) {
+// cdf[0] = 0, cdf[c + 1] = sum of chunks 0..c (block scans in a fixed order, then their totals one
+// after the other), the overall maximum (smallest index on ties) and the total.
+// A CTA scans 1024 chunks: 10 FP64 adds each, on an SM's few FP64 lanes 5 us, so that the blocks
+// run side by side and a second kernel adds what lies before them (8192 chunks: 45 us in one CTA,
+// 9 so).  A block's total, maximum and index stay in its first places of csum, cmax and cidx.
+__device__ __forceinline__ void ro_larger(double &m, long long &i, double m2, long long i2) {
+  if (m2 > m || (m2 == m && i2 < i)) {
+    m = m2;
+    i = i2;
+  }
+}
+__global__ void __launch_bounds__(1024) k_ro_scan(double *csum, double *cmax, long long *cidx, long long nch,
+                                                  double *cdf, double *stats, long long *argmax) {
   __shared__ double buf[1024];
   __shared__ double bm[1024];
   __shared__ long long bi[1024];
   const int tid = threadIdx.x;
-  double carry = 0.0, m = -1.0;
+  const long long b0 = (long long)blockIdx.x << 10, i = b0 + tid;
+  double v = 0.0, m = -1.0;
   long long mi = 0;
-  if (tid == 0) cdf[0] = 0.0;
-  for (long long b0 = 0; b0 < nch; b0 += 1024) {
-    const long long i = b0 + tid;
-    double v = 0.0;
-    if (i < nch) {
-      v = csum[i];
-      const double mm = cmax[i];
-      const long long ii = cidx[i];
-      if (mm > m || (mm == m && ii < mi)) {
-        m = mm;
-        mi = ii;
-      }
-    }
-    buf[tid] = v;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-      const double add = tid >= off ? buf[tid - off] : 0.0;
-      __syncthreads();
-      buf[tid] += add;
-      __syncthreads();
-    }
-    if (i < nch) cdf[i + 1] = carry + buf[tid];
-    carry += buf[1023];
-    __syncthreads();
+  if (i < nch) {
+    v = csum[i];
+    ro_larger(m, mi, cmax[i], cidx[i]);
   }
+  buf[tid] = v;
   bm[tid] = m;
   bi[tid] = mi;
   __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if (tid < w) {
-      const double m2 = bm[tid + w];
-      const long long i2 = bi[tid + w];
-      if (m2 > bm[tid] || (m2 == bm[tid] && i2 < bi[tid])) {
-        bm[tid] = m2;
-        bi[tid] = i2;
-      }
-    }
+  for (int off = 1; off < 1024; off <<= 1) {
+    const double add = tid >= off ? buf[tid - off] : 0.0;
+    __syncthreads();
+    if (tid >= off) buf[tid] += add;
     __syncthreads();
   }
-  if (tid == 0) {
+  for (int w = 512; w > 0; w >>= 1) {
+    if (tid < w) ro_larger(bm[tid], bi[tid], bm[tid + w], bi[tid + w]);
+    __syncthreads();
+  }
+  if (i < nch) cdf[i + 1] = buf[tid];
+  if (tid != 0) return;
+  if (blockIdx.x == 0) cdf[0] = 0.0;
+  if (gridDim.x == 1) {
     stats[0] = bm[0];
-    stats[2] = carry;
+    stats[2] = buf[1023];
     argmax[0] = bi[0];
+  } else {
+    csum[b0] = buf[1023];
+    cmax[b0] = bm[0];
+    cidx[b0] = bi[0];
   }
 }
+__global__ void __launch_bounds__(1024) k_ro_carry(const double *csum, const double *cmax, const long long *cidx,
+                                                   long long nch, double *cdf, double *stats, long long *argmax) {
+  __shared__ double before;
+  const long long i = ((long long)blockIdx.x << 10) + threadIdx.x;
+  if (threadIdx.x == 0) {
+    double carry = 0.0;
+    for (unsigned b = 0; b < blockIdx.x; ++b) carry += csum[(long long)b << 10];
+    before = carry;
+    if (blockIdx.x == gridDim.x - 1) {
+      double m = -1.0;
+      long long mi = 0;
+      for (unsigned b = 0; b < gridDim.x; ++b) ro_larger(m, mi, cmax[(long long)b << 10], cidx[(long long)b << 10]);
+      stats[0] = m;
+      stats[2] = carry + csum[(long long)blockIdx.x << 10];
+      argmax[0] = mi;
+    }
+  }
+  __syncthreads();
+  if (blockIdx.x > 0 && i < nch) cdf[i + 1] = before + cdf[i + 1];
+}
 
-// One warp per shot: t = u * total; the chunk whose cumulative range holds t
-// (binary search), then a warp scan through that chunk for the first x whose
+// p * 2^60 of one amplitude, cut to an integer: for FP32 from the exact square of the mantissa
+// (integer work only), for FP64 from the rounded square.  Below 2^64 for |v| < 2.
+__device__ __forceinline__ unsigned long long qsquare(float v) {
+  const unsigned b = __float_as_uint(v);
+  const int ex = (int)((b >> 23) & 0xFF), e = ex ? ex : 1;
+  const unsigned m = (b & 0x7FFFFFu) | (ex ? 0x800000u : 0u);
+  const unsigned long long m2 = (unsigned long long)m * m;  // p = m2 2^(2 e - 300)
+  const int sh = 2 * e - 240;
+  return sh >= 0 ? (m2 << sh) : (sh > -64 ? (m2 >> -sh) : 0ull);
+}
+__device__ __forceinline__ unsigned long long qsquare(double v) { return __double2ull_rz(v * v * 0x1p60); }
+// four consecutive amplitudes
+__device__ __forceinline__ unsigned long long qsquare4(const float *p) {
+  const float4 v = *reinterpret_cast<const float4 *>(p);
+  return qsquare(v.x) + qsquare(v.y) + qsquare(v.z) + qsquare(v.w);
+}
+__device__ __forceinline__ unsigned long long qsquare4(const double *p) {
+  const double2 v = reinterpret_cast<const double2 *>(p)[0], w = reinterpret_cast<const double2 *>(p)[1];
+  return qsquare(v.x) + qsquare(v.y) + qsquare(w.x) + qsquare(w.y);
+}
+// inclusive scan over the warp
+__device__ __forceinline__ unsigned long long scan_u64(unsigned long long x, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += v;
+  }
+  return x;
+}
+
+// The sample as it is defined: a warp scan through the chunk, 32 amplitudes at a time in FP64, for the first x whose
 // cumulative probability exceeds t.  Where rounding leaves t past the chunk's
 // own running sum, the chunk's last x with p > 0 is taken.
 template <typename T>
-__global__ void __launch_bounds__(RO_NT) k_ro_sample(const T *psi, int cb, long long nch, const double *cdf,
-                                                     const double *u, int nshots, long long *shots) {
-  const int lane = threadIdx.x & 31;
-  const long long k = (blockIdx.x * (long long)RO_NT + threadIdx.x) >> 5;
-  if (k >= nshots) return;  // the whole warp
-  const double total = cdf[nch];
-  double t = u[k] * total;
-  if (!(t < total)) t = nextafter(total, 0.0);
-  long long lo = 0, hi = nch - 1;  // first chunk c with cdf[c + 1] > t
-  while (lo < hi) {
-    const long long mid = (lo + hi) >> 1;
-    if (cdf[mid + 1] > t)
-      hi = mid;
-    else
-      lo = mid + 1;
-  }
-  const long long base = lo << cb;
-  const int len = 1 << cb;
-  double run = cdf[lo];
+__device__ __noinline__ long long ro_scan_chunk(const T *psi, long long base, int len, double run, double t, int lane) {
   long long found = -1, lastnz = -1;
   for (int i0 = 0; i0 < len; i0 += 32) {
     const int i = i0 + lane;
@@ -209,8 +237,75 @@ __global__ void __launch_bounds__(RO_NT) k_ro_sample(const T *psi, int cb, long 
     }
     run += __shfl_sync(0xffffffffu, incl, 31);
   }
-  if (found < 0) found = lastnz >= 0 ? lastnz : base;
-  if (lane == 0) shots[k] = found;
+  return found >= 0 ? found : lastnz >= 0 ? lastnz : base;
+}
+
+// The same in integers, or -1 where they cannot tell.  F, the sum of the cut p * 2^60, is within
+// 2^13 of the sum; the FP64 scan's rounding (at most 262 adds of values below 2), that of t - run
+// and the cuts come to less than 2^17.  So the first x with F > t - run - 2^18 is the scan's if
+// F > t - run + 2^18 there: the scan takes no x before it, and takes it.
+constexpr int RO_SEG = 2048;
+template <typename T>
+__device__ __forceinline__ long long ro_find_chunk(const T *psi, long long base, int len, double run, double t, int lane) {
+  const long long d = __double2ll_rz((t - run) * 0x1p60), lo = d - (1 << 18), hi = d + (1 << 18);
+  const T *p = psi + base;
+  unsigned long long f = 0;
+  int seg = 0;
+  for (; seg < len; seg += RO_SEG) {
+    unsigned long long s = 0;
+#pragma unroll
+    for (int k = 0; k < RO_SEG / 128; ++k) s += qsquare4(p + seg + 128 * k + 4 * lane);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((long long)(f + s) > lo) break;
+    f += s;
+  }
+  if (seg >= len) return -1;
+  // 64 amplitudes a lane, then 2
+  unsigned long long s = 0;
+#pragma unroll
+  for (int k = 0; k < RO_SEG / 128; ++k) s += qsquare4(p + seg + (RO_SEG / 32) * lane + 4 * k);
+  unsigned long long incl = scan_u64(s, lane);
+  int l = __ffs(__ballot_sync(0xffffffffu, (long long)(f + incl) > lo)) - 1;
+  f += __shfl_sync(0xffffffffu, incl - s, l);
+  const T *r = p + seg + (RO_SEG / 32) * l;
+  const unsigned long long q0 = qsquare(r[2 * lane]), q1 = qsquare(r[2 * lane + 1]);
+  incl = scan_u64(q0 + q1, lane);
+  l = __ffs(__ballot_sync(0xffffffffu, (long long)(f + incl) > lo)) - 1;
+  const long long f1 = (long long)(f + incl), f0 = f1 - (long long)q1;
+  const bool first = f0 > lo;
+  const long long x = (first ? f0 : f1) > hi ? (r - psi) + 2 * lane + !first : -1;
+  return __shfl_sync(0xffffffffu, x, l);
+}
+
+// One warp per shot: t = u * total; the chunk whose cumulative range holds t
+// (binary search), then the first x of that chunk whose cumulative probability exceeds t.  Summed
+// in integers, off the few FP64 lanes, with the FP64 scan only where t is within 2e-13 of a
+// step; 26 qubits, 8192 shots: 1010 us with FP64 scans, 87 so.
+template <typename T>
+__global__ void __launch_bounds__(RO_NT) k_ro_sample(const T *psi, int cb, long long nch, const double *cdf,
+                                                     const double *u, int nshots, long long *shots) {
+  const int lane = threadIdx.x & 31;
+  const long long k = (blockIdx.x * (long long)RO_NT + threadIdx.x) >> 5;
+  if (k >= nshots) return;  // the whole warp
+  const double total = cdf[nch];
+  double t = u[k] * total;
+  if (!(t < total)) t = nextafter(total, 0.0);
+  long long lo = 0, hi = nch - 1;  // first chunk c with cdf[c + 1] > t
+  while (lo < hi) {
+    const long long mid = (lo + hi) >> 1;
+    if (cdf[mid + 1] > t)
+      hi = mid;
+    else
+      lo = mid + 1;
+  }
+  const long long base = lo << cb;
+  const int len = 1 << cb;
+  const double run = cdf[lo];
+  long long x = -1;
+  if (len >= RO_SEG && total < 2.0 && run <= t) x = ro_find_chunk(psi, base, len, run, t, lane);
+  if (x < 0) x = ro_scan_chunk(psi, base, len, run, t, lane);
+  if (lane == 0) shots[k] = x;
 }
 
 // Keys of the smallest and largest E over all x: ext[1] (min), ext[2] (max).
@@ -236,8 +331,15 @@ __global__ void __launch_bounds__(RO_NT) k_ro_minmax(const double *E, long long 
       kmax = k[j] > kmax ? k[j] : kmax;
     }
   }
-  atomicMin(&smin, kmin);
-  atomicMax(&smax, kmax);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
+    kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&smin, kmin);
+    atomicMax(&smax, kmax);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     atomicMin(&ext[1], smin);
@@ -251,6 +353,9 @@ __global__ void __launch_bounds__(RO_NT) k_ro_minmax(const double *E, long long 
 // are the keys of evenly spaced energies.  With `below` set, the masses under
 // and above the range are summed too (ext[0], ext[3]); otherwise only x inside
 // the range read their amplitude (the mass below is known from earlier passes).
+//
+// Bound by HBM: 26 qubits 178 us with `below` (0.8 GB; 515 with two loads in flight, a branch
+// for every warp that met the range and atomics from every thread), 88 without (0.5 GB).
 //
 // A key's bin: the range is cut into RO_LUT equal key intervals, lut[j] holds
 // the bin of interval j's first key, so a key of interval j lies in a bin of
@@ -275,14 +380,15 @@ __global__ void __launch_bounds__(RO_NT) k_ro_hist(const T *psi, const double *E
   __shared__ unsigned long long se[RO_BINS + 1];
   __shared__ unsigned long long sm[RO_BINS];
   __shared__ unsigned short lut[RO_LUT + 1];
-  __shared__ unsigned long long smin, smax;
+  __shared__ unsigned long long queue[2][RO_NT / 32][64];
+  __shared__ unsigned long long smin, smax, sbelow, sabove;
   for (int i = threadIdx.x; i <= RO_BINS; i += RO_NT) {
     se[i] = edges[i];
     if (i < RO_BINS) sm[i] = 0ull;
   }
   if (threadIdx.x == 0) {
     smin = ~0ull;
-    smax = 0ull;
+    smax = sbelow = sabove = 0ull;
   }
   __syncthreads();
   const unsigned long long lo = se[0], hi = se[RO_BINS];
@@ -296,6 +402,13 @@ __global__ void __launch_bounds__(RO_NT) k_ro_hist(const T *psi, const double *E
   const unsigned long long lo_read = below ? 0ull : lo;   // keys in [lo_read, hi_read) read psi
   const unsigned long long hi_read = below ? ~0ull : hi;
   unsigned long long kmin = ~0ull, kmax = 0ull, qbelow = 0ull, qabove = 0ull;
+  auto drop = [&](unsigned long long k, unsigned long long q) {
+    const int j = (int)((k - lo) >> lsh);  // < RO_LUT
+    const int b = ro_bin_search(se, k, lut[j], lut[j + 1]);  // largest b with edges[b] <= k
+    if (q) atomicAdd(&sm[b], q);
+    kmin = k < kmin ? k : kmin;
+    kmax = k > kmax ? k : kmax;
+  };
   auto add = [&](unsigned long long k, T v) {
     if (k < lo) {
       qbelow += qmass(v);
@@ -305,15 +418,74 @@ __global__ void __launch_bounds__(RO_NT) k_ro_hist(const T *psi, const double *E
       qabove += qmass(v);
       return;
     }
-    const unsigned long long q = qmass(v);
-    const int j = (int)((k - lo) >> lsh);  // < RO_LUT
-    const int b = ro_bin_search(se, k, lut[j], lut[j + 1]);  // largest b with edges[b] <= k
-    if (q) atomicAdd(&sm[b], q);
-    kmin = k < kmin ? k : kmin;
-    kmax = k > kmax ? k : kmax;
+    drop(k, qmass(v));
   };
   const long long N2 = N >> 1, st = (long long)gridDim.x * RO_NT;
-  for (long long i = blockIdx.x * (long long)RO_NT + threadIdx.x; i < N2; i += 2 * st) {
+  long long i = blockIdx.x * (long long)RO_NT + threadIdx.x;
+  if (below) {
+    // Every amplitude is read: all loads at once.  The few keys inside the range (a few per warp, so
+    // that most warps would take that branch for them) queue up in shared memory until there are 32.
+    // (i and N2 - 3 st are multiples of 32 across a warp: the loop is the same for all of it.)
+    const int lane = threadIdx.x & 31;
+    unsigned long long *qk = queue[0][threadIdx.x >> 5], *qq = queue[1][threadIdx.x >> 5];
+    int cnt = 0;
+    for (; i + 3 * st < N2; i += 4 * st) {
+      unsigned long long k[8], r0, r1;
+      T v[8];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        key_pair(E, i + j * st, k[2 * j], k[2 * j + 1], r0, r1);
+        amp_pair(psi, i + j * st, v[2 * j], v[2 * j + 1]);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const unsigned long long q = qmass(v[j]);
+        const bool in = k[j] >= lo && k[j] < hi;
+        if (k[j] < lo)
+          qbelow += q;
+        else if (!in)
+          qabove += q;
+        const unsigned mask = __ballot_sync(0xffffffffu, in);
+        if (in) {
+          const int at = cnt + __popc(mask & ((1u << lane) - 1));
+          qk[at] = k[j];
+          qq[at] = q;
+        }
+        cnt += __popc(mask);
+        if (cnt >= 32) {
+          __syncwarp();
+          drop(qk[lane], qq[lane]);
+          cnt -= 32;
+          const unsigned long long a = qk[32 + lane], b = qq[32 + lane];
+          __syncwarp();
+          if (lane < cnt) {
+            qk[lane] = a;
+            qq[lane] = b;
+          }
+          __syncwarp();
+        }
+      }
+    }
+    __syncwarp();
+    if (lane < cnt) drop(qk[lane], qq[lane]);
+  } else {
+    for (; i + 7 * st < N2; i += 8 * st) {
+      unsigned long long k[16], r0, r1;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) key_pair(E, i + j * st, k[2 * j], k[2 * j + 1], r0, r1);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const bool in0 = k[2 * j] >= lo && k[2 * j] < hi, in1 = k[2 * j + 1] >= lo && k[2 * j + 1] < hi;
+        if (in0 || in1) {
+          T v0, v1;
+          amp_pair(psi, i + j * st, v0, v1);
+          if (in0) add(k[2 * j], v0);
+          if (in1) add(k[2 * j + 1], v1);
+        }
+      }
+    }
+  }
+  for (; i < N2; i += 2 * st) {
     unsigned long long k[4], raw[4];
     key_pair(E, i, k[0], k[1], raw[0], raw[1]);
     const bool two = i + st < N2;
@@ -333,16 +505,29 @@ __global__ void __launch_bounds__(RO_NT) k_ro_hist(const T *psi, const double *E
       if (in3) add(k[3], v3);
     }
   }
-  atomicMin(&smin, kmin);
-  atomicMax(&smax, kmax);
-  if (qbelow) atomicAdd(&ext[0], qbelow);  // integer: order-independent
-  if (qabove) atomicAdd(&ext[3], qabove);
+  // one atomic per warp and CTA: with two from every thread, all on the same two words of L2, they took
+  // 150 of this pass's 330 us (26 qubits)
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
+    kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
+    qbelow += __shfl_xor_sync(0xffffffffu, qbelow, o);
+    qabove += __shfl_xor_sync(0xffffffffu, qabove, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&smin, kmin);
+    atomicMax(&smax, kmax);
+    if (qbelow) atomicAdd(&sbelow, qbelow);  // integer: order-independent
+    if (qabove) atomicAdd(&sabove, qabove);
+  }
   __syncthreads();
   for (int i = threadIdx.x; i < RO_BINS; i += RO_NT)
     if (sm[i]) atomicAdd(&gmass[i], sm[i]);
   if (threadIdx.x == 0) {
     atomicMin(&ext[1], smin);
     atomicMax(&ext[2], smax);
+    if (sbelow) atomicAdd(&ext[0], sbelow);
+    if (sabove) atomicAdd(&ext[3], sabove);
   }
 }
 
@@ -350,6 +535,56 @@ __global__ void __launch_bounds__(RO_NT) k_ro_hist(const T *psi, const double *E
 __global__ void k_ro_gather(const double *E, const long long *shots, int nshots, double *out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < nshots) out[k] = E[shots[k]];
+}
+
+// The energies of rank r0 (CTA 0) and r1 (CTA 1) among the shots', out[0..1]: their keys' bytes from the top,
+// counted in shared memory among the shots that share the bytes before.  Equal bytes of a warp
+// are counted once (the top bytes are nearly all the same).  8192 shots: 21 us; copying and
+// sorting them on the host took 290.
+constexpr int RANK_NT = 1024;
+__global__ void __launch_bounds__(RANK_NT) k_ro_rank(const double *es, int n, int r0, int r1, double *out) {
+  __shared__ int count[256], digit_s, rank_s;
+  const int tid = threadIdx.x, lane = tid & 31;
+  int rank = blockIdx.x ? r1 : r0;
+  unsigned long long prefix = 0ull;
+  for (int sh = 56; sh >= 0; sh -= 8) {
+    if (tid < 256) count[tid] = 0;
+    __syncthreads();
+    const unsigned long long above = sh == 56 ? 0ull : ~0ull << (sh + 8);
+    for (int i0 = 0; i0 < n; i0 += RANK_NT) {
+      const int i = i0 + tid;
+      int d = -1;
+      if (i < n) {
+        const unsigned long long k = key_of_bits((unsigned long long)__double_as_longlong(es[i]));
+        if ((k & above) == prefix) d = (int)(k >> sh) & 255;
+      }
+      const unsigned same = __match_any_sync(0xffffffffu, d);
+      if (d >= 0 && lane == __ffs(same) - 1) atomicAdd(&count[d], __popc(same));
+    }
+    __syncthreads();
+    if (tid < 32) {  // 8 digits a lane: the first whose running count passes the rank
+      int c[8], s = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) s += c[j] = count[8 * lane + j];
+      int incl = s;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const int l = __ffs(__ballot_sync(0xffffffffu, incl > rank)) - 1;
+      if (lane == l) {
+        int left = rank - (incl - s), d = 0;
+        while (d < 7 && left >= c[d]) left -= c[d++];
+        digit_s = 8 * lane + d;
+        rank_s = left;
+      }
+    }
+    __syncthreads();
+    rank = rank_s;
+    prefix |= (unsigned long long)digit_s << sh;
+  }
+  if (tid == 0) out[blockIdx.x] = __longlong_as_double((long long)((prefix >> 63) ? prefix & 0x7fffffffffffffffull : ~prefix));
 }
 
 // Tail sums for the CVaR: per CTA sum of p*E and p over E < tau, and of p over
@@ -367,6 +602,7 @@ struct KSum {
   }
 };
 
+// Bound by HBM: 26 qubits 163 us (0.8 GB), 208 with two loads in flight instead of eight.
 template <typename T>
 __global__ void __launch_bounds__(RO_NT) k_ro_tail(const T *psi, const double *E, long long N,
                                                    unsigned long long ktau, double *part) {
@@ -382,7 +618,22 @@ __global__ void __launch_bounds__(RO_NT) k_ro_tail(const T *psi, const double *E
     }
   };
   const long long N2 = N >> 1, st = (long long)gridDim.x * RO_NT;
-  for (long long i = blockIdx.x * (long long)RO_NT + threadIdx.x; i < N2; i += 2 * st) {
+  long long i = blockIdx.x * (long long)RO_NT + threadIdx.x;
+  for (; i + 7 * st < N2; i += 8 * st) {  // eight loads at once, the sums in the same order
+    unsigned long long k[16], raw[16];
+    T v[16];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) key_pair(E, i + j * st, k[2 * j], k[2 * j + 1], raw[2 * j], raw[2 * j + 1]);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[2 * j] = v[2 * j + 1] = T(0);
+      if (k[2 * j] <= ktau || k[2 * j + 1] <= ktau) amp_pair(psi, i + j * st, v[2 * j], v[2 * j + 1]);
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (k[j] <= ktau) add(k[j], v[j], raw[j]);
+  }
+  for (; i < N2; i += 2 * st) {
     unsigned long long k[4], raw[4];
     key_pair(E, i, k[0], k[1], raw[0], raw[1]);
     const bool two = i + st < N2;
@@ -416,14 +667,22 @@ __global__ void __launch_bounds__(RO_NT) k_ro_tail(const T *psi, const double *E
 // CVaR_alpha = (S + clamp(alpha T - P, 0, Pa) tau) / (alpha T), T = stats[2]:
 // the lowest-energy alpha fraction of the outcomes, the outcomes at E == tau
 // counted for the remainder.
-__global__ void k_ro_cvar(const double *part, int nparts, double alpha, double tau, double *stats) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double S = 0.0, P = 0.0, Pa = 0.0;
-  for (int i = 0; i < nparts; ++i) {
-    S += part[3 * i];
-    P += part[3 * i + 1];
-    Pa += part[3 * i + 2];
+// Three threads add the parts, one sum each, from shared memory: 29 us for 608 parts, the latency of the
+// FP64 adds in their order (88 with one thread reading them from L2).
+__global__ void __launch_bounds__(256) k_ro_cvar(const double *part, int nparts, double alpha, double tau, double *stats) {
+  extern __shared__ double sp[];
+  __shared__ double sums[3];
+  for (int i = threadIdx.x; i < 3 * nparts; i += blockDim.x) sp[i] = part[i];
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < nparts; ++i) s += sp[3 * i + threadIdx.x];
+    sums[threadIdx.x] = s;
   }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  const double S = sums[0], P = sums[1], Pa = sums[2];
   const double aT = alpha * stats[2];
   double rest = aT - P;
   rest = rest < 0.0 ? 0.0 : (rest > Pa ? Pa : rest);
@@ -467,7 +726,9 @@ cudaError_t launch_ro_prob(int prec, const void *psi, int n, double *csum, doubl
     k_ro_chunks<float><<<(unsigned)nch, RO_NT, 0, s>>>((const float *)psi, cb, csum, cmax, cidx);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_ro_scan<<<1, 1024, 0, s>>>(csum, cmax, cidx, nch, cdf, stats, argmax);
+  const unsigned nb = (unsigned)((nch + 1023) / 1024);
+  k_ro_scan<<<nb, 1024, 0, s>>>(csum, cmax, cidx, nch, cdf, stats, argmax);
+  if (nb > 1) k_ro_carry<<<nb, 1024, 0, s>>>(csum, cmax, cidx, nch, cdf, stats, argmax);
   return cudaGetLastError();
 }
 
@@ -504,6 +765,11 @@ cudaError_t launch_ro_gather(const double *E, const long long *shots, int nshots
   return cudaGetLastError();
 }
 
+cudaError_t launch_ro_rank(const double *es, int nshots, int r0, int r1, double *out, cudaStream_t s) {
+  k_ro_rank<<<2, RANK_NT, 0, s>>>(es, nshots, r0, r1, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_ro_cvar(int prec, const void *psi, const double *E, int n, double alpha, double tau,
                            double *part, double *stats, cudaStream_t s) {
   const int g = ro_grid();
@@ -516,7 +782,7 @@ cudaError_t launch_ro_cvar(int prec, const void *psi, const double *E, int n, do
     k_ro_tail<float><<<g, RO_NT, 0, s>>>((const float *)psi, E, 1LL << n, kt, part);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_ro_cvar<<<1, 32, 0, s>>>(part, g, alpha, tau, stats);
+  k_ro_cvar<<<1, 256, 24 * (size_t)g, s>>>(part, g, alpha, tau, stats);
   return cudaGetLastError();
 }
 

@@ -145,3 +145,30 @@ def test_readout_large_register_properties(fp64):
     r2 = gv.readout(a, h, tht, alpha=0.2, shots=1024, seed=9, fp64=fp64)
     assert r1.cvar == r2.cvar and r1.argmax == r2.argmax
     assert torch.equal(r1.shots, r2.shots)
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("n", [10, 11, 12, 14, 24])
+def test_shots_at_steps_of_the_cumulative_probability(n, fp64):
+    # u at, just under and just over a step: the first x whose cumulative probability exceeds u, or beside it
+    # where rounding (2^-40 here) leaves the step itself open; and the alpha = 0 call, which only samples
+    reps = 1
+    th = wl.thetas(n, reps, 1, seed=n)[0].copy()
+    th[: n // 2] = np.round(th[: n // 2] / math.pi) * math.pi  # exact zeros among the probabilities
+    a = gv.Ansatz(n, reps)
+    tht = torch.as_tensor(th, device="cuda")
+    rng = np.random.default_rng(n)
+    u = rng.random(300)
+    first = gv.readout(a, None, tht, alpha=0.0, uniforms=torch.as_tensor(u, device="cuda"), fp64=fp64)
+    p = ro.probabilities(oracle.state(n, reps, th))
+    cdf = np.cumsum(p.astype(np.longdouble))  # (2^24 adds in float64 would be 5e-12 off)
+    cdf = (cdf / cdf[-1]).astype(np.float64)
+    tol = _tol(fp64) * 4
+    assert np.all(p[first.shots.cpu().numpy()] > 0)
+    steps = cdf[rng.integers(0, 1 << n, 100)]
+    u = np.clip(np.concatenate([steps, steps - 2.0**-40, steps + 2.0**-40, [0.0, 1.0 - 2.0**-53]]), 0.0, 1.0 - 2.0**-53)
+    s = gv.readout(a, None, tht, alpha=0.0, uniforms=torch.as_tensor(u, device="cuda"), fp64=fp64).shots.cpu().numpy()
+    assert np.all(cdf[s] > u - tol) and np.all(np.where(s > 0, cdf[np.maximum(s - 1, 0)], 0.0) <= u + tol)
+    again = gv.readout(a, None, tht, alpha=0.0, uniforms=torch.as_tensor(u, device="cuda"), fp64=fp64).shots.cpu().numpy()
+    assert np.array_equal(s, again)
+    a.close()
