@@ -590,7 +590,8 @@ int mps_layers_for(int n, int reps, int prec, int ent, int gates, int want) {
 }
 
 Plan build_plan(int n, int reps, int prec, int tile_bits, bool want_grad, bool diag, bool tile_grad_l0,
-                bool state_only, int ent, int gates, int split, int xy_tb, int mps_layers, bool mps_tc) {
+                bool state_only, int ent, int gates, int split, int xy_tb, int mps_layers, bool mps_tc,
+                int cut_layers) {
   if (gates == 2) return build_plan_su2(n, reps, prec, tile_bits, want_grad, diag, ent, state_only, split);
   Plan pl;
   pl.n = n;
@@ -620,7 +621,8 @@ Plan build_plan(int n, int reps, int prec, int tile_bits, bool want_grad, bool d
   // pair (energy path), the lambda ping-pong pair, and psi_0 for X/Y terms at reps = 0.
   // closed-form leading layers 1..R; with gradients, theirs come from lambda_R
   // and the matrix product (mgrad), so only layer R's final state is stored
-  const int R = (mps_layers > 0 && reps >= 2) ? std::min(mps_layers, reps - 1) : 0;
+  const int RC = (!want_grad && !state_only && reps > cut_layers) ? cut_layers : 0;
+  const int R = (RC == 0 && mps_layers > 0 && reps >= 2) ? std::min(mps_layers, reps - 1) : 0;
   const bool mgrad = want_grad && !state_only && R >= 1 && R <= MPS_MAX_LAYERS;
   int nb = 0;
   const int first_state = nb;
@@ -713,7 +715,11 @@ Plan build_plan(int n, int reps, int prec, int tile_bits, bool want_grad, bool d
       cur = st.out;
     }
   }
-  for (int r = R + 1; r <= reps; ++r) {
+  if (RC > 0) {
+    pl.cut_layers = RC;
+    pl.cut_buf = cur = PP0;
+  }
+  for (int r = std::max(R, RC) + 1; r <= reps; ++r) {
     for (int j = 0; j < p; ++j) {
       const LayerPass &lp = pl.lp[j];
       PassStep st;
@@ -1157,15 +1163,35 @@ static int ensure_tables(gvqe_hamiltonian_s *h, int prec, cudaStream_t s, bool c
 }
 
 // --------------------------------------------------------- plan execution --
-Plan *gvqe::get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state_only, bool allow_mps) {
+// Energies of a circuit with too many crossing CNOTs for the whole of it (circular and SCA
+// entanglers from 4 layers): how many leading layers have at most 64 terms.  Their state is
+// written from the halves in one pass, the passes over it begin with the layer after.  Pays once
+// the passes are long against the half circuits' latency, 2^23 amplitudes in a call: 4 circular
+// layers, one vector of 22 qubits 112 us (105 with passes alone), 8 vectors of 20 qubits 115 (140),
+// one vector of 24 qubits 180 (315), of 28 qubits 1.59 ms (4.44).
+constexpr double CUT_STATE_AMPS = 0x1p23;
+static int cut_state_layers(gvqe_ansatz_s *a) {
+  if (a->gates != 1 || a->mps != 0 || a->mps_tc != 0) return 0;
+  gvqe_cut_plan &c = a->cut[3];
+  if (!c.known) {
+    c.known = true;
+    for (int r = std::min(a->reps - 1, CUT_MAX_LAYERS); r >= 2 && !c.ok; --r)
+      c.ok = cut_build(a->n, r, a->ent, 0, 1, &c.d);
+  }
+  return c.ok ? c.d.reps : 0;
+}
+
+Plan *gvqe::get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state_only, bool allow_mps,
+                     bool allow_cut) {
   const int key = prec | (want_grad ? 2 : 0) | (diag ? 4 : 0) | (state_only ? 8 : 0) | (a->gates == 2 ? 16 : 0) |
-                  (allow_mps ? 0 : 32);
+                  (allow_mps ? 0 : 32) | (allow_cut ? 64 : 0);
   auto it = a->plans.find(key);
   const int tb = eff_tile_bits(a, prec);
   if (it != a->plans.end() && it->second.tile_bits == tb) return &it->second;
   const int mps = allow_mps ? mps_layers_for(a->n, a->reps, prec, a->ent, a->gates, a->mps) : 0;
   Plan pl = build_plan(a->n, a->reps, prec, tb, want_grad, diag, false, state_only, a->ent, a->gates,
-                       eff_split(a, prec), eff_xy_tb(a, prec), mps, a->mps_tc >= 0);
+                       eff_split(a, prec), eff_xy_tb(a, prec), mps, a->mps_tc >= 0,
+                       allow_cut && mps == 0 && !prec && !want_grad && !state_only ? cut_state_layers(a) : 0);
   pl.tile_bits = tb;
   a->plans[key] = std::move(pl);
   return &a->plans[key];
@@ -1179,11 +1205,22 @@ static int upload_dir(Plan *pl) {
   return GVQE_OK;
 }
 
+static CutGrid cut_grid(const CutDesc &d) {
+  CutGrid g{};
+  g.cx = d.cx;
+  g.m0 = d.half[0].m;
+  g.m1 = d.half[1].m;
+  g.D = d.D;
+  g.reps = d.reps;
+  for (int r = 1; r <= d.reps; ++r) g.bits[r] = d.half[0].L[r - 1].shift + d.half[0].L[r - 1].nb;
+  return g;
+}
+
 // Run the plan for `batch` parameter vectors (already converted to cs on device).
 // With a state-only plan, *state receives job 0's final state (batch must be 1).
 static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const void *cs_all, const uint8_t *mask,
                     int batch, double *E, double *grad, const int *minlayer, cudaStream_t s,
-                    void **state = nullptr) {
+                    void **state = nullptr, const void *cs64 = nullptr) {
   const int prec = pl->prec;
   const size_t es = prec ? 8 : 4;
   const long long S = pl->state_elems;
@@ -1191,7 +1228,22 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
   // jobs per launch: enough tiles to fill the GPU, bounded by memory
   const long long tilesA = 1LL << (pl->n - pl->lp[0].tb);
   int J = (int)std::min<long long>(batch, std::max<long long>(1, 4096 / tilesA));
-  const size_t per_job = (size_t)pl->n_bufs * S * es + (size_t)pl->part_stride * 8 + (size_t)pl->mps_elems * 4;
+  CutArgs C;
+  memset(&C, 0, sizeof(C));
+  CutGrid cgrid{};
+  if (pl->cut_layers > 0) {
+    gvqe_cut_plan &c = a->cut[3];
+    GV_TRY(cut_upload(&c));
+    C.job0.lay = cut_layout(c.d, 0, false);
+    C.job0.desc = (const CutDesc *)c.dev.ptr;
+    C.ws_stride = C.job0.lay.total;
+    C.cs_stride = (long long)pl->P * 16;
+    C.P = pl->P;
+    C.state_stride = S;
+    cgrid = cut_grid(c.d);
+  }
+  const size_t per_job = (size_t)pl->n_bufs * S * es + (size_t)pl->part_stride * 8 + (size_t)pl->mps_elems * 4 +
+                         (size_t)C.ws_stride;
   size_t freeb = 0, total = 0;
   GV_CUDA(cudaMemGetInfo(&freeb, &total));
   size_t have = freeb + a->ws.bytes;
@@ -1202,7 +1254,7 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
     return fail(GVQE_ENOMEM, "one evaluation needs %.3f GiB of workspace, %.3f GiB available", per_job / 1073741824.0,
                 budget / 1073741824.0);
   J = (int)std::max<size_t>(1, std::min<size_t>((size_t)J, budget / per_job));
-  const size_t need = per_job * (size_t)J + 256;
+  const size_t need = per_job * (size_t)J + 512;
   GV_TRY(a->ws.reserve(need));
   char *base = (char *)a->ws.ptr;
   double *part = (double *)base;
@@ -1213,12 +1265,22 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
   };
   // closed-form layer tables after the state buffers (a multiple of 64 floats per job)
   float *mps_tab = (float *)(bufs + (size_t)pl->n_bufs * J * S * es);
+  C.job0.ws = (char *)(mps_tab + (size_t)pl->mps_elems * J) + 255;
+  C.job0.ws -= (uintptr_t)C.job0.ws % 256;
   const bool cplx = a->gates == 2;
   const void *table = h ? (cplx ? h->TC[prec].ptr : (prec ? h->T64.ptr : h->T32.ptr)) : nullptr;
   const void *tc = h ? (prec ? (const void *)h->d_tc64 : (const void *)h->d_tc32) : nullptr;
   if (state) *state = buf_ptr(pl->final_buf);
   for (int j0 = 0; j0 < batch; j0 += J) {
     const int jobs = std::min(J, batch - j0);
+    if (pl->cut_layers > 0) {
+      C.njobs = jobs;
+      C.job0.cs = (const char *)cs64 + (long long)j0 * C.cs_stride;
+      C.state = (float *)buf_ptr(pl->cut_buf);
+      int nl = 0;
+      GV_CUDA(launch_cut_state(C, cgrid, s, &nl));
+      count_launches(nl);
+    }
     for (const PassStep &st : pl->steps) {
       PassArgs A = st.A;
       A.job0 = j0;
@@ -1500,13 +1562,7 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
   A.ws_stride = (long long)per_job;
   A.cs_stride = (long long)P * 16;
   A.P = P;
-  CutGrid grid{};
-  grid.cx = c->d.cx;
-  grid.m0 = c->d.half[0].m;
-  grid.m1 = c->d.half[1].m;
-  grid.D = c->d.D;
-  grid.reps = c->d.reps;
-  for (int r = 1; r <= c->d.reps; ++r) grid.bits[r] = c->d.half[0].L[r - 1].shift + c->d.half[0].L[r - 1].nb;
+  const CutGrid grid = cut_grid(c->d);
   for (int j0 = 0; j0 < batch; j0 += J) {
     A.njobs = std::min(J, batch - j0);
     A.job0.cs = (const char *)cs + (long long)j0 * A.cs_stride;
@@ -1546,22 +1602,27 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
     return run_cut(a, h, c, a->aux.ptr, mask, batch, E, grad, prec, s);
   }
   GV_TRY(ensure_tables(h, prec, s, cplx));
-  Plan *pl = get_plan(a, prec, grad != nullptr, diag);
+  Plan *pl = get_plan(a, prec, grad != nullptr, diag, false, true, std::ldexp((double)batch, a->n) >= CUT_STATE_AMPS);
   const int P = pl->P;
   // trig table and per-job lowest active layer
   const size_t cs_bytes = (size_t)batch * P * (prec ? 16 : 8);
-  GV_TRY(a->aux.reserve(cs_bytes + (size_t)batch * 4 + 256));
-  void *cs = a->aux.ptr;
+  const size_t cs64_at = (cs_bytes + (size_t)batch * 4 + 511) / 256 * 256;
+  GV_TRY(a->aux.reserve(cs64_at + (pl->cut_layers > 0 ? (size_t)batch * P * 16 : 0)));
+  void *cs = a->aux.ptr, *cs64 = (char *)a->aux.ptr + cs64_at;
   int *minlayer = (int *)((char *)a->aux.ptr + ((cs_bytes + 255) / 256) * 256);
   GV_CUDA(launch_trig(prec, params, (long long)batch * P, cs, s));
   count_launches(1);
+  if (pl->cut_layers > 0) {
+    GV_CUDA(launch_trig(1, params, (long long)batch * P, cs64, s));
+    count_launches(1);
+  }
   const int *ml = nullptr;
   if (grad) {
     GV_CUDA(launch_minlayer(mask, batch, a->n * a->gates, P, a->reps + 1, minlayer, s));
     count_launches(1);
     ml = minlayer;
   }
-  return run_plan(a, h, pl, cs, mask, batch, E, grad, ml, s);
+  return run_plan(a, h, pl, cs, mask, batch, E, grad, ml, s, nullptr, cs64);
 }
 
 static int param_shift_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, const uint8_t *mask, int batch,
@@ -2069,6 +2130,13 @@ int gvqe_ansatz_describe(gvqe_ansatz a, int flags, char *buf, int buflen) {
     char line[160];
     snprintf(line, sizeof(line), "diagonal H: evaluated from the halves [0,%d) and [%d,%d), %d terms%s\n", c->d.half[1].q0,
              c->d.half[1].q0, a->n, c->d.D, prec ? "" : " (tensor cores, TF32 split)");
+    s += line;
+  }
+  if (!prec && get_plan(a, prec, false, true, false, true, true)->cut_layers > 0) {
+    const CutDesc &d = a->cut[3].d;
+    char line[160];
+    snprintf(line, sizeof(line), "energies: the state after layer %d written from the halves [0,%d) and [%d,%d), %d terms\n",
+             d.reps, d.half[1].q0, d.half[1].q0, a->n, d.D);
     s += line;
   }
   if (!a->tune_report.empty()) s += a->tune_report;

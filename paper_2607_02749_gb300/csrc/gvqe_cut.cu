@@ -578,6 +578,29 @@ cudaError_t launch_tile_tables(const TableJob *jobs, int njobs, int nmax, cudaSt
 // circuits: one class for every small size, one per size above.
 int cut_class(int prec, int m) { return m <= HALF_SMALL_M(prec) ? HALF_SMALL_M(prec) : m; }
 
+static cudaError_t launch_pack(CutArgs A, const CutGrid &g, int K, cudaStream_t s) {
+  A.items = g.pack_items;
+  A.blk0 = 1 << (g.m0 - 6);
+  A.nblk = A.blk0 + (1 << (g.m1 - 6));
+  auto k = g.cx ? k_cut_pack<true> : k_cut_pack<false>;
+  k<<<g.pack_items ? g.pack_blocks : A.njobs * A.nblk, 256, K * 65 * (g.cx ? 4 : 8), s>>>(A, K);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cut_state(const CutArgs &A0, const CutGrid &g, cudaStream_t s, int *launches) {
+  CutArgs A = A0;
+  const int K = cut_k(g.D);
+  A.blk0 = g.D;
+  A.items = nullptr;
+  cudaError_t e = launch_cut_fwd32(A, g, false, s, launches);
+  if (e == cudaSuccess) e = launch_pack(A, g, K, s);
+  if (e != cudaSuccess) return e;
+  A.blk0 = A.job0.lay.rb[0] * A.job0.lay.ns[0];
+  A.nblk = A.njobs * A.blk0;
+  *launches += 2;
+  return launch_cut_tc(A, K, CUT_STATE, s);
+}
+
 cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
                        const CutXyDims *xy) {
   CutArgs A = A0;
@@ -593,12 +616,7 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
     CUT_CHECK(launch_half<double>(A, cut_class(1, g.m0), grad ? 1 : 0, half_blocks, s));
   } else {
     CUT_CHECK(g.cx ? launch_halfc(A, g.m0, grad ? 1 : 0, half_blocks, s) : launch_cut_fwd32(A, g, grad, s, launches));
-    A.items = g.pack_items;
-    A.blk0 = 1 << (g.m0 - 6);
-    A.nblk = A.blk0 + (1 << (g.m1 - 6));
-    auto k = g.cx ? k_cut_pack<true> : k_cut_pack<false>;
-    k<<<g.pack_items ? g.pack_blocks : A.njobs * A.nblk, 256, K * 65 * (g.cx ? 4 : 8), s>>>(A, K);
-    CUT_CHECK(cudaGetLastError());
+    CUT_CHECK(launch_pack(A, g, K, s));
     *launches += 1;
   }
   A.blk0 = l.rb[0] * l.ns[0];
@@ -621,7 +639,7 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
     }
     CUT_CHECK(cudaGetLastError());
   } else {
-    CUT_CHECK(launch_cut_tc(A, K, grad, s));
+    CUT_CHECK(launch_cut_tc(A, K, grad ? CUT_GRAD : CUT_ENERGY, s));
   }
   *launches += 3;
   if (xy) CUT_CHECK(launch_cut_xy(A, g, *xy, grad, s, launches));

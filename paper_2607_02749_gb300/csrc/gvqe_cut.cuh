@@ -113,6 +113,8 @@ struct CutArgs {
   int P;                // parameters per job (with jobs == NULL)
   int njobs, nblk;
   int blk0;             // blocks of half 0 per job (without items)
+  float *state;         // launch_cut_state: the states, state_stride floats apart
+  long long state_stride;
 };
 
 // The cut plan of a circuit; false when it has none (no layer, too many layers or
@@ -137,6 +139,8 @@ int cut_k(int D);  // terms of the tensor-core operands
 cudaError_t launch_cut(int prec, const CutArgs &A, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
                        const CutXyDims *xy = nullptr);
 int cut_xy_dp(int D);  // row length of its matrices
+// The state itself, S of every tile, for circuits that go on after these layers (FP32, RY).
+cudaError_t launch_cut_state(const CutArgs &A, const CutGrid &g, cudaStream_t s, int *launches);
 cudaError_t launch_cut_xy(const CutArgs &A, const CutGrid &g, const CutXyDims &x, bool grad, cudaStream_t s, int *launches);
 // The diagonal table in the order the FP32 contractions read it, rounded from FP64:
 // d0 for contraction 0 (rows x_lo), d1 for contraction 1 (rows x_hi; may be NULL).  Tiles
@@ -173,7 +177,8 @@ struct SmemLimit {
   }
 };
 // FP32 contraction on the tensor cores (gvqe_cut_tc.cu).
-cudaError_t launch_cut_tc(const CutArgs &A, int K, bool grad, cudaStream_t s);
+enum CutUse { CUT_ENERGY = 0, CUT_GRAD = 1, CUT_STATE = 2 };
+cudaError_t launch_cut_tc(const CutArgs &A, int K, CutUse use, cudaStream_t s);
 
 // What a kernel uses of job k (the layout is indexed in place, not copied).
 struct CutView {

@@ -162,12 +162,15 @@ struct Cfg {
   static constexpr int PARTS = 64 * K;  // floats of one operand image part
 };
 
-template <int K, bool GRAD>
+// CUT_STATE: S is the result, stored row by row (a warp's 32 rows of a column are 128 bytes);
+// bound by the stores, and by S's MMAs at 64 terms.
+template <int K, CutUse USE>
 __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant__ CutArgs A) {
   using C = Cfg<K>;
+  constexpr bool GRAD = USE == CUT_GRAD, STATE = USE == CUT_STATE;
   constexpr int HALF = 2 * C::PARTS;  // floats of one half of B: its hi and lo parts
   constexpr int ETILE = 128 * COLS;   // floats of a tile of E (complex: half of them used)
-  constexpr int ES = C::ES;
+  constexpr int ES = STATE ? 0 : C::ES;
   extern __shared__ __align__(128) float dyn[];
   float *sR = dyn, *sE = dyn + C::RS * HALF, *sC = sE + ES * ETILE;
   __shared__ __align__(8) unsigned long long bars[2 * (C::RS + C::CS + ES) + 2 * C::BUFS + C::GBUFS];
@@ -296,7 +299,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     constexpr int AHEAD = C::GBUFS == 4 ? 2 : 0;  // tiles between a tile's lambda and its G
     const f2 neg1 = pk2(-1.f, -1.f);
     int t = g;
-    if constexpr (!ES) load(t);  // (2 tiles at least)
+    if constexpr (!ES && !STATE) load(t);  // (2 tiles at least)
     for (; t < nt; t += 2) {
       const int b = t % C::BUFS, ee = ES ? t % (ES + !ES) : 0;
       if constexpr (ES > 0)
@@ -306,6 +309,9 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
       const uint32_t ts = tw + C::S0 + 128 * b;
       const float4 *et = reinterpret_cast<const float4 *>(sE + ee * ETILE) + (r >> cx);
       f2 e0 = 0, e1 = 0, z0 = 0, z1 = 0;
+      float *out = nullptr;
+      if constexpr (STATE)
+        out = A.state + (size_t)job * A.state_stride + ((size_t)(t0 + t) << (mr + 6)) + row0 + r;
       auto tile = [&](auto energy) {
 #pragma unroll(ES ? 1 : COLS / 16)
         for (int c = 0; c < COLS; c += 16) {
@@ -328,6 +334,13 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
             const f2 s = add2(pk2(v[j], v[j + 1]), pk2(l[j], l[j + 1]));
+            if constexpr (STATE) {
+              float x, y;
+              unpk2(s, x, y);
+              out[(size_t)(c + j) << mr] = x;
+              out[(size_t)(c + j + 1) << mr] = y;
+              continue;
+            }
             const f2 lam = mul2(s, tv[j / 2]);
             if constexpr (decltype(energy)::value) {
               f2 &e = (j & 2) ? e1 : e0, &z = (j & 2) ? z1 : z0;
@@ -347,7 +360,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
           }
         }
       };
-      if (h == 0)
+      if (h == 0 && !STATE)
         tile(Yes{});
       else
         tile(No{});
@@ -358,9 +371,9 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
         arrive(lbar(b));
         if constexpr (ES > 0) arrive(eempty(ee));
       }
-      if constexpr (!ES)
+      if constexpr (!ES && !STATE)
         if (t + 2 < nt) load(t + 2);
-      if (h == 0) {
+      if (h == 0 && !STATE) {
         float x, y;
         unpk2(add2(e0, e1), x, y);
         two_sum(e_hi, e_lo, x + y);
@@ -372,7 +385,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     }
     if constexpr (GRAD && AHEAD > 0)
       if (t >= 2 && !*bad) drain(t - 2);
-    if (h == 0) {
+    if (h == 0 && !STATE) {
       double e = (double)e_hi + e_lo, z = (double)z_hi + z_lo;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -399,7 +412,8 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
       for (int k = 0; k < K; ++k)
         if (k < D) gout[(size_t)k << mr] = good ? acc[k] + x[k * 128 + r] : __int_as_float(0x7fc00000);
     }
-    if (h == 0 && tid == 0) {
+    if (STATE && !good && w < 4) A.state[(size_t)job * A.state_stride + row0 + r] = __int_as_float(0x7fc00000);
+    if (h == 0 && tid == 0 && !STATE) {
       double e = 0.0, z = 0.0;
       for (int k = 0; k < 8; ++k) {
         e += es[0][k];
@@ -508,12 +522,13 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
   if (w == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-template <int K, bool GRAD>
+template <int K, CutUse USE>
 cudaError_t launch_k(const CutArgs &A, cudaStream_t s) {
   using C = Cfg<K>;
   // (the copies' stages, then reused for the rows' sums: K x 128 floats)
-  const size_t need = (size_t)4 * ((C::RS + (GRAD ? C::CS : 0)) * 2 * C::PARTS + C::ES * 128 * COLS);
-  auto k = k_cut_contract_tc<K, GRAD>;
+  const size_t need = (size_t)4 * ((C::RS + (USE == CUT_GRAD ? C::CS : 0)) * 2 * C::PARTS +
+                                   (USE == CUT_STATE ? 0 : C::ES) * 128 * COLS);
+  auto k = k_cut_contract_tc<K, USE>;
   static SmemLimit limit;
   if (const cudaError_t e = limit.set(k, need)) return e;
   k<<<A.nblk, NT, need, s>>>(A);
@@ -522,10 +537,12 @@ cudaError_t launch_k(const CutArgs &A, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_cut_tc(const CutArgs &A, int K, bool grad, cudaStream_t s) {
-  if (K == 16) return grad ? launch_k<16, true>(A, s) : launch_k<16, false>(A, s);
-  if (K == 32) return grad ? launch_k<32, true>(A, s) : launch_k<32, false>(A, s);
-  return grad ? launch_k<64, true>(A, s) : launch_k<64, false>(A, s);
+template <int K>
+static cudaError_t launch_use(const CutArgs &A, CutUse use, cudaStream_t s) {
+  return use == CUT_GRAD ? launch_k<K, CUT_GRAD>(A, s) : use == CUT_STATE ? launch_k<K, CUT_STATE>(A, s) : launch_k<K, CUT_ENERGY>(A, s);
+}
+cudaError_t launch_cut_tc(const CutArgs &A, int K, CutUse use, cudaStream_t s) {
+  return K == 16 ? launch_use<16>(A, use, s) : K == 32 ? launch_use<32>(A, use, s) : launch_use<64>(A, use, s);
 }
 
 }  // namespace gvqe

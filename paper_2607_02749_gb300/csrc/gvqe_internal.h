@@ -65,6 +65,8 @@ struct Plan {
   bool mps_grad = false;      // ... and their gradients from lambda and the matrix product
   bool mps_tc = false;        // ... with the bond-16 chunk contractions on the tensor cores
   long long mps_elems = 0;    // floats of closed-form tables per job (one stage at a time)
+  int cut_layers = 0;         // leading layers whose state is written from the halves (energies), ...
+  int cut_buf = -1;           // ... into this buffer
   DevBuf d_dir;
   int d_dir_count = 0;
 };
@@ -84,7 +86,7 @@ void count_launches(int k);
 // the writer and the gradient pass over lambda contract on the tensor cores (F_MPS_TC).
 Plan build_plan(int n, int reps, int prec, int tile_bits, bool want_grad, bool diag, bool tile_grad_l0 = false,
                 bool state_only = false, int ent = ENT_LINEAR, int gates = 1, int split = SPLIT_AUTO, int xy_tb = 0,
-                int mps_layers = 0, bool mps_tc = true);
+                int mps_layers = 0, bool mps_tc = true, int cut_layers = 0);
 // How many leading layers a plan may write in closed form: FP32, RY layers,
 // an entangler whose index map ties each qubit only to the one below it
 // (linear, full, reverse linear), n >= MPS_MIN_QUBITS, and never the last
@@ -158,7 +160,7 @@ struct gvqe_ansatz_s {
   int mps = 0;                   // GVQE_OPT_MPS_LAYERS (0 auto, -1 none, 1..4 at most that many)
   int mps_tc = 0;                // GVQE_OPT_MPS_TENSOR (0 auto = tensor cores, -1 = FP32 pipe)
   std::map<int, gvqe::Plan> plans;
-  gvqe_cut_plan cut[3];          // FP32, FP64, FP32 with RZ layers
+  gvqe_cut_plan cut[4];          // FP32, FP64, FP32 with RZ layers, FP32 leading layers (state)
   gvqe::DevBuf ws, aux, shift, ro, tune;
   std::string tune_report;  // the last gvqe_autotune sweep and its choice (empty: not tuned)
 };
@@ -175,7 +177,8 @@ inline int eff_xy_tb(const gvqe_ansatz_s *a, int prec) { return a->tuned_xy_tb[p
 // state only); it and its host-side reduction directory live until the
 // ansatz is destroyed or one of its options changes.
 // allow_mps = false: no closed-form layers (callers without a table region).
-Plan *get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state_only = false, bool allow_mps = true);
+Plan *get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state_only = false, bool allow_mps = true,
+               bool allow_cut = false);
 // The ansatz's two-half plan for this precision when its options and circuit let it take
 // the place of the tile passes for a diagonal H, else NULL.  cut_upload: its descriptor
 // on the device.  ensure_cut_tables: what its contraction reads of the Hamiltonian.

@@ -175,3 +175,26 @@ def test_fp64_many_terms(n, reps, ent, batch):
     with oracle.entangler(ent):
         er, gr = oracle.energy_grad(n, reps, th[0], ham.strings, ham.coeffs)
     assert abs(e[0] - er) <= 1e-10 * scale and np.max(np.abs(g[0] - gr)) <= 1e-9 * scale
+
+
+@pytest.mark.parametrize("n,reps,ent,batch,xy", [(18, 4, gv.GVQE_ENT_CIRCULAR, 35, 0), (19, 5, gv.GVQE_ENT_SCA, 16, 0),
+                                                 (20, 4, gv.GVQE_ENT_SCA, 9, 0.4), (23, 4, gv.GVQE_ENT_CIRCULAR, 1, 0),
+                                                 (24, 5, gv.GVQE_ENT_CIRCULAR, 1, 0), (25, 7, gv.GVQE_ENT_SCA, 2, 0)])
+def test_energies_with_the_leading_layers_from_halves(n, reps, ent, batch, xy):
+    # FP32 energies of circuits with more than 64 terms: the state after layer 3 (64 terms) comes from the halves.
+    # Each amplitude is within a few 2^-23 of its value on either route: 2e-6 of sum |c| against FP64.
+    ham = wl.pauli_hamiltonian(n, 6 * n, seed=n, xy_fraction=xy) if xy else wl.z_hamiltonian(n, 6 * n, seed=n)
+    th = torch.as_tensor(wl.thetas(n, reps, batch, seed=n + ent), device="cuda")
+    h = gv.Hamiltonian.from_workload(ham)
+    a, b = gv.Ansatz(n, reps, entangler=ent), gv.Ansatz(n, reps, entangler=ent)
+    b.set_mps_layers(-1)
+    assert "state after layer 3" in a.describe() and "64 terms" in a.describe()
+    assert "state after layer" not in b.describe()
+    e, ep = gv.energy(a, h, th).cpu().numpy(), gv.energy(b, h, th).cpu().numpy()
+    e64 = gv.energy(a, h, th, fp64=True).cpu().numpy()
+    tol = 2e-6 * ham.abs_sum()
+    assert np.abs(e - e64).max() <= tol and np.abs(ep - e64).max() <= tol
+    assert np.array_equal(e, gv.energy(a, h, th).cpu().numpy())
+    a.close()
+    b.close()
+    h.close()
