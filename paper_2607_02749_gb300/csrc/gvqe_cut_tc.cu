@@ -25,6 +25,9 @@
 // where the sums of G take the registers: one vector of 30 qubits, 64 terms, 2.20 ms with loads and
 // 2.03 ms with copies; 24 qubits, 16 terms, 0.303 and 0.369 ms (each tile then waits
 // for a second barrier).
+// Nothing is full (24 qubits, 16 vectors: L2 30%, tensor pipe 29%, issue 37%): the chain of a tile,
+// S's MMAs, two waits, lambda, G's MMAs, over 2 or 3 buffers of S.  A third group of row warps does not
+// help (312 us for 296), nor does a tile shared by both groups (399 us: twice the waits).
 #include "gvqe_cut.cuh"
 
 namespace gvqe {
@@ -104,12 +107,21 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, vola
   return done != 0;
 }
 
-// The same for a whole warp: one lane polls (32 would keep the barrier unit busy and every
-// other wait of the CTA, above all the MMA warp's, behind them).
+// The same for a whole warp, all of it leaving together.  (All lanes ask: one lane asking and a
+// shuffle of its answer took longer; 24 qubits, 16 vectors 321 us so, 296 with all.)
 __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int *bad) {
-  int ok = 1;
-  if ((threadIdx.x & 31) == 0) ok = wait_bounded(bar, parity, bad);
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+  for (int it = 0; it < (1 << 16); ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2, 20000;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (__all_sync(0xffffffffu, done)) return true;
+    if (__any_sync(0xffffffffu, *bad)) return false;
+  }
+  *bad = 1;
+  return false;
 }
 
 __device__ __forceinline__ void two_sum(float &hi, float &lo, float x) {
@@ -384,7 +396,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
         if (t >= AHEAD && !drain(t - AHEAD)) break;
     }
     if constexpr (GRAD && AHEAD > 0)
-      if (t >= 2 && !*bad) drain(t - 2);
+      if (t >= 2 && !__any_sync(0xffffffffu, *bad)) drain(t - 2);
     if (h == 0 && !STATE) {
       double e = (double)e_hi + e_lo, z = (double)z_hi + z_lo;
 #pragma unroll

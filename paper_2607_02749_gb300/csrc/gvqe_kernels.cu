@@ -323,6 +323,7 @@ __global__ void k_reduce(const double *__restrict__ part, long long part_stride,
   const RedEntry d = dir[e];
   const double *p = part + job * part_stride + d.off;
   double s = 0.0;
+#pragma unroll 16  // (loads in flight; the adds stay in order)
   for (int i = lane; i < d.count; i += 32) s += p[i];
   s = warp_sum(s);
   if (lane == 0) {
