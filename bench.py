@@ -11,8 +11,9 @@ gradient).  Inputs are synthetic and seeded.
 Printed JSON line (rank 0): metric/value/unit (E+grad evaluations per second,
 device-timed with CUDA events on the launching stream), e2e (same metric through
 the public API with pinned host inputs copied in and results copied out every
-step), roofline of the dominant kernel (algorithmic bytes / measured launch
-time vs the measured HBM copy bandwidth), the FP64 parameter-shift comparator
+step), roofline of the dominant kernel (the contraction of the half tables: TF32
+tensor operations / measured launch time vs half the measured bf16 rate; tile passes:
+algorithmic bytes vs the measured HBM copy bandwidth), the FP64 parameter-shift comparator
 on the same GPU, FP32-vs-FP64 errors, clocks during the timed region and the
 CPU oracle baseline.
 
@@ -97,14 +98,14 @@ def max_over_ranks(value: float, dist, device) -> float:
     return t.item()
 
 
-def measured_peaks():
+def measured_peaks(key="hbm_gbs", fallback=FALLBACK_HBM_GBS):
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     try:
         with open(p) as f:
             d = json.load(f)
-        return float(d["hbm_gbs"]), "measured"
+        return float(d[key]), "measured"
     except Exception:
-        return FALLBACK_HBM_GBS, "fallback"
+        return fallback, "fallback"
 
 
 def workload_sweeps(n: int, reps: int, n_terms: int):
@@ -283,52 +284,12 @@ def cluster_leg(steps: int):
     torch.cuda.synchronize()
     dt_loop = time.perf_counter() - t0
     amps = sum(2 ** i.n_qubits for i in insts)
-    # algorithmic bytes of one run (FP32, every layer's passes): per amplitude 4 (layer 1's
-    # first pass writes only) + 8 per other forward pass + 12 per backward pass + 4 (layer 0)
-    lib = _lib.load()
-    nbytes = 0
-    for i in insts:
-        p = lib.gvqe_plan_describe(i.n_qubits, i.reps, _lib.GVQE_FP32, 0, None, 0)
-        nbytes += 2 ** i.n_qubits * (4 + 8 * (i.reps * p - 1) + 12 * i.reps * p + 4)
-    peak, peak_src = measured_peaks()
-    gbps = nbytes / dt / 1e9
-    tuned = _tuned_ms(tune)
-    l2 = l2_copy_gbps()
     return {"value": len(insts) / dt, "unit": "E+grad/s", "instances": len(insts), "ms_per_run": dt * 1e3,
-            "tuned_GBps": nbytes / (tuned / 1e3) / 1e9 if tuned else None,
-            "tuned_frac_of_hbm_peak": (nbytes / (tuned / 1e3) / 1e9 / peak) if (tuned and peak) else None,
-            "l2_copy_GBps": l2, "frac_of_l2_copy": (nbytes / (tuned / 1e3) / 1e9 / l2) if tuned else None,
             "launches_per_run": launches, "per_instance_calls_ms": dt_loop * 1e3,
-            "total_amplitudes": amps, "algorithmic_GB_per_run": nbytes / 1e9, "GBps": gbps,
-            "frac_of_hbm_peak": gbps / peak if peak else None,
-            "schedule": tune.strip().splitlines(),
+            "total_amplitudes": amps, "schedule": tune.strip().splitlines(),
             "tuned_ms_per_run": _tuned_ms(tune),
-            "note": "algorithmic bytes: per amplitude 4 + 8 per further forward pass + 12 per backward pass + 4 "
-                    "(every pass of the 2^12-tile plans); at 256 instances a stage's states exceed L2, so the "
-                    "traffic is DRAM traffic (ncu) and the HBM copy peak is the denominator; the L2 copy rate "
-                    "is given for reference",
+            "note": "evaluated from the registers' halves: no state is stored, so there are no bytes of state passes to count",
             "timing": "wall clock around synchronous gvqe_batch_run calls (tuned_ms_per_run: CUDA events)"}
-
-
-def l2_copy_gbps(reps: int = 200) -> float:
-    """Read + write GB/s of a device copy whose source and destination (32 MB in all)
-    stay in the 129 MB L2: the same-job reference for traffic that stays on chip."""
-    import torch
-
-    n = 4 << 20
-    a = torch.ones(n, dtype=torch.float32, device="cuda")
-    b = torch.empty_like(a)
-    for _ in range(5):
-        b.copy_(a)
-    torch.cuda.synchronize()
-    e0 = torch.cuda.Event(enable_timing=True)
-    e1 = torch.cuda.Event(enable_timing=True)
-    e0.record()
-    for _ in range(reps):
-        b.copy_(a)
-    e1.record()
-    torch.cuda.synchronize()
-    return 2.0 * n * 4 * reps / (e0.elapsed_time(e1) / 1e3) / 1e9
 
 
 def _tuned_ms(report: str):
@@ -782,9 +743,10 @@ def run_gvqe(args):
     # Each kind's share over its measured time is its algorithmic GB/s; the
     # implementation's own per-pass bytes (every tile pass reads and writes the
     # whole state) give the per-pass figure beside it.
-    prof = {k: _lib.gvqe_profile_read(k) for k in range(11)}
+    prof = {k: _lib.gvqe_profile_read(k) for k in range(12)}
     names = {0: "k_fwd", 1: "k_bwd", 2: "k_grad_l0", 3: "k_lambda_xy", 4: "k_wht", 5: "k_mps_write",
-             6: "k_mps_tab", 7: "k_mps_grad", 8: "k_mps_gtree", 9: "k_mps_gred", 10: "k_mps_genv"}
+             6: "k_mps_tab", 7: "k_mps_grad", 8: "k_mps_gtree", 9: "k_mps_gred", 10: "k_mps_genv",
+             11: "k_cut_contract_tc"}
     dom = max(prof, key=lambda k: prof[k]["ms"])
     pk = prof[dom]
     peak, peak_src = measured_peaks()
@@ -831,7 +793,26 @@ def run_gvqe(args):
                      for k in prof if prof[k]["launches"]},
     }
     fwd_ms = sum(prof[k]["ms"] for k in (0, 5, 6))
-    if fwd_ms > 0:
+    cut = re.search(r"evaluated from the halves .* (\d+) terms", a.describe())
+    if dom == 11 and cut:
+        # no state is stored: per E+grad S and G once for either half, 2 D 2^n multiply-adds each
+        # way, every product as three TF32 ones
+        D = int(cut.group(1))
+        tf = 24.0 * max(16, D) * 2.0 ** n * evals / (pk["ms"] / 1000.0) / 1e12
+        bf16 = measured_peaks("bf16_tflops", 1900.0)
+        roofline = {
+            "bound": "tensor", "achieved": tf, "peak": bf16[0] / 2, "unit": "TFLOP/s", "frac": tf / (bf16[0] / 2),
+            "traffic": None, "kernel": names[dom], "launches": pk["launches"], "avg_launch_ms": pk["ms"] / launches_dom,
+            "algorithmic_flops_per_launch": 6.0 * D * 2.0 ** n * evals / launches_dom,
+            "tf32_flops_per_launch": 24.0 * max(16, D) * 2.0 ** n * evals / launches_dom,
+            "flops_rule": "TF32: S = A B^T and G = lambda B for either half, 3 products each (hi/lo split), 2 K 2^n "
+                          "operations a product; algorithmic: S once and G for either half in one product each",
+            "terms": D, "share_of_step": pk["ms"] / ms,
+            "table_GBps": pk["bytes"] / (pk["ms"] / 1000.0) / 1e9,
+            "peak_source": f"{bf16[1]} (half of MEASURED_PEAKS.json bf16_tflops)" if bf16[1] == "measured" else "fallback",
+            "per_kind": {names[k]: {"launches": prof[k]["launches"], "ms": prof[k]["ms"]} for k in prof if prof[k]["launches"]},
+        }
+    if fwd_ms > 0 and dom != 11:
         roofline["per_kind"]["forward"] = {
             "kinds": "k_fwd + k_mps_write + k_mps_tab", "ms": fwd_ms,
             "GBps_algorithmic": alg_share[0] * evals / (fwd_ms / 1000.0) / 1e9}
@@ -868,7 +849,7 @@ def run_gvqe(args):
         "config": {"workload": args.workload, "n_qubits": n, "reps": reps, "n_params": P,
                    "n_terms": w["terms"], "batch_per_gpu": B, "global_batch": B * ws,
                    "amplitudes": "fp32 (real: RY+CX keeps the state real), fp64 table and reductions",
-                   "l2": "inputs larger than L2 (4 GiB state per pass)", "parallelism": f"replicas x{ws}"},
+                   "l2": "inputs larger than L2 (two 4 GiB tables per evaluation)", "parallelism": f"replicas x{ws}"},
         "e2e": e2e, "gpu_launches": launches, "roofline": roofline, "clocks": clk,
         "plan": {"autotune": tune_report.strip().splitlines(), "tune_seconds": tune_s, "cache": tune_cache,
                  "layer_passes": [ln.strip() for ln in a.describe().splitlines() if "layer pass" in ln]},

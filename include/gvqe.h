@@ -87,12 +87,18 @@ extern "C" {
                                  from contracted tables of those matrices (a write-only pass per state)
                                  instead of running their tile passes.  Same results up to FP32 rounding;
                                  the last layer always runs as tile passes.
-                                 At 0, evaluations of a diagonal H (gvqe_energy, gvqe_energy_grad, parameter
-                                 shift, staged batches) whose CNOTs cross the middle of the register at most
-                                 six times in all (linear, full, reverse linear, pairwise: once per layer;
-                                 circular, SCA: twice) are taken from the circuits of its two halves, with no
-                                 2^n state at all (FP32 from 14 qubits, FP64 from 10 to 28); any other value
-                                 keeps them on stored states.  Same results up to rounding in either precision. */
+                                 At 0, evaluations (gvqe_energy, gvqe_energy_grad, parameter shift, staged
+                                 batches) of circuits whose CNOTs cross the middle of the register few
+                                 times (linear, full, reverse linear, pairwise: once per layer; circular,
+                                 SCA: twice) are taken from the circuits of its two halves, with no 2^n
+                                 state at all: FP32 up to six crossings from 14 qubits, diagonal H or, where
+                                 they are the cheaper, X/Y strings; FP32 RY+RZ layers up to five crossings,
+                                 14 to 28 qubits, diagonal H; FP64 RY layers, diagonal H, 10 to 28
+                                 qubits, up to eight crossings (2^crossings terms: up to n reps of them
+                                 always, more where the call leaves the GPU idle).  FP32 energies with more
+                                 crossings begin with the state after the last layer that has at most six, from
+                                 2^23 amplitudes in a call.  Any other value keeps them on stored states.
+                                 Same results up to rounding in either precision. */
 #define GVQE_OPT_MPS_TENSOR 6 /* closed-form layers at bond dimension 16 (four closed-form layers): 0 = auto
                                  (the writer's product per 2^13-amplitude chunk, 128 x 16 x 64, and the
                                  gradient pass's two lambda contractions, 64 x 128 x 16 and 128 x 64 x 16, on
@@ -192,7 +198,10 @@ int gvqe_energy_grad(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, co
  * (gvqe_batch_set_option: staged by default, or one persistent kernel
  * launch); the others (X/Y strings, RY+RZ layers) are evaluated by single
  * gvqe_energy_grad calls on the same stream in the same gvqe_batch_run, after
- * the graph.  Staged results equal single calls bit for bit; the persistent
+ * the graph.  Staged results equal single calls bit for bit, but for FP64
+ * instances whose halves have more than n reps terms (GVQE_OPT_MPS_LAYERS): those
+ * take their halves only where the call leaves the GPU idle, which a single call
+ * does and a large batch does not, and the two agree to FP64 rounding.  The persistent
  * kernel's 2^12-amplitude tiles fix another summation order, so its results
  * agree with single calls within the precision bounds.
  *   n_inst: >= 1.  ansatze, hams: host arrays of n_inst handles (borrowed: they
@@ -234,8 +243,10 @@ int gvqe_batch_run(gvqe_batch b, const double *const *params, const uint8_t *con
  *     all its jobs (as gvqe_energy_grad runs a batch of vectors), on its own
  *     branch of the graph; the branches run side by side (the instances evaluated
  *     from their halves share their launches instead, see GVQE_OPT_MPS_LAYERS).
- *     Results equal those of single gvqe_energy_grad calls bit for bit, and every instance with RY
- *     layers and a diagonal H takes part, whatever its n.
+ *     Results equal those of single gvqe_energy_grad calls bit for bit (but see
+ *     gvqe_batch_create), and every instance with RY layers and a diagonal H takes part, except
+ *     those whose single energies begin with a state written from the halves
+ *     (GVQE_OPT_MPS_LAYERS), which run as single calls.
  *     GVQE_BATCH_PERSISTENT: one persistent launch whose CTAs claim items
  *     (one 2^tile-bits tile of one pass) in ticket order and wait, with a
  *     bounded spin, for the previous step of the item's instance.  Both are

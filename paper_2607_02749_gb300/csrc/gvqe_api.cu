@@ -149,7 +149,7 @@ struct ProfRec {
 static std::mutex g_prof_mu;
 static bool g_prof_on = false;
 static std::vector<ProfRec> g_prof_pending;
-constexpr int PROF_KINDS = 11;  // PassKind values
+constexpr int PROF_KINDS = 12;  // PassKind values
 static long long g_prof_n[PROF_KINDS] = {};
 static double g_prof_ms[PROF_KINDS] = {};
 static double g_prof_bytes[PROF_KINDS] = {};
@@ -214,6 +214,29 @@ cudaError_t launch_step(int prec, const PassArgs &A, int jobs, int nterm, cudaSt
   }
   return e;
 }
+
+// The contraction of a two-half evaluation: it reads the table in one order, with gradients two.
+struct ProfCut : CutMark {
+  ProfRec rec{};
+  cudaStream_t s;
+  bool on;
+  ProfCut(double bytes, cudaStream_t s) : s(s) {
+    std::lock_guard<std::mutex> lk(g_prof_mu);
+    on = g_prof_on;
+    rec.kind = K_CUT;
+    rec.kernels = 1;
+    rec.bytes = bytes;
+  }
+  void mark(bool begin) override {
+    if (!on) return;
+    cudaEvent_t &e = begin ? rec.a : rec.b;
+    cudaEventCreate(&e);
+    cudaEventRecord(e, s);
+    if (begin) return;
+    std::lock_guard<std::mutex> lk(g_prof_mu);
+    g_prof_pending.push_back(rec);
+  }
+};
 
 static void prof_drain() {
   std::lock_guard<std::mutex> lk(g_prof_mu);
@@ -1181,6 +1204,11 @@ static int cut_state_layers(gvqe_ansatz_s *a) {
   return c.ok ? c.d.reps : 0;
 }
 
+bool gvqe::cut_writes_state(gvqe_ansatz_s *a, int prec, int vectors) {
+  return !prec && std::ldexp((double)vectors, a->n) >= CUT_STATE_AMPS &&
+         mps_layers_for(a->n, a->reps, prec, a->ent, a->gates, a->mps) == 0 && cut_state_layers(a) > 0;
+}
+
 Plan *gvqe::get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state_only, bool allow_mps,
                      bool allow_cut) {
   const int key = prec | (want_grad ? 2 : 0) | (diag ? 4 : 0) | (state_only ? 8 : 0) | (a->gates == 2 ? 16 : 0) |
@@ -1191,7 +1219,7 @@ Plan *gvqe::get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool
   const int mps = allow_mps ? mps_layers_for(a->n, a->reps, prec, a->ent, a->gates, a->mps) : 0;
   Plan pl = build_plan(a->n, a->reps, prec, tb, want_grad, diag, false, state_only, a->ent, a->gates,
                        eff_split(a, prec), eff_xy_tb(a, prec), mps, a->mps_tc >= 0,
-                       allow_cut && mps == 0 && !prec && !want_grad && !state_only ? cut_state_layers(a) : 0);
+                       allow_cut && !want_grad && !state_only ? cut_state_layers(a) : 0);
   pl.tile_bits = tb;
   a->plans[key] = std::move(pl);
   return &a->plans[key];
@@ -1570,7 +1598,8 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
     A.job0.E = E + j0;
     A.job0.grad = grad ? grad + (size_t)j0 * P : nullptr;
     int nl = 0;
-    GV_CUDA(launch_cut(prec, A, grid, grad != nullptr, s, &nl, xy ? &h->xy : nullptr));
+    ProfCut prof(std::ldexp((prec ? 8.0 : 4.0) * (grad ? 2 : 1) * A.njobs, a->n), s);
+    GV_CUDA(launch_cut(prec, A, grid, grad != nullptr, s, &nl, xy ? &h->xy : nullptr, &prof));
     count_launches(nl);
   }
   return GVQE_OK;
@@ -1602,7 +1631,7 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
     return run_cut(a, h, c, a->aux.ptr, mask, batch, E, grad, prec, s);
   }
   GV_TRY(ensure_tables(h, prec, s, cplx));
-  Plan *pl = get_plan(a, prec, grad != nullptr, diag, false, true, std::ldexp((double)batch, a->n) >= CUT_STATE_AMPS);
+  Plan *pl = get_plan(a, prec, grad != nullptr, diag, false, true, !grad && cut_writes_state(a, prec, batch));
   const int P = pl->P;
   // trig table and per-job lowest active layer
   const size_t cs_bytes = (size_t)batch * P * (prec ? 16 : 8);
@@ -2132,7 +2161,7 @@ int gvqe_ansatz_describe(gvqe_ansatz a, int flags, char *buf, int buflen) {
              c->d.half[1].q0, a->n, c->d.D, prec ? "" : " (tensor cores, TF32 split)");
     s += line;
   }
-  if (!prec && get_plan(a, prec, false, true, false, true, true)->cut_layers > 0) {
+  if (cut_writes_state(a, prec, 1 << 23) && !get_cut(a, prec, 1, false)) {
     const CutDesc &d = a->cut[3].d;
     char line[160];
     snprintf(line, sizeof(line), "energies: the state after layer %d written from the halves [0,%d) and [%d,%d), %d terms\n",

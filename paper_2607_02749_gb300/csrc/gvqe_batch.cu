@@ -1020,7 +1020,9 @@ int prepare_tables(gvqe_hamiltonian h, int prec, cudaStream_t s);
 
 namespace {
 // Which instances the persistent kernel takes: RY layers, a diagonal Hamiltonian
-// and n at least the batch tile bits; the others are evaluated by single calls.
+// and n at least the batch tile bits; the others are evaluated by single calls.  So are, under
+// the staged schedule, those whose single energies begin with a state written from the halves
+// (from 23 qubits, which fill the GPU by themselves), so that both give the same bits.
 void classify(gvqe_batch_s *b) {
   b->pidx.clear();
   b->sidx.clear();
@@ -1028,7 +1030,8 @@ void classify(gvqe_batch_s *b) {
     const gvqe_ansatz a = b->a[i];
     const gvqe_hamiltonian h = b->h[i];
     const bool small = b->schedule != GVQE_BATCH_STAGED && a->n < tile_bits_for(b);
-    if (small || !h->gm.empty() || a->gates != 1)
+    const bool writes = b->schedule == GVQE_BATCH_STAGED && !get_cut(a, b->prec, 1, false) && cut_writes_state(a, b->prec, 1);
+    if (small || !h->gm.empty() || a->gates != 1 || writes)
       b->sidx.push_back((int)i);
     else
       b->pidx.push_back((int)i);

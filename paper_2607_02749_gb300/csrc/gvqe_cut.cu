@@ -602,7 +602,7 @@ cudaError_t launch_cut_state(const CutArgs &A0, const CutGrid &g, cudaStream_t s
 }
 
 cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
-                       const CutXyDims *xy) {
+                       const CutXyDims *xy, CutMark *mark) {
   CutArgs A = A0;
   const CutLayout &l = A.job0.lay;
   const int half_blocks = g.half_items ? g.half_blocks : A.njobs * 2 * g.D;
@@ -622,6 +622,7 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
   A.blk0 = l.rb[0] * l.ns[0];
   A.nblk = g.con_items ? g.con_blocks : A.njobs * (A.blk0 + (grad ? l.rb[1] * l.ns[1] : 0));
   A.items = g.con_items;
+  if (mark) mark->mark(true);
   if (prec && cut_by_rows(g.m0, g.D)) {
     auto k = grad ? k_cut_rows64<true> : k_cut_rows64<false>;
     k<<<A.nblk, 256, 0, s>>>(A);
@@ -641,6 +642,7 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
   } else {
     CUT_CHECK(launch_cut_tc(A, K, grad ? CUT_GRAD : CUT_ENERGY, s));
   }
+  if (mark) mark->mark(false);
   *launches += 3;
   if (xy) CUT_CHECK(launch_cut_xy(A, g, *xy, grad, s, launches));
   if (grad) {

@@ -136,8 +136,11 @@ struct CutGrid {
 int cut_class(int prec, int m);
 int cut_k(int D);  // terms of the tensor-core operands
 // The kernels of one evaluation, in order.  `grad`: also the gradients.
+struct CutMark {  // told before and after the contraction (for the event profiler)
+  virtual void mark(bool begin) = 0;
+};
 cudaError_t launch_cut(int prec, const CutArgs &A, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
-                       const CutXyDims *xy = nullptr);
+                       const CutXyDims *xy = nullptr, CutMark *mark = nullptr);
 int cut_xy_dp(int D);  // row length of its matrices
 // The state itself, S of every tile, for circuits that go on after these layers (FP32, RY).
 cudaError_t launch_cut_state(const CutArgs &A, const CutGrid &g, cudaStream_t s, int *launches);

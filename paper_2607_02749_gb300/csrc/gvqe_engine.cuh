@@ -32,6 +32,7 @@ enum PassKind : int {
   K_MPS_GHIGH = 8,  // ... the qubits above the 2^13-amplitude chunk, per chunk and qubit
   K_MPS_GRED = 9,   // ... fixed-order FP64 sums of the per-CTA partials
   K_MPS_GENV = 10,  // ... the qubits inside the chunk, from the summed environments
+  K_CUT = 11,       // (the event profiler) the two-half evaluation's contraction
 };
 
 enum LoadMode : int {

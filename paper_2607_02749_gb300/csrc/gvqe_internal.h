@@ -184,6 +184,8 @@ Plan *get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state
 // on the device.  ensure_cut_tables: what its contraction reads of the Hamiltonian.
 // vectors, grad: of the call.
 gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad);
+// Whether energies of `vectors` vectors begin with a state written from the halves (FP32).
+bool cut_writes_state(gvqe_ansatz_s *a, int prec, int vectors);
 int cut_upload(gvqe_cut_plan *c);
 int ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool grad, cudaStream_t s);
 // The X/Y strings split into parts on the halves (host only); and whether their two-half
