@@ -168,6 +168,10 @@ struct Cfg {
   static constexpr int GBUFS = K <= 32 ? 4 : 2;  // G buffers: two per warp group where they fit
   // stages of the copies: the row-form and column-form halves of B (freed by S and by G), and E
   static constexpr int RS = K <= 32 ? 4 : 2, CS = K <= 32 ? 4 : 2, ES = K <= 32 ? 0 : 3;
+  // Full barriers of S and of E: a barrier's tiles all belong to one group of row warps, which so sees
+  // every phase of it.  With one per stage and an odd number of stages a group skips the other's
+  // phases, and cannot tell "mine is here" from "the one before the other group's is not yet here".
+  static constexpr int SB = BUFS % 2 ? 2 * BUFS : BUFS, EB = ES % 2 ? 2 * ES : ES;
   // tensor-memory columns
   static constexpr int A_HI = 0, A_LO = K, S0 = 2 * K, G0 = S0 + 128 * BUFS;
   static_assert(G0 + GBUFS * K <= 512, "tensor memory");
@@ -182,10 +186,10 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
   constexpr bool GRAD = USE == CUT_GRAD, STATE = USE == CUT_STATE;
   constexpr int HALF = 2 * C::PARTS;  // floats of one half of B: its hi and lo parts
   constexpr int ETILE = 128 * COLS;   // floats of a tile of E (complex: half of them used)
-  constexpr int ES = STATE ? 0 : C::ES;
+  constexpr int ES = STATE ? 0 : C::ES, EB = STATE ? 0 : C::EB;
   extern __shared__ __align__(128) float dyn[];
   float *sR = dyn, *sE = dyn + C::RS * HALF, *sC = sE + ES * ETILE;
-  __shared__ __align__(8) unsigned long long bars[2 * (C::RS + C::CS + ES) + 2 * C::BUFS + C::GBUFS];
+  __shared__ __align__(8) unsigned long long bars[2 * (C::RS + C::CS) + EB + ES + C::SB + C::BUFS + C::GBUFS + 2];
   __shared__ uint32_t tslot;
   __shared__ int bad_s;
   __shared__ double es[2][8];
@@ -214,16 +218,17 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
   const float *bp = reinterpret_cast<const float *>(J.ws + J.lay->pack[1 - h]);
   const float *E = reinterpret_cast<const float *>(h ? J.table_t : J.table);  // in tile order
   const uint32_t bar0 = smem_addr(bars);
-  // per stage a full barrier, then the empty ones
+  // full barriers, then the empty ones
   auto rfull = [&](int s) { return bar0 + 8 * s; };
   auto rempty = [&](int s) { return rfull(C::RS + s); };
   auto cfull = [&](int s) { return rfull(2 * C::RS + s); };
   auto cempty = [&](int s) { return cfull(C::CS + s); };
   auto efull = [&](int s) { return cfull(2 * C::CS + s); };
-  auto eempty = [&](int s) { return efull(ES + s); };
-  auto sbar = [&](int b) { return efull(2 * ES + b); };
-  auto lbar = [&](int b) { return sbar(C::BUFS + b); };
+  auto eempty = [&](int s) { return efull(EB + s); };
+  auto sbar = [&](int b) { return eempty(ES + b); };
+  auto lbar = [&](int b) { return sbar(C::SB + b); };
   auto gbar = [&](int b) { return lbar(C::BUFS + b); };
+  auto last = [&](int i) { return gbar(C::GBUFS + i); };  // an issuer's MMAs, when it has given up
   if (w == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(&tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -233,13 +238,12 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     auto init = [](uint32_t bar, int count) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
     };
-    for (int s = 0; s < 2 * C::RS + 2 * C::CS + ES; ++s) init(bar0 + 8 * s, 1);
+    for (int s = 0; s < 2 * (C::RS + C::CS) + EB; ++s) init(bar0 + 8 * s, 1);
     for (int s = 0; s < ES; ++s) init(eempty(s), 4);
-    for (int b = 0; b < C::BUFS; ++b) {
-      init(sbar(b), 1);
-      init(lbar(b), 4);
-    }
+    for (int b = 0; b < C::SB; ++b) init(sbar(b), 1);
+    for (int b = 0; b < C::BUFS; ++b) init(lbar(b), 4);
     for (int b = 0; b < C::GBUFS; ++b) init(gbar(b), 1);
+    for (int i = 0; i < 2; ++i) init(last(i), 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -315,8 +319,8 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     for (; t < nt; t += 2) {
       const int b = t % C::BUFS, ee = ES ? t % (ES + !ES) : 0;
       if constexpr (ES > 0)
-        if (!wait_warp(efull(ee), (t / ES) & 1, bad)) break;
-      if (!wait_warp(sbar(b), (t / C::BUFS) & 1, bad)) break;
+        if (!wait_warp(efull(t % EB), (t / EB) & 1, bad)) break;
+      if (!wait_warp(sbar(t % C::SB), (t / C::SB) & 1, bad)) break;
       fence_after();
       const uint32_t ts = tw + C::S0 + 128 * b;
       const float4 *et = reinterpret_cast<const float4 *>(sE + ee * ETILE) + (r >> cx);
@@ -456,7 +460,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
           if constexpr (ES > 0) {
             const int e = t % ES;
             if (t >= ES && !wait_bounded(eempty(e), (t / ES - 1) & 1, bad)) break;
-            copy(sE + e * ETILE, Ei + (size_t)t * et, et * 4, efull(e));
+            copy(sE + e * ETILE, Ei + (size_t)t * et, et * 4, efull(t % EB));
           }
         }
         // the last commits have arrived before the CTA leaves
@@ -495,7 +499,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
         mmas<HI, ID, false, K / 8>(d, tu + C::A_HI, bl);
         mmas<HI, ID, false, K / 16>(d, tu + C::A_HI, bh);
         mmas<HI, ID, true, K / 16>(d + 64, tu + C::A_HI + K / 2, bh + K);  // (16 per step of 8)
-        commit(sbar(b));
+        commit(sbar(t % C::SB));
         commit(rempty(s));
       }
     } else if (GRAD && el && w == 10) {
@@ -514,6 +518,11 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
         commit(cempty(s));
       }
     }
+    if (el && *bad && (w == 9 || (GRAD && w == 10))) {  // the MMAs in flight end before the CTA does
+      int none = 0;
+      commit(last(w - 9));
+      wait_bounded(last(w - 9), 0, &none);
+    }
   }
   __syncwarp();
   fence_before();
@@ -525,7 +534,7 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
     int none = 0;
     for (int s = 0; s < C::RS; ++s)
       for (int p = 0; p < 2; ++p) wait_bounded(rfull(s), p, &none);
-    for (int s = 0; s < ES; ++s)
+    for (int s = 0; s < EB; ++s)
       for (int p = 0; p < 2; ++p) wait_bounded(efull(s), p, &none);
     for (int s = 0; GRAD && s < C::CS; ++s)
       for (int p = 0; p < 2; ++p) wait_bounded(cfull(s), p, &none);
