@@ -1278,11 +1278,19 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
   const long long left = budget_left();
   if (left >= 0) have = std::min(have, (size_t)left + a->ws.bytes + ((size_t)512 << 20));
   const size_t budget = have > (size_t)512 << 20 ? have - ((size_t)512 << 20) : 0;
-  if (per_job > budget)
+  if (per_job > budget) {
+    if (pl->cut_layers > 0)  // the passes alone need less
+      return run_plan(a, h, get_plan(a, prec, false, h->gm.empty()), cs_all, mask, batch, E, grad, minlayer, s);
     return fail(GVQE_ENOMEM, "one evaluation needs %.3f GiB of workspace, %.3f GiB available", per_job / 1073741824.0,
                 budget / 1073741824.0);
+  }
   J = (int)std::max<size_t>(1, std::min<size_t>((size_t)J, budget / per_job));
-  const size_t need = per_job * (size_t)J + 512;
+  // the half tables of several launches' vectors at once, where there is room: their circuits are chains
+  // of small launches (26 qubits, 64 terms: 55 us for one vector, 157 for 8)
+  int G = J;
+  if (pl->cut_layers > 0 && J < 8 && batch > J) G = std::min(8 / J, (batch + J - 1) / J) * J;
+  if (per_job * (size_t)J + (size_t)C.ws_stride * (G - J) > budget) G = J;
+  const size_t need = per_job * (size_t)J + (size_t)C.ws_stride * (G - J) + 512;
   GV_TRY(a->ws.reserve(need));
   char *base = (char *)a->ws.ptr;
   double *part = (double *)base;
@@ -1293,8 +1301,8 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
   };
   // closed-form layer tables after the state buffers (a multiple of 64 floats per job)
   float *mps_tab = (float *)(bufs + (size_t)pl->n_bufs * J * S * es);
-  C.job0.ws = (char *)(mps_tab + (size_t)pl->mps_elems * J) + 255;
-  C.job0.ws -= (uintptr_t)C.job0.ws % 256;
+  char *halves = (char *)(mps_tab + (size_t)pl->mps_elems * J) + 255;
+  halves -= (uintptr_t)halves % 256;
   const bool cplx = a->gates == 2;
   const void *table = h ? (cplx ? h->TC[prec].ptr : (prec ? h->T64.ptr : h->T32.ptr)) : nullptr;
   const void *tc = h ? (prec ? (const void *)h->d_tc64 : (const void *)h->d_tc32) : nullptr;
@@ -1302,10 +1310,16 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
   for (int j0 = 0; j0 < batch; j0 += J) {
     const int jobs = std::min(J, batch - j0);
     if (pl->cut_layers > 0) {
-      C.njobs = jobs;
-      C.job0.cs = (const char *)cs64 + (long long)j0 * C.cs_stride;
-      C.state = (float *)buf_ptr(pl->cut_buf);
       int nl = 0;
+      C.job0.cs = (const char *)cs64 + (long long)j0 * C.cs_stride;
+      if (j0 % G == 0) {
+        C.job0.ws = halves;
+        C.njobs = std::min(G, batch - j0);
+        GV_CUDA(launch_cut_halves(C, cgrid, s, &nl));
+      }
+      C.job0.ws = halves + (long long)(j0 % G) * C.ws_stride;
+      C.njobs = jobs;
+      C.state = (float *)buf_ptr(pl->cut_buf);
       GV_CUDA(launch_cut_state(C, cgrid, s, &nl));
       count_launches(nl);
     }
@@ -1605,6 +1619,21 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
   return GVQE_OK;
 }
 
+// Whether a device memory limit leaves room for a two-half evaluation of one vector: many
+// terms on a small register need more than its stored states.
+static bool cut_fits(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const gvqe_cut_plan *c, int prec, bool grad) {
+  const long long left = budget_left();
+  if (left < 0) return true;
+  const bool xy = !h->gm.empty();
+  size_t need = 0;
+  auto want = [&](const DevBuf &b, size_t bytes) { need += bytes > b.bytes ? bytes : 0; };
+  want(a->ws, (size_t)cut_layout(c->d, prec, grad, xy ? &h->xy : nullptr).total);
+  want(h->T64, (size_t)8 << h->n);
+  for (int k = 0; !prec && k < (grad ? 2 : 1); ++k) want(h->TT[c->d.cx][k], (size_t)4 << h->n);
+  if (xy) want(h->XY, 64 * (size_t)(h->xy.U[0] + h->xy.U[1]) + 64 * h->tz.size());
+  return need <= (size_t)left + a->ws.bytes;
+}
+
 static bool is_ham(const void *p) { return p && ((const gvqe_hamiltonian_s *)p)->magic == MAGIC_HAM; }
 static bool is_ansatz(const void *p) { return p && ((const gvqe_ansatz_s *)p)->magic == MAGIC_ANSATZ; }
 
@@ -1621,7 +1650,7 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
   const bool cplx = a->gates == 2;
   const bool diag = cplx ? h->cgm.empty() : h->gm.empty();
   gvqe_cut_plan *c = diag || (!cplx && !prec) ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
-  if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr))) {
+  if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr)) && cut_fits(a, h, c, prec, grad != nullptr)) {
     GV_TRY(ensure_cut_tables(h, prec, c->d, grad != nullptr, s));
     if (!diag) GV_TRY(ensure_cut_xy(h, c->d.half[0].m));
     const long long count = (long long)batch * a->gates * a->n * (a->reps + 1);

@@ -587,18 +587,20 @@ static cudaError_t launch_pack(CutArgs A, const CutGrid &g, int K, cudaStream_t 
   return cudaGetLastError();
 }
 
+cudaError_t launch_cut_halves(const CutArgs &A0, const CutGrid &g, cudaStream_t s, int *launches) {
+  CutArgs A = A0;
+  A.blk0 = g.D;
+  const cudaError_t e = launch_cut_fwd32(A, g, false, s, launches);
+  *launches += 1;
+  return e == cudaSuccess ? launch_pack(A, g, cut_k(g.D), s) : e;
+}
+
 cudaError_t launch_cut_state(const CutArgs &A0, const CutGrid &g, cudaStream_t s, int *launches) {
   CutArgs A = A0;
-  const int K = cut_k(g.D);
-  A.blk0 = g.D;
-  A.items = nullptr;
-  cudaError_t e = launch_cut_fwd32(A, g, false, s, launches);
-  if (e == cudaSuccess) e = launch_pack(A, g, K, s);
-  if (e != cudaSuccess) return e;
   A.blk0 = A.job0.lay.rb[0] * A.job0.lay.ns[0];
   A.nblk = A.njobs * A.blk0;
-  *launches += 2;
-  return launch_cut_tc(A, K, CUT_STATE, s);
+  *launches += 1;
+  return launch_cut_tc(A, cut_k(g.D), CUT_STATE, s);
 }
 
 cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad, cudaStream_t s, int *launches,

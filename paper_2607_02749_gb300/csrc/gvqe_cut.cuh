@@ -142,7 +142,9 @@ struct CutMark {  // told before and after the contraction (for the event profil
 cudaError_t launch_cut(int prec, const CutArgs &A, const CutGrid &g, bool grad, cudaStream_t s, int *launches,
                        const CutXyDims *xy = nullptr, CutMark *mark = nullptr);
 int cut_xy_dp(int D);  // row length of its matrices
-// The state itself, S of every tile, for circuits that go on after these layers (FP32, RY).
+// The state itself, S of every tile, for circuits that go on after these layers (FP32, RY): the
+// half tables of all jobs, then the states of some.
+cudaError_t launch_cut_halves(const CutArgs &A, const CutGrid &g, cudaStream_t s, int *launches);
 cudaError_t launch_cut_state(const CutArgs &A, const CutGrid &g, cudaStream_t s, int *launches);
 cudaError_t launch_cut_xy(const CutArgs &A, const CutGrid &g, const CutXyDims &x, bool grad, cudaStream_t s, int *launches);
 // The diagonal table in the order the FP32 contractions read it, rounded from FP64:

@@ -198,3 +198,33 @@ def test_energies_with_the_leading_layers_from_halves(n, reps, ent, batch, xy):
     a.close()
     b.close()
     h.close()
+
+
+@pytest.mark.parametrize("n,fp64,grad", [(14, True, True), (23, False, False)])
+def test_falls_back_to_stored_states_under_a_memory_limit(n, fp64, grad):
+    # 256 terms need more than the stored states they stand for: with room for those alone, the call runs on them
+    reps, ent = 4, gv.GVQE_ENT_CIRCULAR
+    h = gv.Hamiltonian.from_workload(wl.z_hamiltonian(n, 4 * n, seed=n))
+    t = torch.as_tensor(wl.thetas(n, reps, 1, seed=n), device="cuda")
+
+    def run(mps):
+        a = gv.Ansatz(n, reps, entangler=ent)
+        a.set_mps_layers(mps)
+        out = gv.energy_grad(a, h, t, fp64=fp64) if grad else (gv.energy(a, h, t, fp64=fp64),)
+        torch.cuda.synchronize()
+        used = gv._lib.gvqe_device_memory_in_use()
+        a.close()
+        return [x.cpu() for x in out], used
+
+    run(0)  # (its tables)
+    passes, used = run(-1)
+    free, more = run(0)
+    assert more > used + (1 << 18)
+    try:
+        gv._lib.gvqe_set_device_memory_limit(used + (1 << 18))
+        limited, _ = run(0)
+    finally:
+        gv._lib.gvqe_set_device_memory_limit(0)
+    assert all(torch.equal(x, y) for x, y in zip(limited, passes))
+    assert not all(torch.equal(x, y) for x, y in zip(free, passes))
+    h.close()
