@@ -428,7 +428,9 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
       for (int k = 0; k < K; ++k)
         if (k < D) gout[(size_t)k << mr] = good ? acc[k] + x[k * 128 + r] : __int_as_float(0x7fc00000);
     }
-    if (STATE && !good && w < 4) A.state[(size_t)job * A.state_stride + row0 + r] = __int_as_float(0x7fc00000);
+    // (in this item's own first column: the rows' column 0 is another split's to write)
+    if (STATE && !good && w < 4)
+      A.state[(size_t)job * A.state_stride + ((size_t)t0 << (mr + 6)) + row0 + r] = __int_as_float(0x7fc00000);
     if (h == 0 && tid == 0 && !STATE) {
       double e = 0.0, z = 0.0;
       for (int k = 0; k < 8; ++k) {
