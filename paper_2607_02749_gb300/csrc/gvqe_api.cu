@@ -1619,19 +1619,28 @@ static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, co
   return GVQE_OK;
 }
 
-// Whether a device memory limit leaves room for a two-half evaluation of one vector: many
-// terms on a small register need more than its stored states.
+// Whether a two-half evaluation of one vector has room: under the device memory limit and in
+// the device's free memory (asked only where something is still to be allocated).  Many terms on a
+// small register need more than its stored states, X/Y strings with many parts more than those of
+// any register: 4 D^2 bytes per part, half and run of M.
 static bool cut_fits(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const gvqe_cut_plan *c, int prec, bool grad) {
-  const long long left = budget_left();
-  if (left < 0) return true;
   const bool xy = !h->gm.empty();
-  size_t need = 0;
-  auto want = [&](const DevBuf &b, size_t bytes) { need += bytes > b.bytes ? bytes : 0; };
+  size_t need = 0, freed = 0;
+  auto want = [&](const DevBuf &b, size_t bytes) {
+    if (bytes <= b.bytes) return;
+    need += bytes;
+    freed += b.bytes;  // (a buffer that grows is given back first)
+  };
   want(a->ws, (size_t)cut_layout(c->d, prec, grad, xy ? &h->xy : nullptr).total);
   want(h->T64, (size_t)8 << h->n);
   for (int k = 0; !prec && k < (grad ? 2 : 1); ++k) want(h->TT[c->d.cx][k], (size_t)4 << h->n);
   if (xy) want(h->XY, 64 * (size_t)(h->xy.U[0] + h->xy.U[1]) + 64 * h->tz.size());
-  return need <= (size_t)left + a->ws.bytes;
+  if (need == 0) return true;
+  const long long left = budget_left();
+  if (left >= 0 && need > (size_t)left + freed) return false;
+  size_t freeb = 0, total = 0;
+  if (cudaMemGetInfo(&freeb, &total) != cudaSuccess) return false;
+  return need + ((size_t)64 << 20) <= freeb + freed;  // (64 MiB: the allocations' granularity, and the small buffers)
 }
 
 static bool is_ham(const void *p) { return p && ((const gvqe_hamiltonian_s *)p)->magic == MAGIC_HAM; }
@@ -1645,22 +1654,32 @@ static int check_pair(gvqe_ansatz a, gvqe_hamiltonian h) {
 }
 
 // energies (and optionally adjoint gradients) for a batch
+static int energy_halves(gvqe_ansatz a, gvqe_hamiltonian h, gvqe_cut_plan *c, const double *params, const uint8_t *mask,
+                         int batch, double *E, double *grad, int prec, cudaStream_t s) {
+  GV_TRY(ensure_cut_tables(h, prec, c->d, grad != nullptr, s));
+  if (!h->gm.empty()) GV_TRY(ensure_cut_xy(h, c->d.half[0].m));
+  const long long count = (long long)batch * a->gates * a->n * (a->reps + 1);
+  GV_TRY(a->aux.reserve((size_t)count * 16));
+  GV_CUDA(launch_trig(1, params, count, a->aux.ptr, s));
+  count_launches(1);
+  return run_cut(a, h, c, a->aux.ptr, mask, batch, E, grad, prec, s);
+}
+
 int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, const uint8_t *mask, int batch,
                       double *E, double *grad, int prec, cudaStream_t s) {
   const bool cplx = a->gates == 2;
   const bool diag = cplx ? h->cgm.empty() : h->gm.empty();
   gvqe_cut_plan *c = diag || (!cplx && !prec) ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
-  if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr)) && cut_fits(a, h, c, prec, grad != nullptr)) {
-    GV_TRY(ensure_cut_tables(h, prec, c->d, grad != nullptr, s));
-    if (!diag) GV_TRY(ensure_cut_xy(h, c->d.half[0].m));
-    const long long count = (long long)batch * a->gates * a->n * (a->reps + 1);
-    GV_TRY(a->aux.reserve((size_t)count * 16));
-    GV_CUDA(launch_trig(1, params, count, a->aux.ptr, s));
-    count_launches(1);
-    return run_cut(a, h, c, a->aux.ptr, mask, batch, E, grad, prec, s);
+  bool room = true;
+  if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr))) {
+    const int rc = cut_fits(a, h, c, prec, grad != nullptr) ? energy_halves(a, h, c, params, mask, batch, E, grad, prec, s)
+                                                           : GVQE_ENOMEM;
+    if (rc != GVQE_ENOMEM) return rc;
+    room = false;  // (where the allocation itself failed, nothing was launched that writes a result)
+    g_err.clear();
   }
   GV_TRY(ensure_tables(h, prec, s, cplx));
-  Plan *pl = get_plan(a, prec, grad != nullptr, diag, false, true, !grad && cut_writes_state(a, prec, batch));
+  Plan *pl = get_plan(a, prec, grad != nullptr, diag, false, true, room && !grad && cut_writes_state(a, prec, batch));
   const int P = pl->P;
   // trig table and per-job lowest active layer
   const size_t cs_bytes = (size_t)batch * P * (prec ? 16 : 8);

@@ -401,7 +401,7 @@ long long wait_budget_cycles() {
     if (e_ != cudaSuccess) return fail(GVQE_ECUDA, "%s: %s", #expr, cudaGetErrorString(e_));  \
   } while (0)
 
-int build_grouped(gvqe_batch_s *b, int want_grad);
+int build_grouped(gvqe_batch_s *b, int want_grad, bool halves = true);
 
 int build_schedule(gvqe_batch_s *b, int want_grad) {
   if (b->schedule == GVQE_BATCH_STAGED) return build_grouped(b, want_grad);
@@ -652,8 +652,8 @@ int batch_loop(gvqe_batch_s *b, const double *const *params, const uint8_t *cons
 // and gradient into the caller's buffers).  The branches run side by side.
 // Instances with a two-half evaluation (gvqe_cut.cuh) take one branch per number of
 // terms and class of half circuit instead, whatever their circuits: a PREP launch and the kernels of
-// that evaluation, each over all of the branch's instances, largest first.
-int build_grouped(gvqe_batch_s *b, int want_grad) {
+// that evaluation, each over all of the branch's instances, largest first (halves = false: none do).
+int build_grouped(gvqe_batch_s *b, int want_grad, bool halves) {
   BatchSchedule &sc = b->sched[want_grad];
   const int prec = b->prec;
   const size_t es = prec ? 8 : 4;
@@ -672,7 +672,8 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
   };
   std::map<std::pair<int, int>, CutGroup> cuts;  // (terms, class of the larger half)
   for (int k = 0; k < ni; ++k) {
-    if (const gvqe_cut_plan *c = get_cut(A_of(k), prec, ni, want_grad != 0)) {
+    const gvqe_cut_plan *c = halves ? get_cut(A_of(k), prec, ni, want_grad != 0) : nullptr;
+    if (c) {
       cuts[{cut_k(c->d.D), cut_class(prec, c->d.half[0].m)}].slots.push_back(k);
     } else {
       by_plan[{A_of(k)->n, A_of(k)->reps, A_of(k)->ent, eff_split(A_of(k), prec)}].push_back(k);
@@ -769,6 +770,11 @@ int build_grouped(gvqe_batch_s *b, int want_grad) {
   });
   {
     const int rc = sc.dev.reserve(off);
+    // many terms on a small register need more than its stored states: where they don't fit, those may
+    if (rc == GVQE_ENOMEM && !cuts.empty()) {
+      g_err.clear();
+      return build_grouped(b, want_grad, false);
+    }
     if (rc != GVQE_OK) return rc;
   }
   char *base = (char *)sc.dev.ptr;

@@ -1,0 +1,95 @@
+"""Which evaluation a call takes, and that it has one to take: from the register's halves or
+on stored states, told apart by the launches that the event profiler counts.  Results of the two are
+compared in test_gpu_cut.py; where a call is moved from one to the other, its bits are the other's."""
+import numpy as np
+import pytest
+
+from paper_2607_02749_gb300 import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - CPU containers
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2607_02749_gb300 as gv  # noqa: E402
+from paper_2607_02749_gb300 import _lib  # noqa: E402
+
+K_FWD, K_BWD, K_CUT = 0, 1, 11  # gvqe_engine.cuh, PassKind
+
+
+def _profiled(f, kinds):
+    """f() and how many launches of each kind it made."""
+    _lib.gvqe_profile_reset()
+    _lib.gvqe_profile_enable(True)
+    try:
+        r = f()
+        torch.cuda.synchronize()
+    finally:
+        _lib.gvqe_profile_enable(False)
+    return r, [_lib.gvqe_profile_read(k)["launches"] for k in kinds]
+
+
+def test_xy_strings_run_on_stored_states_where_their_parts_do_not_fit():
+    # 10,000 parts of 64 terms take 3 GB, a state of 24 qubits 64 MiB: with 1.25 GiB left on the device (and no
+    # declared limit) the call runs on stored states (pairwise: no closed-form layers, the same passes as -1)
+    n, reps = 24, 6
+    h = gv.Hamiltonian.from_workload(wl.pauli_hamiltonian(n, 20000, seed=3, xy_fraction=1.0, max_weight=8))
+    t = torch.as_tensor(wl.thetas(n, reps, 1, seed=n), device="cuda")
+
+    def run(mps):
+        a = gv.Ansatz(n, reps, entangler=gv.GVQE_ENT_PAIRWISE)
+        a.set_mps_layers(mps)
+        e, k = _profiled(lambda: gv.energy(a, h, t), (K_CUT, K_FWD))
+        a.close()
+        return e.item(), k
+
+    stored, k = run(-1)
+    assert k[0] == 0 and k[1] > 0
+    halves, k = run(0)
+    assert k == [1, 0]
+    torch.cuda.empty_cache()
+    block = torch.empty(torch.cuda.mem_get_info()[0] - (5 << 28), dtype=torch.uint8, device="cuda")
+    try:
+        short, k = run(0)
+    finally:
+        del block
+        torch.cuda.empty_cache()
+    assert k[0] == 0 and k[1] > 0
+    assert short == stored and halves != stored
+    h.close()
+
+
+@pytest.mark.parametrize("n,reps,ent,fp64", [(14, 3, gv.GVQE_ENT_CIRCULAR, False), (12, 6, gv.GVQE_ENT_LINEAR, True)])
+def test_staged_batch_runs_on_stored_states_where_the_halves_do_not_fit(n, reps, ent, fp64):
+    # 64 terms of a small register need more than its stored states: with room for those alone the batch runs on them
+    count = 12
+    hams = [gv.Hamiltonian.from_workload(wl.z_hamiltonian(n, 4 * n, seed=k)) for k in range(count)]
+    params = [torch.as_tensor(wl.thetas(n, reps, 1, seed=k)[0], device="cuda") for k in range(count)]
+
+    def run(mps):
+        ans = [gv.Ansatz(n, reps, entangler=ent) for _ in range(count)]
+        for a in ans:
+            a.set_mps_layers(mps)
+        b = gv.Batch(ans, hams, fp64=fp64)
+        grads = [torch.empty_like(p) for p in params]
+        e = b.run(params, grads=grads)
+        torch.cuda.synchronize()
+        used = _lib.gvqe_device_memory_in_use()
+        for x in [b] + ans:
+            x.close()
+        return [e.cpu()] + [g.cpu() for g in grads], used
+
+    run(-1)  # (the Hamiltonians' tables)
+    stored, used = run(-1)
+    halves, more = run(0)
+    assert more > used + (1 << 18)
+    try:
+        _lib.gvqe_set_device_memory_limit(used + (1 << 18))
+        limited, _ = run(0)
+    finally:
+        _lib.gvqe_set_device_memory_limit(0)
+    assert all(torch.equal(x, y) for x, y in zip(limited, stored))
+    assert not all(torch.equal(x, y) for x, y in zip(halves, stored))
+    for h in hams:
+        h.close()
