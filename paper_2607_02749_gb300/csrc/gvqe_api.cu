@@ -1666,10 +1666,10 @@ static int energy_halves(gvqe_ansatz a, gvqe_hamiltonian h, gvqe_cut_plan *c, co
 }
 
 int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, const uint8_t *mask, int batch,
-                      double *E, double *grad, int prec, cudaStream_t s) {
+                      double *E, double *grad, int prec, cudaStream_t s, bool halves) {
   const bool cplx = a->gates == 2;
   const bool diag = cplx ? h->cgm.empty() : h->gm.empty();
-  gvqe_cut_plan *c = diag || (!cplx && !prec) ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
+  gvqe_cut_plan *c = halves && (diag || (!cplx && !prec)) ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
   bool room = true;
   if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr))) {
     const int rc = cut_fits(a, h, c, prec, grad != nullptr) ? energy_halves(a, h, c, params, mask, batch, E, grad, prec, s)

@@ -193,7 +193,7 @@ int ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool gr
 void split_xy(const gvqe_hamiltonian_s *h, int m0, CutXyDims *dims, std::vector<uint32_t> *xm, std::vector<uint32_t> *zm,
               std::vector<int> *start, std::vector<int> *other, std::vector<double> *coef, std::vector<int> *gstart);
 // Energies (and adjoint gradients when grad != NULL) of a batch: the body of
-// gvqe_energy / gvqe_energy_grad after their argument checks.
+// gvqe_energy / gvqe_energy_grad after their argument checks.  halves = false: on stored states.
 int energy_impl(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const double *params, const uint8_t *mask, int batch,
-                double *E, double *grad, int prec, cudaStream_t s);
+                double *E, double *grad, int prec, cudaStream_t s, bool halves = true);
 }  // namespace gvqe

@@ -10,7 +10,10 @@
 // distinct plan among tile bits 10 .. the precision's maximum and the two
 // strided layouts runs the requested evaluation (energy, or energy and adjoint
 // gradient) on the caller's parameters, timed with CUDA events on the caller's
-// stream, and the fastest becomes the ansatz's plan.
+// stream, and the fastest becomes the ansatz's plan.  They run on stored states, which
+// are what a plan cuts, also where the evaluation itself would be taken from the register's
+// halves (gvqe_cut.cuh): those calls read no plan and would time the same for every candidate;
+// the plan then serves the calls that keep stored states (readout, a memory limit, other options).
 //
 // Winners are kept in a JSON file, one entry per key (GPU name, n, reps,
 // entangler, gate set, precision, gradient or not, diagonal H or not, batch):
@@ -395,7 +398,7 @@ int gvqe_autotune(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, int b
     a->tuned_split[prec] = sp;
     a->tuned_xy_tb[prec] = xtb;
     a->plans.clear();
-    int r = energy_impl(a, h, params, nullptr, batch, E, G, prec, s);
+    int r = energy_impl(a, h, params, nullptr, batch, E, G, prec, s, false);
     if (r == GVQE_ENOMEM) {
       *per = -1.0;
       return GVQE_OK;
@@ -407,7 +410,7 @@ int gvqe_autotune(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, int b
     int calls = 0;
     while (calls < timed) {
       GT_CUDA(cudaEventRecord(ev.a, s));
-      r = energy_impl(a, h, params, nullptr, batch, E, G, prec, s);
+      r = energy_impl(a, h, params, nullptr, batch, E, G, prec, s, false);
       GT_CUDA(cudaEventRecord(ev.b, s));
       GT_CUDA(cudaEventSynchronize(ev.b));
       if (r != GVQE_OK) return r;

@@ -93,3 +93,20 @@ def test_staged_batch_runs_on_stored_states_where_the_halves_do_not_fit(n, reps,
     assert not all(torch.equal(x, y) for x, y in zip(halves, stored))
     for h in hams:
         h.close()
+
+
+@pytest.mark.parametrize("xy", [0.0, 0.4])
+def test_autotuner_times_the_passes_it_chooses_between(xy):
+    # the evaluation itself takes the halves, which read no tile plan: every candidate must run its passes
+    n, reps = 17, 2
+    h = gv.Hamiltonian.from_workload(wl.pauli_hamiltonian(n, 30, seed=1, xy_fraction=xy))
+    t = torch.as_tensor(wl.thetas(n, reps, 1, seed=2), device="cuda")
+    a = gv.Ansatz(n, reps, entangler=gv.GVQE_ENT_PAIRWISE)
+    rep, k = _profiled(lambda: a.autotune(h, t, cache=None), (K_CUT, K_FWD, K_BWD))
+    candidates = rep.count(" ms") - 1
+    assert candidates >= 2
+    assert k[0] == 0 and k[1] >= 2 * candidates and k[2] >= 2 * candidates, (rep, k)
+    if not xy:
+        assert _profiled(lambda: gv.energy_grad(a, h, t), (K_CUT, K_FWD))[1] == [1, 0]
+    a.close()
+    h.close()
