@@ -69,6 +69,9 @@ extern "C" {
 #define GVQE_ENT_SCA 5
 
 /* options for gvqe_ansatz_set_option */
+/* GVQE_OPT_TILE_BITS and GVQE_OPT_SPLIT_PASSES (and, for strings with X/Y letters, GVQE_OPT_XY_TILE_BITS) say
+ * how passes over a stored 2^n state are cut: set to anything but 0 they also keep the evaluation on stored states
+ * (see GVQE_OPT_MPS_LAYERS).  A plan chosen by gvqe_autotune does not. */
 #define GVQE_OPT_TILE_BITS 1 /* log2 amplitudes per on-chip tile, 10..13 (FP64: 10..12); 0 = auto (13 FP32, 12 FP64) */
 #define GVQE_OPT_GATES 2     /* rotation layer: GVQE_GATES_RY (default) or GVQE_GATES_RY_RZ */
 #define GVQE_OPT_SPLIT_PASSES 3 /* strided-pass bit layout: 0 auto, 1 never split, 2 always split (when a layer
@@ -97,7 +100,8 @@ extern "C" {
                                  qubits, up to eight crossings (2^crossings terms: up to n reps of them
                                  always, more where the call leaves the GPU idle).  FP32 energies with more
                                  crossings begin with the state after the last layer that has at most six, from
-                                 2^23 amplitudes in a call.  Any other value keeps them on stored states.
+                                 2^23 amplitudes in a call.  Any other value keeps them on stored states, and so
+                                 do a tile size or a strided layout set by the options above.
                                  Same results up to rounding in either precision. */
 #define GVQE_OPT_MPS_TENSOR 6 /* closed-form layers at bond dimension 16 (four closed-form layers): 0 = auto
                                  (the writer's product per 2^13-amplitude chunk, 128 x 16 x 64, and the

@@ -1427,6 +1427,7 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
 // operations on 152 SMs against 0.25 M on one).
 gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad) {
   if (a->mps != 0 || (!prec && a->mps_tc != 0) || (a->gates == 2 && prec)) return nullptr;
+  if (a->tile_bits != 0 || a->split != 0) return nullptr;  // (they say how stored states are cut)
   gvqe_cut_plan &c = a->cut[a->gates == 2 ? 2 : prec];
   if (!c.known) {
     c.ok = cut_build(a->n, a->reps, a->ent, prec, a->gates, &c.d);
@@ -1669,7 +1670,8 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
                       double *E, double *grad, int prec, cudaStream_t s, bool halves) {
   const bool cplx = a->gates == 2;
   const bool diag = cplx ? h->cgm.empty() : h->gm.empty();
-  gvqe_cut_plan *c = halves && (diag || (!cplx && !prec)) ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
+  const bool may = halves && (diag || (!cplx && !prec && a->xy_tb == 0));
+  gvqe_cut_plan *c = may ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
   bool room = true;
   if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr))) {
     const int rc = cut_fits(a, h, c, prec, grad != nullptr) ? energy_halves(a, h, c, params, mask, batch, E, grad, prec, s)

@@ -110,3 +110,23 @@ def test_autotuner_times_the_passes_it_chooses_between(xy):
         assert _profiled(lambda: gv.energy_grad(a, h, t), (K_CUT, K_FWD))[1] == [1, 0]
     a.close()
     h.close()
+
+
+@pytest.mark.parametrize("option", ["tile_bits", "split", "xy_tile_bits"])
+@pytest.mark.parametrize("fp64", [False, True])
+def test_tile_options_name_the_passes_that_run(option, fp64):
+    # an option that says how stored states are cut is honoured by the call it is set for
+    n, reps = 18, 2
+    xy = option == "xy_tile_bits"
+    h = gv.Hamiltonian.from_workload(wl.pauli_hamiltonian(n, 40, seed=4, xy_fraction=0.4 if xy else 0.0))
+    t = torch.as_tensor(wl.thetas(n, reps, 1, seed=5), device="cuda")
+    a = gv.Ansatz(n, reps, **({} if xy else {"tile_bits": 11} if option == "tile_bits" else {"split": 2}))
+    if xy:
+        _lib.gvqe_ansatz_set_option(a.handle, _lib.GVQE_OPT_XY_TILE_BITS, 11)
+    _, k = _profiled(lambda: gv.energy_grad(a, h, t, fp64=fp64), (K_CUT, K_FWD, K_BWD))
+    assert k[0] == 0 and k[1] > 0 and k[2] > 0
+    _lib.gvqe_ansatz_set_option(a.handle, {"tile_bits": 1, "split": 3}.get(option, _lib.GVQE_OPT_XY_TILE_BITS), 0)
+    if not (fp64 and xy):
+        assert _profiled(lambda: gv.energy_grad(a, h, t, fp64=fp64), (K_CUT, K_FWD))[1] == [1, 0]
+    a.close()
+    h.close()
