@@ -97,8 +97,9 @@ extern "C" {
                                  state at all: FP32 up to six crossings from 14 qubits, diagonal H or, where
                                  they are the cheaper, X/Y strings; FP32 RY+RZ layers up to five crossings,
                                  14 to 28 qubits, diagonal H; FP64 RY layers, diagonal H, 10 to 28
-                                 qubits, up to eight crossings (2^crossings terms: up to n reps of them
-                                 always, more where the call leaves the GPU idle).  FP32 energies with more
+                                 qubits, up to eight crossings (2^crossings terms) where that is the faster: from 16
+                                 terms on registers of up to 16 qubits that depends on the vectors of the
+                                 call, few of which leave the GPU idle.  FP32 energies with more
                                  crossings begin with the state after the last layer that has at most six, from
                                  2^23 amplitudes in a call.  Any other value keeps them on stored states, and so
                                  do a tile size or a strided layout set by the options above.
@@ -203,9 +204,9 @@ int gvqe_energy_grad(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, co
  * launch); the others (X/Y strings, RY+RZ layers) are evaluated by single
  * gvqe_energy_grad calls on the same stream in the same gvqe_batch_run, after
  * the graph.  Staged results equal single calls bit for bit, but for FP64
- * instances whose halves have more than n reps terms (GVQE_OPT_MPS_LAYERS): those
- * take their halves only where the call leaves the GPU idle, which a single call
- * does and a large batch does not, and the two agree to FP64 rounding.  The persistent
+ * instances of up to 16 qubits whose halves have 16 terms or more
+ * (GVQE_OPT_MPS_LAYERS): those take their halves where that is the faster for the number of vectors
+ * or instances at hand, and the two ways agree to FP64 rounding.  The persistent
  * kernel's 2^12-amplitude tiles fix another summation order, so its results
  * agree with single calls within the precision bounds.
  *   n_inst: >= 1.  ansatze, hams: host arrays of n_inst handles (borrowed: they

@@ -1417,14 +1417,31 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
 }
 
 // ------------------------------------------------- two-half evaluation --
-// A diagonal H and RY layers whose crossing CNOTs leave at most 64 terms: the state is
-// never stored (gvqe_cut.cuh).  GVQE_OPT_MPS_LAYERS other than 0 and GVQE_OPT_MPS_TENSOR = -1
-// name the other evaluations.  FP64 is a matter of FP64 operations: D (energies) or 4 D
-// multiply-adds per amplitude and the half circuits, spread over all SMs, against about 2
-// or 6 per gate and amplitude of the tile passes, on as many SMs as the call has tiles.
-// Up to n reps terms the halves win at any number of vectors; above, only where a call leaves
-// most SMs without a tile (10 qubits, 4 circular repetitions, one vector: 256 terms, 3.5 M
-// operations on 152 SMs against 0.25 M on one).
+// A diagonal H, or X/Y strings in FP32, whose circuit has few enough CNOTs across the cut: the
+// state is never stored (gvqe_cut.cuh).  GVQE_OPT_MPS_LAYERS other than 0, GVQE_OPT_MPS_TENSOR = -1 and
+// the options that say how stored states are cut name the other evaluations.
+
+// FP64, from 17 qubits: up to 64 terms always (64 terms, 17 to 20 qubits, 1 to 16 vectors: 0.35 to
+// 1.0 of the passes' time), 256 never (1.5 to 2.8).  To 16 qubits the times of both in us, fitted to 740
+// calls of 10 to 16 qubits, 2 to 256 terms and 1 to 4096 vectors (nine in ten within 12 to 15
+// percent): launches, then FP64 operations, those of the halves (a small half leaves lanes idle) and of the
+// contraction over all SMs, those of the passes at one 4096-amplitude tile per SM.  So up to 8 terms
+// the halves win at any number of vectors, 16 terms from 12 qubits and 32 from 13; many terms only
+// where a call leaves most SMs without a tile (10 qubits, 4 circular layers: one vector 95 us for 378, 64
+// vectors 1281 for 381).
+static bool cut64_pays(const CutDesc &d, double vectors, bool grad) {
+  if (d.n > 16) return d.D <= 64;
+  const int m = d.half[0].m;
+  const double S = std::ldexp(1.0, d.n), sms = 152.0;
+  const double half = 2.0 * d.D * std::ldexp(m, m) * (d.reps + 1) * (grad ? 6 : 2) * vectors / sms;
+  const double con = (grad ? 4 : 1) * d.D * S * vectors / sms;
+  const double halves = 48 + 1.9 * d.reps + (grad ? 20 + 4.9 * d.reps : 0) +
+                        half * (m == 5 ? 0.93e-3 : m == 6 ? 0.44e-3 : 0.2e-3) + con * 0.31e-3;
+  const double wave = 4.096 * d.n * d.reps * (grad ? 6 : 2), waves = vectors * S / 4096 / sms;
+  const double passes = (grad ? 77 : 66) + wave * (0.343 + 0.334 * std::max(0.0, waves - 1));
+  return halves < 0.95 * passes;
+}
+
 gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad) {
   if (a->mps != 0 || (!prec && a->mps_tc != 0) || (a->gates == 2 && prec)) return nullptr;
   if (a->tile_bits != 0 || a->split != 0) return nullptr;  // (they say how stored states are cut)
@@ -1434,14 +1451,7 @@ gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool
     c.known = true;
   }
   if (!c.ok) return nullptr;
-  if (prec && c.d.D > a->n * a->reps) {
-    const double S = std::ldexp(1.0, a->n), m = c.d.half[0].m;
-    const double half = 2.0 * c.d.D * std::ldexp(m, c.d.half[0].m) * (a->reps + 1) * (grad ? 6 : 2);
-    const double cut = ((grad ? 4 : 1) * c.d.D * S + half) / 152.0;
-    const double sms = std::min(152.0, vectors * std::max(1.0, S / 4096.0));
-    const double tile = (grad ? 6 : 2) * a->n * a->reps * S / sms;
-    if (cut * 1.5 > tile) return nullptr;
-  }
+  if (prec && !cut64_pays(c.d, (double)vectors, grad)) return nullptr;
   return &c;
 }
 

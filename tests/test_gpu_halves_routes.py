@@ -130,3 +130,32 @@ def test_tile_options_name_the_passes_that_run(option, fp64):
         assert _profiled(lambda: gv.energy_grad(a, h, t, fp64=fp64), (K_CUT, K_FWD))[1] == [1, 0]
     a.close()
     h.close()
+
+
+@pytest.mark.parametrize("n,reps,ent,batch,grad,cut", [
+    (12, 6, gv.GVQE_ENT_LINEAR, 128, True, 0),    # 64 terms: 1274 us from the halves, 654 on stored states
+    (12, 6, gv.GVQE_ENT_LINEAR, 1, True, 1),      # 107, 645
+    (10, 2, gv.GVQE_ENT_CIRCULAR, 1024, False, 0),  # 16 terms: 250, 158
+    (10, 2, gv.GVQE_ENT_CIRCULAR, 16, False, 1),  # 52, 119
+    (14, 6, gv.GVQE_ENT_LINEAR, 256, True, 1),    # 64 terms: 4178, 4417
+    (16, 5, gv.GVQE_ENT_LINEAR, 64, False, 1),    # 32 terms: 483, 1380
+    (12, 2, gv.GVQE_ENT_LINEAR, 1024, True, 1),   # 4 terms: 404, 1260
+    (17, 4, gv.GVQE_ENT_CIRCULAR, 1, True, 0)])   # 256 terms: 1326, 650
+def test_fp64_calls_take_the_faster_evaluation(n, reps, ent, batch, grad, cut):
+    # by the terms and the vectors of the call; both within FP64 rounding of each other at either choice
+    h = gv.Hamiltonian.from_workload(wl.z_hamiltonian(n, 5 * n, seed=n))
+    t = torch.as_tensor(wl.thetas(n, reps, batch, seed=n + reps), device="cuda")
+    out = []
+    for mps in (0, -1):
+        a = gv.Ansatz(n, reps, entangler=ent)
+        a.set_mps_layers(mps)
+        f = (lambda: gv.energy_grad(a, h, t, fp64=True)) if grad else (lambda: (gv.energy(a, h, t, fp64=True),))
+        r, k = _profiled(f, (K_CUT, K_FWD))
+        assert (k[0] > 0) == (cut == 1 and mps == 0) and (k[1] > 0) == (k[0] == 0), k
+        out.append([x.cpu().numpy() for x in r])
+        a.close()
+    scale = np.abs(out[1][0]).max()
+    assert np.abs(out[0][0] - out[1][0]).max() <= 1e-12 * scale
+    if grad:
+        assert np.linalg.norm(out[0][1] - out[1][1]) <= 1e-12 * np.linalg.norm(out[1][1])
+    h.close()
