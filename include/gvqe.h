@@ -94,8 +94,9 @@ extern "C" {
                                  batches) of circuits whose CNOTs cross the middle of the register few
                                  times (linear, full, reverse linear, pairwise: once per layer; circular,
                                  SCA: twice) are taken from the circuits of its two halves, with no 2^n
-                                 state at all: FP32 up to six crossings from 14 qubits, diagonal H or, where
-                                 they are the cheaper, X/Y strings; FP32 RY+RZ layers up to five crossings,
+                                 state at all: FP32 up to six crossings from 14 qubits, diagonal H (to 17
+                                 qubits, entanglers without closed-form layers: up to the number of vectors from
+                                 which the passes are the faster) or, where they are the cheaper, X/Y strings; FP32 RY+RZ layers up to five crossings,
                                  14 to 28 qubits, diagonal H; FP64 RY layers, diagonal H, 10 to 28
                                  qubits, up to eight crossings (2^crossings terms) where that is the faster: from 16
                                  terms on registers of up to 16 qubits that depends on the vectors of the
@@ -203,10 +204,10 @@ int gvqe_energy_grad(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, co
  * (gvqe_batch_set_option: staged by default, or one persistent kernel
  * launch); the others (X/Y strings, RY+RZ layers) are evaluated by single
  * gvqe_energy_grad calls on the same stream in the same gvqe_batch_run, after
- * the graph.  Staged results equal single calls bit for bit, but for FP64
- * instances of up to 16 qubits whose halves have 16 terms or more
- * (GVQE_OPT_MPS_LAYERS): those take their halves where that is the faster for the number of vectors
- * or instances at hand, and the two ways agree to FP64 rounding.  The persistent
+ * the graph.  Staged results equal single calls bit for bit, but for small
+ * registers whose evaluation depends on the number of vectors or instances at hand
+ * (GVQE_OPT_MPS_LAYERS: FP64, up to 16 qubits, 16 terms or more; FP32, up to 17 qubits, no closed-form
+ * layers): where a batch and a single call differ in it, they agree to the rounding of the precision.  The persistent
  * kernel's 2^12-amplitude tiles fix another summation order, so its results
  * agree with single calls within the precision bounds.
  *   n_inst: >= 1.  ansatze, hams: host arrays of n_inst handles (borrowed: they

@@ -1442,7 +1442,24 @@ static bool cut64_pays(const CutDesc &d, double vectors, bool grad) {
   return halves < 0.95 * passes;
 }
 
-gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad) {
+// FP32, RY layers: from 18 qubits, and wherever the passes would write closed-form layers (2 to 20
+// times as long), the halves always.  To 17 qubits without those, the same comparison, fitted to 304
+// calls of 14 to 18 qubits, 2 to 64 terms and 1 to 2048 vectors (within 10 percent): per vector the halves cost
+// D circuits whatever n, so that on the smallest registers 64 terms lose from some 50 vectors on (14 qubits,
+// 3 circular layers, energies: one vector 66 us for 90, 128 vectors 154 for 101).
+static bool cut32_pays(const CutDesc &d, double vectors, bool grad) {
+  const double S = std::ldexp(vectors, d.n) * 1e-6, reps = d.reps;
+  const double D = d.D * vectors * std::max(1.0, d.n * std::exp2(0.5 * d.n) / 4096);
+  double halves = 51 + 2.5 * reps + 0.033 * vectors + D * (0.0033 * reps + 0.0026) + 0.85 * S;
+  double passes = 58 + 9.9 * reps + S * (0.3 + 0.166 * d.n * reps);
+  if (grad) {
+    halves += 12 + 2.3 * reps + 0.028 * vectors + D * (0.0024 * reps + 0.0044) + 0.8 * S;
+    passes += 15 + 15.5 * reps + S * (1.5 + 0.337 * d.n * reps);
+  }
+  return halves < 0.95 * passes;
+}
+
+gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad, bool diag) {
   if (a->mps != 0 || (!prec && a->mps_tc != 0) || (a->gates == 2 && prec)) return nullptr;
   if (a->tile_bits != 0 || a->split != 0) return nullptr;  // (they say how stored states are cut)
   gvqe_cut_plan &c = a->cut[a->gates == 2 ? 2 : prec];
@@ -1452,6 +1469,9 @@ gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool
   }
   if (!c.ok) return nullptr;
   if (prec && !cut64_pays(c.d, (double)vectors, grad)) return nullptr;
+  if (!prec && diag && a->gates == 1 && a->n < 18 && !mps_layers_for(a->n, a->reps, 0, a->ent, 1, 0) &&
+      !cut32_pays(c.d, (double)vectors, grad))
+    return nullptr;
   return &c;
 }
 
@@ -1681,7 +1701,7 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
   const bool cplx = a->gates == 2;
   const bool diag = cplx ? h->cgm.empty() : h->gm.empty();
   const bool may = halves && (diag || (!cplx && !prec && a->xy_tb == 0));
-  gvqe_cut_plan *c = may ? get_cut(a, prec, batch, grad != nullptr) : nullptr;
+  gvqe_cut_plan *c = may ? get_cut(a, prec, batch, grad != nullptr, diag) : nullptr;
   bool room = true;
   if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr))) {
     const int rc = cut_fits(a, h, c, prec, grad != nullptr) ? energy_halves(a, h, c, params, mask, batch, E, grad, prec, s)

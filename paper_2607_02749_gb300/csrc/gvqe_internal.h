@@ -180,10 +180,11 @@ inline int eff_xy_tb(const gvqe_ansatz_s *a, int prec) { return a->tuned_xy_tb[p
 Plan *get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state_only = false, bool allow_mps = true,
                bool allow_cut = false);
 // The ansatz's two-half plan for this precision when its options and circuit let it take
-// the place of the tile passes for a diagonal H, else NULL.  cut_upload: its descriptor
+// the place of the tile passes for a diagonal H (diag = false: for X/Y strings, which have a rule of
+// their own), else NULL.  cut_upload: its descriptor
 // on the device.  ensure_cut_tables: what its contraction reads of the Hamiltonian.
 // vectors, grad: of the call.
-gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad);
+gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad, bool diag = true);
 // Whether energies of `vectors` vectors begin with a state written from the halves (FP32).
 bool cut_writes_state(gvqe_ansatz_s *a, int prec, int vectors);
 int cut_upload(gvqe_cut_plan *c);
