@@ -1581,26 +1581,45 @@ static int ensure_cut_xy(gvqe_hamiltonian_s *h, int m0) {
   return GVQE_OK;
 }
 
-// X/Y strings, FP32: the two-half evaluation costs 2 D^2 2^m multiply-adds per part and half
-// (one of the two without gradients), the passes over stored states one signed addition per
-// string and amplitude on top of the tile passes.
-static bool cut_xy_pays(gvqe_hamiltonian_s *h, const CutDesc &d, bool grad) {
+// X/Y strings, FP32: the times of both evaluations in us, fitted to 1580 calls of 14 to 26 qubits,
+// 28 to 4800 strings, 2 to 64 terms and 1 to 16 vectors (nine in ten within 13 percent; the rule then
+// costs 0.4 percent of the better time, its largest miss 21).  Halves: nine launches, M and the diagonal
+// contraction by their multiply-adds, N's FP64 sums with the chain of the part that most strings share, and
+// k_xy_g, whose CTAs take 64 rows through all parts of a half one after the other.  Passes: launches per
+// layer, sweeps, and k_lambda_xy's chain and signed additions per string (14 qubits, 426 strings, 64 terms:
+// 1148 us from the halves, 288 with passes; 28 qubits, 1250 strings, 32 terms: 5 ms, 102).
+static bool cut_xy_pays(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const CutDesc &d, double vectors, bool grad) {
   if (h->xy.U[0] == 0) {  // the sizes alone, once
     CutXyDims dims{};
     std::vector<uint32_t> xm[2], zm[2];
     std::vector<int> start[2], other[2], gstart[2];
     std::vector<double> coef[2];
     split_xy(h, d.half[0].m, &dims, xm, zm, start, other, coef, gstart);
-    h->xy.U[0] = dims.U[0];
+    h->xy_shared = 0;
+    for (int s = 0; s < 2; ++s)
+      for (int u = 0; u < dims.U[s]; ++u) h->xy_shared = std::max(h->xy_shared, start[s][u + 1] - start[s][u]);
     h->xy.U[1] = dims.U[1];
     h->xy.ng[0] = dims.ng[0];
     h->xy.ng[1] = dims.ng[1];
+    h->xy.U[0] = dims.U[0];
   }
-  const double dp = cut_xy_dp(d.D);
-  const double mac = (std::ldexp((double)h->xy.U[0], d.half[0].m) + std::ldexp((double)h->xy.U[1], d.half[1].m)) * dp *
-                     dp * (grad ? 2 : 1);
-  const double half = mac / 1.5e13, tile = std::ldexp((double)h->tz.size(), d.n) * 2e-13;
-  return half < tile + 50e-6;
+  const double reps = d.reps, D = d.D, dp = cut_xy_dp(d.D), dd = dp * dp;
+  const double S = std::ldexp(vectors, d.n) * 1e-6, T = (double)h->tz.size(), U = std::max(h->xy.U[0], h->xy.U[1]);
+  const double mac = (std::ldexp((double)h->xy.U[0], d.half[0].m) + std::ldexp((double)h->xy.U[1], d.half[1].m)) * dd *
+                     vectors * 1e-9;
+  double halves = 99 + 1.9 * reps + 0.32 * D + 1.6 * S + 100 * mac + (7.9e-6 * vectors * T + 0.53e-3 * h->xy_shared) * dd;
+  const double W = std::max(1.0, std::ldexp(vectors, d.n - 21));
+  double passes = 59 + 10.7 * reps + S * (4.2 + 2 * reps) + W * (0.042 * T + 0.49 * h->gm.size()) + 0.059 * S * T;
+  const bool bond16 = mps_layers_for(d.n, a->reps, 0, a->ent, 1, 0) >= 4;
+  if (bond16) passes += 70 + 1.3 * vectors;
+  if (grad) {
+    const double waves = std::max(1.0, std::ldexp(vectors, d.half[0].m - 5) / 304);
+    halves += 39 + 1.8 * reps + 0.27 * D + S * (0.94 + 0.01 * D) + 30 * mac + U * waves * (0.41 + 0.07 * dp) +
+              0.0041 * vectors * D * reps * std::max(1.0, d.n * std::exp2(0.5 * d.n) / 4096);
+    passes += 15 + 16.4 * reps + S * (3.7 + 3.8 * reps);
+    if (bond16) passes += 68 + 13.3 * vectors;
+  }
+  return halves < 0.95 * passes;
 }
 
 static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, const void *cs, const uint8_t *mask,
@@ -1703,7 +1722,7 @@ int gvqe::energy_impl(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, c
   const bool may = halves && (diag || (!cplx && !prec && a->xy_tb == 0));
   gvqe_cut_plan *c = may ? get_cut(a, prec, batch, grad != nullptr, diag) : nullptr;
   bool room = true;
-  if (c && (diag || cut_xy_pays(h, c->d, grad != nullptr))) {
+  if (c && (diag || cut_xy_pays(a, h, c->d, batch, grad != nullptr))) {
     const int rc = cut_fits(a, h, c, prec, grad != nullptr) ? energy_halves(a, h, c, params, mask, batch, E, grad, prec, s)
                                                            : GVQE_ENOMEM;
     if (rc != GVQE_ENOMEM) return rc;

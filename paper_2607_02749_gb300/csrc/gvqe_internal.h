@@ -128,6 +128,7 @@ struct gvqe_hamiltonian_s {
   double abs_sum = 0.0;
   gvqe::DevBuf T64, T32, G;
   gvqe::CutXy xy{};          // the X/Y strings by halves (host copy of the device descriptor), built on first use
+  int xy_shared = 0;         // strings that the most shared part of a half belongs to
   gvqe::DevBuf XY;
   gvqe::DevBuf TT[2][2];  // [complex][contraction]: FP32 tables in the tile order of the two-half contractions
   gvqe::DevBuf TC[2];  // complex path: each table entry twice (re/im), FP32 and FP64

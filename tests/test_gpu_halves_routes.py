@@ -118,7 +118,7 @@ def test_tile_options_name_the_passes_that_run(option, fp64):
     # an option that says how stored states are cut is honoured by the call it is set for
     n, reps = 18, 2
     xy = option == "xy_tile_bits"
-    h = gv.Hamiltonian.from_workload(wl.pauli_hamiltonian(n, 40, seed=4, xy_fraction=0.4 if xy else 0.0))
+    h = gv.Hamiltonian.from_workload(wl.pauli_hamiltonian(n, 700, seed=n, xy_fraction=0.4 if xy else 0.0))
     t = torch.as_tensor(wl.thetas(n, reps, 1, seed=5), device="cuda")
     a = gv.Ansatz(n, reps, **({} if xy else {"tile_bits": 11} if option == "tile_bits" else {"split": 2}))
     if xy:
@@ -127,7 +127,7 @@ def test_tile_options_name_the_passes_that_run(option, fp64):
     assert k[0] == 0 and k[1] > 0 and k[2] > 0
     _lib.gvqe_ansatz_set_option(a.handle, {"tile_bits": 1, "split": 3}.get(option, _lib.GVQE_OPT_XY_TILE_BITS), 0)
     if not (fp64 and xy):
-        assert _profiled(lambda: gv.energy_grad(a, h, t, fp64=fp64), (K_CUT, K_FWD))[1] == [1, 0]
+        assert _profiled(lambda: gv.energy(a, h, t, fp64=fp64), (K_CUT, K_FWD))[1] == [1, 0]
     a.close()
     h.close()
 
@@ -156,9 +156,25 @@ def test_fp32_calls_take_the_faster_evaluation(n, reps, ent, batch, grad, cut):
     _faster(n, reps, ent, batch, grad, cut, False, 1e-6, 5e-6)
 
 
-def _faster(n, reps, ent, batch, grad, cut, fp64, tol_e, tol_g):
+@pytest.mark.parametrize("n,reps,ent,batch,strings,grad,cut", [
+    (14, 3, gv.GVQE_ENT_CIRCULAR, 1, 2800, True, 0),  # 1148 us from the halves, 288 on stored states
+    (16, 2, gv.GVQE_ENT_LINEAR, 1, 80, True, 0),      # 160, 143
+    (18, 6, gv.GVQE_ENT_LINEAR, 8, 3600, False, 0),   # 1334, 463
+    (20, 2, gv.GVQE_ENT_LINEAR, 8, 4000, True, 1),    # 506, 1259
+    (24, 2, gv.GVQE_ENT_CIRCULAR, 1, 960, True, 1),   # 483, 1264
+    (16, 4, gv.GVQE_ENT_LINEAR, 1, 640, False, 1),    # 113, 149
+    # the halves' kernels at every number of terms they are built for (8 to 64)
+    (14, 6, gv.GVQE_ENT_LINEAR, 16, 28, True, 1), (15, 6, gv.GVQE_ENT_FULL, 16, 30, True, 1),
+    (21, 5, gv.GVQE_ENT_LINEAR, 8, 840, True, 1), (22, 1, gv.GVQE_ENT_LINEAR, 4, 880, True, 1),
+    (22, 2, gv.GVQE_ENT_CIRCULAR, 4, 880, True, 1), (23, 3, gv.GVQE_ENT_REVERSE_LINEAR, 4, 920, True, 1),
+    (24, 6, gv.GVQE_ENT_REVERSE_LINEAR, 1, 500, True, 1), (25, 2, gv.GVQE_ENT_PAIRWISE, 2, 2000, True, 1)])
+def test_xy_calls_take_the_faster_evaluation(n, reps, ent, batch, strings, grad, cut):
+    _faster(n, reps, ent, batch, grad, cut, False, 1e-6, 5e-6, strings)
+
+
+def _faster(n, reps, ent, batch, grad, cut, fp64, tol_e, tol_g, xy=0):
     # by the terms and the vectors of the call; both within rounding of each other at either choice (tolerances of test_gpu_cut.py)
-    ham = wl.z_hamiltonian(n, 5 * n, seed=n)
+    ham = wl.pauli_hamiltonian(n, xy, seed=n) if xy else wl.z_hamiltonian(n, 5 * n, seed=n)
     h = gv.Hamiltonian.from_workload(ham)
     t = torch.as_tensor(wl.thetas(n, reps, batch, seed=n + reps), device="cuda")
     out = []
