@@ -14,6 +14,12 @@
 // that x_lo has no sign of its own and the dropped x_lo y_lo averages out; lambda's x_hi is
 // cut (one instruction).  For the same reason G is taken out after every tile (8 full-size
 // steps) and summed on the FP32 pipe.
+// What rounding toward zero takes away has a known mean, since it depends on the last bit's size
+// alone: TRUNC of the partial sum per step, k / N of the whole at step k of N; and of lambda the
+// bits below its 22, on average 0.875 units of its last one.  The sums are scaled back by it once, at
+// their end.  Without that every gradient came out short: by 2.0e-7 (20 qubits, 32 terms) to 4.0e-7
+// (25 qubits, 2 terms) of itself, as much as its other errors; with it 0 to 1.8e-7.  (Rounding lambda's x_hi to nearest
+// instead takes its 7.5e-8 away too, for 1 to 3% of the time.)
 //
 // Both A operands (the rows, and lambda) sit in tensor memory: lambda never touches shared
 // memory, its parts overwrite the two of S in place, and the MMAs read only B from shared
@@ -161,6 +167,11 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+
+constexpr double TRUNC = 0.36 / (1 << 23);  // mean loss of a sum cut to 24 bits: half of its last bit, 0.72 x 2^-23
+constexpr double LOST_LAMBDA = 0.875 * 0.72 / (1 << 23);
+// k / N summed over the steps k = 1 .. N
+constexpr double steps(int n) { return 0.5 * (n + 1); }
 
 template <int K>
 struct Cfg {
@@ -426,7 +437,11 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
       float *gout = reinterpret_cast<float *>(J.ws + J.lay->g[h]) + ((size_t)split * D << mr) + row0 + r;
 #pragma unroll
       for (int k = 0; k < K; ++k)
-        if (k < D) gout[(size_t)k << mr] = good ? acc[k] + x[k * 128 + r] : __int_as_float(0x7fc00000);
+        if (k < D) {
+          constexpr float up = (float)(TRUNC * (steps(COLS / 8) + steps(K / 16)) + LOST_LAMBDA);  // G's, S's and lambda's
+          const float sum = acc[k] + x[k * 128 + r];
+          gout[(size_t)k << mr] = good ? fmaf(sum, up, sum) : __int_as_float(0x7fc00000);
+        }
     }
     // (in this item's own first column: the rows' column 0 is another split's to write)
     if (STATE && !good && w < 4)
@@ -437,6 +452,9 @@ __global__ void __launch_bounds__(NT, 1) k_cut_contract_tc(const __grid_constant
         e += es[0][k];
         z += es[1][k];
       }
+      constexpr double up = 1.0 + 2.0 * TRUNC * steps(K / 16);  // (of E / z none is left: for X/Y strings' energies)
+      e *= up;
+      z *= up;
       double *ep = reinterpret_cast<double *>(J.ws + J.lay->ep) + 2 * idx;
       ep[0] = good ? e : __longlong_as_double(0x7ff8000000000000ll);
       ep[1] = good ? z : 1.0;

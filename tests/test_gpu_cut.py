@@ -228,3 +228,23 @@ def test_falls_back_to_stored_states_under_a_memory_limit(n, fp64, grad):
     assert all(torch.equal(x, y) for x, y in zip(limited, passes))
     assert not all(torch.equal(x, y) for x, y in zip(free, passes))
     h.close()
+
+
+@pytest.mark.parametrize("n,reps,ent", [(16, 1, gv.GVQE_ENT_LINEAR), (18, 2, gv.GVQE_ENT_CIRCULAR), (20, 5, gv.GVQE_ENT_PAIRWISE),
+                                        (19, 6, gv.GVQE_ENT_LINEAR)])
+def test_fp32_gradients_are_not_short(n, reps, ent):
+    # The tensor cores' accumulators round toward zero: 8 full-size steps a tile take 4.5 x 4.3e-8 of it, lambda's
+    # cut 7.5e-8, S's steps 0.4 to 1.1e-7 (against 0.9 to 2.2e-7 of the norm), in all 1.6 to 2.7e-7 of every gradient unless
+    # it is put back.  The other errors have no sign: 7e-8 a vector, 1e-8 in the mean of 64.
+    ham = wl.z_hamiltonian(n, 40 * n, seed=n)
+    th = wl.thetas(n, reps, 64, seed=n + 1).astype(np.float32).astype(np.float64)
+    h = gv.Hamiltonian.from_workload(ham)
+    a = gv.Ansatz(n, reps, entangler=ent)
+    t = torch.as_tensor(th, device="cuda")
+    g = gv.energy_grad(a, h, t)[1].cpu().numpy()
+    g64 = gv.energy_grad(a, h, t, fp64=True)[1].cpu().numpy()
+    short = np.mean(np.sum((g - g64) * g64, axis=1) / np.sum(g64 * g64, axis=1))
+    print(f"n={n} reps={reps} ent={ent}: common factor off by {short:.1e}")
+    assert abs(short) <= 1.2e-7
+    a.close()
+    h.close()
