@@ -1422,7 +1422,7 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
 // the options that say how stored states are cut name the other evaluations.
 
 // FP64, from 17 qubits: up to 64 terms always (64 terms, 17 to 20 qubits, 1 to 16 vectors: 0.35 to
-// 1.0 of the passes' time), 256 never (1.5 to 2.8).  To 16 qubits the times of both in us, fitted to 740
+// 1.0 of the passes' time; 256 took 1.5 to 2.8 and have no plan).  To 16 qubits the times of both in us, fitted to 740
 // calls of 10 to 16 qubits, 2 to 256 terms and 1 to 4096 vectors (nine in ten within 12 to 15
 // percent): launches, then FP64 operations, those of the halves (a small half leaves lanes idle) and of the
 // contraction over all SMs, those of the passes at one 4096-amplitude tile per SM.  So up to 8 terms
@@ -1430,7 +1430,7 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
 // where a call leaves most SMs without a tile (10 qubits, 4 circular layers: one vector 95 us for 378, 64
 // vectors 1281 for 381).
 static bool cut64_pays(const CutDesc &d, double vectors, bool grad) {
-  if (d.n > 16) return d.D <= 64;
+  if (d.n > 16) return true;
   const int m = d.half[0].m;
   const double S = std::ldexp(1.0, d.n), sms = 152.0;
   const double half = 2.0 * d.D * std::ldexp(m, m) * (d.reps + 1) * (grad ? 6 : 2) * vectors / sms;

@@ -139,7 +139,8 @@ bool cut_build(int n, int reps, int ent, int prec, int gates, CutDesc *d) {
       }
     }
     kappa += nb;
-    if (kappa > (prec ? CUT_MAX_PATH64 : CUT_MAX_PATH) - d->cx) return false;  // complex: two real terms per term
+    // FP64 above 64 terms: the row form alone (k_cut_rows64); complex: two real terms per term
+    if (kappa > (prec && h <= 8 ? CUT_MAX_PATH64 : CUT_MAX_PATH) - d->cx) return false;
   }
   d->kappa = kappa;
   d->D = 1 << kappa;
@@ -302,7 +303,8 @@ __global__ void __launch_bounds__(256) k_cut_pack(const __grid_constant__ CutArg
 // amplitude and contraction against 6 (reps + 1) n of the gate-by-gate sweeps.
 constexpr int C64 = CUT_TILE64, C64LD = C64 + 1;
 
-template <bool GRAD, int NA>  // NA: terms per thread of G, 8 NA in all
+constexpr int NA = 8;  // terms per thread of G: 64 in all (more are taken by rows, on registers of up to 16 qubits)
+template <bool GRAD>
 __global__ void __launch_bounds__(256) k_cut_contract64(const __grid_constant__ CutArgs A) {
   extern __shared__ __align__(16) unsigned char cut_smem[];
   int job, h, idx;
@@ -630,16 +632,9 @@ cudaError_t launch_cut(int prec, const CutArgs &A0, const CutGrid &g, bool grad,
     k<<<A.nblk, 256, 0, s>>>(A);
     CUT_CHECK(cudaGetLastError());
   } else if (prec) {
-    const size_t sm = (size_t)8 * C64LD * (2 * g.D + (grad ? C64 : 0));
-    if (g.D <= 64) {
-      auto k = grad ? k_cut_contract64<true, 8> : k_cut_contract64<false, 8>;
-      k<<<A.nblk, 256, sm, s>>>(A);
-    } else {
-      static SmemLimit lim[2];
-      auto k = grad ? k_cut_contract64<true, 32> : k_cut_contract64<false, 32>;
-      CUT_CHECK(lim[grad].set(k, (size_t)8 * C64LD * (2 * 256 + C64)));
-      k<<<A.nblk, 256, sm, s>>>(A);
-    }
+    const size_t sm = (size_t)8 * C64LD * (2 * g.D + (grad ? C64 : 0));  // (64 terms at most: 42 KB)
+    auto k = grad ? k_cut_contract64<true> : k_cut_contract64<false>;
+    k<<<A.nblk, 256, sm, s>>>(A);
     CUT_CHECK(cudaGetLastError());
   } else {
     CUT_CHECK(launch_cut_tc(A, K, grad ? CUT_GRAD : CUT_ENERGY, s));

@@ -20,8 +20,8 @@
 namespace gvqe {
 
 constexpr int CUT_MAX_LAYERS = 6;  // entangler layers, each with at least one crossing CNOT
-constexpr int CUT_MAX_PATH = 6;    // FP32: crossing CNOTs in all, at most 64 terms
-constexpr int CUT_MAX_PATH64 = 8;  // FP64: at most 256
+constexpr int CUT_MAX_PATH = 6;    // crossing CNOTs in all, at most 64 terms
+constexpr int CUT_MAX_PATH64 = 8;  // FP64 to 16 qubits: at most 256
 constexpr int CUT_MAX_M = 15;      // qubits of a half
 
 // One entangler layer as seen by one half: the GF(2)-affine map of its basis indices
