@@ -230,6 +230,18 @@ def test_falls_back_to_stored_states_under_a_memory_limit(n, fp64, grad):
     h.close()
 
 
+def test_uneven_halves_of_the_largest_register():
+    # 29 qubits: a half of 15 (two chunks a state) beside one of 14 in the same launches
+    n, reps = 29, 3
+    ham = wl.z_hamiltonian(n, 300, seed=n)
+    th = wl.thetas(n, reps, 1, seed=n)
+    e0, e, g, d = _run(n, reps, gv.GVQE_ENT_LINEAR, ham, th, False)
+    assert "8 terms" in d
+    _, et, gt, _ = _run(n, reps, gv.GVQE_ENT_LINEAR, ham, th, False, mps=-1)
+    assert abs(e[0] - et[0]) <= 1e-7 * ham.abs_sum() and abs(e0[0] - et[0]) <= 1e-7 * ham.abs_sum()
+    assert np.linalg.norm(g - gt) <= 5e-6 * np.linalg.norm(gt)
+
+
 @pytest.mark.parametrize("n,reps,ent", [(16, 1, gv.GVQE_ENT_LINEAR), (18, 2, gv.GVQE_ENT_CIRCULAR), (20, 5, gv.GVQE_ENT_PAIRWISE),
                                         (19, 6, gv.GVQE_ENT_LINEAR)])
 def test_fp32_gradients_are_not_short(n, reps, ent):
