@@ -1684,7 +1684,7 @@ static bool cut_fits(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const gvqe_cut_pla
   want(a->ws, (size_t)cut_layout(c->d, prec, grad, xy ? &h->xy : nullptr).total);
   want(h->T64, (size_t)8 << h->n);
   for (int k = 0; !prec && k < (grad ? 2 : 1); ++k) want(h->TT[c->d.cx][k], (size_t)4 << h->n);
-  if (xy) want(h->XY, 64 * (size_t)(h->xy.U[0] + h->xy.U[1]) + 64 * h->tz.size());
+  if (xy && !h->XY.ptr) want(h->XY, 64 * (size_t)(h->xy.U[0] + h->xy.U[1]) + 64 * h->tz.size());  // (an upper bound)
   if (need == 0) return true;
   const long long left = budget_left();
   if (left >= 0 && need > (size_t)left + freed) return false;
