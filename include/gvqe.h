@@ -170,7 +170,10 @@ int gvqe_ansatz_set_option(gvqe_ansatz a, int option, int value);
  *   energies: device, batch doubles (written).
  *   flags:    GVQE_FP32 or GVQE_FP64.
  *   stream:   cudaStream_t as void*.
- * The energy reduction always accumulates in FP64.
+ * The energy reduction always accumulates in FP64 (FP32 mode from the register's
+ * halves: sums of 64 products in FP32, those in pairs of floats, then FP64).
+ * Device-side waits inside the tensor-core kernels are bounded; one that runs out (none is expected to) leaves
+ * NaN in the energies and gradients it belongs to.
  * Errors: GVQE_EINVAL (NULL, batch < 1, n of ansatz != n of H), GVQE_ENOMEM, GVQE_ECUDA.
  */
 int gvqe_energy(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, int batch,
@@ -188,7 +191,8 @@ int gvqe_energy(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, int bat
  *             (Eq. 13; this path copies the mask to the host and synchronises
  *             `stream`).
  * Gradient reductions accumulate in FP64 (FP32 mode sums at most one warp's
- * products in FP32 first).
+ * products in FP32 first; from the register's halves, GVQE_OPT_MPS_LAYERS, also
+ * the contraction of each half's rows with the other half's columns).
  * Errors: as gvqe_energy.
  */
 int gvqe_energy_grad(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, const uint8_t *mask,

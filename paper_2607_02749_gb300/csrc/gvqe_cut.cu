@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(256) k_cut_rows64(const __grid_constant__ CutA
 // One warp sums the energy's parts (the FP64 adds of a sum over all warps, by all of them, took
 // longer than the rest), all of them the parameters' path values: a few lanes for a parameter, in
 // an order that depends on the number of terms alone, the parameters next to each other along
-// the lanes as in memory.  8 CTAs for a job where there are few jobs, each a share of the
+// the lanes as in memory.  8 CTAs for a job where there are few jobs (8 x 19 = 152 SMs), each a share of the
 // parameters.  The FP32 contraction also sums psi^2: E and the gradients are divided by
 // that norm, which takes the rounding of cos, sin and of the tensor cores' accumulation out
 // of the results to first order (it is 1 up to that rounding).

@@ -1,11 +1,12 @@
 // gvqe_cut_fwd.cu -- the forward half circuits in FP32 (RY layers) with about 45 bits.
 //
 // Every error of a half's table meets all 2^(n/2) columns of the other half, so the energy
-// does not average it away as it does the rounding of a 2^n state: tables computed in plain
-// FP32 left 2e-6 to 6e-6 of error in E at 20 qubits (rounded-once tables: 2e-7), which is more
-// than a stored state's where E is near zero.  So amplitudes are carried as unevaluated sums
-// hi + lo of two floats, cos and sin too, and the tables are rounded once, into the
-// tensor cores' hi and lo parts.  13 FP32 operations per rotated amplitude, a tenth of
+// does not average it away as it does the rounding of a 2^n state.  In plain FP32 the tables still leave
+// no more than a stored state does (RMS error of E per sum |c|, RY+RZ layers, whose halves are plain FP32, 20 to
+// 25 qubits: 2.7e-10 to 5.7e-10; stored states 6.6e-10 to 1.0e-9); rounded once, a small part of it (RY
+// layers, 14 to 26 qubits: 0.5e-10 to 7e-10; stored states 0.8e-9 to 2.9e-9).  So amplitudes are carried as
+// unevaluated sums hi + lo of two floats, cos and sin too, and the tables are rounded once, into
+// the tensor cores' hi and lo parts.  13 FP32 operations per rotated amplitude, a tenth of
 // the FP64 pipe's time.
 //
 // From 11 qubits a half runs layer by layer, one launch each: a state after layer r depends on

@@ -483,7 +483,7 @@ int gvqe_autotune(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, int b
   a->plans.clear();
   char line[256];
   snprintf(line, sizeof(line),
-           "autotune: measured: tile_bits=%d strided=%s%s %.3f ms per call (batch %d, %s, %s)\n", cands[best].tb,
+           "autotune: measured: tile_bits=%d strided=%s%s %.3f ms per call on stored states (batch %d, %s, %s)\n", cands[best].tb,
            split_name(cands[best].split).c_str(),
            best_xy ? (" xy_tile_bits=" + std::to_string(best_xy)).c_str() : "", best_ms, batch,
            want_grad ? "energy+gradient" : "energy", prec ? "fp64" : "fp32");
