@@ -102,7 +102,7 @@ extern "C" {
                                  terms on registers of up to 16 qubits that depends on the vectors of the
                                  call, few of which leave the GPU idle.  FP32 energies with more
                                  crossings begin with the state after the last layer that has at most six, from
-                                 2^23 amplitudes in a call.  Any other value keeps them on stored states, and so
+                                 18 qubits and 2^23 amplitudes in a call.  Any other value keeps them on stored states, and so
                                  do a tile size or a strided layout set by the options above.
                                  Same results up to rounding in either precision. */
 #define GVQE_OPT_MPS_TENSOR 6 /* closed-form layers at bond dimension 16 (four closed-form layers): 0 = auto

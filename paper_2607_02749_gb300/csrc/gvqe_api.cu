@@ -1191,8 +1191,11 @@ static int ensure_tables(gvqe_hamiltonian_s *h, int prec, cudaStream_t s, bool c
 // written from the halves in one pass, the passes over it begin with the layer after.  Pays once
 // the passes are long against the half circuits' latency, 2^23 amplitudes in a call: 4 circular
 // layers, one vector of 22 qubits 112 us (105 with passes alone), 8 vectors of 20 qubits 115 (140),
-// one vector of 24 qubits 180 (315), of 28 qubits 1.59 ms (4.44).
+// one vector of 24 qubits 180 (315), of 28 qubits 1.59 ms (4.44).  And against their work, 64 terms whatever
+// the register, from 18 qubits: the same 2^25 amplitudes take 1790 us as 14 qubits (493 with passes
+// alone), 694 as 16 (493), 677 as 17 (492), 496 as 18 (494), 423 as 19 (497), 337 as 20 (494).
 constexpr double CUT_STATE_AMPS = 0x1p23;
+constexpr int CUT_STATE_QUBITS = 18;
 static int cut_state_layers(gvqe_ansatz_s *a) {
   if (a->gates != 1 || a->mps != 0 || a->mps_tc != 0) return 0;
   gvqe_cut_plan &c = a->cut[3];
@@ -1205,7 +1208,7 @@ static int cut_state_layers(gvqe_ansatz_s *a) {
 }
 
 bool gvqe::cut_writes_state(gvqe_ansatz_s *a, int prec, int vectors) {
-  return !prec && std::ldexp((double)vectors, a->n) >= CUT_STATE_AMPS &&
+  return !prec && a->n >= CUT_STATE_QUBITS && std::ldexp((double)vectors, a->n) >= CUT_STATE_AMPS &&
          mps_layers_for(a->n, a->reps, prec, a->ent, a->gates, a->mps) == 0 && cut_state_layers(a) > 0;
 }
 

@@ -190,3 +190,19 @@ def _faster(n, reps, ent, batch, grad, cut, fp64, tol_e, tol_g, xy=0):
     if grad:
         assert np.linalg.norm(out[0][1] - out[1][1]) <= tol_g * np.linalg.norm(out[1][1])
     h.close()
+
+
+@pytest.mark.parametrize("n,reps,ent,batch", [(14, 4, gv.GVQE_ENT_CIRCULAR, 512), (17, 7, gv.GVQE_ENT_PAIRWISE, 64)])
+def test_leading_layers_of_small_registers_run_as_passes(n, reps, ent, batch):
+    # 529 us with them from the halves, 184 with passes; 307 and 279: one route and its bits, at every option
+    h = gv.Hamiltonian.from_workload(wl.z_hamiltonian(n, 5 * n, seed=n))
+    t = torch.as_tensor(wl.thetas(n, reps, batch, seed=n), device="cuda")
+    out = []
+    for mps in (0, -1):
+        a = gv.Ansatz(n, reps, entangler=ent)
+        a.set_mps_layers(mps)
+        out.append(gv.energy(a, h, t))
+        assert "state after layer" not in a.describe()
+        a.close()
+    assert torch.equal(*out)
+    h.close()
