@@ -908,6 +908,15 @@ int build_grouped(gvqe_batch_s *b, int want_grad, bool halves) {
   }
   sc.waves = (int)wave_start.size() - 1;
   if (e == cudaSuccess) {
+    // the branches evaluated from the halves fork before the first wave of groups and join after the last
+    cudaEvent_t cfork = nullptr;
+    if (!cuts.empty()) {
+      le = cudaEventCreateWithFlags(&cfork, cudaEventDisableTiming);
+      if (le == cudaSuccess) {
+        evs.push_back(cfork);
+        le = cudaEventRecord(cfork, cap);
+      }
+    }
     cudaEvent_t fork = nullptr;
     size_t first = 0;
     for (size_t gi = 0; gi < groups.size() && le == cudaSuccess; ++gi) {
@@ -960,12 +969,6 @@ int build_grouped(gvqe_batch_s *b, int want_grad, bool halves) {
       first += (size_t)J;
     }
     if (le == cudaSuccess && !cuts.empty()) {
-      cudaEvent_t cfork = nullptr;
-      le = cudaEventCreateWithFlags(&cfork, cudaEventDisableTiming);
-      if (le == cudaSuccess) {
-        evs.push_back(cfork);
-        le = cudaEventRecord(cfork, cap);
-      }
       size_t at = cut_ids;
       for (auto &kv : cuts) {
         if (le != cudaSuccess) break;
