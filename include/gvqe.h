@@ -210,8 +210,7 @@ int gvqe_energy_grad(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, co
  * gvqe_energy_grad calls on the same stream in the same gvqe_batch_run, after
  * the graph.  Staged results equal single calls bit for bit, but for small
  * registers whose evaluation depends on the number of vectors or instances at hand
- * (GVQE_OPT_MPS_LAYERS: FP64, up to 16 qubits, 16 terms or more; FP32, up to 17 qubits, no closed-form
- * layers): where a batch and a single call differ in it, they agree to the rounding of the precision.  The persistent
+ * (GVQE_OPT_MPS_LAYERS: FP64, up to 16 qubits, 16 terms or more; FP32, up to 17 qubits): where a batch and a single call differ in it, they agree to the rounding of the precision.  The persistent
  * kernel's 2^12-amplitude tiles fix another summation order, so its results
  * agree with single calls within the precision bounds.
  *   n_inst: >= 1.  ansatze, hams: host arrays of n_inst handles (borrowed: they

@@ -1462,7 +1462,7 @@ static bool cut32_pays(const CutDesc &d, double vectors, bool grad) {
   return halves < 0.95 * passes;
 }
 
-gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad, bool diag) {
+gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad, bool diag, bool batch) {
   if (a->mps != 0 || (!prec && a->mps_tc != 0) || (a->gates == 2 && prec)) return nullptr;
   if (a->tile_bits != 0 || a->split != 0) return nullptr;  // (they say how stored states are cut)
   gvqe_cut_plan &c = a->cut[a->gates == 2 ? 2 : prec];
@@ -1471,8 +1471,12 @@ gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool
     c.known = true;
   }
   if (!c.ok) return nullptr;
+  // A staged batch runs its passes without closed-form layers, and side by side with those of its other
+  // instances: what counts is the work, not the chain of launches (255 problems of 14 to 16 qubits, 3
+  // circular layers, gradients: 487 us by the chains of 255 vectors of one problem, 429 on stored states).
+  if (batch) vectors *= 8;
   if (prec && !cut64_pays(c.d, (double)vectors, grad)) return nullptr;
-  if (!prec && diag && a->gates == 1 && a->n < 18 && !mps_layers_for(a->n, a->reps, 0, a->ent, 1, 0) &&
+  if (!prec && diag && a->gates == 1 && a->n < 18 && (batch || !mps_layers_for(a->n, a->reps, 0, a->ent, 1, 0)) &&
       !cut32_pays(c.d, (double)vectors, grad))
     return nullptr;
   return &c;

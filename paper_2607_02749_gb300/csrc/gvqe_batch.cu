@@ -672,7 +672,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad, bool halves) {
   };
   std::map<std::pair<int, int>, CutGroup> cuts;  // (terms, class of the larger half)
   for (int k = 0; k < ni; ++k) {
-    const gvqe_cut_plan *c = halves ? get_cut(A_of(k), prec, ni, want_grad != 0) : nullptr;
+    const gvqe_cut_plan *c = halves ? get_cut(A_of(k), prec, ni, want_grad != 0, true, true) : nullptr;
     if (c) {
       cuts[{cut_k(c->d.D), cut_class(prec, c->d.half[0].m)}].slots.push_back(k);
     } else {
@@ -725,7 +725,7 @@ int build_grouped(gvqe_batch_s *b, int want_grad, bool halves) {
     CutGroup &g = kv.second;
     std::stable_sort(g.slots.begin(), g.slots.end(), [&](int x, int y) { return A_of(x)->n > A_of(y)->n; });
     for (int k : g.slots) {
-      const CutDesc &d = get_cut(A_of(k), prec, ni, want_grad != 0)->d;
+      const CutDesc &d = get_cut(A_of(k), prec, ni, want_grad != 0, true, true)->d;
       const int j = (int)g.jobs.size();
       CutJob job{};
       job.lay = cut_layout(d, prec, want_grad != 0);

@@ -184,8 +184,8 @@ Plan *get_plan(gvqe_ansatz_s *a, int prec, bool want_grad, bool diag, bool state
 // the place of the tile passes for a diagonal H (diag = false: for X/Y strings, which have a rule of
 // their own), else NULL.  cut_upload: its descriptor
 // on the device.  ensure_cut_tables: what its contraction reads of the Hamiltonian.
-// vectors, grad: of the call.
-gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad, bool diag = true);
+// vectors, grad: of the call; batch: of a staged batch (its instances).
+gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad, bool diag = true, bool batch = false);
 // Whether energies of `vectors` vectors begin with a state written from the halves (FP32).
 bool cut_writes_state(gvqe_ansatz_s *a, int prec, int vectors);
 int cut_upload(gvqe_cut_plan *c);

@@ -68,3 +68,23 @@ def test_staged_batch_equals_single_calls(shapes, grad):
         a.close()
     for x in [b] + ans + handles[:-2]:
         x.close()
+
+
+@pytest.mark.parametrize("n,reps,ent,count,fp64,halves", [(15, 6, LI, 64, False, False), (14, 3, CI, 64, False, False), (16, 1, LI, 64, False, True),
+                                                          (18, 3, CI, 16, False, True), (10, 2, CI, 256, True, False), (12, 2, LI, 64, True, True)])
+def test_staged_batch_takes_the_faster_evaluation(n, reps, ent, count, fp64, halves):
+    # as gvqe_energy does (test_gpu_halves_routes.py), by the work alone; on stored states the bits of that option
+    handles = [gv.Hamiltonian.from_workload(wl.z_hamiltonian(n, 3 * n, seed=k)) for k in range(count)]
+    p = [torch.as_tensor(t, device="cuda") for t in wl.thetas(n, reps, count, seed=n)]
+    out = []
+    for mps in (0, -1):
+        ans = [gv.Ansatz(n, reps, entangler=ent) for _ in range(count)]
+        for a in ans:
+            a.set_mps_layers(mps)
+        b = gv.Batch(ans, handles, fp64=fp64)
+        out.append(b.run(p).cpu().numpy())
+        for x in [b] + ans:
+            x.close()
+    assert np.array_equal(*out) == (not halves)
+    for x in handles:
+        x.close()

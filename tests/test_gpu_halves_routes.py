@@ -60,10 +60,9 @@ def test_xy_strings_run_on_stored_states_where_their_parts_do_not_fit():
     h.close()
 
 
-@pytest.mark.parametrize("n,reps,ent,fp64", [(14, 3, gv.GVQE_ENT_CIRCULAR, False), (12, 6, gv.GVQE_ENT_LINEAR, True)])
-def test_staged_batch_runs_on_stored_states_where_the_halves_do_not_fit(n, reps, ent, fp64):
-    # 64 terms of a small register need more than its stored states: with room for those alone the batch runs on them
-    count = 12
+@pytest.mark.parametrize("n,reps,ent,count,fp64", [(14, 3, gv.GVQE_ENT_CIRCULAR, 4, False), (10, 4, gv.GVQE_ENT_CIRCULAR, 1, True)])
+def test_staged_batch_runs_on_stored_states_where_the_halves_do_not_fit(n, reps, ent, count, fp64):
+    # 64 or 256 terms of a small register need more than its stored states: with room for those alone the batch runs on them
     hams = [gv.Hamiltonian.from_workload(wl.z_hamiltonian(n, 4 * n, seed=k)) for k in range(count)]
     params = [torch.as_tensor(wl.thetas(n, reps, 1, seed=k)[0], device="cuda") for k in range(count)]
 
