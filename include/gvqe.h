@@ -253,8 +253,8 @@ int gvqe_batch_run(gvqe_batch b, const double *const *params, const uint8_t *con
  *     branch of the graph; the branches run side by side (the instances evaluated
  *     from their halves share their launches instead, see GVQE_OPT_MPS_LAYERS).
  *     Results equal those of single gvqe_energy_grad calls bit for bit (but see
- *     gvqe_batch_create), and every instance with RY layers and a diagonal H takes part, except
- *     those whose single energies begin with a state written from the halves
+ *     gvqe_batch_create), and every instance with RY layers and a diagonal H takes part, except,
+ *     in runs of energies alone, those whose single energies begin with a state written from the halves
  *     (GVQE_OPT_MPS_LAYERS), which run as single calls.
  *     GVQE_BATCH_PERSISTENT: one persistent launch whose CTAs claim items
  *     (one 2^tile-bits tile of one pass) in ticket order and wait, with a

@@ -334,14 +334,13 @@ struct BatchSchedule {
 struct gvqe_batch_s {
   uint32_t magic = 0;
   int prec = 0;
-  bool persistent = false;
   long long wave_bytes = kDefaultWaveBytes;  // GVQE_BATCH_OPT_WAVE_BYTES
   int schedule = GVQE_BATCH_STAGED;         // GVQE_BATCH_OPT_SCHEDULE
   int tile_bits = 12;                        // GVQE_BATCH_OPT_TILE_BITS (FP64: always 12)
   std::string tune_report;
-  // instances of the persistent launch (slot k -> instance pidx[k]) and the
-  // ones evaluated by single calls in the same run (n < 12, X/Y strings, RY+RZ)
-  std::vector<int> pidx, sidx;
+  // of runs without and with gradients: instances of the graph (slot k -> instance pidx[g][k]) and
+  // the ones evaluated by single calls in the same run (n < 12, X/Y strings, RY+RZ; classify)
+  std::vector<int> pidx[2], sidx[2];
   std::vector<gvqe_ansatz> a;
   std::vector<gvqe_hamiltonian> h;
   BatchSchedule sched[2];  // [0] energies only, [1] energies + gradients
@@ -409,9 +408,9 @@ int build_schedule(gvqe_batch_s *b, int want_grad) {
   const int prec = b->prec;
   const int TB = tile_bits_for(b);
   const size_t es = prec ? 8 : 4;
-  const int ni = (int)b->pidx.size();  // slots of the persistent launch
-  auto A_of = [&](int k) { return b->a[b->pidx[k]]; };
-  auto H_of = [&](int k) { return b->h[b->pidx[k]]; };
+  const int ni = (int)b->pidx[want_grad].size();  // slots of the persistent launch
+  auto A_of = [&](int k) { return b->a[b->pidx[want_grad][k]]; };
+  auto H_of = [&](int k) { return b->h[b->pidx[want_grad][k]]; };
   sc.plans.clear();
   sc.plans.reserve(ni);
   for (int i = 0; i < ni; ++i)
@@ -658,9 +657,9 @@ int build_grouped(gvqe_batch_s *b, int want_grad, bool halves) {
   const int prec = b->prec;
   const size_t es = prec ? 8 : 4;
   const int tbg = max_tile_bits(prec);
-  const int ni = (int)b->pidx.size();
-  auto A_of = [&](int k) { return b->a[b->pidx[k]]; };
-  auto H_of = [&](int k) { return b->h[b->pidx[k]]; };
+  const int ni = (int)b->pidx[want_grad].size();
+  auto A_of = [&](int k) { return b->a[b->pidx[want_grad][k]]; };
+  auto H_of = [&](int k) { return b->h[b->pidx[want_grad][k]]; };
   std::map<std::vector<int>, std::vector<int>> by_plan;  // plan key -> slots
   struct CutGroup {
     std::vector<int> slots;
@@ -1028,29 +1027,31 @@ int energy_one(gvqe_ansatz a, gvqe_hamiltonian h, const double *params, const ui
 int prepare_tables(gvqe_hamiltonian h, int prec, cudaStream_t s);
 
 namespace {
-// Which instances the persistent kernel takes: RY layers, a diagonal Hamiltonian
-// and n at least the batch tile bits; the others are evaluated by single calls.  So are, under
-// the staged schedule, those whose single energies begin with a state written from the halves
-// (from 23 qubits, which fill the GPU by themselves), so that both give the same bits.
+// Which instances the graph takes: RY layers, a diagonal Hamiltonian and, under the persistent
+// schedule, n at least the batch tile bits; the others are evaluated by single calls.  So are, under
+// the staged schedule, the energies of those whose single energies begin with a state written from the
+// halves (from 23 qubits, which fill the GPU by themselves), so that both give the same bits.
 void classify(gvqe_batch_s *b) {
-  b->pidx.clear();
-  b->sidx.clear();
-  for (size_t i = 0; i < b->a.size(); ++i) {
-    const gvqe_ansatz a = b->a[i];
-    const gvqe_hamiltonian h = b->h[i];
-    const bool small = b->schedule != GVQE_BATCH_STAGED && a->n < tile_bits_for(b);
-    const bool writes = b->schedule == GVQE_BATCH_STAGED && !get_cut(a, b->prec, 1, false) && cut_writes_state(a, b->prec, 1);
-    if (small || !h->gm.empty() || a->gates != 1 || writes)
-      b->sidx.push_back((int)i);
-    else
-      b->pidx.push_back((int)i);
+  for (int g = 0; g < 2; ++g) {
+    b->pidx[g].clear();
+    b->sidx[g].clear();
+    for (size_t i = 0; i < b->a.size(); ++i) {
+      const gvqe_ansatz a = b->a[i];
+      const gvqe_hamiltonian h = b->h[i];
+      const bool small = b->schedule != GVQE_BATCH_STAGED && a->n < tile_bits_for(b);
+      const bool writes =
+          g == 0 && b->schedule == GVQE_BATCH_STAGED && !get_cut(a, b->prec, 1, false) && cut_writes_state(a, b->prec, 1);
+      if (small || !h->gm.empty() || a->gates != 1 || writes)
+        b->sidx[g].push_back((int)i);
+      else
+        b->pidx[g].push_back((int)i);
+    }
   }
-  b->persistent = !b->pidx.empty();
 }
 
 int batch_loop(gvqe_batch_s *b, const double *const *params, const uint8_t *const *masks, double *energies,
                double *const *grads, cudaStream_t s) {
-  for (int i : b->sidx) {
+  for (int i : b->sidx[grads ? 1 : 0]) {
     const int rc = energy_one(b->a[i], b->h[i], params[i], masks ? masks[i] : nullptr, energies + i,
                               grads ? grads[i] : nullptr, b->prec, s);
     if (rc != GVQE_OK) return rc;
@@ -1143,7 +1144,7 @@ int gvqe_batch_autotune(gvqe_batch b, const double *const *params, const uint8_t
       report[m] = 0;
     }
   };
-  if (!b->persistent) {
+  if (b->pidx[grads ? 1 : 0].empty()) {
     rep = "batch autotune: instance by instance (no persistent schedule to tune)\n";
     put();
     return GVQE_OK;
@@ -1189,11 +1190,11 @@ int gvqe_batch_autotune(gvqe_batch b, const double *const *params, const uint8_t
     char line[200];
     if (cd.sched == GVQE_BATCH_STAGED)
       snprintf(line, sizeof(line), "%sstaged wave=%lldMiB (%d plan groups in %d waves, %zu of %zu instances in it): %.3f ms",
-               sweep.empty() ? "" : "; ", cd.wb >> 20, b->sched[g].groups, b->sched[g].waves, b->pidx.size(),
+               sweep.empty() ? "" : "; ", cd.wb >> 20, b->sched[g].groups, b->sched[g].waves, b->pidx[g].size(),
                b->a.size(), per);
     else
       snprintf(line, sizeof(line), "%spersistent tiles=2^%d wave=%lldMiB (%d waves, %zu of %zu instances in it): %.3f ms",
-               sweep.empty() ? "" : "; ", cd.tb, cd.wb >> 20, b->sched[g].waves, b->pidx.size(), b->a.size(), per);
+               sweep.empty() ? "" : "; ", cd.tb, cd.wb >> 20, b->sched[g].waves, b->pidx[g].size(), b->a.size(), per);
     sweep += line;
     if (best.tb < 0 || per < best_ms) {
       best = cd;
@@ -1238,17 +1239,17 @@ int gvqe_batch_run(gvqe_batch b, const double *const *params, const uint8_t *con
     if (grads && !grads[i]) return fail(GVQE_EINVAL, "grads[%zu] is NULL", i);
   }
   cudaStream_t s = (cudaStream_t)stream;
-  if (!b->persistent) return batch_loop(b, params, masks, energies, grads, s);
   const int g = grads ? 1 : 0;
+  if (b->pidx[g].empty()) return batch_loop(b, params, masks, energies, grads, s);
   BatchSchedule &sc = b->sched[g];
   if (!sc.built) {
     const int rc = build_schedule(b, g);
     if (rc != GVQE_OK) return rc;
   }
-  const size_t np = b->pidx.size();
+  const size_t np = b->pidx[g].size();
   std::vector<BatchIO> io(np);
   for (size_t k = 0; k < np; ++k) {
-    const int i = b->pidx[k];
+    const int i = b->pidx[g][k];
     io[k].params = params[i];
     io[k].mask = masks ? masks[i] : nullptr;
     io[k].grad = grads ? grads[i] : nullptr;
@@ -1263,7 +1264,7 @@ int gvqe_batch_run(gvqe_batch b, const double *const *params, const uint8_t *con
   GB_CUDA(cudaGraphLaunch(sc.exec, s));
   count_launches(1);
   // the instances outside the persistent launch, on the same stream after it
-  if (!b->sidx.empty()) {
+  if (!b->sidx[g].empty()) {
     const int rc = batch_loop(b, params, masks, energies, grads, s);
     if (rc != GVQE_OK) return rc;
   }

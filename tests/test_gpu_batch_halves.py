@@ -15,6 +15,7 @@ if not torch.cuda.is_available():  # pragma: no cover - CPU containers
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
 import paper_2607_02749_gb300 as gv  # noqa: E402
+from paper_2607_02749_gb300 import _lib  # noqa: E402
 
 LI, CI, FU, RV, PW, SC = range(6)
 # (n, reps, entangler): the groups are 16 terms (1 to 16), 32 and 64, by the larger half
@@ -87,4 +88,26 @@ def test_staged_batch_takes_the_faster_evaluation(n, reps, ent, count, fp64, hal
             x.close()
     assert np.array_equal(*out) == (not halves)
     for x in handles:
+        x.close()
+
+
+def test_staged_gradients_of_deep_circuits_stay_in_the_graph():
+    # energies of these begin with a state written from the halves and run as single calls; gradients have no
+    # such state (3193 us as four single calls, 2865 in the graph): one launch, the bits of a single call either way
+    insts = [(23, 4, CI), (14, 2, LI), (23, 5, SC)]
+    handles = [gv.Hamiltonian.from_workload(wl.z_hamiltonian(n, 3 * n, seed=n + r)) for n, r, _ in insts]
+    ans = [gv.Ansatz(n, r, entangler=e) for n, r, e in insts]
+    p = [torch.as_tensor(wl.thetas(n, r, 1, seed=n)[0], device="cuda") for n, r, _ in insts]
+    grads = [torch.empty_like(x) for x in p]
+    b = gv.Batch(ans, handles)
+    b.run(p, grads=grads)
+    before = _lib.gvqe_launch_count()
+    e = b.run(p, grads=grads).cpu()
+    assert _lib.gvqe_launch_count() - before == 1
+    e0 = b.run(p).cpu()
+    for k in range(len(insts)):
+        e1, g1 = gv.energy_grad(ans[k], handles[k], p[k])
+        assert e[k].item() == e1.item() and torch.equal(grads[k], g1[0])
+        assert e0[k].item() == gv.energy(ans[k], handles[k], p[k]).item()
+    for x in [b] + ans + handles:
         x.close()
