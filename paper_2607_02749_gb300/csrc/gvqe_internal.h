@@ -2,6 +2,7 @@
 #pragma once
 #include <cstdint>
 #include <map>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -100,6 +101,14 @@ std::string describe_plan(const Plan &pl);
 // profiler when it is on.
 cudaError_t launch_step(int prec, const PassArgs &A, int jobs, int nterm, cudaStream_t s);
 
+// The X/Y strings of a Hamiltonian as parts on the halves (CutXy), on the host.
+struct CutXySplit : CutXyDims {
+  std::vector<uint32_t> xm[2], zm[2];
+  std::vector<int> start[2], other[2], gstart[2];
+  std::vector<double> coef[2];
+  int shared = 0;  // strings of the part that most share
+};
+
 }  // namespace gvqe
 
 struct gvqe_hamiltonian_s {
@@ -128,6 +137,7 @@ struct gvqe_hamiltonian_s {
   double abs_sum = 0.0;
   gvqe::DevBuf T64, T32, G;
   gvqe::CutXy xy{};          // the X/Y strings by halves (host copy of the device descriptor), built on first use
+  std::unique_ptr<gvqe::CutXySplit> xy_split;  // ... and its arrays until they are on the device
   int xy_shared = 0;         // strings that the most shared part of a half belongs to
   gvqe::DevBuf XY;
   gvqe::DevBuf TT[2][2];  // [complex][contraction]: FP32 tables in the tile order of the two-half contractions
@@ -190,10 +200,6 @@ gvqe_cut_plan *get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad,
 bool cut_writes_state(gvqe_ansatz_s *a, int prec, int vectors);
 int cut_upload(gvqe_cut_plan *c);
 int ensure_cut_tables(gvqe_hamiltonian_s *h, int prec, const CutDesc &d, bool grad, cudaStream_t s);
-// The X/Y strings split into parts on the halves (host only); and whether their two-half
-// evaluation is the cheaper one.
-void split_xy(const gvqe_hamiltonian_s *h, int m0, CutXyDims *dims, std::vector<uint32_t> *xm, std::vector<uint32_t> *zm,
-              std::vector<int> *start, std::vector<int> *other, std::vector<double> *coef, std::vector<int> *gstart);
 // Energies (and adjoint gradients when grad != NULL) of a batch: the body of
 // gvqe_energy / gvqe_energy_grad after their argument checks.  halves = false: on stored states.
 int energy_impl(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const double *params, const uint8_t *mask, int batch,
