@@ -805,7 +805,7 @@ def run_gvqe(args):
             "traffic": None, "kernel": names[dom], "launches": pk["launches"], "avg_launch_ms": pk["ms"] / launches_dom,
             "algorithmic_flops_per_launch": 6.0 * D * 2.0 ** n * evals / launches_dom,
             "tf32_flops_per_launch": 24.0 * max(16, D) * 2.0 ** n * evals / launches_dom,
-            "flops_rule": "TF32: S = A B^T and G = lambda B for either half, 3 products each (hi/lo split), 2 K 2^n "
+            "flops_rule": "TF32: S = A B^T (formed for either half) and G = lambda B, 3 products each (hi/lo split), 2 K 2^n "
                           "operations a product; algorithmic: S once and G for either half in one product each",
             "terms": D, "share_of_step": pk["ms"] / ms,
             "table_GBps": pk["bytes"] / (pk["ms"] / 1000.0) / 1e9,
