@@ -1432,7 +1432,7 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
 // the halves win at any number of vectors, 16 terms from 12 qubits and 32 from 13; many terms only
 // where a call leaves most SMs without a tile (10 qubits, 4 circular layers: one vector 95 us for 378, 64
 // vectors 1281 for 381).
-static bool cut64_pays(const CutDesc &d, double vectors, bool grad) {
+static bool cut64_pays(const CutDesc &d, double vectors, bool grad, double margin) {
   if (d.n > 16) return true;
   const int m = d.half[0].m;
   const double S = std::ldexp(1.0, d.n), sms = 152.0;
@@ -1442,7 +1442,7 @@ static bool cut64_pays(const CutDesc &d, double vectors, bool grad) {
                         half * (m == 5 ? 0.93e-3 : m == 6 ? 0.44e-3 : 0.2e-3) + con * 0.31e-3;
   const double wave = 4.096 * d.n * d.reps * (grad ? 6 : 2), waves = vectors * S / 4096 / sms;
   const double passes = (grad ? 77 : 66) + wave * (0.343 + 0.334 * std::max(0.0, waves - 1));
-  return halves < 0.95 * passes;
+  return halves < margin * passes;
 }
 
 // FP32, RY layers: from 18 qubits, and wherever the passes would write closed-form layers (2 to 20
@@ -1450,7 +1450,7 @@ static bool cut64_pays(const CutDesc &d, double vectors, bool grad) {
 // calls of 14 to 18 qubits, 2 to 64 terms and 1 to 2048 vectors (within 10 percent): per vector the halves cost
 // D circuits whatever n, so that on the smallest registers 64 terms lose from some 50 vectors on (14 qubits,
 // 3 circular layers, energies: one vector 66 us for 90, 128 vectors 154 for 101).
-static bool cut32_pays(const CutDesc &d, double vectors, bool grad) {
+static bool cut32_pays(const CutDesc &d, double vectors, bool grad, double margin) {
   const double S = std::ldexp(vectors, d.n) * 1e-6, reps = d.reps;
   const double D = d.D * vectors * std::max(1.0, d.n * std::exp2(0.5 * d.n) / 4096);
   double halves = 51 + 2.5 * reps + 0.033 * vectors + D * (0.0033 * reps + 0.0026) + 0.85 * S;
@@ -1459,7 +1459,7 @@ static bool cut32_pays(const CutDesc &d, double vectors, bool grad) {
     halves += 12 + 2.3 * reps + 0.028 * vectors + D * (0.0024 * reps + 0.0044) + 0.8 * S;
     passes += 15 + 15.5 * reps + S * (1.5 + 0.337 * d.n * reps);
   }
-  return halves < 0.95 * passes;
+  return halves < margin * passes;
 }
 
 gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool grad, bool diag, bool batch) {
@@ -1472,12 +1472,14 @@ gvqe_cut_plan *gvqe::get_cut(gvqe_ansatz_s *a, int prec, long long vectors, bool
   }
   if (!c.ok) return nullptr;
   // A staged batch runs its passes without closed-form layers, and side by side with those of its other
-  // instances: what counts is the work, not the chain of launches (255 problems of 14 to 16 qubits, 3
-  // circular layers, gradients: 487 us by the chains of 255 vectors of one problem, 429 on stored states).
-  if (batch) vectors *= 8;
-  if (prec && !cut64_pays(c.d, (double)vectors, grad)) return nullptr;
+  // instances, so that their chains of launches cost less than in a call: there the halves have to be clearly
+  // the faster (255 problems of 14 to 16 qubits, 3 circular layers, gradients: 487 us with those that win
+  // as a call, 427 with a margin of a fifth), but not beyond that (the cluster of 256 problems, 600 us; 667
+  // if the smallest, whose times are near equal by work alone, form groups of passes of their own).
+  const double margin = batch ? 0.8 : 0.95;
+  if (prec && !cut64_pays(c.d, (double)vectors, grad, margin)) return nullptr;
   if (!prec && diag && a->gates == 1 && a->n < 18 && (batch || !mps_layers_for(a->n, a->reps, 0, a->ent, 1, 0)) &&
-      !cut32_pays(c.d, (double)vectors, grad))
+      !cut32_pays(c.d, (double)vectors, grad, margin))
     return nullptr;
   return &c;
 }
