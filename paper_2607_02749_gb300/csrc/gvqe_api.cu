@@ -1601,9 +1601,9 @@ static int ensure_cut_xy(gvqe_hamiltonian_s *h, int m0) {
   return GVQE_OK;
 }
 
-// X/Y strings, FP32: the times of both evaluations in us, fitted to 1580 calls of 14 to 26 qubits,
+// X/Y strings, FP32: the times of both evaluations in us, fitted to 2016 calls of 14 to 26 qubits,
 // 28 to 4800 strings, 2 to 64 terms and 1 to 16 vectors (nine in ten within 13 percent; the rule then
-// costs 0.4 percent of the better time, its largest miss 21).  Halves: nine launches, M and the diagonal
+// costs 0.3 percent of the better time on average, above 10 in 12 calls).  Halves: nine launches, M and the diagonal
 // contraction by their multiply-adds, N's FP64 sums with the chain of the part that most strings share, and
 // k_xy_g, whose CTAs take 64 rows through all parts of a half one after the other.  Passes: launches per
 // layer, sweeps, and k_lambda_xy's chain and signed additions per string (14 qubits, 426 strings, 64 terms:
@@ -1618,7 +1618,9 @@ static bool cut_xy_pays(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const CutDesc &
   const double S = std::ldexp(vectors, d.n) * 1e-6, T = (double)h->tz.size(), U = std::max(h->xy.U[0], h->xy.U[1]);
   const double mac = (std::ldexp((double)h->xy.U[0], d.half[0].m) + std::ldexp((double)h->xy.U[1], d.half[1].m)) * dd *
                      vectors * 1e-9;
-  double halves = 99 + 1.9 * reps + 0.32 * D + 1.6 * S + 100 * mac + (7.9e-6 * vectors * T + 0.53e-3 * h->xy_shared) * dd;
+  // (from 21 qubits the half circuits are a launch per layer)
+  const double launches = d.n < 21 ? 1.9 * reps : 7 + 7 * reps + (grad ? 17 : 0);
+  double halves = 99 + launches + 0.32 * D + 1.4 * S + 98 * mac + (7.9e-6 * vectors * T + 0.53e-3 * h->xy_shared) * dd;
   const double W = std::max(1.0, std::ldexp(vectors, d.n - 21));
   double passes = 59 + 10.7 * reps + S * (4.2 + 2 * reps) + W * (0.042 * T + 0.49 * h->gm.size()) + 0.059 * S * T;
   const bool bond16 = mps_layers_for(d.n, a->reps, 0, a->ent, 1, 0) >= 4;
@@ -1630,7 +1632,7 @@ static bool cut_xy_pays(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, const CutDesc &
     passes += 15 + 16.4 * reps + S * (3.7 + 3.8 * reps);
     if (bond16) passes += 68 + 13.3 * vectors;
   }
-  return halves < 0.95 * passes;
+  return halves < 0.98 * passes;
 }
 
 static int run_cut(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, gvqe_cut_plan *c, const void *cs, const uint8_t *mask,
