@@ -1275,25 +1275,31 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
   }
   const size_t per_job = (size_t)pl->n_bufs * S * es + (size_t)pl->part_stride * 8 + (size_t)pl->mps_elems * 4 +
                          (size_t)C.ws_stride;
-  size_t freeb = 0, total = 0;
-  GV_CUDA(cudaMemGetInfo(&freeb, &total));
-  size_t have = freeb + a->ws.bytes;
-  const long long left = budget_left();
-  if (left >= 0) have = std::min(have, (size_t)left + a->ws.bytes + ((size_t)512 << 20));
-  const size_t budget = have > (size_t)512 << 20 ? have - ((size_t)512 << 20) : 0;
-  if (per_job > budget) {
-    if (pl->cut_layers > 0)  // the passes alone need less
-      return run_plan(a, h, get_plan(a, prec, false, h->gm.empty()), cs_all, mask, batch, E, grad, minlayer, s);
-    return fail(GVQE_ENOMEM, "one evaluation needs %.3f GiB of workspace, %.3f GiB available", per_job / 1073741824.0,
-                budget / 1073741824.0);
-  }
-  J = (int)std::max<size_t>(1, std::min<size_t>((size_t)J, budget / per_job));
   // the half tables of several launches' vectors at once, where there is room: their circuits are chains
   // of small launches (26 qubits, 64 terms: 55 us for one vector, 157 for 8)
-  int G = J;
-  if (pl->cut_layers > 0 && J < 8 && batch > J) G = std::min(8 / J, (batch + J - 1) / J) * J;
-  if (per_job * (size_t)J + (size_t)C.ws_stride * (G - J) > budget) G = J;
-  const size_t need = per_job * (size_t)J + (size_t)C.ws_stride * (G - J) + 512;
+  auto group = [&](int J) { return pl->cut_layers > 0 && J < 8 && batch > J ? std::min(8 / J, (batch + J - 1) / J) * J : J; };
+  auto bytes = [&](int J, int G) { return per_job * (size_t)J + (size_t)C.ws_stride * (G - J) + 512; };
+  int G = group(J);
+  // the workspace of an earlier call serves a call of its size: the device is asked for its free memory (22 us)
+  // only where it has to grow
+  if (bytes(J, G) > a->ws.bytes) {
+    size_t freeb = 0, total = 0;
+    GV_CUDA(cudaMemGetInfo(&freeb, &total));
+    size_t have = freeb + a->ws.bytes;
+    const long long left = budget_left();
+    if (left >= 0) have = std::min(have, (size_t)left + a->ws.bytes + ((size_t)512 << 20));
+    const size_t budget = have > (size_t)512 << 20 ? have - ((size_t)512 << 20) : 0;
+    if (per_job > budget) {
+      if (pl->cut_layers > 0)  // the passes alone need less
+        return run_plan(a, h, get_plan(a, prec, false, h->gm.empty()), cs_all, mask, batch, E, grad, minlayer, s);
+      return fail(GVQE_ENOMEM, "one evaluation needs %.3f GiB of workspace, %.3f GiB available", per_job / 1073741824.0,
+                  budget / 1073741824.0);
+    }
+    J = (int)std::max<size_t>(1, std::min<size_t>((size_t)J, budget / per_job));
+    G = group(J);
+    if (bytes(J, G) - 512 > budget) G = J;
+  }
+  const size_t need = bytes(J, G);
   GV_TRY(a->ws.reserve(need));
   char *base = (char *)a->ws.ptr;
   double *part = (double *)base;
@@ -1432,6 +1438,8 @@ static int run_plan(gvqe_ansatz_s *a, gvqe_hamiltonian_s *h, Plan *pl, const voi
 // the halves win at any number of vectors, 16 terms from 12 qubits and 32 from 13; many terms only
 // where a call leaves most SMs without a tile (10 qubits, 4 circular layers: one vector 95 us for 378, 64
 // vectors 1281 for 381).
+// (The passes' times of this fit and the two below hold a memory query, 22 us, that run_plan makes only where its
+// workspace grows since; the halves keep the calls between.)
 static bool cut64_pays(const CutDesc &d, double vectors, bool grad, double margin) {
   if (d.n > 16) return true;
   const int m = d.half[0].m;
